@@ -1,12 +1,14 @@
-"""ctypes binding of libclv.so: argument marshalling only.
+"""Python binding of libclv.so: argument marshalling only.
 
 Every function has the name of the C entry point it forwards to (see ``include/clv.h``) and takes
 torch CUDA tensors; all arithmetic of the verify step runs in the library's kernels.  There is no
-CPU fallback: if the shared library has not been built, :func:`lib` raises.
+CPU fallback: if the shared library has not been built, :func:`lib` raises.  The calls of a decode
+loop are marshalled natively (``csrc/py_calls.c``), the set-up calls through ctypes.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional
 
@@ -132,6 +134,26 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_calls = None
+
+
+def _load_calls():
+    """The CPython module through which the calls of a decode loop go (``csrc/py_calls.c``)."""
+    global _calls
+    if _calls is None:
+        lib()                # the one missing-library error, and the same loaded file
+        path = os.path.join(_PKG, "_calls.so")
+        if not os.path.exists(path):
+            raise RuntimeError("_calls.so is missing at %s: build it with `python -m paper_2408_00264_b200.build`" % path)
+        torch.cuda.init()    # so that a device and a current stream exist
+        spec = importlib.util.spec_from_file_location("_calls", path)
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        m.init(torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+        _calls = m
+    return _calls
+
+
 def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
@@ -185,22 +207,16 @@ def new_workspace(shape: ClvShape, cache: Optional[ClvKvCache], max_ctx_len: int
 
 def clv_tree_attn(shape, cache, q, k_tree, v_tree, parent, ctx_len, max_ctx_len, softmax_scale,
                   out, lse, status, workspace, stream=None, check=True) -> int:
-    code = lib().clv_tree_attn(_ref(shape), _ref(cache), _ptr(q), _ptr(k_tree), _ptr(v_tree),
-                               _ptr(parent), _ptr(ctx_len), int(max_ctx_len), float(softmax_scale),
-                               _ptr(out), _ptr(lse), _ptr(status), _ptr(workspace),
-                               0 if workspace is None else workspace.numel() * workspace.element_size(),
-                               _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).tree_attn(shape, cache, q, k_tree, v_tree, parent, ctx_len, max_ctx_len,
+                                               softmax_scale, out, lse, status, workspace, stream)
+    if code and check:
         _check(code, "clv_tree_attn")
     return code
 
 
 def clv_accept_argmax(shape, logits, ld, argmax_ids, workspace, stream=None, check=True) -> int:
-    code = lib().clv_accept_argmax(_ref(shape), _ptr(logits), int(ld), _ptr(argmax_ids),
-                                   _ptr(workspace),
-                                   0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                   _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).accept_argmax(shape, logits, ld, argmax_ids, workspace, stream)
+    if code and check:
         _check(code, "clv_accept_argmax")
     return code
 
@@ -208,9 +224,8 @@ def clv_accept_argmax(shape, logits, ld, argmax_ids, workspace, stream=None, che
 def clv_accept_argmax_noalloc(shape, logits, ld, argmax_ids, stream=None, check=True) -> int:
     """clv_accept_argmax for callers that may not allocate device memory: no workspace argument,
     the scratch is a fixed array inside the library (limits and sharing rules in clv.h)."""
-    code = lib().clv_accept_argmax_noalloc(_ref(shape), _ptr(logits), int(ld), _ptr(argmax_ids),
-                                           _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).accept_argmax_noalloc(shape, logits, ld, argmax_ids, stream)
+    if code and check:
         _check(code, "clv_accept_argmax_noalloc")
     return code
 
@@ -218,12 +233,10 @@ def clv_accept_argmax_noalloc(shape, logits, ld, argmax_ids, stream=None, check=
 def clv_accept_walk_commit(shape, cache, parent, tokens, argmax_ids, k_tree, v_tree, ctx_len, accept_len,
                            accept_idx, next_token, ctx_len_out, walk_status, commit_status, stream=None,
                            check=True) -> int:
-    code = lib().clv_accept_walk_commit(_ref(shape), _ref(cache), _ptr(parent), _ptr(tokens),
-                                        _ptr(argmax_ids), _ptr(k_tree), _ptr(v_tree), _ptr(ctx_len),
-                                        _ptr(accept_len), _ptr(accept_idx), _ptr(next_token),
-                                        _ptr(ctx_len_out), _ptr(walk_status), _ptr(commit_status),
-                                        _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).accept_walk_commit(shape, cache, parent, tokens, argmax_ids, k_tree, v_tree,
+                                                        ctx_len, accept_len, accept_idx, next_token, ctx_len_out,
+                                                        walk_status, commit_status, stream)
+    if code and check:
         _check(code, "clv_accept_walk_commit")
     return code
 
@@ -231,11 +244,9 @@ def clv_accept_walk_commit(shape, cache, parent, tokens, argmax_ids, k_tree, v_t
 def clv_accept_sample(shape, logits, ld, parent, tokens, uniforms, temperature, accept_len, accept_idx,
                       next_token, status, workspace, stream=None, check=True) -> int:
     """uniforms: float32 [B, N + 1] in [0, 1); temperature: python float > 0."""
-    code = lib().clv_accept_sample(_ref(shape), _ptr(logits), int(ld), _ptr(parent), _ptr(tokens),
-                                   _ptr(uniforms), float(temperature), _ptr(accept_len), _ptr(accept_idx),
-                                   _ptr(next_token), _ptr(status), _ptr(workspace),
-                                   workspace.numel() * workspace.element_size(), _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).accept_sample(shape, logits, ld, parent, tokens, uniforms, temperature, accept_len,
+                                                   accept_idx, next_token, status, workspace, stream)
+    if code and check:
         _check(code, "clv_accept_sample")
     return code
 
@@ -243,18 +254,16 @@ def clv_accept_sample(shape, logits, ld, parent, tokens, uniforms, temperature, 
 def clv_tree_to_intervals(parent, tin, tout, status, stream=None, check=True) -> int:
     """parent, tin, tout: int32 [B, N]; status int32 [B]."""
     B, N = parent.shape
-    code = lib().clv_tree_to_intervals(int(B), int(N), _ptr(parent), _ptr(tin), _ptr(tout), _ptr(status),
-                                       _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).tree_to_intervals(B, N, parent, tin, tout, status, stream)
+    if code and check:
         _check(code, "clv_tree_to_intervals")
     return code
 
 
 def clv_tree_from_intervals(tin, tout, parent, status, stream=None, check=True) -> int:
     B, N = tin.shape
-    code = lib().clv_tree_from_intervals(int(B), int(N), _ptr(tin), _ptr(tout), _ptr(parent), _ptr(status),
-                                         _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).tree_from_intervals(B, N, tin, tout, parent, status, stream)
+    if code and check:
         _check(code, "clv_tree_from_intervals")
     return code
 
@@ -262,11 +271,10 @@ def clv_tree_from_intervals(tin, tout, parent, status, stream=None, check=True) 
 def clv_kv_commit_layers(shape, cache, n_layers, cache_layer_stride, k_tree, v_tree, tree_layer_stride,
                          accept_idx, accept_len, ctx_len, ctx_len_out, status, stream=None, check=True) -> int:
     """cache: descriptor of layer 0; the strides are in bf16 elements between consecutive layers."""
-    code = lib().clv_kv_commit_layers(_ref(shape), _ref(cache), int(n_layers), int(cache_layer_stride),
-                                      _ptr(k_tree), _ptr(v_tree), int(tree_layer_stride), _ptr(accept_idx),
-                                      _ptr(accept_len), _ptr(ctx_len), _ptr(ctx_len_out), _ptr(status),
-                                      _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).kv_commit_layers(shape, cache, n_layers, cache_layer_stride, k_tree, v_tree,
+                                                      tree_layer_stride, accept_idx, accept_len, ctx_len, ctx_len_out,
+                                                      status, stream)
+    if code and check:
         _check(code, "clv_kv_commit_layers")
     return code
 
@@ -284,10 +292,9 @@ def make_draft_head(weights: dict, rms_eps: float = 1e-5) -> ClvDraftHead:
 def clv_draft_head_step(head, h, e, k_top, hidden_out, top_ids, top_logits, status, workspace, stream=None,
                         check=True) -> int:
     """h, e, hidden_out: bf16 [rows, hidden]; top_ids int32 / top_logits float32 [rows, k_top]; status int32 [5]."""
-    code = lib().clv_draft_head_step(_ref(head), int(h.shape[0]), _ptr(h), _ptr(e), int(k_top), _ptr(hidden_out),
-                                     _ptr(top_ids), _ptr(top_logits), _ptr(status), _ptr(workspace),
-                                     workspace.numel() * workspace.element_size(), _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).draft_head_step(head, h.shape[0], h, e, k_top, hidden_out, top_ids, top_logits,
+                                                     status, workspace, stream)
+    if code and check:
         _check(code, "clv_draft_head_step")
     return code
 
@@ -304,10 +311,9 @@ def clv_build_token_tree(root_token, cand, cand_len, tokens, parent, n_nodes, no
     """cand int32 [B, n_cand, max_len], cand_len [B, n_cand], root_token [B]; outputs tokens and
     parent [B, node_cap], n_nodes [B], node_of [B, n_cand, max_len], status [B] (all int32)."""
     B, C, D = cand.shape
-    code = lib().clv_build_token_tree(int(B), int(C), int(D), int(tokens.shape[1]), _ptr(root_token),
-                                      _ptr(cand), _ptr(cand_len), _ptr(tokens), _ptr(parent),
-                                      _ptr(n_nodes), _ptr(node_of), _ptr(status), _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).build_token_tree(B, C, D, tokens.shape[1], root_token, cand, cand_len, tokens,
+                                                      parent, n_nodes, node_of, status, stream)
+    if code and check:
         _check(code, "clv_build_token_tree")
     return code
 
@@ -316,33 +322,27 @@ def clv_lm_head_argmax(hidden, weight, argmax_ids, status, workspace, stream=Non
     """hidden bf16 [rows, hidden_dim], weight bf16 [vocab, hidden_dim] (row strides taken from the
     tensors), argmax_ids int32 [rows], status int32 [1]."""
     rows, hidden_dim = hidden.shape
-    vocab = weight.shape[0]
-    code = lib().clv_lm_head_argmax(_ptr(hidden), int(hidden.stride(0)), _ptr(weight),
-                                    int(weight.stride(0)), int(rows), int(hidden_dim), int(vocab),
-                                    _ptr(argmax_ids), _ptr(status), _ptr(workspace),
-                                    0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                    _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).lm_head_argmax(hidden, hidden.stride(0), weight, weight.stride(0), rows, hidden_dim,
+                                                    weight.shape[0], argmax_ids, status, workspace, stream)
+    if code and check:
         _check(code, "clv_lm_head_argmax")
     return code
 
 
 def clv_accept_walk(shape, parent, tokens, argmax_ids, accept_len, accept_idx, next_token, status,
                     stream=None, check=True) -> int:
-    code = lib().clv_accept_walk(_ref(shape), _ptr(parent), _ptr(tokens), _ptr(argmax_ids),
-                                 _ptr(accept_len), _ptr(accept_idx), _ptr(next_token), _ptr(status),
-                                 _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).accept_walk(shape, parent, tokens, argmax_ids, accept_len, accept_idx, next_token,
+                                                 status, stream)
+    if code and check:
         _check(code, "clv_accept_walk")
     return code
 
 
 def clv_kv_commit(shape, cache, k_tree, v_tree, accept_idx, accept_len, ctx_len, ctx_len_out, status,
                   stream=None, check=True) -> int:
-    code = lib().clv_kv_commit(_ref(shape), _ref(cache), _ptr(k_tree), _ptr(v_tree),
-                               _ptr(accept_idx), _ptr(accept_len), _ptr(ctx_len), _ptr(ctx_len_out),
-                               _ptr(status), _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).kv_commit(shape, cache, k_tree, v_tree, accept_idx, accept_len, ctx_len, ctx_len_out,
+                                               status, stream)
+    if code and check:
         _check(code, "clv_kv_commit")
     return code
 
@@ -354,13 +354,9 @@ def clv_staging_bytes(shape: ClvShape, ld: int) -> int:
 def clv_verify_step_host(shape, cache, host_in: ClvHostInputs, host_out: ClvHostOutputs, ctx_len,
                          max_ctx_len, softmax_scale, staging, workspace, stream=None,
                          check=True) -> int:
-    code = lib().clv_verify_step_host(_ref(shape), _ref(cache), _ref(host_in), _ref(host_out),
-                                      _ptr(ctx_len), int(max_ctx_len), float(softmax_scale),
-                                      _ptr(staging), staging.numel() * staging.element_size(),
-                                      _ptr(workspace),
-                                      0 if workspace is None else workspace.numel() * workspace.element_size(),
-                                      _stream(stream))
-    if check:
+    code = (_calls or _load_calls()).verify_step_host(shape, cache, host_in, host_out, ctx_len, max_ctx_len,
+                                                      softmax_scale, staging, workspace, stream)
+    if code and check:
         _check(code, "clv_verify_step_host")
     return code
 

@@ -6,11 +6,13 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libclv.so")
+CALLS = os.path.join(PKG, "_calls.so")      # the CPython side of the calls (csrc/py_calls.c)
 OBJ_DIR = os.path.join(PKG, "_build")
 
 NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -60,6 +62,13 @@ def build(force: bool = False, verbose: bool = False) -> str:
         subprocess.check_call([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a",
                                "-o", tmp] + objs)
         os.replace(tmp, LIB)
+    calls_src = os.path.join(CSRC, "py_calls.c")
+    if force or _stale(CALLS, [calls_src] + headers):
+        tmp = CALLS + ".tmp%d" % os.getpid()
+        subprocess.check_call(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"),
+                               "-I", sysconfig.get_paths()["include"], calls_src, "-o", tmp,
+                               "-L", PKG, "-l:libclv.so", "-Wl,-rpath,$ORIGIN"])
+        os.replace(tmp, CALLS)
     return LIB
 
 
