@@ -73,9 +73,8 @@ extern "C" {
 size_t clv_workspace_bytes(const clv_shape* shape, const clv_kv_cache* cache, int32_t max_ctx_len) {
   (void)cache;
   if (check_shape(shape) != CLV_OK) return 0;
-  if (max_ctx_len < 0) max_ctx_len = 0;
-  size_t scratch = (tc2_attn_wanted(*shape) ? tc2_attn_plan(*shape, max_ctx_len)
-                                            : tc_attn_plan(*shape, max_ctx_len)).scratch_bytes;
+  (void)max_ctx_len;
+  size_t scratch = 0;   // attention merges on chip
   if (shape->vocab > 0) {
     const ArgmaxPlan gp = argmax_plan(shape->batch * shape->n_nodes, shape->vocab);
     if (gp.scratch_bytes > scratch) scratch = gp.scratch_bytes;
@@ -93,12 +92,11 @@ clv_status clv_workspace_init(void* workspace, size_t workspace_bytes, void* cud
   return e == cudaSuccess ? CLV_OK : cuda_fail(e);
 }
 
-// Argument checks of clv_tree_attn (nothing is enqueued); fills the plan on success.
+// Argument checks of clv_tree_attn (nothing is enqueued).
 static clv_status validate_tree_attn(const clv_shape* shape, const clv_kv_cache* cache, const void* q,
                                      const void* k_tree, const void* v_tree, const int32_t* parent,
                                      const int32_t* ctx_len, int32_t max_ctx_len, const void* out,
-                                     const int32_t* status, const void* workspace, size_t workspace_bytes,
-                                     AttnPlan* plan) {
+                                     const int32_t* status, const void* workspace, size_t workspace_bytes) {
   clv_status st = check_shape(shape);
   if (st != CLV_OK) return st;
   st = check_cache(cache);
@@ -108,10 +106,9 @@ static clv_status validate_tree_attn(const clv_shape* shape, const clv_kv_cache*
   if (max_ctx_len < 0) return CLV_ERR_SHAPE;
   if (shape->n_q_heads / shape->n_kv_heads > 128) return CLV_ERR_UNSUPPORTED;
   if (shape->batch > kTickets / 2) return CLV_ERR_UNSUPPORTED;   // two counters per sequence
-  *plan = tc2_attn_wanted(*shape) ? tc2_attn_plan(*shape, max_ctx_len) : tc_attn_plan(*shape, max_ctx_len);
-  if (!workspace || workspace_bytes < kWsFixedBytes + plan->scratch_bytes) return CLV_ERR_WORKSPACE;
+  if (!workspace || workspace_bytes < kWsFixedBytes) return CLV_ERR_WORKSPACE;
   if (!aligned16(workspace)) return CLV_ERR_ALIGN;
-  if (!tc_attn_supported(*shape, *cache)) return CLV_ERR_UNSUPPORTED;   // asks the driver: last
+  if (!tree_attn_supported(*shape, *cache)) return CLV_ERR_UNSUPPORTED;   // asks the driver: last
   return CLV_OK;
 }
 
@@ -120,17 +117,11 @@ clv_status clv_tree_attn(const clv_shape* shape, const clv_kv_cache* cache, cons
                          const int32_t* ctx_len, int32_t max_ctx_len, float softmax_scale,
                          void* out, float* lse, int32_t* status, void* workspace,
                          size_t workspace_bytes, void* cuda_stream) {
-  AttnPlan plan;
   const clv_status st = validate_tree_attn(shape, cache, q, k_tree, v_tree, parent, ctx_len, max_ctx_len,
-                                           out, status, workspace, workspace_bytes, &plan);
+                                           out, status, workspace, workspace_bytes);
   if (st != CLV_OK) return st;
-  cudaError_t e = tc2_attn_wanted(*shape)
-                      ? launch_tree_attn_tc2(plan, *shape, *cache, q, k_tree, v_tree, parent, ctx_len, softmax_scale,
-                                             out, lse, status, ws_tickets(workspace), ws_scratch(workspace),
-                                             static_cast<cudaStream_t>(cuda_stream))
-                      : launch_tree_attn_tc(plan, *shape, *cache, q, k_tree, v_tree, parent, ctx_len, softmax_scale,
-                                            out, lse, status, ws_tickets(workspace), ws_scratch(workspace),
-                                            static_cast<cudaStream_t>(cuda_stream));
+  cudaError_t e = launch_tree_attn(*shape, *cache, q, k_tree, v_tree, parent, ctx_len, max_ctx_len, softmax_scale,
+                                   out, lse, status, ws_tickets(workspace), static_cast<cudaStream_t>(cuda_stream));
   return e == cudaSuccess ? CLV_OK : cuda_fail(e);
 }
 
@@ -452,11 +443,10 @@ clv_status clv_verify_step_host(const clv_shape* shape, const clv_kv_cache* cach
   const size_t tb = B * N * shape->n_kv_heads * CLV_HEAD_DIM * 2;
   int32_t* const dstat = reinterpret_cast<int32_t*>(d + L.status);
   // every check of the three calls first: a mistake the host can see must leave the stream empty
-  AttnPlan attn_plan_unused;
   ArgmaxPlan argmax_plan_unused;
   st = validate_tree_attn(shape, cache, d + L.q, d + L.k_tree, d + L.v_tree,
                           reinterpret_cast<int32_t*>(d + L.parent), ctx_len, max_ctx_len, d + L.out, dstat,
-                          workspace, workspace_bytes, &attn_plan_unused);
+                          workspace, workspace_bytes);
   if (st != CLV_OK) return st;
   st = validate_accept_argmax(shape, d + L.logits, in->ld, reinterpret_cast<int32_t*>(d + L.ids), workspace,
                               workspace_bytes, &argmax_plan_unused);
@@ -520,6 +510,6 @@ int clv_last_cuda_error(void) { return g_last_cuda_error; }
 void clv_test_set_wait_limit(int64_t sm_cycles) {
   g_wait_limit.store(sm_cycles > 0 ? (long long)sm_cycles : 2000000000ll, std::memory_order_relaxed);
 }
-int clv_version(void) { return 111; }
+int clv_version(void) { return 112; }
 
 }  // extern "C"

@@ -75,28 +75,11 @@ cudaError_t launch_tree_from_intervals(int batch, int n_nodes, const int32_t* ti
                                        int32_t* parent, int32_t* status, cudaStream_t stream);
 
 // ---- tree attention (tcgen05 / TMA; a row tile holds whole nodes: any group size G up to 128) -------
-struct AttnPlan {
-  int m_tiles;   // row tiles per (sequence, kv head)
-  int splits;    // thread blocks along the key axis per row tile
-  size_t scratch_bytes;
-  int tickets;   // counters used
-};
-bool tc_attn_supported(const clv_shape& s, const clv_kv_cache& c);
-AttnPlan tc_attn_plan(const clv_shape& s, int max_ctx_len);
-cudaError_t launch_tree_attn_tc(const AttnPlan& plan, const clv_shape& s, const clv_kv_cache& c,
-                                const void* q, const void* k_tree, const void* v_tree,
-                                const int32_t* parent, const int32_t* ctx_len, float scale, void* out,
-                                float* lse, int32_t* status, unsigned* tickets, void* scratch,
-                                cudaStream_t stream);
-// units of four or more row tiles per (sequence, kv head): blocks of two row tiles that share every
-// staged K/V tile (same results, same plan fields; m_tiles counts pairs of row tiles)
-bool tc2_attn_wanted(const clv_shape& s);
-AttnPlan tc2_attn_plan(const clv_shape& s, int max_ctx_len);
-cudaError_t launch_tree_attn_tc2(const AttnPlan& plan, const clv_shape& s, const clv_kv_cache& c,
-                                 const void* q, const void* k_tree, const void* v_tree,
-                                 const int32_t* parent, const int32_t* ctx_len, float scale, void* out,
-                                 float* lse, int32_t* status, unsigned* tickets, void* scratch,
-                                 cudaStream_t stream);
+bool tree_attn_supported(const clv_shape& s, const clv_kv_cache& c);
+cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const void* q, const void* k_tree,
+                             const void* v_tree, const int32_t* parent, const int32_t* ctx_len, int max_ctx_len,
+                             float scale, void* out, float* lse, int32_t* status, unsigned* tickets,
+                             cudaStream_t stream);
 
 // ---- LM head fused with the argmax (tcgen05 GEMM whose logits stay in tensor memory) ---------------
 bool lm_head_supported(int rows, int hidden, int vocab);

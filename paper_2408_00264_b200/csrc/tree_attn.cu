@@ -1,0 +1,1098 @@
+// Tree attention (Sec. 2.1) on the 5th-generation tensor cores: tcgen05.mma with accumulators in
+// tensor memory, K/V/Q tiles staged by TMA into 128-byte-swizzled shared memory.
+//
+// Query row = (tree node, head-in-group) pair, so all G heads of a GQA group and all tree nodes
+// reuse every K/V byte.  A row tile of 128 rows holds whole nodes: 128 / G of them (rounded down;
+// its other rows idle).  The key axis (cache keys first, then the tree's own) is walked in tiles of
+// 128 keys that are loaded as 64-key pieces (also the page size of a paged cache).
+//
+// A thread block has two SLOTS, each with a score buffer and an output accumulator of its own in
+// tensor memory (4 x 128 columns) and four softmax warps of its own, one thread per query row:
+//   kRows2    the slots are two row tiles of the same (sequence, kv head); both take every key tile,
+//             so a staged K/V tile serves 256 rows;
+//   otherwise the slots share one row tile and take the key tiles in turn (even, odd); their two
+//             partial results are combined like those of two blocks.
+// What bounds a key tile of 128 x 128 scores: Q K^T and P V are 16 MMAs of 64 cycles, the
+// exponentials 1024 cycles of the special-function units, and within a slot the two alternate (scores
+// -> exponentials -> P V -> next scores).  With two slots the tensor core works for one while the
+// other is in its exponentials, and P is handed over in three parts (64, 32, 32 keys), so that only
+// the last quarter of P V is left when the exponentials are done.
+//
+// Softmax: a thread takes its row's 128 scores into registers and writes P (bf16) back over the score
+// columns.  The exponentials of the first 64 keys are computed with the row's reference as it stands,
+// beside the maximum of all 128; the reference is replaced (O rescaled, those exponentials redone) only
+// when a score exceeds it by 2^32: P is bf16 and the sums are fp32, so a probability above 1 costs
+// no precision, and after a row's first tile the replacement is a rare event.
+// The tree columns are masked with ancestor bitsets derived from parent[]; masked scores are replaced
+// by -inf, not added to, so they contribute exactly zero.
+//
+// Split-KV: the blocks that share row tiles form a thread-block cluster (1..8 along the key axis).
+// Each sends the accumulator rows that another one finalises as fp16 (half a row scaled by a power of
+// two of its own: 2^-11 relative, against the output's 2^-9) with their reference and sum, by bulk
+// copies from its shared memory to the other's, into tile memory that is idle by then.
+// No partial result touches global memory.
+// Every wait is bounded: on expiry the block raises a flag, all roles leave their loops, in-flight
+// copies and MMAs are drained and CLV_ERR_TIMEOUT is reported for the sequence.
+#include <cuda.h>
+#include <cuda_fp16.h>
+#include <math.h>
+
+#include "clv_internal.cuh"
+#include "tc_ptx.cuh"
+#include "tmem_access.cuh"
+
+namespace clv {
+namespace {
+
+constexpr int PG = CLV_PAGE_SIZE;      // 64: keys per TMA piece (= page size)
+constexpr int HD = CLV_HEAD_DIM;       // 128
+constexpr int BM = 128;                // rows per slot
+constexpr int BN = 128;                // keys per tile
+constexpr int CH = 32;                 // keys whose scores one load brings
+constexpr int kThreads = 384;          // warps 0-3 and 4-7: the slots' softmax; 8: TMA producer; 9: MMA issuer; 10, 11 idle
+// Registers per thread: the launch's 168 cannot hold a row's 128 scores and the rest of a softmax
+// thread, so the third warpgroup's go to the first two while the roles work (256 x 216 + 128 x 72 =
+// 384 x 168; 4 x 64 nodes x 4096 keys: 28.0 -> 26.5 us).
+constexpr int kSoftmaxRegs = 216, kOtherRegs = 72, kLaunchRegs = 168;
+constexpr int kSoftmaxWarps = 8, kProducer = 8, kIssuer = 9;
+constexpr int kMaxSplits = 8;          // portable cluster size
+constexpr uint32_t kQTile = BM * HD * 2;      // 32 KB: two [128 rows][64 d] swizzled halves
+constexpr uint32_t kPiece = PG * 64 * 2;       // 8 KB: [64 keys][64 d] swizzled, one TMA box
+constexpr uint32_t kStage = BN * HD * 2;       // 32 KB: a K (or V) tile, [64-wide half of d][128 keys][64 d]
+constexpr uint32_t kHalf = kStage / 2;
+constexpr uint32_t kTmemCols = 512;
+constexpr float kRefSlack = 32.f;      // log2 units a score may exceed the row's reference by
+constexpr uint32_t kIdescQK = make_idesc(BM, BN, false);  // S[128 rows x 128 keys] = Q K^T
+constexpr uint32_t kIdescPV = make_idesc(BM, HD, true);   // O[128 rows x 128 d] += P V
+
+template <bool kRows2>
+struct Cfg {
+  static constexpr int kQ = kRows2 ? 2 : 1;      // row tiles
+  static constexpr int NST = kRows2 ? 5 : 6;     // ring stages: K and V tiles in turn
+  static constexpr int kStep = kRows2 ? 2 : 4;   // loads from one tile of a slot to its next
+};
+
+// barriers: stage full [6] | stage empty [6] | S full [2] | part of P [2][3] | last P V done [2] | Q | merge | drain
+constexpr int B_FULL = 0, B_EMPTY = 6, B_S = 12, B_P = 14, B_LAST = 20, B_Q = 22, B_RX = 23, B_DR = 24, NBAR = 25;
+
+struct Misc {                           // behind the tiles in dynamic shared memory
+  float2 ml[2 * BM];                    // (reference, sum) of every row of both slots
+  unsigned long long bar[NBAR];
+  uint32_t tmem;
+  int abort_flag;
+  int seq, len;                         // the block's sequence and its context length
+  int issued;                           // loads issued (producer)
+  signed char parent[CLV_MAX_NODES];    // as far as valid, -1 otherwise
+};
+constexpr uint32_t kMiscAt = 7 * kStage;   // either way: Q tiles + ring = 224 KB
+constexpr uint32_t kSmem = kMiscAt + (uint32_t)sizeof(Misc);
+static_assert(Cfg<true>::kQ + Cfg<true>::NST == 7 && Cfg<false>::kQ + Cfg<false>::NST == 7 && kSmem <= 232448, "shared memory");
+
+struct Params {
+  const int32_t* block_table;
+  const int32_t* parent;
+  const int32_t* ctx_len;
+  uint16_t* out;
+  float* lse;
+  int32_t* status;
+  int B, N, Hq, Hkv, G;
+  int paged, cap_tokens, n_pages, max_pages;
+  int longest_first;  // hand out sequences in order of decreasing context length
+  int pair_boxes;     // the 4-D tensor maps exist: a whole 128-key tile of a contiguous cache is one copy
+  int tiles;          // row tiles per (sequence, kv head)
+  int groups;         // blocks along the rows: tiles, or pairs of tiles (kRows2)
+  int splits;         // blocks along the key axis = cluster size
+  float scale_log2;
+  long long wait_limit;   // SM cycles a bounded wait may last
+  unsigned* tickets;      // per sequence: [2b] blocks that have finished, [2b+1] error bits; zero between calls
+  int blocks_per_seq;
+};
+
+struct Maps {
+  CUtensorMap q, out;    // [B][N][Hq][128], box = 64 x G x 128/G nodes
+  CUtensorMap kc, vc;    // cache rows, box = 64 x 1 head x 64 rows
+  CUtensorMap kt, vt;    // tree rows, likewise
+  CUtensorMap kc2, vc2;  // cache rows as [head][half of d][row][64], box = a whole key tile
+};
+
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float y;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(reinterpret_cast<unsigned long long&>(d))
+      : "l"(reinterpret_cast<unsigned long long&>(a)), "l"(reinterpret_cast<unsigned long long&>(b)),
+        "l"(reinterpret_cast<unsigned long long&>(c)));
+  return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("add.rn.f32x2 %0, %1, %2;"
+      : "=l"(reinterpret_cast<unsigned long long&>(d))
+      : "l"(reinterpret_cast<unsigned long long&>(a)), "l"(reinterpret_cast<unsigned long long&>(b)));
+  return d;
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<uint32_t*>(&v);
+}
+__device__ __forceinline__ float2 half2_bits_to_float2(uint32_t u) {
+  return __half22float2(*reinterpret_cast<const __half2*>(&u));
+}
+// bounded wait of a whole warp for a phase of a barrier: the same verdict for every lane
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit) {
+  return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag, limit)) != 0;
+}
+__device__ __forceinline__ void named_barrier(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+template <int kRegs>
+__device__ __forceinline__ void more_registers() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs)); }
+template <int kRegs>
+__device__ __forceinline__ void fewer_registers() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs)); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// bulk copy to a peer's shared memory; its barrier counts the bytes
+__device__ __forceinline__ void bulk_to_peer(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "r"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* tm, uint32_t src, int c0, int c1, int c2, int c3) {
+  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];"
+               ::"l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(src)
+               : "memory");
+}
+__device__ __forceinline__ void st_shared16(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+__device__ __forceinline__ void st_shared8(uint32_t a, float x, float y) {
+  asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(a), "f"(x), "f"(y) : "memory");
+}
+
+// a position in the ring of stages and the parity of its current round
+template <int NST>
+struct RingPos {
+  int idx;
+  uint32_t ph;
+  __device__ __forceinline__ explicit RingPos(int n) : idx(n % NST), ph((uint32_t)(n / NST) & 1u) {}   // of load n
+  __device__ __forceinline__ void advance(int k) {
+    idx += k;
+    if (idx >= NST) { idx -= NST; ph ^= 1u; }
+  }
+};
+
+// What a thread knows about its block: its place in the grid, its share of the key axis, its row.
+template <bool kRows2>
+struct Block {
+  uint8_t* smem;
+  uint32_t smem0, sRing, bar0, tmem;
+  volatile int* abort_flag;
+  int tid, warp, lane;
+  int CS, split, group, kvh, b;            // cluster size, rank in the cluster, rows' group, kv head, sequence
+  int N, G, tile_nodes, RT, tile0, users;  // whole nodes of a row tile and the rows they take; first row tile; slots that read one K/V tile
+  int R, per, first, mine;                 // rows in use, numbered through the row tiles; rank d finalises [d * per, (d + 1) * per)
+  int L, p_cache, p_total, pc_begin, pc_end, T, t_plain;
+  bool len_bad;
+  int slot, row, node, my_tiles;           // of the softmax threads
+  bool row_valid;
+  uint32_t lane_addr;
+
+  __device__ __forceinline__ Misc& misc() const { return *reinterpret_cast<Misc*>(smem + kMiscAt); }
+  __device__ __forceinline__ uint32_t bar(int idx) const { return bar0 + 8u * (uint32_t)idx; }
+  __device__ __forceinline__ uint32_t tmem_S(int s) const { return tmem + (uint32_t)(s * BN); }   // P overwrites columns 0-63
+  __device__ __forceinline__ uint32_t tmem_O(int s) const { return tmem + (uint32_t)(2 * BN + s * HD); }
+  // real keys of piece g (0: not of this block)
+  __device__ __forceinline__ int piece_keys(int g) const {
+    return g >= pc_end ? 0 : g < p_cache ? min(PG, L - g * PG) : min(PG, N - (g - p_cache) * PG);
+  }
+  __device__ __forceinline__ int slot_tiles(int s) const { return kRows2 ? (s < users ? T : 0) : (T - s + 1) / 2; }
+
+  // the place in the grid (blocks of a cluster are neighbours along x)
+  __device__ __forceinline__ void place(const Params& p, uint8_t* sm, unsigned block, int thread) {
+    smem = sm;
+    smem0 = smem_u32(sm);
+    sRing = smem0 + Cfg<kRows2>::kQ * kQTile;
+    bar0 = smem_u32(&misc().bar[0]);
+    abort_flag = &misc().abort_flag;
+    tid = thread; warp = tid >> 5; lane = tid & 31;
+    CS = p.splits;
+    split = (int)(block % (unsigned)CS);
+    const int cluster_id = (int)(block / (unsigned)CS), unit = cluster_id / p.groups;
+    group = cluster_id - unit * p.groups;
+    b = unit / p.Hkv;
+    kvh = unit - b * p.Hkv;
+    N = p.N; G = p.G;
+    tile_nodes = BM / G; RT = tile_nodes * G;
+    tile0 = kRows2 ? 2 * group : group;
+    users = (kRows2 && tile0 + 1 < p.tiles) ? 2 : 1;
+    R = (kRows2 ? (users - 1) * BM : 0) + min(RT, (N - (tile0 + users - 1) * tile_nodes) * G);
+    per = ((R + CS - 1) / CS + 7) & ~7;
+    first = min(R, split * per);
+    mine = min(R, first + per) - first;
+  }
+  // The sequence's length and this block's range of the key axis.  The axis is cut in 64-key pieces:
+  // p_cache pieces of context, then the tree's own pieces.  A split takes a contiguous range of pieces
+  // and walks it in tiles of two; the last tile of a range may hold one piece only.  A bad length
+  // reads the tree's own rows only.  Tiles [0, t_plain) consist of two complete pieces of context.
+  __device__ __forceinline__ void range(const Params& p, int len) {
+    L = len;
+    len_bad = (L < 0) || (p.paged ? ((L + PG - 1) / PG > p.max_pages) : (L > p.cap_tokens));
+    p_cache = (!len_bad && L > 0) ? (L + PG - 1) / PG : 0;
+    p_total = p_cache + (N + PG - 1) / PG;
+    pc_begin = (int)((unsigned)split * (unsigned)p_total / (unsigned)CS);
+    pc_end = (int)((unsigned)(split + 1) * (unsigned)p_total / (unsigned)CS);
+    T = (pc_end - pc_begin + 1) / 2;
+    t_plain = max(0, (min(pc_end, len_bad ? 0 : L / PG) - pc_begin) / 2);
+    tmem = misc().tmem;
+    slot = (warp >> 2) & 1;
+    row = (warp & 3) * 32 + lane;   // a warp may touch the 32 tensor-memory lanes of its number modulo 4
+    lane_addr = (uint32_t)((warp & 3) * 32) << 16;
+    const int rtile = kRows2 ? tile0 + slot : tile0;
+    node = rtile * tile_nodes + row / G;
+    row_valid = warp < kSoftmaxWarps && row < RT && rtile < p.tiles && node < N;
+    my_tiles = slot_tiles(slot);
+  }
+};
+
+// ---- the roles' work on the block's share of the keys
+
+template <bool kRows2>
+__device__ __forceinline__ void produce(const Block<kRows2>& k, const Maps& tm, const Params& p) {
+  constexpr int NST = Cfg<kRows2>::NST;
+  if (k.lane == 0 && k.T > 0) {
+    mbar_expect_tx(k.bar(B_Q), (uint32_t)(k.users * k.RT * HD * 2));   // a box holds RT rows, absent nodes as zeros
+#pragma unroll
+    for (int m = 0; m < Cfg<kRows2>::kQ; ++m) {
+      if (m >= k.users) break;
+      tma_load_4d(k.smem0 + m * kQTile, &tm.q, 0, k.kvh * k.G, (k.tile0 + m) * k.tile_nodes, k.b, k.bar(B_Q));
+      tma_load_4d(k.smem0 + m * kQTile + kQTile / 2, &tm.q, 64, k.kvh * k.G, (k.tile0 + m) * k.tile_nodes, k.b, k.bar(B_Q));
+    }
+  }
+  int page = 0, page_base = -64;   // lane j: pool page of context piece (page_base + j)
+  RingPos<NST> pos(0);
+  int issued = 0;
+  bool ok = true;
+  for (int t = 0; t < k.T && ok; ++t) {
+    const int g0 = k.pc_begin + 2 * t;
+    if (p.paged && g0 < k.p_cache && g0 + 2 > page_base + 32) {
+      page_base = g0;
+      const int pc = g0 + k.lane;
+      page = (pc < k.p_cache) ? p.block_table[(int64_t)k.b * p.max_pages + pc] : 0;
+    }
+    int row0[2];
+    bool is_tree[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int g = g0 + j;
+      int pg = __shfl_sync(0xFFFFFFFFu, page, (g - page_base) & 31);
+      is_tree[j] = g >= k.p_cache;
+      if (g >= k.pc_end) row0[j] = -1;     // the range ended inside this tile
+      else if (is_tree[j]) row0[j] = k.b * k.N + (g - k.p_cache) * PG;
+      else if (p.paged) {
+        if (pg < 0 || pg >= p.n_pages) pg = 0;   // the reporter flags the sequence; any page will do
+        row0[j] = pg * PG;
+      } else row0[j] = k.b * p.cap_tokens + g * PG;
+    }
+#pragma unroll
+    for (int kv = 0; kv < 2; ++kv) {   // K, then V
+      if (issued >= NST) ok = wait_warp(k.bar(B_EMPTY + pos.idx), pos.ph ^ 1u, k.abort_flag, p.wait_limit);
+      if (!ok) break;
+      if (k.lane == 0) {
+        const uint32_t full = k.bar(B_FULL + pos.idx), stage = k.sRing + (uint32_t)pos.idx * kStage;
+        if (p.pair_boxes && row0[0] >= 0 && !is_tree[1] && row0[1] == row0[0] + PG) {
+          // both pieces are neighbours in the cache: the whole tile, both halves of d, in one copy
+          mbar_expect_tx(full, kStage);
+          tma_load_4d(stage, kv == 0 ? &tm.kc2 : &tm.vc2, 0, row0[0], 0, k.kvh, full);
+        } else {
+          mbar_expect_tx(full, (row0[1] >= 0 ? 2u : 1u) * 2u * kPiece);
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            if (row0[j] < 0) continue;
+            const CUtensorMap* m = is_tree[j] ? (kv == 0 ? &tm.kt : &tm.vt) : (kv == 0 ? &tm.kc : &tm.vc);
+            const uint32_t dst = stage + (uint32_t)j * kPiece;
+            tma_load_3d(dst, m, 0, k.kvh, row0[j], full);
+            tma_load_3d(dst + kHalf, m, 64, k.kvh, row0[j], full);
+          }
+        }
+      }
+      ++issued;
+      pos.advance(1);
+    }
+  }
+  if (k.lane == 0) k.misc().issued = issued;   // for the drain of an aborted block
+}
+
+// The whole warp walks the schedule and one elected lane issues: inside a divergent branch every
+// operand is moved to the uniform registers for each MMA, and an MMA of 64 cycles took 110 to 200 to
+// issue (long contexts, 8 x 32768 keys: 1090 -> 740 us for the branch under elect.sync alone).  Fixed
+// order: Q K^T of both slots, then per tile and slot P V of the tile's parts as they are handed over and
+// Q K^T of the slot's next tile.  The tensor core queues a few MMAs, so what lies between two groups
+// of them is hidden.
+template <bool kRows2>
+__device__ __forceinline__ void issue(const Block<kRows2>& k, const Params& p) {
+  constexpr int NST = Cfg<kRows2>::NST;
+  const uint32_t el = elect_one();
+  if (k.T == 0 || !wait_warp(k.bar(B_Q), 0, k.abort_flag, p.wait_limit)) return;
+  const uint64_t q_desc = smem_desc(k.smem0, 16, 1024);
+  const uint64_t k_desc = smem_desc(k.sRing, 16, 1024);
+  const uint64_t v_desc = smem_desc(k.sRing, kHalf, 1024);   // lbo: the other half of d
+  RingPos<NST> kpos[2] = {RingPos<NST>(0), RingPos<NST>(kRows2 ? 0 : 2)};
+  uint32_t ph = 0u;   // bit 3 s + h: parity of the next use of the barrier for part h of slot s's P
+  auto issue_qk = [&](int s) -> bool {
+    if (!wait_warp(k.bar(B_FULL + kpos[s].idx), kpos[s].ph, k.abort_flag, p.wait_limit)) return false;
+    tc_fence_after();
+    const uint64_t qd = q_desc + (uint64_t)(((kRows2 ? s : 0) * kQTile) >> 4);
+    const uint64_t kd = k_desc + (uint64_t)((uint32_t)(kpos[s].idx * (int)kStage) >> 4);
+#pragma unroll
+    for (int ks = 0; ks < HD / 16; ++ks) {
+      const uint32_t qo = (ks >> 2) * (kQTile / 2) + (ks & 3) * 32;
+      const uint32_t ko = (ks >> 2) * kHalf + (ks & 3) * 32;
+      umma_bf16_if(el, k.tmem_S(s), qd + (qo >> 4), kd + (ko >> 4), kIdescQK, ks > 0 ? 1u : 0u);
+    }
+    umma_commit_if(el, k.bar(B_S + s));
+    umma_commit_if(el, k.bar(B_EMPTY + kpos[s].idx));
+    return true;
+  };
+  bool ok = issue_qk(0);
+  if (ok && k.slot_tiles(1) > 0) ok = issue_qk(1);
+#pragma unroll 1
+  for (int r = 0; r < k.slot_tiles(0) && ok; ++r) {
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      if (!ok || r >= k.slot_tiles(s)) continue;
+      const int g0 = k.pc_begin + 2 * (kRows2 ? r : 2 * r + s);
+      RingPos<NST> vpos = kpos[s];
+      vpos.advance(1);
+      ok = wait_warp(k.bar(B_FULL + vpos.idx), vpos.ph, k.abort_flag, p.wait_limit);
+      const uint64_t vd = v_desc + (uint64_t)((uint32_t)(vpos.idx * (int)kStage) >> 4);
+      const int keys[2] = {k.piece_keys(g0), k.piece_keys(g0 + 1)};
+#pragma unroll
+      for (int h = 0; h < 3; ++h) {   // keys 0-63, 64-95, 96-127 of the tile
+        if (!ok || (h > 0 && keys[1] <= (h - 1) * CH)) continue;
+        ok = wait_warp(k.bar(B_P + 3 * s + h), (ph >> (3 * s + h)) & 1u, k.abort_flag, p.wait_limit);
+        if (!ok) continue;
+        ph ^= 1u << (3 * s + h);
+        tc_fence_after();
+#pragma unroll
+        for (int kk = h == 0 ? 0 : 2 + 2 * h; kk < 4 + 2 * h; ++kk)
+          if (h > 0 || kk < 2 || keys[0] > CH)
+            umma_bf16_ts_if(el, k.tmem_O(s), k.tmem_S(s) + (uint32_t)(kk * 8), vd + (uint64_t)((kk * 16 * 128) >> 4), kIdescPV,
+                            (r > 0 || kk > 0) ? 1u : 0u);
+      }
+      if (!ok) continue;
+      umma_commit_if(el, k.bar(B_EMPTY + vpos.idx));
+      kpos[s].advance(Cfg<kRows2>::kStep);
+      if (r + 1 < k.slot_tiles(s)) ok = issue_qk(s);
+      else umma_commit_if(el, k.bar(B_LAST + s));
+    }
+  }
+}
+
+template <bool kRows2>
+__device__ __forceinline__ void softmax(const Block<kRows2>& k, const Params& p) {
+  constexpr int NST = Cfg<kRows2>::NST;
+  Misc& ms = k.misc();
+  const int tid = k.tid, lane = k.lane, slot = k.slot, row = k.row;
+  if (tid < CLV_MAX_NODES) {
+    bool bad = false;
+    int par = -1;
+    if (tid < k.N) {
+      par = p.parent[(int64_t)k.b * k.N + tid];
+      if (par < -1 || par >= tid) { bad = true; par = -1; }
+    }
+    ms.parent[tid] = (signed char)par;
+    // one block per sequence reports what is wrong with it: the length, the tree, the block table
+    if (k.group == 0 && k.split == 0 && k.kvh == 0) {
+      bad |= k.len_bad;
+      if (p.paged && k.warp == 0)
+        for (int pg = lane; pg < k.p_cache; pg += 32) {
+          const int e = p.block_table[(int64_t)k.b * p.max_pages + pg];
+          bad |= (e < 0 || e >= p.n_pages);
+        }
+      if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(p.tickets + 2 * k.b + 1, 1u);  // before this block's ticket
+    }
+  }
+  __syncwarp();
+  named_barrier(1, 32 * kSoftmaxWarps);
+  uint32_t anc[4] = {0u, 0u, 0u, 0u};   // row of the tree's topology matrix: the node and its ancestors
+  if (k.row_valid) {
+    for (int j = k.node; j >= 0; j = ms.parent[j]) {
+#pragma unroll
+      for (int w = 0; w < 4; ++w) anc[w] |= (j >> 5) == w ? 1u << (j & 31) : 0u;
+    }
+  }
+  __syncwarp();
+  const bool warp_active = __any_sync(0xFFFFFFFFu, k.row_valid), warp_full = __all_sync(0xFFFFFFFFu, k.row_valid);
+  const uint32_t s_addr = k.tmem_S(slot) + k.lane_addr;   // this row's scores, then its P
+  const float sc = p.scale_log2;
+  float m_ref = k.row_valid ? -INFINITY : 0.f, l_run = 0.f;
+  auto hand_over = [&](int h) {   // part h of P: keys 0-63, 64-95, 96-127 of the tile
+    tmem_wait_st();
+    tc_fence_before();
+    __syncwarp();
+    mbar_arrive_if(lane == 0 ? 1u : 0u, k.bar(B_P + 3 * slot + h));
+  };
+  RingPos<NST> vpos(kRows2 || slot == 0 ? 1 : 3);   // V stage of the current tile
+#pragma unroll 1
+  for (int r = 0; r < k.my_tiles; ++r) {
+    const int t = kRows2 ? r : 2 * r + slot;
+    if (!wait_warp(k.bar(B_S + slot), (uint32_t)r & 1u, k.abort_flag, p.wait_limit)) break;
+    tc_fence_after();
+    int keys0 = PG, keys1 = PG;    // real keys of the tile's pieces
+    const bool plain = t < k.t_plain;
+    if (!plain) {
+      keys0 = k.piece_keys(k.pc_begin + 2 * t);
+      keys1 = k.piece_keys(k.pc_begin + 2 * t + 1);
+      // Rows of V beyond a piece's real keys hold whatever lies behind them in memory; their
+      // probabilities are exactly 0, but 0 * NaN would poison O: clear them, up to the end of the
+      // last 32 keys that P V takes.
+      if ((keys0 | keys1) & (CH - 1)) {
+        if (!wait_warp(k.bar(B_FULL + vpos.idx), vpos.ph, k.abort_flag, p.wait_limit)) break;
+        uint8_t* vt = k.smem + (k.sRing - k.smem0) + (uint32_t)vpos.idx * kStage;
+#pragma unroll 1
+        for (int j = 0; j < 2; ++j) {
+          const int v = j ? keys1 : keys0;
+          const int n = ((v + CH - 1) & ~(CH - 1)) - v;
+          for (int i = row; i < n * 16; i += BM) {
+            const int vr = j * PG + v + (i >> 4), chk = i & 15;
+            *reinterpret_cast<uint4*>(vt + (chk >> 3) * kHalf + vr * 128 + (chk & 7) * 16) = make_uint4(0, 0, 0, 0);
+          }
+        }
+        fence_async_smem();   // cleared V rows visible to the tensor core's reads
+        __syncwarp();
+      }
+    }
+    vpos.advance(Cfg<kRows2>::kStep);
+    if (!warp_active) {   // no row of this warp exists: its lanes of P may hold anything
+      hand_over(0);
+      if (keys1 > 0) hand_over(1);
+      if (keys1 > CH) hand_over(2);
+      continue;
+    }
+    const bool masked = !plain || !warp_full;
+    auto mask = [&](int c, uint32_t (&a)[CH]) {   // columns that this row may not see become -inf
+      const int g = k.pc_begin + 2 * t + (c >> 1), keys = ((c >> 1) ? keys1 : keys0) - (c & 1) * CH;
+      uint32_t bits = 0u;
+      if (k.row_valid && keys > 0) {
+        if (g < k.p_cache) bits = keys >= CH ? 0xFFFFFFFFu : (1u << keys) - 1u;
+        else bits = g == k.p_cache ? ((c & 1) ? anc[1] : anc[0]) : ((c & 1) ? anc[3] : anc[2]);
+      }
+#pragma unroll
+      for (int j = 0; j < CH; ++j)
+        if (!((bits >> j) & 1u)) a[j] = 0xFF800000u;
+    };
+    float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+    auto take_max = [&](const uint32_t (&a)[CH]) {
+#pragma unroll
+      for (int j = 0; j < CH; j += 2) mx[(j >> 1) & 3] = max3(mx[(j >> 1) & 3], __uint_as_float(a[j]), __uint_as_float(a[j + 1]));
+    };
+    float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    float neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
+    auto exps = [&](uint32_t (&a)[CH]) {   // the first half of `a` becomes P
+      const float2 sc2 = make_float2(sc, sc), nm2 = make_float2(neg_m, neg_m);
+#pragma unroll
+      for (int j = 0; j < CH / 2; ++j) {
+        const float2 e = fma2(make_float2(__uint_as_float(a[2 * j]), __uint_as_float(a[2 * j + 1])), sc2, nm2);
+        const float2 pr = make_float2(ex2(e.x), ex2(e.y));
+        sum[j & 1] = add2(sum[j & 1], pr);
+        a[j] = pack_bf16(pr.x, pr.y);
+      }
+    };
+    auto load = [&](int c, uint32_t (&a)[CH]) { tmem_ld_x32(s_addr + (uint32_t)(c * CH), a); };
+    auto store_p = [&](int c, const uint32_t (&a)[CH]) {
+      tmem_st_x16(s_addr + (uint32_t)(c * (CH / 2)), *reinterpret_cast<const uint32_t(*)[CH / 2]>(&a[0]));
+    };
+    uint32_t x0[CH], x1[CH], x2[CH], x3[CH];
+    load(0, x0);
+    tmem_wait_ld();
+    load(1, x1);
+    load(2, x2);
+    load(3, x3);
+    if (masked) mask(0, x0);
+    take_max(x0);
+    exps(x0);
+    tmem_wait_ld();
+    if (masked) {
+      mask(1, x1);
+      mask(2, x2);
+      mask(3, x3);
+    }
+    take_max(x1);
+    take_max(x2);
+    take_max(x3);
+    exps(x1);
+    const float m_new = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]) * sc;   // scale > 0; no allowed key: -inf
+    const bool need = m_new > m_ref + kRefSlack;
+    if (__any_sync(0xFFFFFFFFu, need)) {
+      // A new reference.  O is at rest: these scores were asked for after P V of the slot's previous
+      // tile.  The scores of the first 64 keys are still in place.
+      const float alpha = need ? ex2(m_ref - m_new) : 1.f;   // ex2(-inf) = 0
+      if (need) { m_ref = m_new; l_run *= alpha; }
+      neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
+      if (r > 0) {
+#pragma unroll 1
+        for (int cc = 0; cc < HD; cc += 16) {
+          uint32_t ov[16];
+          tmem_ld_x16(k.tmem_O(slot) + k.lane_addr + (uint32_t)cc, ov);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * alpha);
+          tmem_st_x16(k.tmem_O(slot) + k.lane_addr + (uint32_t)cc, ov);
+        }
+      }
+      sum[0] = sum[1] = make_float2(0.f, 0.f);
+      load(0, x0);
+      load(1, x1);
+      tmem_wait_ld();
+      if (masked) {
+        mask(0, x0);
+        mask(1, x1);
+      }
+      exps(x0);
+      exps(x1);
+    }
+    store_p(0, x0);
+    store_p(1, x1);
+    if (keys1 > CH) {   // a part's stores have the time of the next exponentials before they are waited for
+      exps(x2);
+      hand_over(0);
+      store_p(2, x2);
+      exps(x3);
+      hand_over(1);
+      store_p(3, x3);
+      hand_over(2);
+    } else if (keys1 > 0) {
+      exps(x2);
+      hand_over(0);
+      store_p(2, x2);
+      hand_over(1);
+    } else {
+      hand_over(0);
+    }
+    const float2 tot = add2(sum[0], sum[1]);
+    l_run += tot.x + tot.y;
+  }
+  ms.ml[slot * BM + row] = make_float2(m_ref, l_run);
+}
+
+// ------------------------------------------------------------------------------------ kernel
+template <bool kRows2>
+__global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Params p) {
+  constexpr int NST = Cfg<kRows2>::NST;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  Misc& ms = *reinterpret_cast<Misc*>(smem + kMiscAt);
+  {
+  Block<kRows2> k;
+  k.place(p, smem, blockIdx.x, threadIdx.x);
+  const int tid = k.tid, warp = k.warp;
+  auto bar = [&](int idx) { return k.bar(idx); };
+
+  // ---- set-up that reads no global memory: barriers, tensor memory, descriptor prefetch.  The
+  //      kernel is launched with programmatic stream serialisation, so this part may run while the
+  //      previous kernel of the stream drains.
+  if (tid == 0) {
+    for (int i = 0; i < NST; ++i) { mbar_init(bar(B_FULL + i), 1); mbar_init(bar(B_EMPTY + i), (uint32_t)k.users); }
+    for (int i = 0; i < 2; ++i) { mbar_init(bar(B_S + i), 1); mbar_init(bar(B_LAST + i), 1); }
+    for (int i = 0; i < 6; ++i) mbar_init(bar(B_P + i), 4);
+    mbar_init(bar(B_Q), 1);
+    mbar_init(bar(B_RX), 1);
+    mbar_init(bar(B_DR), 1);
+    if (k.CS > 1) mbar_expect_tx(bar(B_RX), (uint32_t)((k.CS - 1) * k.mine) * 272u);   // what the other ranks will send
+    ms.abort_flag = 0;
+    ms.issued = 0;
+    fence_barrier_init();
+    fence_async_smem();
+  }
+  if (warp == kIssuer) tmem_alloc(smem_u32(&ms.tmem), kTmemCols);
+  if (tid == 32 * kProducer) {
+    tma_prefetch_desc(&tm.q);
+    if (p.pair_boxes) { tma_prefetch_desc(&tm.kc2); tma_prefetch_desc(&tm.vc2); }
+    tma_prefetch_desc(&tm.kc); tma_prefetch_desc(&tm.vc);
+    tma_prefetch_desc(&tm.kt); tma_prefetch_desc(&tm.vt);
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  cudaGridDependencySynchronize();
+
+  if (p.longest_first) {
+    // More blocks than SMs and contexts of different lengths (ragged batch): hand the sequences
+    // out longest first, so that the block scheduler packs the short ones into the gaps.  Block
+    // group `b` takes the sequence whose length has rank b (ties by index).
+    int* len = reinterpret_cast<int*>(smem);   // the tiles are not in use yet
+    for (int i = tid; i < p.B; i += kThreads) len[i] = p.ctx_len[i];
+    __syncthreads();
+    for (int i = tid; i < p.B; i += kThreads) {
+      const int Li = len[i];
+      int rank = 0;
+      for (int j = 0; j < p.B; ++j) rank += (len[j] > Li) || (len[j] == Li && j < i);
+      if (rank == k.b) ms.seq = i;
+    }
+    __syncthreads();
+    k.b = ms.seq;
+    fence_async_smem();   // the tiles are written by TMA next
+    __syncthreads();
+  }
+  k.range(p, p.ctx_len[k.b]);
+  if (tid == 0) { ms.seq = k.b; ms.len = k.L; }
+  if (warp < kSoftmaxWarps) {
+    more_registers<kSoftmaxRegs>();
+    softmax<kRows2>(k, p);
+    __syncwarp();
+    fewer_registers<kLaunchRegs>();   // before the third warpgroup takes its own back
+    named_barrier(2, kThreads);
+  } else {
+    fewer_registers<kOtherRegs>();
+    if (warp == kProducer) produce<kRows2>(k, tm, p);
+    else if (warp == kIssuer) issue<kRows2>(k, p);
+    __syncwarp();
+    named_barrier(2, kThreads);
+    more_registers<kLaunchRegs>();
+  }
+  }
+
+  // ---- every role has met here ------------------------------------------------------------------
+  // What is known about the block is worked out once more: kept in registers it would push the softmax
+  // threads' scores out of theirs (4 x 64 nodes x 4096 keys: 29.8 -> 27.7 us).
+  Block<kRows2> k;
+  {
+    unsigned block;
+    int thread;
+    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(block));
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(thread));
+    k.place(p, smem, block, thread);
+    k.b = ms.seq;
+    k.range(p, ms.len);
+  }
+  const int tid = k.tid, warp = k.warp, lane = k.lane, CS = k.CS, split = k.split, kvh = k.kvh, N = k.N, G = k.G;
+  const int tile_nodes = k.tile_nodes, tile0 = k.tile0, users = k.users, b = k.b, T = k.T;
+  const int R = k.R, per = k.per, first = k.first, mine = k.mine;
+  const uint32_t smem0 = k.smem0, sRing = k.sRing;
+  auto bar = [&](int idx) { return k.bar(idx); };
+  const bool aborted = *k.abort_flag != 0;
+  if (CS > 1) cluster_arrive();   // all Q K^T of this block are done: what the merge uses is idle (see there)
+  if (aborted) {
+    // copies that were issued land on their own, MMAs that were issued finish: wait for both
+    if (warp == kProducer && lane == 0) {
+      const int issued = ms.issued;
+      for (int i = max(0, issued - NST); i < issued; ++i) {
+        const RingPos<NST> pos(i);
+        mbar_drain(bar(B_FULL + pos.idx), pos.ph);
+      }
+      if (T > 0) mbar_drain(bar(B_Q), 0);
+    }
+    if (warp == kIssuer) {
+      umma_commit_if(elect_one(), bar(B_DR));
+      mbar_drain(bar(B_DR), 0);
+    }
+    __syncthreads();
+  }
+  // status[b] is written once, by whichever block of the sequence finishes last: every block adds
+  // its error bits (1 malformed input, 2 a wait ran out) to the sequence's word in the workspace
+  // and then takes a ticket; the holder of the last ticket turns the bits into the status code and
+  // leaves both words zero for the next call.  The ticket is taken here and looked at when the block
+  // leaves, so that its round trip is hidden behind the merge.
+  unsigned my_ticket = 0;
+  if (tid == 32 * kIssuer) {
+    if (aborted) atomicOr(p.tickets + 2 * b + 1, 2u);
+    if (aborted || (k.group == 0 && split == 0 && kvh == 0)) __threadfence();   // error bits before the ticket
+    my_ticket = atomicInc(p.tickets + 2 * b, (unsigned)p.blocks_per_seq - 1);  // wraps to 0
+  }
+  auto publish = [&]() {
+    if (tid != 32 * kIssuer || my_ticket != (unsigned)p.blocks_per_seq - 1) return;
+    __threadfence();
+    const unsigned bits = atomicExch(p.tickets + 2 * b + 1, 0u);
+    p.status[b] = (bits & 1u) ? CLV_ERR_TREE : (bits & 2u) ? CLV_ERR_TIMEOUT : CLV_OK;
+  };
+
+  // ---- merge.  Idle once all Q K^T of a block are done, which is when it arrives at the cluster
+  //      barrier: the Q tiles (staging of the rows to be sent), and all ring stages but those of the
+  //      last V tiles.  Two neighbouring stages receive; since other ranks write there, the place is a
+  //      function of the receiver's number of tiles.  A third one holds what goes with this block's
+  //      own rows: 16 bytes per row (reference, sum, scales of its halves) | where each row's output
+  //      starts | the weights of the final sum.
+  auto rx_index = [&](int tiles_of_rank) {
+    const int i = (2 * tiles_of_rank) % NST;
+    return i == NST - 1 ? 0 : i;
+  };
+  auto rank_tiles = [&](int d) {
+    return ((int)((unsigned)(d + 1) * (unsigned)k.p_total / (unsigned)CS) - (int)((unsigned)d * (unsigned)k.p_total / (unsigned)CS) + 1) / 2;
+  };
+  auto rx_meta = [&](uint32_t rx_base) { return rx_base + (uint32_t)((CS - 1) * per) * 256u; };   // behind the rows
+  const uint32_t rx = sRing + (uint32_t)rx_index(T) * kStage;
+  const uint32_t meta = sRing + (uint32_t)((rx_index(T) + 2) % NST) * kStage;
+  const uint32_t row_at = meta + 4096u, weights = meta + 8192u;
+  __syncwarp();
+  if (warp < kSoftmaxWarps) {
+    const int slot = k.slot, row = k.row, row_in_out = (b * N + k.node) * p.Hq + kvh * G + (row - (row / G) * G);
+    float2 ml = ms.ml[slot * BM + row];
+    float w0 = 1.f, w1 = 0.f;
+    if (!kRows2) {   // combine the slots' shares of the keys
+      const float2 a = ms.ml[row], c = ms.ml[BM + row];
+      ml.x = fmaxf(a.x, c.x);
+      const float mu = ml.x == -INFINITY ? 0.f : ml.x;
+      w0 = ex2(a.x - mu);   // ex2(-inf) = 0
+      w1 = ex2(c.x - mu);
+      ml.y = a.y * w0 + c.y * w1;
+    }
+    if (CS == 1) {
+      const float inv = ml.y > 0.f ? 1.f / ml.y : 0.f;
+      w0 *= inv;
+      w1 *= inv;
+      if (p.lse != nullptr && k.row_valid && (kRows2 || slot == 0)) p.lse[row_in_out] = (ml.x + log2f(ml.y)) * 0.6931471805599453f;
+    }
+    // the last P V of the accumulators this thread reads
+    const bool has0 = kRows2 ? k.my_tiles > 0 : T > 0, has1 = !kRows2 && T > 1;
+    if (!aborted) {
+      if (has0) mbar_drain(bar(B_LAST + (kRows2 ? slot : 0)), 0);
+      if (has1) mbar_drain(bar(B_LAST + 1), 0);
+    }
+    __syncwarp();
+    tc_fence_after();
+    // half a row (64 columns) at a time: bf16 output if the block is alone, else fp16 for the rank
+    // that finalises the row
+    const int seq_row = (kRows2 ? slot * BM : 0) + row;   // number of this row within the block
+    const uint32_t acc0 = (kRows2 ? k.tmem_O(slot) : k.tmem_O(0)) + k.lane_addr, acc1 = k.tmem_O(1) + k.lane_addr;
+#pragma unroll 1
+    for (int half = kRows2 ? 0 : slot; half < (kRows2 ? 2 : slot + 1); ++half) {
+      float v[64];
+      {
+        uint32_t u[64];
+        if (has0) {
+          tmem_ld_x64(acc0 + (uint32_t)(half * 64), u);
+          tmem_wait_ld();
+        }
+#pragma unroll
+        for (int j = 0; j < 64; ++j) v[j] = has0 ? __uint_as_float(u[j]) * w0 : 0.f;
+      }
+      if (has1) {
+#pragma unroll
+        for (int q = 0; q < 64; q += 32) {
+          uint32_t u[32];
+          tmem_ld_x32(acc1 + (uint32_t)(half * 64 + q), u);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[q + j] = fmaf(__uint_as_float(u[j]), w1, v[q + j]);
+        }
+      }
+      if (CS == 1) {   // into the Q tile's place and layout; TMA stores it
+        const uint32_t dst = smem0 + (kRows2 ? slot * kQTile : 0u) + (uint32_t)half * (kQTile / 2) + (uint32_t)row * 128u;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          st_shared16(dst + (uint32_t)((c ^ (row & 7)) << 4), pack_bf16(v[8 * c], v[8 * c + 1]), pack_bf16(v[8 * c + 2], v[8 * c + 3]),
+                      pack_bf16(v[8 * c + 4], v[8 * c + 5]), pack_bf16(v[8 * c + 6], v[8 * c + 7]));
+      } else {
+        float amax = 0.f;
+#pragma unroll
+        for (int j = 0; j < 64; j += 2) amax = max3(amax, fabsf(v[j]), fabsf(v[j + 1]));
+        // scale 2^lc with amax * 2^lc in [2^13, 2^14); lc is clamped so that the scale and its
+        // inverse are normal numbers (zeros stay zeros, inf or NaN stay what they are)
+        const int biased = (int)((__float_as_uint(amax) >> 23) & 255u);
+        const int lc = max(-100, min(100, 140 - biased));
+        const float up = __uint_as_float((uint32_t)(127 + lc) << 23);
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(meta + (uint32_t)seq_row * 16u + 8u + (uint32_t)half * 4u),
+                     "f"(__uint_as_float((uint32_t)(127 - lc) << 23)) : "memory");
+        // 256 bytes per row; 16-byte piece c of row r sits at c ^ (r & 15)
+        const uint32_t dst = smem0 + (uint32_t)seq_row * 256u;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          uint32_t h[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const __half2 hv = __floats2half2_rn(v[8 * c + 2 * e] * up, v[8 * c + 2 * e + 1] * up);
+            h[e] = *reinterpret_cast<const uint32_t*>(&hv);
+          }
+          st_shared16(dst + (uint32_t)(((half * 8 + c) ^ (row & 15)) << 4), h[0], h[1], h[2], h[3]);
+        }
+      }
+    }
+    if (CS > 1 && (kRows2 || slot == 0)) {
+      st_shared8(meta + (uint32_t)seq_row * 16u, ml.x, ml.y);
+      // where the row's output starts (in rows of 128), -1: the row does not exist
+      asm volatile("st.shared.b32 [%0], %1;" ::"r"(row_at + (uint32_t)seq_row * 4u), "r"(k.row_valid ? row_in_out : -1) : "memory");
+    }
+    fence_async_smem();
+    tc_fence_before();
+  }
+  __syncthreads();
+  if (warp == kIssuer) { tc_fence_after(); tmem_dealloc(k.tmem, kTmemCols); }
+
+  if (CS == 1) {
+    if (tid == 0) {
+#pragma unroll
+      for (int m = 0; m < Cfg<kRows2>::kQ; ++m) {
+        if (m >= users) break;
+        tma_store_4d(&tm.out, smem0 + m * kQTile, 0, kvh * G, (tile0 + m) * tile_nodes, b);
+        tma_store_4d(&tm.out, smem0 + m * kQTile + kQTile / 2, 64, kvh * G, (tile0 + m) * tile_nodes, b);
+      }
+      asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    }
+    publish();
+    return;
+  }
+
+  cluster_wait();   // every rank's receiving stages are idle
+  if (tid < CS && tid != split) {   // a peer's rows, then what goes with them
+    const int d = tid, f = min(R, d * per), n = min(R, f + per) - f;
+    if (n > 0) {
+      const uint32_t base = sRing + (uint32_t)rx_index(rank_tiles(d)) * kStage, at = (uint32_t)((split < d ? split : split - 1) * per);
+      const uint32_t their_bar = cluster_map(bar(B_RX), (uint32_t)d);
+      bulk_to_peer(cluster_map(base + at * 256u, (uint32_t)d), smem0 + (uint32_t)f * 256u, (uint32_t)n * 256u, their_bar);
+      bulk_to_peer(cluster_map(rx_meta(base) + at * 16u, (uint32_t)d), meta + (uint32_t)f * 16u, (uint32_t)n * 16u, their_bar);
+    }
+  }
+  mbar_drain(bar(B_RX), 0);
+  __syncwarp();
+  cluster_arrive();   // what this block was sent has arrived: its peers may leave
+  // ---- final rows.  First the weight of every source of a row (with the source's scales and the sum
+  //      of all in it): a thread per row; then 16 threads per row, 8 columns each.  Sources in rank
+  //      order, so that the result does not depend on timing.
+  auto source = [&](int q, int i) { return (uint32_t)((q < split ? q : q - 1) * per + i); };
+  auto row_out = [&](int i) {
+    int o;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(o) : "r"(row_at + (uint32_t)(first + i) * 4u));
+    return o;
+  };
+  for (int i = tid; i < mine; i += kThreads) {
+    float4 m[kMaxSplits];
+    float M = -INFINITY;
+#pragma unroll
+    for (int q = 0; q < kMaxSplits; ++q) {
+      m[q] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
+      if (q < CS)
+        asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(m[q].x), "=f"(m[q].y), "=f"(m[q].z), "=f"(m[q].w)
+                     : "r"(q == split ? meta + (uint32_t)(first + i) * 16u : rx_meta(rx) + source(q, i) * 16u));
+      M = fmaxf(M, m[q].x);
+    }
+    const float mu = M == -INFINITY ? 0.f : M;
+    float total = 0.f;
+#pragma unroll
+    for (int q = 0; q < kMaxSplits; ++q) {
+      m[q].x = ex2(m[q].x - mu);   // ex2(-inf) = 0
+      total = fmaf(m[q].y, m[q].x, total);
+    }
+    const float inv = total > 0.f ? 1.f / total : 0.f;
+#pragma unroll
+    for (int q = 0; q < kMaxSplits; ++q)
+      if (q < CS) st_shared8(weights + (uint32_t)(i * kMaxSplits + q) * 8u, m[q].x * m[q].z * inv, m[q].x * m[q].w * inv);
+    const int o = row_out(i);
+    if (p.lse != nullptr && o >= 0) p.lse[o] = (M + log2f(total)) * 0.6931471805599453f;
+  }
+  __syncthreads();
+  for (int it = tid; it < mine * 16; it += kThreads) {
+    const int i = it >> 4, c = it & 15, o = row_out(i);
+    const uint32_t at = (uint32_t)((c ^ ((first + i) & 15)) << 4);
+    float acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+#pragma unroll 4
+    for (int q = 0; q < CS; ++q) {
+      uint32_t u[4];
+      float w;
+      asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3])
+                   : "r"((q == split ? smem0 + (uint32_t)(first + i) * 256u : rx + source(q, i) * 256u) + at));
+      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w) : "r"(weights + (uint32_t)(i * kMaxSplits + q) * 8u + (uint32_t)(c >> 3) * 4u));
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 f = half2_bits_to_float2(u[e]);
+        acc[2 * e] = fmaf(f.x, w, acc[2 * e]);
+        acc[2 * e + 1] = fmaf(f.y, w, acc[2 * e + 1]);
+      }
+    }
+    if (o >= 0)
+      *reinterpret_cast<uint4*>(p.out + (int64_t)o * HD + c * 8) =
+          make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
+  }
+  __syncwarp();
+  cluster_wait();   // no block may leave while a copy still reads its shared memory
+  publish();
+}
+
+// ------------------------------------------------------------------------------------ host side
+bool encode(CUtensorMap* tm, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// bf16 tensor [rows][heads][128]; box = 64 elements x 1 head x box_rows, 128-byte swizzle
+bool make_map(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t heads, uint32_t box_rows) {
+  const cuuint64_t dims[3] = {(cuuint64_t)HD, heads, rows};
+  const cuuint64_t strides[2] = {(cuuint64_t)HD * 2, (cuuint64_t)HD * 2 * heads};
+  const cuuint32_t box[3] = {64, 1, box_rows};
+  return encode(tm, base, 3, dims, strides, box);
+}
+
+// Q and the output: [B][N][Hq][128], box = 64 elements x G heads x `nodes` nodes of one sequence, so
+// that nodes beyond the sequence's last are read as zeros and never written
+bool make_map_nodes(CUtensorMap* tm, const void* base, const clv_shape& s, uint32_t G, uint32_t nodes) {
+  const cuuint64_t dims[4] = {(cuuint64_t)HD, (cuuint64_t)s.n_q_heads, (cuuint64_t)s.n_nodes, (cuuint64_t)s.batch};
+  const cuuint64_t row = (cuuint64_t)HD * 2 * s.n_q_heads;
+  const cuuint64_t strides[3] = {(cuuint64_t)HD * 2, row, row * s.n_nodes};
+  const cuuint32_t box[4] = {64, G, nodes, 1};
+  return encode(tm, base, 4, dims, strides, box);
+}
+
+// The cache seen as [rows][heads][2 halves of d][64]: a box of 64 x box_rows x 2 x 1 in the order
+// (d, row, half, head) lands in shared memory as [half][row][64], the layout of a K or V stage, so a
+// tile of 128 neighbouring rows is one copy instead of four.
+bool make_map_halves(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t heads, uint32_t box_rows) {
+  const cuuint64_t dims[4] = {64, rows, 2, heads};
+  const cuuint64_t strides[3] = {(cuuint64_t)HD * 2 * heads, 128, (cuuint64_t)HD * 2};
+  const cuuint32_t box[4] = {64, box_rows, 2, 1};
+  return encode(tm, base, 4, dims, strides, box);
+}
+
+void* kernel_of(bool rows2) {
+  return rows2 ? reinterpret_cast<void*>(tree_attn_kernel<true>) : reinterpret_cast<void*>(tree_attn_kernel<false>);
+}
+
+// Once per device: the kernels' shared memory, and how many clusters of each size run at once (one
+// block per SM; a cluster lives inside one GPC, so sizes that do not divide a GPC's SMs leave some idle).
+int g_clusters[kMaxDevices][kMaxSplits + 1];
+
+cudaError_t set_up() {
+  for (int r = 0; r < 2; ++r) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel_of(r != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    if (e != cudaSuccess) return e;
+  }
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  for (int s = 1; s <= kMaxSplits; ++s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(s * sm_count()), 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = kSmem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)s;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, kernel_of(false), &cfg);
+    if (e != cudaSuccess) return e;
+    g_clusters[dev][s] = n > 0 ? n : 1;
+  }
+  return cudaSuccess;
+}
+
+struct AttnPlan {
+  bool rows2;
+  int tiles, groups, splits;
+};
+
+// Blocks along the rows and along the keys: the cheapest choice by a cost in SM cycles, rounds of
+// clusters over the machine times (key tiles of a block x cycles per tile + what a block takes
+// besides).  The figures are fitted to measurements of 22 shapes (batch 1-32, 1-8 row tiles, 350-16424
+// keys).
+AttnPlan make_plan(const clv_shape& s, int max_ctx_len, const int* clusters) {
+  const int G = s.n_q_heads / s.n_kv_heads;
+  const int tiles = (s.n_nodes + BM / G - 1) / (BM / G);   // row tiles of BM / G whole nodes
+  const int pieces = (max_ctx_len + PG - 1) / PG + (s.n_nodes + PG - 1) / PG;
+  const int64_t units = (int64_t)s.batch * s.n_kv_heads;
+  AttnPlan best = {false, tiles, tiles, 1};
+  double best_cost = 1e300;
+  for (int r = 0; r < 2; ++r) {
+    if (r && tiles < 2) break;
+    const int groups = r ? (tiles + 1) / 2 : tiles;
+    for (int sp = 1; sp <= kMaxSplits; ++sp) {
+      if (sp > 1 && pieces < 2 * sp) break;   // at least one key tile per block
+      const double rounds = (double)((units * groups + clusters[sp] - 1) / clusters[sp]);
+      const double key_tiles = (double)((pieces + sp - 1) / sp) * 0.5;
+      const double cost = rounds * (key_tiles * (r ? 3200.0 : 1650.0) + (sp == 1 ? 18000.0 : r ? 36000.0 : 22500.0));
+      if (cost < best_cost) { best_cost = cost; best = {r != 0, tiles, groups, sp}; }
+    }
+  }
+  return best;
+}
+
+}  // namespace
+
+bool tree_attn_supported(const clv_shape& s, const clv_kv_cache& c) {
+  const int G = s.n_q_heads / s.n_kv_heads;
+  if (G > BM) return false;                            // a row tile must hold at least one whole node
+  const int64_t cache_rows = c.paged ? (int64_t)c.n_pages * CLV_PAGE_SIZE : (int64_t)s.batch * c.cap_tokens;
+  if (cache_rows >= (1ll << 31) || (int64_t)s.batch * s.n_nodes * s.n_q_heads >= (1ll << 31)) return false;
+  return encode_fn() != nullptr;
+}
+
+cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const void* q, const void* k_tree,
+                             const void* v_tree, const int32_t* parent, const int32_t* ctx_len, int max_ctx_len,
+                             float scale, void* out, float* lse, int32_t* status, unsigned* tickets,
+                             cudaStream_t stream) {
+  static OncePerDevice once;
+  cudaError_t e = run_once_per_device(once, set_up);
+  if (e != cudaSuccess) return e;
+  int dev = 0;
+  e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const AttnPlan plan = make_plan(s, max_ctx_len, g_clusters[dev]);
+  const int G = s.n_q_heads / s.n_kv_heads;
+  alignas(64) Maps tm;
+  const uint64_t cache_rows = c.paged ? (uint64_t)c.n_pages * CLV_PAGE_SIZE : (uint64_t)s.batch * c.cap_tokens;
+  const uint64_t tree_rows = (uint64_t)s.batch * s.n_nodes;
+  if (!make_map_nodes(&tm.q, q, s, (uint32_t)G, (uint32_t)(BM / G)) ||
+      !make_map_nodes(&tm.out, out, s, (uint32_t)G, (uint32_t)(BM / G)) ||
+      !make_map(&tm.kc, c.k, cache_rows, s.n_kv_heads, PG) || !make_map(&tm.vc, c.v, cache_rows, s.n_kv_heads, PG) ||
+      !make_map(&tm.kt, k_tree, tree_rows, s.n_kv_heads, PG) || !make_map(&tm.vt, v_tree, tree_rows, s.n_kv_heads, PG))
+    return cudaErrorInvalidValue;
+  // whole-tile copies: only if the driver accepts the 4-D view (else the piece-wise copies do it all)
+  const bool pair_boxes = make_map_halves(&tm.kc2, c.k, cache_rows, s.n_kv_heads, BN) &&
+                          make_map_halves(&tm.vc2, c.v, cache_rows, s.n_kv_heads, BN);
+  if (!pair_boxes) { tm.kc2 = tm.kc; tm.vc2 = tm.vc; }
+
+  Params p;
+  p.pair_boxes = pair_boxes ? 1 : 0;
+  p.block_table = c.block_table;
+  p.parent = parent;
+  p.ctx_len = ctx_len;
+  p.out = static_cast<uint16_t*>(out);
+  p.lse = lse;
+  p.status = status;
+  const int64_t clusters = (int64_t)s.batch * s.n_kv_heads * plan.groups;
+  p.B = s.batch; p.N = s.n_nodes; p.Hq = s.n_q_heads; p.Hkv = s.n_kv_heads; p.G = G;
+  p.paged = c.paged; p.cap_tokens = c.cap_tokens; p.n_pages = c.n_pages; p.max_pages = c.max_pages_per_seq;
+  p.tiles = plan.tiles;
+  p.groups = plan.groups;
+  p.splits = plan.splits;
+  p.longest_first = (clusters * plan.splits > sm_count() && s.batch > 1 && s.batch <= 256) ? 1 : 0;
+  p.scale_log2 = scale * 1.4426950408889634f;
+  p.wait_limit = wait_limit_cycles();
+  p.tickets = tickets;
+  p.blocks_per_seq = s.n_kv_heads * plan.groups * plan.splits;
+
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(clusters * plan.splits), 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = kSmem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;  // the blocks that share row tiles
+  attr[0].val.clusterDim.x = (unsigned)plan.splits;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // set-up overlaps the previous kernel's tail
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return plan.rows2 ? cudaLaunchKernelEx(&cfg, tree_attn_kernel<true>, tm, p)
+                    : cudaLaunchKernelEx(&cfg, tree_attn_kernel<false>, tm, p);
+}
+
+}  // namespace clv

@@ -247,6 +247,38 @@ def test_attention_units_of_many_row_tiles(clv, oracle, paged):
     check_attention(oracle, w, st)
 
 
+@pytest.mark.parametrize("batch,hq,hkv,ctx,n_nodes", [
+    (5, 8, 8, (130, 700), 20),      # 40 units: the keys of a unit over 3 blocks
+    (3, 8, 8, (64, 1200), 33),      # 24 units: over 5
+    (11, 2, 2, (1, 900), 40),       # 22 units: over 6
+    (1, 15, 15, (2050, 2050), 65),  # 15 units: over 7 or 8, an odd number of tiles
+    (7, 32, 8, (60, 390), 96),      # three row tiles per unit and more units than half the machine: two per block
+])
+def test_attention_splits_and_row_tiles(clv, oracle, batch, hq, hkv, ctx, n_nodes):
+    cfg = W.small_config(batch=batch, n_q_heads=hq, n_kv_heads=hkv, ctx=ctx, n_nodes=n_nodes, vocab=64,
+                         seed=W.BASE_SEED + 31 * batch)
+    w = W.generate(cfg)
+    st = make_step(w)
+    st.tree_attn()
+    torch.cuda.synchronize()
+    check_attention(oracle, w, st)
+
+
+@pytest.mark.parametrize("n_nodes", [16, 128])
+def test_attention_scores_that_outgrow_the_first_tile(clv, oracle, n_nodes):
+    # Keys 128 times larger from position 300 on: scores rise by far more than 2^32 between the tiles,
+    # so the running reference of a row is replaced and its accumulator rescaled.  Scores reach about
+    # 500, where float32 resolves 6e-5: within the tolerance of the check.
+    cfg = W.small_config(batch=2, n_q_heads=8, n_kv_heads=2, ctx=(500, 1400), n_nodes=n_nodes, vocab=64,
+                         seed=W.BASE_SEED + 606)
+    w = W.generate(cfg)
+    w.k_cache[:, 300:] = _scale_bf16_by_pow2(w.k_cache[:, 300:], 7)
+    st = make_step(w)
+    st.tree_attn()
+    torch.cuda.synchronize()
+    check_attention(oracle, w, st)
+
+
 @pytest.mark.parametrize("n_nodes", [24, 128])   # one row tile per block / two row tiles per block
 def test_attention_wait_that_runs_out_is_reported_and_leaves_the_library_usable(clv, oracle, n_nodes):
     # Every on-chip wait of the attention kernel is bounded.  With the bound cut to a few dozen SM
