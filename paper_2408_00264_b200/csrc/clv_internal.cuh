@@ -12,7 +12,7 @@
 namespace clv {
 
 // ---- workspace layout -------------------------------------------------------------------------
-// [0, 256)                     header (reserved)
+// [0, 256)                     header: a queue's two counters (zero between calls), the rest reserved
 // [256, 256 + 4*kTickets)      arrival counters, zero between calls (self-resetting atomicInc)
 // [kWsFixedBytes, ...)         scratch for partial results (contents are garbage between calls)
 constexpr size_t kWsHeaderBytes = 256;
@@ -22,6 +22,7 @@ constexpr size_t kWsFixedBytes = kWsHeaderBytes + sizeof(unsigned) * (size_t)kTi
 inline unsigned* ws_tickets(void* ws) {
   return reinterpret_cast<unsigned*>(static_cast<char*>(ws) + kWsHeaderBytes);
 }
+inline unsigned* ws_queue(unsigned* tickets) { return tickets - kWsHeaderBytes / sizeof(unsigned); }
 inline void* ws_scratch(void* ws) { return static_cast<char*>(ws) + kWsFixedBytes; }
 
 // ---- argmax -----------------------------------------------------------------------------------
@@ -89,9 +90,9 @@ cudaError_t launch_lm_head_argmax(const void* hidden, int64_t ld_hidden, const v
 
 int rows_linear_splits(int rows, int in_dim, int out_dim, int n);
 cudaError_t launch_rows_linear(int n, const void* const* x, int64_t ld_x, const void* const* weight,
-                               int64_t ld_weight, const void* const* bias, int rows, int in_dim, int out_dim,
-                               float* const* out, int64_t ld_out, int splits, int64_t split_stride, int32_t* status,
-                               unsigned* tickets, cudaStream_t stream);
+                               int64_t ld_weight, int rows, int in_dim, int out_dim,
+                               float* const* out, int64_t ld_out, bool in_parts, int64_t split_stride, bool early_weights,
+                               int32_t* status, unsigned* tickets, cudaStream_t stream);
 
 // ---- one step of a Clover-2 draft head
 size_t draft_head_scratch_bytes(int rows, int hidden, int vocab);

@@ -3,12 +3,17 @@
 // v on ties.  The logits are never written: each 256 x 256 tile of them lives in tensor memory
 // only, and its row maxima go to one 64-bit key per row with atomicMax.
 //
-// A persistent block per SM walks (vocabulary tile, row block) pairs.  Warp 0 streams 64-wide
-// K chunks of the weight tile ([256 vocabulary rows][64]) and of the hidden rows ([2 x 128][64])
-// through a three-deep TMA ring, warp 1 issues tcgen05.mma (M 128, N 256, K 16; two accumulators
-// of 256 columns fill the tensor memory), warps 2..9 are the epilogue: one thread per row scans
-// the accumulator for the row's best (value, lowest index).  The weight matrix is read from HBM
+// A persistent block per SM takes (vocabulary tile, row block) pairs from a queue.  Warp 0 streams
+// 64-wide K chunks of the weight tile ([up to 256 vocabulary rows][64]) and of the hidden rows ([1 or 2 x
+// 128][64]) through a TMA ring, warp 1 issues tcgen05.mma (M 128, N = the tile's width, K 16; two
+// accumulators of 256 columns fill the tensor memory), warps 2..9 are the epilogue: one thread per row
+// scans the accumulator for the row's best (value, lowest index).  The weight matrix is read from HBM
 // once per row block; the hidden rows are re-read from L2 by every block.
+// With a handful of rows the kernel is a stream over the weights, and what is in flight sets its rate:
+// the ring is as deep as shared memory allows and holds only the rows there are (4 rows x 128256 x 4096:
+// 172.9 -> 159.5 us, the measured copy rate).  The width of a tile is chosen so that the tiles divide
+// evenly over the SMs (plan()).  With many rows the tensor core bounds it, at the power cap
+// (1024 rows: 795 -> 780 us, of which the queue is the most).
 #include <cuda_bf16.h>
 #include <limits.h>
 #include <math.h>
@@ -23,39 +28,40 @@ namespace {
 constexpr int kThreads = 320;
 constexpr int BM = 128;              // rows per accumulator
 constexpr int MB = 2 * BM;           // rows per block step (two accumulators)
-constexpr int BN = 256;              // vocabulary entries per tile
+constexpr int BN = 256;              // columns of an accumulator: the most vocabulary entries per tile
 constexpr int BK = 64;               // K elements per ring stage (one 128-byte swizzle row)
-constexpr int kStages = 3;
+constexpr int kMaxStages = 12;
+constexpr int kItems = 16;           // more than the ring, the accumulators and the producer's next item can hold at a time
 constexpr int kMaxProb = 3;          // products of one shape that one launch can take
 constexpr uint32_t kATile = BM * BK * 2;      // 16 KB
-constexpr uint32_t kWTile = BN * BK * 2;      // 32 KB
-constexpr uint32_t kStageBytes = 2 * kATile + kWTile;
-constexpr uint32_t kSmem = kStages * kStageBytes + 1024;
+constexpr uint32_t kSmemMost = 232448 - 1024;   // the ring (its alignment included); static shared memory is small
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kIdesc = make_idesc(BM, BN, false);
-constexpr uint32_t kIdescHalf = make_idesc(BM, BN / 2, false);
 
 struct Params {
   int M, K, V;
   int n_tiles, m_blocks;
-  int full_items;   // work items that are whole tiles; the rest are half tiles (128 vocabulary entries)
-  int n_items;
+  int bn;                     // vocabulary entries per tile, a multiple of 16
+  uint32_t idesc;
+  int stages;                 // depth of the ring
+  uint32_t stage_bytes;       // row operand tile(s), then the weight tile
+  int early_weights;          // no launch that may still be running writes the weights: ask for the first tiles before
+                              //   the previous kernel's results are waited for
   int32_t* ids;
-  float* out;                 // not NULL: the products (+ bias) are written here, fp32 [M, ld_out], and no argmax is taken
+  float* out;                 // not NULL: the products are written here, fp32 [M, ld_out], and no argmax is taken
   int n_prob;                 // with `out`: up to kMaxProb products of one shape in one launch, each with its own
-  float* outs[3];             //   operands (tensor maps), destination and bias; out == outs[0]
-  const uint16_t* biases[3];
+  float* outs[3];             //   operands (tensor maps) and destination; out == outs[0]
   int64_t ld_out;
   int k_splits;               // with `out`: the K axis is cut in this many parts, part s writes its partial
   int64_t out_split_stride;   //   products to out + s * out_split_stride (the reader adds the parts up)
-  int out_vec;                // `out`, its strides and `bias` allow 16-byte accesses
+  int out_vec;                // `out` and its strides allow 16-byte accesses
   int two_acc;                // M <= 128: the two accumulators alternate between tiles, so that the
                               //   epilogue of one tile runs under the MMAs of the next
   uint32_t a_tile_bytes;      // bytes one load of the row operand brings (a box of 8..128 rows)
   unsigned long long* keys;   // [M], zero between calls
+  unsigned* queue;            // [0] items handed out beyond each block's first, [1] blocks that have stopped drawing; zero between calls
   unsigned* counter;          // zero between calls
   unsigned* aborts;           // blocks that gave up a wait; zero between calls
-  int32_t* status;            // one word: CLV_OK or CLV_ERR_TIMEOUT
+  int32_t* status;            // CLV_OK or CLV_ERR_TIMEOUT; with `out` one word per product, which holds CLV_OK before the launch
   long long wait_limit;       // SM cycles a bounded wait may last
 };
 
@@ -69,50 +75,47 @@ __device__ __forceinline__ float round_bf16(float x) {
   return __bfloat162float(__float2bfloat16_rn(x));
 }
 
-// Work item -> (first vocabulary entry, entries, row block).  Items are whole tiles, all row
-// blocks of a tile in a row so that a weight tile is read from HBM once and from L2 afterwards;
-// when the last round would leave more than half of the blocks idle, its tiles are cut in two
-// halves of 128 entries so that twice as many blocks share it.
+// What a work item is: a vocabulary tile, a row block, with `out` also a part of the K axis and a
+// product.  Products are innermost, so that blocks working side by side read different weights; the
+// row blocks of a tile follow each other, so that a weight tile is read from HBM once and from L2
+// afterwards.
 struct Item {
-  int col0, cols, mb;
+  int col0, mb, prob, part;
 };
 __device__ __forceinline__ Item decode_item(const Params& p, int item) {
-  int tile = item, half = -1;
-  if (item >= p.full_items) {
-    const int j = item - p.full_items;
-    tile = p.full_items + (j >> 1);
-    half = j & 1;
-  }
-  const int n = tile / p.m_blocks;
+  const int per_tile = p.k_splits * p.n_prob;
+  const int tile = item / per_tile, sub = item - tile * per_tile, n = tile / p.m_blocks;
   Item it;
+  it.part = sub / p.n_prob;
+  it.prob = sub - it.part * p.n_prob;
   it.mb = tile - n * p.m_blocks;
-  it.col0 = n * BN + (half > 0 ? BN / 2 : 0);
-  it.cols = half < 0 ? BN : BN / 2;
+  it.col0 = n * p.bn;
   return it;
 }
 
 struct Maps {
-  CUtensorMap a[kMaxProb], w[kMaxProb], w_half;   // w_half: 128-entry boxes of w[0] (single product only)
+  CUtensorMap a[kMaxProb], w[kMaxProb];
 };
 
 __global__ void __launch_bounds__(kThreads, 1)
 lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) unsigned long long s_bar[2 * kStages + 5];
+  __shared__ __align__(8) unsigned long long s_bar[2 * kMaxStages + 5];
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
   __shared__ int s_last;
+  __shared__ volatile int s_item[kItems];   // the block's items in turn, -1 behind the last
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t bar0 = smem_u32(&s_bar[0]);
   auto bar_full = [&](int s) { return bar0 + 8u * s; };
-  auto bar_empty = [&](int s) { return bar0 + 8u * (kStages + s); };
+  auto bar_empty = [&](int s) { return bar0 + 8u * (kMaxStages + s); };
   // a tile's accumulators are complete / the epilogue has read them; index 1 only with two_acc
-  auto bar_acc_full = [&](int b) { return bar0 + 8u * (2 * kStages + b); };
-  auto bar_acc_empty = [&](int b) { return bar0 + 8u * (2 * kStages + 2 + b); };
-  const uint32_t bar_drain = bar0 + 8u * (2 * kStages + 4);
+  auto bar_acc_full = [&](int b) { return bar0 + 8u * (2 * kMaxStages + b); };
+  auto bar_acc_empty = [&](int b) { return bar0 + 8u * (2 * kMaxStages + 2 + b); };
+  const uint32_t bar_drain = bar0 + 8u * (2 * kMaxStages + 4);
   if (tid == 0) {
-    for (int i = 0; i < 2 * kStages; ++i) mbar_init(bar0 + 8u * i, 1);
+    for (int i = 0; i < 2 * kMaxStages; ++i) mbar_init(bar0 + 8u * i, 1);
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar_acc_full(b), 1);
       mbar_init(bar_acc_empty(b), p.two_acc ? BM : 2 * BM);
@@ -126,18 +129,8 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
   if (tid >= 64 && tid < 64 + p.n_prob) {
     tma_prefetch_desc(&tm.a[tid - 64]);
     tma_prefetch_desc(&tm.w[tid - 64]);
-    if (tid == 64) tma_prefetch_desc(&tm.w_half);
   }
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  if (p.a_tile_bytes < kATile) {
-    // a box of fewer than 128 rows leaves the rest of the operand tile as it was: make that zeros
-    uint8_t* base = smem_raw + (smem_base - smem_u32(smem_raw));
-    for (int s = 0; s < kStages; ++s)
-      for (uint32_t o = (uint32_t)tid * 16u; o < kATile; o += kThreads * 16u)
-        *reinterpret_cast<uint4*>(base + (size_t)s * kStageBytes + o) = make_uint4(0u, 0u, 0u, 0u);
-    fence_async_smem();
-  }
-  cudaGridDependencySynchronize();  // programmatic launch: the previous kernel's results are complete
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -145,74 +138,108 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
   volatile int* abort_flag = &s_abort;
   const long long wlim = p.wait_limit;
 
-  auto sA = [&](int s, int mt) { return smem_base + (uint32_t)s * kStageBytes + (uint32_t)mt * kATile; };
-  auto sW = [&](int s) { return smem_base + (uint32_t)s * kStageBytes + 2 * kATile; };
-
-  // work item -> (tile and row block, part of the K axis, product): products innermost, so that
-  // blocks working side by side read different weights
-  const int per_tile = p.k_splits * p.n_prob;
-  const int n_items = p.n_items * per_tile;
+  // Within a stage: the row operand, then the weight tile.  With fewer than 128 rows the operand takes the
+  // box that was loaded; the rest of its 128 rows is whatever lies behind it (the weights): rows of
+  // a product do not mix, and nobody reads those.
+  const uint32_t w_at = p.two_acc ? p.a_tile_bytes : 2u * kATile;
+  auto sA = [&](int s, int mt) { return smem_base + (uint32_t)s * p.stage_bytes + (uint32_t)mt * kATile; };
+  auto sW = [&](int s) { return smem_base + (uint32_t)s * p.stage_bytes + w_at; };
+  const int n_items = p.n_tiles * p.m_blocks * p.k_splits * p.n_prob;
   const int k_chunks = p.K / BK / p.k_splits;
   int issued = 0;  // ring stages filled by the producer (for the drain)
+  if (!p.early_weights || warp != 0) cudaGridDependencySynchronize();  // programmatic launch: the previous kernel's results are complete
+  cudaTriggerProgrammaticLaunchCompletion();
 
   if (warp == 0) {
     // =========================== TMA producer ===============================================
+    // A block's first item is its number; the others come from a queue, because the SMs do not get
+    // equal shares of the memory's bandwidth (with equal numbers of tiles the fastest was done after
+    // 0.75 of the time of the slowest).
     if (lane == 0) {
       bool ok = true;
-      int it = 0;
-      for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-        const Item wi = decode_item(p, item / per_tile);
-        const int sub = item % per_tile, prob = sub % p.n_prob;
-        const int kc0 = (sub / p.n_prob) * k_chunks;
-        const int mb = wi.mb;
-        const int rows_left = p.M - mb * MB;
-        const int m_tiles = rows_left > BM ? 2 : 1;
-        const uint32_t w_bytes = (uint32_t)wi.cols * BK * 2;
-        for (int kc = 0; kc < k_chunks && ok; ++kc, ++it) {
-          const int s = it % kStages;
-          if (it >= kStages) ok = mbar_wait(bar_empty(s), ((it / kStages) - 1) & 1, abort_flag, wlim);
-          if (!ok) break;
-          mbar_expect_tx(bar_full(s), w_bytes + (uint32_t)m_tiles * p.a_tile_bytes);
-          tma_load_2d(sW(s), wi.cols == BN ? &tm.w[prob] : &tm.w_half, (kc0 + kc) * BK, wi.col0, bar_full(s));
-          for (int mt = 0; mt < m_tiles; ++mt)
-            tma_load_2d(sA(s, mt), &tm.a[prob], (kc0 + kc) * BK, mb * MB + mt * BM, bar_full(s));
-          issued = it + 1;
-        }
+      int s = 0, n = 0, item = blockIdx.x;
+      uint32_t round = 0;
+      auto load_w = [&](const Item& wi, int chunk, int st) {
+        mbar_expect_tx(bar_full(st), (uint32_t)p.bn * BK * 2 + ((p.M - wi.mb * MB) > BM ? 2u : 1u) * p.a_tile_bytes);
+        tma_load_2d(sW(st), &tm.w[wi.prob], (wi.part * k_chunks + chunk) * BK, wi.col0, bar_full(st));
+      };
+      int early = 0;
+      if (p.early_weights) {   // the weights of the first item's first stages; the rows follow below
+        const Item wi = decode_item(p, item);
+        early = min(p.stages, k_chunks);
+        for (int i = 0; i < early; ++i) load_w(wi, i, i);
+        cudaGridDependencySynchronize();
       }
+      for (; ok; ++n) {
+        const bool end = item >= n_items;
+        unsigned ticket = 0;
+        if (!end) ticket = atomicAdd(p.queue, 1u);   // the next item, looked at when this one has been asked for
+        const Item wi = decode_item(p, item);
+        if (end) s_item[(n + 1) % kItems] = -1;
+        s_item[n % kItems] = end ? -1 : item;
+        for (int kc = 0; kc < (end ? 1 : k_chunks) && ok; ++kc) {
+          if (issued >= p.stages) ok = mbar_wait(bar_empty(s), (round & 1u) ^ 1u, abort_flag, wlim);
+          if (!ok) break;
+          if (end) {
+            mbar_arrive(bar_full(s));   // nothing to load: the issuer finds the end in s_item
+          } else {
+            if (issued >= early) load_w(wi, kc, s);
+            for (int mt = 0; mt < ((p.M - wi.mb * MB) > BM ? 2 : 1); ++mt)
+              tma_load_2d(sA(s, mt), &tm.a[wi.prob], (wi.part * k_chunks + kc) * BK, wi.mb * MB + mt * BM, bar_full(s));
+          }
+          ++issued;
+          if (++s == p.stages) { s = 0; ++round; }
+        }
+        if (end) break;
+        item = (int)(ticket + gridDim.x);
+      }
+      // the last block to stop drawing leaves the queue empty for the next call
+      __threadfence();
+      if (atomicInc(p.queue + 1, gridDim.x - 1) == gridDim.x - 1) *p.queue = 0u;
     }
   } else if (warp == 1) {
     // =========================== MMA issuer ===================================================
-    if (lane == 0) {
-      bool ok = true;
-      int it = 0, tile = 0;
-      for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++tile) {
-        const Item wi = decode_item(p, item / per_tile);
-        const int m_tiles = (p.M - wi.mb * MB) > BM ? 2 : 1;
-        const uint32_t idesc = wi.cols == BN ? kIdesc : kIdescHalf;
-        const int acc = p.two_acc ? (tile & 1) : 0;          // accumulator (pair) of this tile
-        const int use = p.two_acc ? (tile >> 1) : tile;      // how often it has been used before
-        if (use > 0) {  // the epilogue has taken its previous tile out of tensor memory
-          ok = mbar_wait(bar_acc_empty(acc), (use - 1) & 1, abort_flag, wlim);
-          if (!ok) break;
-          tc_fence_after();
-        }
-        for (int kc = 0; kc < k_chunks && ok; ++kc, ++it) {
-          const int s = it % kStages;
-          ok = mbar_wait(bar_full(s), (it / kStages) & 1, abort_flag, wlim);
-          if (!ok) break;
-          tc_fence_after();
-          const uint64_t wd = smem_desc(sW(s), 16, 1024);
-          for (int mt = 0; mt < m_tiles; ++mt) {
-            const uint64_t ad = smem_desc(sA(s, mt), 16, 1024);
-#pragma unroll
-            for (int ks = 0; ks < BK / 16; ++ks)
-              umma_bf16(tmem + (uint32_t)((mt + acc) * BN), ad + (uint64_t)((ks * 32) >> 4), wd + (uint64_t)((ks * 32) >> 4),
-                        idesc, (kc > 0 || ks > 0) ? 1u : 0u);
-          }
-          umma_commit(bar_empty(s));  // the stage is free once these MMAs have read it
-        }
-        if (ok) umma_commit(bar_acc_full(acc));
+    // The whole warp walks the schedule and one elected lane issues.
+    const uint32_t el = elect_one();
+    bool ok = true;
+    int s = 0;
+    uint32_t round = 0;
+    // accumulator (pair) of tile t is free: the epilogue has taken its previous tile out of tensor memory
+    auto acc_free = [&](int t) {
+      const int acc = p.two_acc ? (t & 1) : 0, use = p.two_acc ? (t >> 1) : t;
+      if (use > 0 && !wait_warp(bar_acc_empty(acc), (use - 1) & 1, abort_flag, wlim)) return false;
+      tc_fence_after();
+      return true;
+    };
+    for (int tile = 0; ok; ++tile) {
+      ok = wait_warp(bar_full(s), round & 1u, abort_flag, wlim);
+      if (!ok) break;
+      const int item = __shfl_sync(0xFFFFFFFFu, (int)s_item[tile % kItems], 0);
+      ok = acc_free(tile);
+      if (!ok) break;
+      const int acc = p.two_acc ? (tile & 1) : 0;
+      if (item < 0) {   // tell the epilogue's groups: with two_acc each waits for an accumulator of its own
+        umma_commit_if(el, bar_acc_full(acc));
+        if (p.two_acc && acc_free(tile + 1)) umma_commit_if(el, bar_acc_full(acc ^ 1));
+        break;
       }
+      const int m_tiles = (p.M - decode_item(p, item).mb * MB) > BM ? 2 : 1;
+      for (int kc = 0; kc < k_chunks && ok; ++kc) {
+        if (kc > 0) ok = wait_warp(bar_full(s), round & 1u, abort_flag, wlim);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t wd = smem_desc(sW(s), 16, 1024);
+        for (int mt = 0; mt < m_tiles; ++mt) {
+          const uint64_t ad = smem_desc(sA(s, mt), 16, 1024);
+#pragma unroll
+          for (int ks = 0; ks < BK / 16; ++ks)
+            umma_bf16_if(el, tmem + (uint32_t)((mt + acc) * BN), ad + (uint64_t)((ks * 32) >> 4), wd + (uint64_t)((ks * 32) >> 4),
+                         p.idesc, (kc > 0 || ks > 0) ? 1u : 0u);
+        }
+        umma_commit_if(el, bar_empty(s));  // the stage is free once these MMAs have read it
+        if (++s == p.stages) { s = 0; ++round; }
+      }
+      if (ok) umma_commit_if(el, bar_acc_full(acc));
     }
   } else {
     // =========================== epilogue: one thread per row ==================================
@@ -220,64 +247,39 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
     const int quarter = warp & 3;            // tensor-memory lanes this warp may touch
     const int row_in_tile = quarter * 32 + lane;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-    bool ok = true;
-    int tile = 0;
-    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++tile) {
-      const Item wi = decode_item(p, item / per_tile);
-      const int sub = item % per_tile, prob = sub % p.n_prob, part = sub / p.n_prob;
-      const int mb = wi.mb;
-      if (p.two_acc && (tile & 1) != mt) continue;   // the other group's tile
+    for (int tile = p.two_acc ? mt : 0;; tile += p.two_acc ? 2 : 1) {
       const int acc = p.two_acc ? mt : 0;
-      const int row = mb * MB + (p.two_acc ? 0 : mt * BM) + row_in_tile;
-      const bool row_valid = row < p.M;
-      ok = mbar_wait(bar_acc_full(acc), (p.two_acc ? (tile >> 1) : tile) & 1, abort_flag, wlim);
-      ok = __all_sync(0xFFFFFFFFu, ok);
-      if (!ok) break;
+      if (!wait_warp(bar_acc_full(acc), (p.two_acc ? (tile >> 1) : tile) & 1, abort_flag, wlim)) break;
+      const int item = s_item[tile % kItems];
+      if (item < 0) break;
       tc_fence_after();
+      const Item wi = decode_item(p, item);
+      const int row = wi.mb * MB + (p.two_acc ? 0 : mt * BM) + row_in_tile;
+      const int lim = min(p.V, wi.col0 + p.bn);   // end of the tile's columns
+      const bool row_valid = row < p.M;
       // the second accumulator is unused for a short row block
-      const bool group_used = p.two_acc || (p.M - mb * MB) > mt * BM;
+      const bool group_used = p.two_acc || (p.M - wi.mb * MB) > mt * BM;
       float best_v = -INFINITY;
       int best_i = INT_MAX;
       if (group_used) {
-        const int col0 = wi.col0;
 #pragma unroll 1
-        for (int c = 0; c < wi.cols; c += 32) {
+        for (int c = 0; c < p.bn; c += 32) {
           uint32_t x[32];
           tmem_ld_x32(tmem + lane_addr + (uint32_t)(mt * BN + c), x);
           tmem_wait_ld();
-          if (p.out != nullptr) {   // plain product: this row's 32 values (+ bias) go to memory
+          if (p.out != nullptr) {   // plain product: this row's 32 values go to memory
             if (row_valid) {
-              const uint16_t* bias = p.biases[0];
-              float* dst = p.outs[0];
-              if (prob == 1) { bias = p.biases[1]; dst = p.outs[1]; }
-              if (prob == 2) { bias = p.biases[2]; dst = p.outs[2]; }
-              dst += part * p.out_split_stride + (int64_t)row * p.ld_out + col0 + c;
-              const bool add_bias = bias != nullptr && part == 0;
-              if (p.out_vec && col0 + c + 32 <= p.V) {   // 128 bytes of this row in eight stores
-                if (add_bias) {
-                  const uint4* b4 = reinterpret_cast<const uint4*>(bias + col0 + c);
+              float* dst = (wi.prob == 0 ? p.outs[0] : wi.prob == 1 ? p.outs[1] : p.outs[2]) +
+                           wi.part * p.out_split_stride + (int64_t)row * p.ld_out + wi.col0 + c;
 #pragma unroll
-                  for (int j = 0; j < 4; ++j) {
-                    const uint4 b = b4[j];
-                    const uint32_t w[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                      x[8 * j + 2 * t] = __float_as_uint(__uint_as_float(x[8 * j + 2 * t]) + __uint_as_float(w[t] << 16));
-                      x[8 * j + 2 * t + 1] =
-                          __float_as_uint(__uint_as_float(x[8 * j + 2 * t + 1]) + __uint_as_float(w[t] & 0xFFFF0000u));
-                    }
-                  }
-                }
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
+              for (int j = 0; j < 8; ++j) {   // four values at a time; the last of a tile or row one by one
+                const int at = wi.col0 + c + 4 * j;
+                if (p.out_vec && at + 4 <= lim) {
                   reinterpret_cast<uint4*>(dst)[j] = make_uint4(x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
-              } else {
+                } else {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                  if (col0 + c + j >= p.V) continue;
-                  float v = __uint_as_float(x[j]);
-                  if (add_bias) v += __uint_as_float((uint32_t)bias[col0 + c + j] << 16);
-                  dst[j] = v;
+                  for (int t = 0; t < 4; ++t)
+                    if (at + t < lim) dst[4 * j + t] = __uint_as_float(x[4 * j + t]);
                 }
               }
             }
@@ -287,7 +289,7 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
           float m = -INFINITY;
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
-            const float v = (col0 + c + j < p.V) ? __uint_as_float(x[j]) : -INFINITY;
+            const float v = (wi.col0 + c + j < lim) ? __uint_as_float(x[j]) : -INFINITY;
             x[j] = __float_as_uint(v);
             m = fmaxf(m, v);   // NaN operands are dropped
           }
@@ -298,7 +300,7 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
             for (int j = 31; j >= 0; --j)
               if (round_bf16(__uint_as_float(x[j])) == mr) first = j;
             best_v = mr;
-            best_i = col0 + c + first;
+            best_i = wi.col0 + c + first;
           }
         }
       }
@@ -312,15 +314,20 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
   __syncwarp();
   if (*abort_flag) {
     if (warp == 0 && lane == 0)
-      for (int i = max(0, issued - kStages); i < issued; ++i) mbar_drain(bar_full(i % kStages), (i / kStages) & 1);
-    if (warp == 1 && lane == 0) {
-      umma_commit(bar_drain);
+      for (int i = max(0, issued - p.stages); i < issued; ++i) mbar_drain(bar_full(i % p.stages), (i / p.stages) & 1);
+    if (warp == 1) {
+      umma_commit_if(elect_one(), bar_drain);
       mbar_drain(bar_drain, 0);
     }
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, kTmemCols);
+  if (p.out != nullptr) {   // no keys were written
+    if (tid == 0 && *abort_flag)
+      for (int i = 0; i < p.n_prob; ++i) p.status[i] = CLV_ERR_TIMEOUT;
+    return;
+  }
   if (tid == 0) {
     if (*abort_flag) atomicAdd(p.aborts, 1u);
     __threadfence();
@@ -331,11 +338,7 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
   if (!s_last) return;
   // the last block turns the keys into indices and leaves keys and counters zero for the next call
   __threadfence();
-  if (tid == 0) {   // one status word per product
-    const int verdict = atomicExch(p.aborts, 0u) ? (int)CLV_ERR_TIMEOUT : (int)CLV_OK;
-    for (int i = 0; i < p.n_prob; ++i) p.status[i] = verdict;
-  }
-  if (p.out != nullptr) return;   // no keys were written
+  if (tid == 0) p.status[0] = atomicExch(p.aborts, 0u) ? (int)CLV_ERR_TIMEOUT : (int)CLV_OK;
   for (int r = tid; r < p.M; r += kThreads) {
     const unsigned long long key = atomicExch(p.keys + r, 0ull);
     const int idx = (int)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
@@ -364,20 +367,45 @@ bool lm_head_supported(int rows, int hidden, int vocab) {
 }
 
 namespace {
-struct Product {   // one product of a launch: rows x[rows, K] times weight[vocab, K]^T (+ bias) -> out
+// How a product is cut: vocabulary entries per tile and parts of the K axis.  A tile of bn entries and
+// k_chunks chunks takes about k_chunks * bn * 5.6 cycles when it streams weights from HBM (one SM's
+// share of the bandwidth) or 4.3 of tensor core (16 columns more count for what a narrow tile costs: the
+// rows are read more often), and some more per tile; what counts is the number of rounds over the SMs
+// times that.  60 rows x vocabulary 32000 x 4096: 143 tiles of 224 keep 143 SMs busy where 125 tiles of
+// 256 left 23 idle, 51.2 -> 47.4 us.  Below 128 entries a stage of the ring would bring too little.
+struct Cut {
+  int bn, splits;
+};
+Cut plan(int rows, int in_dim, int out_dim, int n, bool may_split) {
+  const int m_blocks = (rows + MB - 1) / MB, chunks = in_dim / BK;
+  const bool stream = rows <= BM;
+  Cut best = {BN, 1};
+  double best_cost = 1e300;
+  for (int sp = 1; sp <= (may_split ? 8 : 1); sp *= 2) {
+    if (chunks % sp) break;
+    for (int bn = BN; bn >= 128; bn -= 16) {
+      const int64_t items = (int64_t)((out_dim + bn - 1) / bn) * m_blocks * n * sp;
+      const double rounds = (double)((items + sm_count() - 1) / sm_count());
+      const double cost = rounds * ((double)(chunks / sp) * (stream ? bn * 5.6 : (bn + 16) * 4.3) + (stream ? 700.0 : 4000.0)) + 200.0 * sp;
+      if (cost < best_cost) { best_cost = cost; best = {bn, sp}; }
+    }
+  }
+  return best;
+}
+
+struct Product {   // one product of a launch: rows x[rows, K] times weight[vocab, K]^T -> out
   const void* x;
   const void* weight;
-  const void* bias;
   float* out;
 };
 
 cudaError_t launch_rows_times_weights(int n_prob, const Product* pr, int64_t ld_hidden, int64_t ld_weight, int rows,
-                                      int hidden_dim, int vocab, int32_t* ids, int64_t ld_out, int k_splits,
-                                      int64_t out_split_stride, int32_t* status, unsigned* tickets,
+                                      int hidden_dim, int vocab, int32_t* ids, int64_t ld_out, Cut cut,
+                                      int64_t out_split_stride, bool early_weights, int32_t* status, unsigned* tickets,
                                       cudaStream_t stream) {
   static OncePerDevice once;
   cudaError_t e0 = run_once_per_device(once, [] {
-    return cudaFuncSetAttribute(lm_head_argmax_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    return cudaFuncSetAttribute(lm_head_argmax_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMost);
   });
   if (e0 != cudaSuccess) return e0;
   if (n_prob < 1 || n_prob > kMaxProb) return cudaErrorInvalidValue;
@@ -389,44 +417,43 @@ cudaError_t launch_rows_times_weights(int n_prob, const Product* pr, int64_t ld_
   for (int i = 0; i < kMaxProb; ++i) {
     const Product& q = pr[i < n_prob ? i : 0];   // unused slots repeat the first product
     if (!make_map_2d(&tm.a[i], q.x, (uint64_t)rows, (uint64_t)hidden_dim, ld_hidden, (uint32_t)a_box) ||
-        !make_map_2d(&tm.w[i], q.weight, (uint64_t)vocab, (uint64_t)hidden_dim, ld_weight, BN))
+        !make_map_2d(&tm.w[i], q.weight, (uint64_t)vocab, (uint64_t)hidden_dim, ld_weight, (uint32_t)cut.bn))
       return cudaErrorInvalidValue;
     p.outs[i] = q.out;
-    p.biases[i] = static_cast<const uint16_t*>(q.bias);
-    vec = vec && (reinterpret_cast<uintptr_t>(q.out) % 16) == 0 && (reinterpret_cast<uintptr_t>(q.bias) % 16) == 0;
+    vec = vec && (reinterpret_cast<uintptr_t>(q.out) % 16) == 0;
   }
-  if (!make_map_2d(&tm.w_half, pr[0].weight, (uint64_t)vocab, (uint64_t)hidden_dim, ld_weight, BN / 2))
-    return cudaErrorInvalidValue;
   p.M = rows;
   p.K = hidden_dim;
   p.V = vocab;
-  p.n_tiles = (vocab + BN - 1) / BN;
+  p.n_tiles = (vocab + cut.bn - 1) / cut.bn;
+  p.bn = cut.bn;
+  p.idesc = make_idesc(BM, cut.bn, false);
   p.m_blocks = (rows + MB - 1) / MB;
   p.ids = ids;
   p.out = pr[0].out;
   p.n_prob = n_prob;
   p.ld_out = ld_out;
-  p.k_splits = k_splits;
+  p.k_splits = cut.splits;
+  p.early_weights = early_weights;
   p.out_split_stride = out_split_stride;
   p.out_vec = p.out != nullptr && vec;
   p.two_acc = rows <= BM;
   p.a_tile_bytes = (uint32_t)a_box * BK * 2;
+  p.queue = ws_queue(tickets);
   p.counter = tickets;
   p.aborts = tickets + 1;
   p.keys = reinterpret_cast<unsigned long long*>(tickets + 2);
   p.status = status;
   p.wait_limit = wait_limit_cycles();
-  const int tiles = p.n_tiles * p.m_blocks;
-  const int work = tiles * k_splits * n_prob;
+  p.stage_bytes = (p.two_acc ? p.a_tile_bytes : 2u * kATile) + (uint32_t)cut.bn * BK * 2;   // >= 16 KB: an operand ends inside
+  p.stages = (int)((kSmemMost - 1024) / p.stage_bytes);
+  if (p.stages > kMaxStages) p.stages = kMaxStages;
+  const int work = p.n_tiles * p.m_blocks * cut.splits * n_prob;
   const int grid = work < sm_count() ? work : sm_count();
-  const int rem = tiles % grid;   // tiles of the last, incomplete round
-  const int split = (k_splits == 1 && n_prob == 1 && rem > 0 && 2 * rem <= grid) ? rem : 0;
-  p.full_items = tiles - split;
-  p.n_items = tiles + split;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = kSmem;
+  cfg.dynamicSmemBytes = p.stages * p.stage_bytes + 1024;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -440,35 +467,29 @@ cudaError_t launch_rows_times_weights(int n_prob, const Product* pr, int64_t ld_
 cudaError_t launch_lm_head_argmax(const void* hidden, int64_t ld_hidden, const void* weight, int64_t ld_weight,
                                   int rows, int hidden_dim, int vocab, int32_t* ids, int32_t* status,
                                   unsigned* tickets, cudaStream_t stream) {
-  const Product pr = {hidden, weight, nullptr, nullptr};
-  return launch_rows_times_weights(1, &pr, ld_hidden, ld_weight, rows, hidden_dim, vocab, ids, 0, 1, 0, status,
-                                   tickets, stream);
+  const Product pr = {hidden, weight, nullptr};
+  return launch_rows_times_weights(1, &pr, ld_hidden, ld_weight, rows, hidden_dim, vocab, ids, 0,
+                                   plan(rows, hidden_dim, vocab, 1, false), 0, false, status, tickets, stream);
 }
 
-// How many parts the K axis of a product with few output features is cut into, so that the launch
-// covers the machine: a power of two up to 8 that divides the number of 64-wide K chunks.
-// `n` products of one shape share the launch; up to three rounds of blocks are accepted.
-int rows_linear_splits(int rows, int in_dim, int out_dim, int n) {
-  const int tiles = ((out_dim + BN - 1) / BN) * ((rows + MB - 1) / MB) * n;
-  int s = 1;
-  while (s < 8 && tiles * s * 2 <= 3 * sm_count() && (in_dim / BK) % (s * 2) == 0) s *= 2;
-  return s;
-}
+// How many parts the K axis of `n` products of one shape in one launch is cut into.
+int rows_linear_splits(int rows, int in_dim, int out_dim, int n) { return plan(rows, in_dim, out_dim, n, true).splits; }
 
-// out[i][part][r][o] = sum over part's share of k of x[i][r][k] * weight[i][o][k] (+ bias[i][o] in
-// part 0) for n products of one shape (n <= 3) in one launch: the same kernel with its
-// accumulators written out (fp32) instead of reduced to an argmax.  The reader adds the `splits`
-// parts up (a fixed order: the result does not depend on scheduling).  status gets one word per
-// product.
+// out[i][part][r][o] = sum over part's share of k of x[i][r][k] * weight[i][o][k] for n products of one shape (n <= 3) in one launch: the same kernel with its
+// accumulators written out (fp32) instead of reduced to an argmax.  in_parts: the reader adds
+// rows_linear_splits() parts up (a fixed order: the result does not depend on scheduling); else there
+// is one.  status: one word per product, CLV_OK before the launch.  early_weights: no launch that may
+// still be running when this one starts writes any of the weights, so the first tiles of them are
+// asked for without waiting.
 cudaError_t launch_rows_linear(int n, const void* const* x, int64_t ld_x, const void* const* weight,
-                               int64_t ld_weight, const void* const* bias, int rows, int in_dim, int out_dim,
-                               float* const* out, int64_t ld_out, int splits, int64_t split_stride, int32_t* status,
-                               unsigned* tickets, cudaStream_t stream) {
+                               int64_t ld_weight, int rows, int in_dim, int out_dim,
+                               float* const* out, int64_t ld_out, bool in_parts, int64_t split_stride, bool early_weights,
+                               int32_t* status, unsigned* tickets, cudaStream_t stream) {
   if (n < 1 || n > kMaxProb) return cudaErrorInvalidValue;
   Product pr[kMaxProb];
-  for (int i = 0; i < n; ++i) pr[i] = Product{x[i], weight[i], bias[i], out[i]};
-  return launch_rows_times_weights(n, pr, ld_x, ld_weight, rows, in_dim, out_dim, nullptr, ld_out, splits,
-                                   split_stride, status, tickets, stream);
+  for (int i = 0; i < n; ++i) pr[i] = Product{x[i], weight[i], out[i]};
+  return launch_rows_times_weights(n, pr, ld_x, ld_weight, rows, in_dim, out_dim, nullptr, ld_out,
+                                   plan(rows, in_dim, out_dim, n, in_parts), split_stride, early_weights, status, tickets, stream);
 }
 
 }  // namespace clv

@@ -78,6 +78,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
   }
 }
+// bounded wait of a whole warp for a phase of a barrier: the same verdict for every lane
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit) {
+  return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag, limit)) != 0;
+}
 // Teardown only: waits for work that is already in flight (a TMA copy, issued MMAs) and therefore
 // always keeps the long bound, whatever limit the block's other waits had.
 __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
@@ -115,22 +119,9 @@ __device__ __forceinline__ void tmem_alloc(uint32_t slot_smem, uint32_t cols) {
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
-// D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate; issued by one thread.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// The same for a warp in which every lane holds the operands and one lane (`leader` not 0) issues: no
-// divergent branch, so the operands stay in uniform registers.
+// D[tmem] (+)= A * B, bf16 inputs, fp32 accumulate; A from shared memory, or from tensor memory (_ts).
+// Every lane of the warp holds the operands and one (`leader` not 0) issues: no divergent branch, so the
+// operands stay in uniform registers.
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t leader;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(leader));
