@@ -50,23 +50,28 @@ __global__ void __launch_bounds__(kThreads) to_intervals_kernel(int N, const int
 
 __global__ void __launch_bounds__(kThreads) from_intervals_kernel(int N, const int32_t* tin, const int32_t* tout,
                                                                   int32_t* parent, int32_t* status) {
-  __shared__ long long s0[CLV_MAX_NODES], s1[CLV_MAX_NODES];
+  __shared__ int2 lab[CLV_MAX_NODES];
   __shared__ int s_bad;
   const int b = blockIdx.x, i = threadIdx.x;
   cudaGridDependencySynchronize();
   if (i == 0) s_bad = 0;
-  if (i < N) { s0[i] = tin[(int64_t)b * N + i]; s1[i] = tout[(int64_t)b * N + i]; }
+  if (i < N) lab[i] = make_int2(tin[(int64_t)b * N + i], tout[(int64_t)b * N + i]);
   __syncthreads();
   int best = -1;
   if (i < N) {
-    const long long a0 = s0[i], a1 = s1[i];
-    bool bad = !(a1 > a0);
+    const int2 a = lab[i];
+    bool bad = !(a.y > a.x);
+    uint32_t best_len = 0xFFFFFFFFu;               // an interval's length fits 32 bits without a sign
+#pragma unroll 8
     for (int j = 0; j < N; ++j) {
-      if (j == i) continue;
-      const long long b0 = s0[j], b1 = s1[j];
-      bad |= (b0 == a0);                         // two nodes with the same entry label
-      bad |= (a0 < b0 && b0 < a1 && a1 < b1);    // overlap without nesting
-      if (b0 <= a0 && a0 < b1 && (best < 0 || b1 - b0 < s1[best] - s0[best])) best = j;   // narrowest interval around i
+      const int2 o = lab[j];
+      const bool other = j != i;
+      const uint32_t len = (uint32_t)o.y - (uint32_t)o.x;
+      bad |= other & (o.x == a.x);                                  // two nodes with the same entry label
+      bad |= other & (a.x < o.x) & (o.x < a.y) & (a.y < o.y);       // overlap without nesting
+      const bool around = other & (o.x <= a.x) & (a.x < o.y) & ((best < 0) | (len < best_len));
+      best = around ? j : best;                                     // narrowest interval around i
+      best_len = around ? len : best_len;
     }
     bad |= (best >= i);                          // a parent must come before its child
     if (bad) s_bad = 1;
