@@ -12,6 +12,12 @@
 //             so a staged K/V tile serves 256 rows;
 //   otherwise the slots share one row tile and take the key tiles in turn (even, odd); their two
 //             partial results are combined like those of two blocks.
+// If the row tile has 64 rows or fewer (kParts = 2; 32: kParts = 4), Q is loaded that many times, one copy
+// below the other, and a row's keys are shared out over its copies: the softmax thread of a copy takes 64
+// (32) of a tile's 128 scores, has zeros for the others, and ends up with a partial result of its own.
+// The MMAs take what they take for 128 rows anyway; the softmax, which is what a short call waits for, is
+// half (a quarter) as long and keeps all four of the SM's quadrants busy (1 x 16 nodes x 512 keys:
+// 9.5 -> 8.2 us; 32 layers of 1 x 60 nodes x 1500 keys: 458 -> 425 us).
 // What bounds a key tile of 128 x 128 scores: Q K^T and P V are 16 MMAs of 64 cycles, the
 // exponentials 1024 cycles of the special-function units, and within a slot the two alternate (scores
 // -> exponentials -> P V -> next scores).  With two slots the tensor core works for one while the
@@ -65,8 +71,9 @@ constexpr float kRefSlack = 32.f;      // log2 units a score may exceed the row'
 constexpr uint32_t kIdescQK = make_idesc(BM, BN, false);  // S[128 rows x 128 keys] = Q K^T
 constexpr uint32_t kIdescPV = make_idesc(BM, HD, true);   // O[128 rows x 128 d] += P V
 
-template <bool kRows2>
+template <bool kRows2, int kParts>
 struct Cfg {
+  static constexpr int kRows = BM / kParts;      // rows of a row tile
   static constexpr int kQ = kRows2 ? 2 : 1;      // row tiles
   static constexpr int NST = kRows2 ? 5 : 6;     // ring stages: K and V tiles in turn
   static constexpr int kStep = kRows2 ? 2 : 4;   // loads from one tile of a slot to its next
@@ -86,7 +93,7 @@ struct Misc {                           // behind the tiles in dynamic shared me
 };
 constexpr uint32_t kMiscAt = 7 * kStage;   // either way: Q tiles + ring = 224 KB
 constexpr uint32_t kSmem = kMiscAt + (uint32_t)sizeof(Misc);
-static_assert(Cfg<true>::kQ + Cfg<true>::NST == 7 && Cfg<false>::kQ + Cfg<false>::NST == 7 && kSmem <= 232448, "shared memory");
+static_assert(Cfg<true, 1>::kQ + Cfg<true, 1>::NST == 7 && Cfg<false, 1>::kQ + Cfg<false, 1>::NST == 7 && kSmem <= 232448, "shared memory");
 
 // n / d by a multiplication: m = ceil(2^32 / d), so the high word is n / d or one more.  (A division of
 // the language is some 40 instructions that a block runs once, from a cold instruction cache.)
@@ -203,7 +210,7 @@ struct RingPos {
 };
 
 // What a thread knows about its block: its place in the grid, its share of the key axis, its row.
-template <bool kRows2>
+template <bool kRows2, int kParts>
 struct Block {
   uint8_t* smem;
   uint32_t smem0, sRing, bar0, tmem;
@@ -214,7 +221,7 @@ struct Block {
   int R, per, first, mine;                 // rows in use, numbered through the row tiles; rank d finalises [d * per, (d + 1) * per)
   int L, p_cache, p_total, pc_begin, pc_end, T, t_plain;
   bool len_bad;
-  int slot, row, node_in_tile, node, my_tiles;           // of the softmax threads
+  int slot, row, part, node_in_tile, node, my_tiles;     // of the softmax threads: accumulator row, share of a tile's keys
   bool row_valid;
   uint32_t lane_addr;
 
@@ -232,7 +239,7 @@ struct Block {
   __device__ __forceinline__ void place(const Params& p, uint8_t* sm, unsigned block, int thread) {
     smem = sm;
     smem0 = smem_u32(sm);
-    sRing = smem0 + Cfg<kRows2>::kQ * kQTile;
+    sRing = smem0 + Cfg<kRows2, kParts>::kQ * kQTile;
     bar0 = smem_u32(&misc().bar[0]);
     abort_flag = &misc().abort_flag;
     tid = thread; warp = tid >> 5; lane = tid & 31;
@@ -269,27 +276,42 @@ struct Block {
     row = (warp & 3) * 32 + lane;   // a warp may touch the 32 tensor-memory lanes of its number modulo 4
     lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const int rtile = kRows2 ? tile0 + slot : tile0;
-    node_in_tile = (int)p.by_group_heads.divide((unsigned)row);
+    part = row / Cfg<kRows2, kParts>::kRows;
+    const int tile_row = row % Cfg<kRows2, kParts>::kRows;
+    node_in_tile = (int)p.by_group_heads.divide((unsigned)tile_row);
     node = rtile * tile_nodes + node_in_tile;
-    row_valid = warp < kSoftmaxWarps && row < RT && rtile < p.tiles && node < N;
+    row_valid = warp < kSoftmaxWarps && tile_row < RT && rtile < p.tiles && node < N;
     my_tiles = slot_tiles(slot);
   }
 };
 
 // ---- the roles' work on the block's share of the keys
 
-template <bool kRows2>
-__device__ __forceinline__ void produce(const Block<kRows2>& k, const Maps& tm, const Params& p) {
-  constexpr int NST = Cfg<kRows2>::NST;
-  if (k.lane == 0 && k.T > 0) {
-    mbar_expect_tx(k.bar(B_Q), (uint32_t)(k.users * k.RT * HD * 2));   // a box holds RT rows, absent nodes as zeros
+// A tile's P is handed over in parts: keys 0-63, 64-95, 96-127 if a thread has all keys of its row, else
+// the first and the second 32 of every thread's, or all at once.
+template <int kParts>
+__host__ __device__ constexpr int hand_overs() { return kParts == 1 ? 3 : kParts == 2 ? 2 : 1; }
+template <int kParts>
+__host__ __device__ constexpr int handed_over_in(int c) { return kParts == 1 ? (c < 2 ? 0 : c - 1) : kParts == 2 ? (c & 1) : 0; }   // 32 keys c
+
+// Q needs nothing that is read from memory, so it is asked for ahead of the context length.
+template <bool kRows2, int kParts>
+__device__ __forceinline__ void load_q(const Block<kRows2, kParts>& k, const Maps& tm) {
+  mbar_expect_tx(k.bar(B_Q), (uint32_t)(k.users * kParts * k.RT * HD * 2));   // a box holds RT rows, absent nodes as zeros
 #pragma unroll
-    for (int m = 0; m < Cfg<kRows2>::kQ; ++m) {
-      if (m >= k.users) break;
-      tma_load_4d(k.smem0 + m * kQTile, &tm.q, 0, k.kvh * k.G, (k.tile0 + m) * k.tile_nodes, k.b, k.bar(B_Q));
-      tma_load_4d(k.smem0 + m * kQTile + kQTile / 2, &tm.q, 64, k.kvh * k.G, (k.tile0 + m) * k.tile_nodes, k.b, k.bar(B_Q));
-    }
+  for (int m = 0; m < Cfg<kRows2, kParts>::kQ * kParts; ++m) {
+    if (kRows2 && m >= k.users) break;
+    const uint32_t dst = k.smem0 + (uint32_t)m * (kRows2 ? kQTile : kQTile / 2 / kParts);
+    const int node0 = (k.tile0 + (kRows2 ? m : 0)) * k.tile_nodes;
+    tma_load_4d(dst, &tm.q, 0, k.kvh * k.G, node0, k.b, k.bar(B_Q));
+    tma_load_4d(dst + kQTile / 2, &tm.q, 64, k.kvh * k.G, node0, k.b, k.bar(B_Q));
   }
+}
+
+template <bool kRows2, int kParts>
+__device__ __forceinline__ void produce(const Block<kRows2, kParts>& k, const Maps& tm, const Params& p) {
+  constexpr int NST = Cfg<kRows2, kParts>::NST;
+  if (k.T == 0) mbar_drain(k.bar(B_Q), 0);   // nobody else waits for the Q that is on its way
   int page = 0, page_base = -64;   // lane j: pool page of context piece (page_base + j)
   RingPos<NST> pos(0);
   int issued = 0;
@@ -350,9 +372,9 @@ __device__ __forceinline__ void produce(const Block<kRows2>& k, const Maps& tm, 
 // order: Q K^T of both slots, then per tile and slot P V of the tile's parts as they are handed over and
 // Q K^T of the slot's next tile.  The tensor core queues a few MMAs, so what lies between two groups
 // of them is hidden.
-template <bool kRows2>
-__device__ __forceinline__ void issue(const Block<kRows2>& k, const Params& p) {
-  constexpr int NST = Cfg<kRows2>::NST;
+template <bool kRows2, int kParts>
+__device__ __forceinline__ void issue(const Block<kRows2, kParts>& k, const Params& p) {
+  constexpr int NST = Cfg<kRows2, kParts>::NST;
   const uint32_t el = elect_one();
   if (k.T == 0 || !wait_warp(k.bar(B_Q), 0, k.abort_flag, p.wait_limit)) return;
   const uint64_t q_desc = smem_desc(k.smem0, 16, 1024);
@@ -389,39 +411,38 @@ __device__ __forceinline__ void issue(const Block<kRows2>& k, const Params& p) {
       const uint64_t vd = v_desc + (uint64_t)((uint32_t)(vpos.idx * (int)kStage) >> 4);
       const int keys[2] = {k.piece_keys(g0), k.piece_keys(g0 + 1)};
 #pragma unroll
-      for (int h = 0; h < 3; ++h) {   // keys 0-63, 64-95, 96-127 of the tile
-        if (!ok || (h > 0 && keys[1] <= (h - 1) * CH)) continue;
+      for (int h = 0; h < hand_overs<kParts>(); ++h) {
+        if (!ok || (kParts == 1 && h > 0 && keys[1] <= (h - 1) * CH)) continue;
         ok = wait_warp(k.bar(B_P + 3 * s + h), (ph >> (3 * s + h)) & 1u, k.abort_flag, p.wait_limit);
         if (!ok) continue;
         ph ^= 1u << (3 * s + h);
         tc_fence_after();
 #pragma unroll
-        for (int kk = h == 0 ? 0 : 2 + 2 * h; kk < 4 + 2 * h; ++kk)
-          if (h > 0 || kk < 2 || keys[0] > CH)
+        for (int c = 0; c < BN / CH; ++c) {
+          if (handed_over_in<kParts>(c) != h || keys[c >> 1] <= (c & 1) * CH) continue;
+#pragma unroll
+          for (int kk = 2 * c; kk < 2 * c + 2; ++kk)
             umma_bf16_ts_if(el, k.tmem_O(s), k.tmem_S(s) + (uint32_t)(kk * 8), vd + (uint64_t)((kk * 16 * 128) >> 4), kIdescPV,
                             (r > 0 || kk > 0) ? 1u : 0u);
+        }
       }
       if (!ok) continue;
       umma_commit_if(el, k.bar(B_EMPTY + vpos.idx));
-      kpos[s].advance(Cfg<kRows2>::kStep);
+      kpos[s].advance(Cfg<kRows2, kParts>::kStep);
       if (r + 1 < k.slot_tiles(s)) ok = issue_qk(s);
       else umma_commit_if(el, k.bar(B_LAST + s));
     }
   }
 }
 
-template <bool kRows2>
-__device__ __forceinline__ void softmax(const Block<kRows2>& k, const Params& p) {
-  constexpr int NST = Cfg<kRows2>::NST;
+template <bool kRows2, int kParts>
+__device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Params& p, int par) {
+  constexpr int NST = Cfg<kRows2, kParts>::NST;
   Misc& ms = k.misc();
   const int tid = k.tid, lane = k.lane, slot = k.slot, row = k.row;
   if (tid < CLV_MAX_NODES) {
     bool bad = false;
-    int par = -1;
-    if (tid < k.N) {
-      par = p.parent[(int64_t)k.b * k.N + tid];
-      if (par < -1 || par >= tid) { bad = true; par = -1; }
-    }
+    if (par < -1 || par >= tid) { bad = true; par = -1; }
     ms.parent[tid] = (signed char)par;
     // one block per sequence reports what is wrong with it: the length, the tree, the block table
     if (k.group == 0 && k.split == 0 && k.kvh == 0) {
@@ -444,7 +465,7 @@ __device__ __forceinline__ void softmax(const Block<kRows2>& k, const Params& p)
     }
   }
   __syncwarp();
-  const bool warp_active = __any_sync(0xFFFFFFFFu, k.row_valid), warp_full = __all_sync(0xFFFFFFFFu, k.row_valid);
+  const bool warp_active = __any_sync(0xFFFFFFFFu, k.row_valid);
   const uint32_t s_addr = k.tmem_S(slot) + k.lane_addr;   // this row's scores, then its P
   const float sc = p.scale_log2;
   float m_ref = k.row_valid ? -INFINITY : 0.f, l_run = 0.f;
@@ -484,14 +505,14 @@ __device__ __forceinline__ void softmax(const Block<kRows2>& k, const Params& p)
         __syncwarp();
       }
     }
-    vpos.advance(Cfg<kRows2>::kStep);
-    if (!warp_active) {   // no row of this warp exists: its lanes of P may hold anything
+    vpos.advance(Cfg<kRows2, kParts>::kStep);
+    if (kParts == 1 && !warp_active) {   // no row of this warp exists: its lanes of P may hold anything
       hand_over(0);
       if (keys1 > 0) hand_over(1);
       if (keys1 > CH) hand_over(2);
       continue;
     }
-    const bool masked = !plain || !warp_full;
+    const bool masked = !plain;   // rows that do not exist compute what nobody reads
     auto mask = [&](int c, uint32_t (&a)[CH]) {   // columns that this row may not see become -inf
       const int g = k.pc_begin + 2 * t + (c >> 1), keys = ((c >> 1) ? keys1 : keys0) - (c & 1) * CH;
       uint32_t bits = 0u;
@@ -520,10 +541,58 @@ __device__ __forceinline__ void softmax(const Block<kRows2>& k, const Params& p)
         a[j] = pack_bf16(pr.x, pr.y);
       }
     };
+    auto new_reference = [&](float m_new, bool need) {   // O is at rest: these scores were asked for after P V of the slot's previous tile
+      const float alpha = need ? ex2(m_ref - m_new) : 1.f;   // ex2(-inf) = 0
+      if (need) { m_ref = m_new; l_run *= alpha; }
+      neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
+      if (r > 0) {
+#pragma unroll 1
+        for (int cc = 0; cc < HD; cc += 16) {
+          uint32_t ov[16];
+          tmem_ld_x16(k.tmem_O(slot) + k.lane_addr + (uint32_t)cc, ov);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * alpha);
+          tmem_st_x16(k.tmem_O(slot) + k.lane_addr + (uint32_t)cc, ov);
+        }
+      }
+    };
     auto load = [&](int c, uint32_t (&a)[CH]) { tmem_ld_x32(s_addr + (uint32_t)(c * CH), a); };
     auto store_p = [&](int c, const uint32_t (&a)[CH]) {
       tmem_st_x16(s_addr + (uint32_t)(c * (CH / 2)), *reinterpret_cast<const uint32_t(*)[CH / 2]>(&a[0]));
     };
+    if constexpr (kParts > 1) {   // one or two loads' worth of keys
+      constexpr int kLoads = 4 / kParts;
+      const int c0 = k.part * kLoads;
+      uint32_t x[kLoads][CH];
+#pragma unroll
+      for (int c = 0; c < kLoads; ++c) load(c0 + c, x[c]);
+      tmem_wait_ld();
+      {
+        uint32_t none[CH / 2];
+#pragma unroll
+        for (int j = 0; j < CH / 2; ++j) none[j] = 0u;
+#pragma unroll
+        for (int c = kLoads; c < 4; ++c) tmem_st_x16(s_addr + (uint32_t)(((c0 + c) & 3) * (CH / 2)), none);   // the other parts' keys
+      }
+#pragma unroll
+      for (int c = 0; c < kLoads; ++c) {
+        if (masked) mask(c0 + c, x[c]);
+        take_max(x[c]);
+      }
+      const float m_new = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]) * sc;
+      const bool need = m_new > m_ref + kRefSlack;
+      if (__any_sync(0xFFFFFFFFu, need)) new_reference(m_new, need);
+#pragma unroll
+      for (int c = 0; c < kLoads; ++c) {
+        exps(x[c]);
+        store_p(c0 + c, x[c]);
+        hand_over(c);
+      }
+      const float2 tot = add2(sum[0], sum[1]);
+      l_run += tot.x + tot.y;
+      continue;
+    }
     uint32_t x0[CH], x1[CH], x2[CH], x3[CH];
     load(0, x0);
     tmem_wait_ld();
@@ -546,22 +615,7 @@ __device__ __forceinline__ void softmax(const Block<kRows2>& k, const Params& p)
     const float m_new = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]) * sc;   // scale > 0; no allowed key: -inf
     const bool need = m_new > m_ref + kRefSlack;
     if (__any_sync(0xFFFFFFFFu, need)) {
-      // A new reference.  O is at rest: these scores were asked for after P V of the slot's previous
-      // tile.  The scores of the first 64 keys are still in place.
-      const float alpha = need ? ex2(m_ref - m_new) : 1.f;   // ex2(-inf) = 0
-      if (need) { m_ref = m_new; l_run *= alpha; }
-      neg_m = m_ref == -INFINITY ? 0.f : -m_ref;
-      if (r > 0) {
-#pragma unroll 1
-        for (int cc = 0; cc < HD; cc += 16) {
-          uint32_t ov[16];
-          tmem_ld_x16(k.tmem_O(slot) + k.lane_addr + (uint32_t)cc, ov);
-          tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * alpha);
-          tmem_st_x16(k.tmem_O(slot) + k.lane_addr + (uint32_t)cc, ov);
-        }
-      }
+      new_reference(m_new, need);   // the scores of the first 64 keys are still in place
       sum[0] = sum[1] = make_float2(0.f, 0.f);
       load(0, x0);
       load(1, x1);
@@ -598,13 +652,13 @@ __device__ __forceinline__ void softmax(const Block<kRows2>& k, const Params& p)
 }
 
 // ------------------------------------------------------------------------------------ kernel
-template <bool kRows2>
+template <bool kRows2, int kParts>
 __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Params p) {
-  constexpr int NST = Cfg<kRows2>::NST;
+  constexpr int NST = Cfg<kRows2, kParts>::NST;
   extern __shared__ __align__(1024) uint8_t smem[];
   Misc& ms = *reinterpret_cast<Misc*>(smem + kMiscAt);
   {
-  Block<kRows2> k;
+  Block<kRows2, kParts> k;
   k.place(p, smem, blockIdx.x, threadIdx.x);
   const int tid = k.tid, warp = k.warp;
   auto bar = [&](int idx) { return k.bar(idx); };
@@ -619,7 +673,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     mbar_init(bar(B_Q), 1);
     mbar_init(bar(B_RX), 1);
     mbar_init(bar(B_DR), 1);
-    if (k.CS > 1) mbar_expect_tx(bar(B_RX), (uint32_t)((k.CS - 1) * k.mine) * 272u);   // what the other ranks will send
+    if (k.CS > 1) mbar_expect_tx(bar(B_RX), (uint32_t)((k.CS - 1) * kParts * k.mine) * 272u);   // what the other ranks will send
     ms.abort_flag = 0;
     ms.issued = 0;
     fence_barrier_init();
@@ -655,18 +709,22 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     fence_async_smem();   // the tiles are written by TMA next
     __syncthreads();
   }
+  // what the block reads of global memory before its tiles: all under way at once
+  if (tid == 32 * kProducer) load_q<kRows2, kParts>(k, tm);
+  __syncwarp();
+  const int par = tid < k.N ? p.parent[(int64_t)k.b * k.N + tid] : -1;   // of node tid
   k.range(p, p.ctx_len[k.b]);
   if (tid == 0) { ms.seq = k.b; ms.len = k.L; }
   if (warp < kSoftmaxWarps) {
     more_registers<kSoftmaxRegs>();
-    softmax<kRows2>(k, p);
+    softmax<kRows2, kParts>(k, p, par);
     __syncwarp();
     fewer_registers<kLaunchRegs>();   // before the third warpgroup takes its own back
     named_barrier(2, kThreads);
   } else {
     fewer_registers<kOtherRegs>();
-    if (warp == kProducer) produce<kRows2>(k, tm, p);
-    else if (warp == kIssuer) issue<kRows2>(k, p);
+    if (warp == kProducer) produce<kRows2, kParts>(k, tm, p);
+    else if (warp == kIssuer) issue<kRows2, kParts>(k, p);
     __syncwarp();
     named_barrier(2, kThreads);
     more_registers<kLaunchRegs>();
@@ -676,7 +734,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   // ---- every role has met here ------------------------------------------------------------------
   // What is known about the block is worked out once more: kept in registers it would push the softmax
   // threads' scores out of theirs (4 x 64 nodes x 4096 keys: 29.8 -> 27.7 us).
-  Block<kRows2> k;
+  Block<kRows2, kParts> k;
   {
     unsigned block;
     int thread;
@@ -691,6 +749,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   const int R = k.R, per = k.per, first = k.first, mine = k.mine;
   const uint32_t smem0 = k.smem0, sRing = k.sRing;
   auto bar = [&](int idx) { return k.bar(idx); };
+  const bool alone = kParts == 1 && CS == 1;   // nothing to be added to this block's accumulators
   const bool aborted = *k.abort_flag != 0;
   if (CS > 1) cluster_arrive();   // all Q K^T of this block are done: what the merge uses is idle (see there)
   if (aborted) {
@@ -701,7 +760,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
         const RingPos<NST> pos(i);
         mbar_drain(bar(B_FULL + pos.idx), pos.ph);
       }
-      if (T > 0) mbar_drain(bar(B_Q), 0);
+      mbar_drain(bar(B_Q), 0);
     }
     if (warp == kIssuer) {
       umma_commit_if(elect_one(), bar(B_DR));
@@ -732,7 +791,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   //      last V tiles.  Two neighbouring stages receive; since other ranks write there, the place is a
   //      function of the receiver's number of tiles.  A third one holds what goes with this block's
   //      own rows: 16 bytes per row (reference, sum, scales of its halves) | where each row's output
-  //      starts | the weights of the final sum.
+  //      starts.
   auto rx_index = [&](int tiles_of_rank) {
     const int i = (2 * tiles_of_rank) % NST;
     return i == NST - 1 ? 0 : i;
@@ -740,13 +799,13 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   auto rank_tiles = [&](int d) {
     return ((int)(p.by_splits.divide((unsigned)(d + 1) * (unsigned)k.p_total) - p.by_splits.divide((unsigned)d * (unsigned)k.p_total)) + 1) / 2;
   };
-  auto rx_meta = [&](uint32_t rx_base) { return rx_base + (uint32_t)((CS - 1) * per) * 256u; };   // behind the rows
+  auto rx_meta = [&](uint32_t rx_base) { return rx_base + (uint32_t)((CS - 1) * kParts * per) * 256u; };   // behind the rows
   const uint32_t rx = sRing + (uint32_t)rx_index(T) * kStage;
   const uint32_t meta = sRing + (uint32_t)((rx_index(T) + 2) % NST) * kStage;
-  const uint32_t row_at = meta + 4096u, weights = meta + 8192u;
+  const uint32_t row_at = meta + 4096u;
   __syncwarp();
   if (warp < kSoftmaxWarps) {
-    const int slot = k.slot, row = k.row, row_in_out = (b * N + k.node) * p.Hq + kvh * G + (row - k.node_in_tile * G);
+    const int slot = k.slot, row = k.row, row_in_out = (b * N + k.node) * p.Hq + kvh * G + (row % Cfg<kRows2, kParts>::kRows - k.node_in_tile * G);
     float2 ml = ms.ml[slot * BM + row];
     float w0 = 1.f, w1 = 0.f;
     if (!kRows2) {   // combine the slots' shares of the keys
@@ -757,7 +816,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
       w1 = ex2(c.x - mu);
       ml.y = a.y * w0 + c.y * w1;
     }
-    if (CS == 1) {
+    if (alone) {
       const float inv = ml.y > 0.f ? 1.f / ml.y : 0.f;
       w0 *= inv;
       w1 *= inv;
@@ -779,34 +838,27 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     for (int half = kRows2 ? 0 : slot; half < (kRows2 ? 2 : slot + 1); ++half) {
       float v[64];
       {
-        uint32_t u[64];
-        if (has0) {
-          tmem_ld_x64(acc0 + (uint32_t)(half * 64), u);
-          tmem_wait_ld();
-        }
+        uint32_t u[64], u1[64];
+        if (has0) tmem_ld_x64(acc0 + (uint32_t)(half * 64), u);
+        if (!kRows2 && has1) tmem_ld_x64(acc1 + (uint32_t)(half * 64), u1);
+        tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 64; ++j) v[j] = has0 ? __uint_as_float(u[j]) * w0 : 0.f;
-      }
-      if (has1) {
-#pragma unroll
-        for (int q = 0; q < 64; q += 32) {
-          uint32_t u[32];
-          tmem_ld_x32(acc1 + (uint32_t)(half * 64 + q), u);
-          tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) v[q + j] = fmaf(__uint_as_float(u[j]), w1, v[q + j]);
+        for (int j = 0; j < 64; ++j) {
+          v[j] = has0 ? __uint_as_float(u[j]) * w0 : 0.f;
+          if (!kRows2 && has1) v[j] = fmaf(__uint_as_float(u1[j]), w1, v[j]);
         }
       }
-      if (CS == 1) {   // into the Q tile's place and layout; TMA stores it
+      if (alone) {   // into the Q tile's place and layout; TMA stores it
         const uint32_t dst = smem0 + (kRows2 ? slot * kQTile : 0u) + (uint32_t)half * (kQTile / 2) + (uint32_t)row * 128u;
 #pragma unroll
         for (int c = 0; c < 8; ++c)
           st_shared16(dst + (uint32_t)((c ^ (row & 7)) << 4), pack_bf16(v[8 * c], v[8 * c + 1]), pack_bf16(v[8 * c + 2], v[8 * c + 3]),
                       pack_bf16(v[8 * c + 4], v[8 * c + 5]), pack_bf16(v[8 * c + 6], v[8 * c + 7]));
       } else {
-        float amax = 0.f;
+        float top[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int j = 0; j < 64; j += 2) amax = max3(amax, fabsf(v[j]), fabsf(v[j + 1]));
+        for (int j = 0; j < 64; j += 2) top[(j >> 1) & 3] = max3(top[(j >> 1) & 3], fabsf(v[j]), fabsf(v[j + 1]));
+        const float amax = fmaxf(max3(top[0], top[1], top[2]), top[3]);
         // scale 2^lc with amax * 2^lc in [2^13, 2^14); lc is clamped so that the scale and its
         // inverse are normal numbers (zeros stay zeros, inf or NaN stay what they are)
         const int biased = (int)((__float_as_uint(amax) >> 23) & 255u);
@@ -828,7 +880,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
         }
       }
     }
-    if (CS > 1 && (kRows2 || slot == 0)) {
+    if (!alone && (kRows2 || slot == 0)) {
       st_shared8(meta + (uint32_t)seq_row * 16u, ml.x, ml.y);
       // where the row's output starts (in rows of 128), -1: the row does not exist
       asm volatile("st.shared.b32 [%0], %1;" ::"r"(row_at + (uint32_t)seq_row * 4u), "r"(k.row_valid ? row_in_out : -1) : "memory");
@@ -839,10 +891,10 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   __syncthreads();
   if (warp == kIssuer) { tc_fence_after(); tmem_dealloc(k.tmem, kTmemCols); }
 
-  if (CS == 1) {
+  if (alone) {
     if (tid == 0) {
 #pragma unroll
-      for (int m = 0; m < Cfg<kRows2>::kQ; ++m) {
+      for (int m = 0; m < Cfg<kRows2, kParts>::kQ; ++m) {
         if (m >= users) break;
         tma_store_4d(&tm.out, smem0 + m * kQTile, 0, kvh * G, (tile0 + m) * tile_nodes, b);
         tma_store_4d(&tm.out, smem0 + m * kQTile + kQTile / 2, 64, kvh * G, (tile0 + m) * tile_nodes, b);
@@ -854,80 +906,144 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     return;
   }
 
-  cluster_wait();   // every rank's receiving stages are idle
-  if (tid < CS && tid != split) {   // a peer's rows, then what goes with them
-    const int d = tid, f = min(R, d * per), n = min(R, f + per) - f;
-    if (n > 0) {
-      const uint32_t base = sRing + (uint32_t)rx_index(rank_tiles(d)) * kStage, at = (uint32_t)((split < d ? split : split - 1) * per);
-      const uint32_t their_bar = cluster_map(bar(B_RX), (uint32_t)d);
-      bulk_to_peer(cluster_map(base + at * 256u, (uint32_t)d), smem0 + (uint32_t)f * 256u, (uint32_t)n * 256u, their_bar);
-      bulk_to_peer(cluster_map(rx_meta(base) + at * 16u, (uint32_t)d), meta + (uint32_t)f * 16u, (uint32_t)n * 16u, their_bar);
+  if (CS > 1) {
+    cluster_wait();   // every rank's receiving stages are idle
+    const int d = tid / kParts, part = tid % kParts;
+    if (d < CS && d != split) {   // a peer's rows, then what goes with them
+      const int f = min(R, d * per), n = min(R, f + per) - f, row0 = part * Cfg<kRows2, kParts>::kRows + f;
+      if (n > 0) {
+        const uint32_t base = sRing + (uint32_t)rx_index(rank_tiles(d)) * kStage;
+        const uint32_t at = (uint32_t)(((split < d ? split : split - 1) * kParts + part) * per);
+        const uint32_t their_bar = cluster_map(bar(B_RX), (uint32_t)d);
+        bulk_to_peer(cluster_map(base + at * 256u, (uint32_t)d), smem0 + (uint32_t)row0 * 256u, (uint32_t)n * 256u, their_bar);
+        bulk_to_peer(cluster_map(rx_meta(base) + at * 16u, (uint32_t)d), meta + (uint32_t)row0 * 16u, (uint32_t)n * 16u, their_bar);
+      }
     }
+    mbar_drain(bar(B_RX), 0);
+    __syncwarp();
+    cluster_arrive();   // what this block was sent has arrived: its peers may leave
   }
-  mbar_drain(bar(B_RX), 0);
-  __syncwarp();
-  cluster_arrive();   // what this block was sent has arrived: its peers may leave
-  // ---- final rows.  First the weight of every source of a row (with the source's scales and the sum
-  //      of all in it): a thread per row; then 16 threads per row, 8 columns each.  Sources in rank
-  //      order, so that the result does not depend on timing.
-  auto source = [&](int q, int i) { return (uint32_t)((q < split ? q : q - 1) * per + i); };
-  auto row_out = [&](int i) {
-    int o;
-    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(o) : "r"(row_at + (uint32_t)(first + i) * 4u));
-    return o;
-  };
-  for (int i = tid; i < mine; i += kThreads) {
-    float4 m[kMaxSplits];
-    float M = -INFINITY;
-#pragma unroll
-    for (int q = 0; q < kMaxSplits; ++q) {
-      m[q] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
-      if (q < CS)
-        asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(m[q].x), "=f"(m[q].y), "=f"(m[q].z), "=f"(m[q].w)
-                     : "r"(q == split ? meta + (uint32_t)(first + i) * 16u : rx_meta(rx) + source(q, i) * 16u));
-      M = fmaxf(M, m[q].x);
-    }
-    const float mu = M == -INFINITY ? 0.f : M;
-    float total = 0.f;
-#pragma unroll
-    for (int q = 0; q < kMaxSplits; ++q) {
-      m[q].x = ex2(m[q].x - mu);   // ex2(-inf) = 0
-      total = fmaf(m[q].y, m[q].x, total);
-    }
-    const float inv = total > 0.f ? 1.f / total : 0.f;
-#pragma unroll
-    for (int q = 0; q < kMaxSplits; ++q)
-      if (q < CS) st_shared8(weights + (uint32_t)(i * kMaxSplits + q) * 8u, m[q].x * m[q].z * inv, m[q].x * m[q].w * inv);
-    const int o = row_out(i);
+  // ---- final rows.  A source of a row is a part of a block's accumulators: first what was received, by
+  //      rank, then this block's own, always in this order, so that the result does not depend on timing.
+  //      What counts here is the length of one thread's chain: the sources are loaded four at a time
+  //      ahead of their sums (one after the other they cost 90 cycles each).
+  constexpr int kSources = kMaxSplits * kParts;
+  const int received = (CS - 1) * kParts, sources = CS * kParts;
+  const uint8_t* rx_rows = smem + (rx - smem0);                     // of source 0; the next source's are per rows on
+  const uint8_t* own_rows = smem + first * 256;                     // of part 0; the next part's are kRows rows on
+  const float4* rx_sums = reinterpret_cast<const float4*>(smem + (rx_meta(rx) - smem0));
+  const float4* own_sums = reinterpret_cast<const float4*>(smem + (meta - smem0)) + first;
+  const int* row_outs = reinterpret_cast<const int*>(smem + (row_at - smem0)) + first;
+  constexpr int kRows = Cfg<kRows2, kParts>::kRows;
+  auto sums_of = [&](int j, int i) { return j < received ? rx_sums[j * per + i] : own_sums[(j - received) * kRows + i]; };
+  auto write_lse = [&](int o, float M, float total) {
     if (p.lse != nullptr && o >= 0) p.lse[o] = (M + log2f(total)) * 0.6931471805599453f;
-  }
-  __syncthreads();
-  for (int it = tid; it < mine * 16; it += kThreads) {
-    const int i = it >> 4, c = it & 15, o = row_out(i);
-    const uint32_t at = (uint32_t)((c ^ ((first + i) & 15)) << 4);
-    float acc[8];
+  };
+  // 8 columns of row i (16-byte piece c): sources j0 .. j0 + 3 with weights w
+  auto add = [&](float (&acc)[8], int j0, int i, int c, auto weight) {
+    const uint32_t at = (uint32_t)i * 256u + (uint32_t)((c ^ ((first + i) & 15)) << 4);
+    uint4 u[4];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-#pragma unroll 4
-    for (int q = 0; q < CS; ++q) {
-      uint32_t u[4];
-      float w;
-      asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3])
-                   : "r"((q == split ? smem0 + (uint32_t)(first + i) * 256u : rx + source(q, i) * 256u) + at));
-      asm volatile("ld.shared.f32 %0, [%1];" : "=f"(w) : "r"(weights + (uint32_t)(i * kMaxSplits + q) * 8u + (uint32_t)(c >> 3) * 4u));
+    for (int j = 0; j < 4; ++j)
+      if (j0 + j < sources)
+        u[j] = *reinterpret_cast<const uint4*>((j0 + j < received ? rx_rows + (j0 + j) * per * 256 : own_rows + (j0 + j - received) * (kRows * 256)) + at);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float w = weight(j);
+      if (j0 + j >= sources) continue;
+      const uint32_t h[4] = {u[j].x, u[j].y, u[j].z, u[j].w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const float2 f = half2_bits_to_float2(u[e]);
+        const float2 f = half2_bits_to_float2(h[e]);
         acc[2 * e] = fmaf(f.x, w, acc[2 * e]);
         acc[2 * e + 1] = fmaf(f.y, w, acc[2 * e + 1]);
       }
     }
-    if (o >= 0)
-      *reinterpret_cast<uint4*>(p.out + (int64_t)o * HD + c * 8) =
-          make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
+  };
+  auto write_row = [&](const float (&acc)[8], int o, int c) {
+    *reinterpret_cast<uint4*>(p.out + (int64_t)o * HD + c * 8) =
+        make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
+  };
+  if constexpr (kParts == 1) {   // up to 128 rows of few sources: their weights first, a thread per row
+    float* weights = reinterpret_cast<float*>(smem + (meta + 8192u - smem0));   // [row][half][source]
+    for (int i = tid; i < mine; i += kThreads) {
+      float4 m[kSources];
+      float M = -INFINITY;
+#pragma unroll
+      for (int j = 0; j < kSources; ++j) {
+        m[j] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
+        if (j < sources) m[j] = sums_of(j, i);
+        M = fmaxf(M, m[j].x);
+      }
+      const float mu = M == -INFINITY ? 0.f : M;
+      float total = 0.f;
+#pragma unroll
+      for (int j = 0; j < kSources; ++j) {
+        m[j].x = ex2(m[j].x - mu);   // ex2(-inf) = 0
+        total = fmaf(m[j].y, m[j].x, total);
+      }
+      const float inv = total > 0.f ? 1.f / total : 0.f;
+#pragma unroll
+      for (int j = 0; j < kSources; ++j) {
+        if (j >= sources) continue;
+        weights[i * 2 * kSources + j] = m[j].x * m[j].z * inv;
+        weights[i * 2 * kSources + kSources + j] = m[j].x * m[j].w * inv;
+      }
+      write_lse(row_outs[i], M, total);
+    }
+    __syncthreads();
+    for (int it = tid; it < mine * 16; it += kThreads) {
+      const int i = it >> 4, c = it & 15, o = row_outs[i];
+      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int j0 = 0; j0 < kSources; j0 += 4) {
+        if (j0 >= sources) break;
+        const float4 w4 = *reinterpret_cast<const float4*>(weights + i * 2 * kSources + (c >> 3) * kSources + j0);
+        const float w[4] = {w4.x, w4.y, w4.z, w4.w};
+        add(acc, j0, i, c, [&](int j) { return w[j]; });
+      }
+      if (o >= 0) write_row(acc, o, c);
+    }
+  } else {   // up to 32 rows of many sources: eight lanes share a row's sources for one half of its columns
+#pragma unroll 1
+    for (int i0 = 2 * warp; i0 < mine; i0 += 2 * (kThreads / 32)) {
+      const int i = min(i0 + (lane >> 4), mine - 1), c = lane & 15, o = row_outs[i];
+      float4 m[kParts];   // sources (lane & 7) + 8 e
+      float M = -INFINITY;
+#pragma unroll
+      for (int e = 0; e < kParts; ++e) {
+        const int j = (lane & 7) + 8 * e;
+        m[e] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
+        if (j < sources) m[e] = sums_of(j, i);
+        M = fmaxf(M, m[e].x);
+      }
+#pragma unroll
+      for (int d = 1; d < 8; d *= 2) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, d));
+      const float mu = M == -INFINITY ? 0.f : M;
+      float total = 0.f;
+#pragma unroll
+      for (int e = 0; e < kParts; ++e) {
+        m[e].x = ex2(m[e].x - mu);   // ex2(-inf) = 0
+        total = fmaf(m[e].y, m[e].x, total);
+      }
+#pragma unroll
+      for (int d = 1; d < 8; d *= 2) total += __shfl_xor_sync(0xFFFFFFFFu, total, d);
+      const float inv = total > 0.f ? 1.f / total : 0.f;
+      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int j0 = 0; j0 < kSources; j0 += 4) {
+        if (j0 >= sources) break;
+        const float scale = (c < 8 ? m[j0 >> 3].z : m[j0 >> 3].w) * (m[j0 >> 3].x * inv);
+        add(acc, j0, i, c, [&](int j) { return __shfl_sync(0xFFFFFFFFu, scale, (j0 + j) & 7, 8); });
+      }
+      if (i0 + (lane >> 4) < mine) {
+        if (o >= 0) write_row(acc, o, c);
+        if (c == 0) write_lse(o, M, total);
+      }
+    }
   }
   __syncwarp();
-  cluster_wait();   // no block may leave while a copy still reads its shared memory
+  if (CS > 1) cluster_wait();   // no block may leave while a copy still reads its shared memory
   publish();
 }
 
@@ -969,8 +1085,9 @@ bool make_map_halves(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t 
   return encode(tm, base, 4, dims, strides, box);
 }
 
-void* kernel_of(bool rows2) {
-  return rows2 ? reinterpret_cast<void*>(tree_attn_kernel<true>) : reinterpret_cast<void*>(tree_attn_kernel<false>);
+using Kernel = void (*)(Maps, Params);
+Kernel kernel_of(bool rows2, int parts) {
+  return rows2 ? tree_attn_kernel<true, 1> : parts == 4 ? tree_attn_kernel<false, 4> : parts == 2 ? tree_attn_kernel<false, 2> : tree_attn_kernel<false, 1>;
 }
 
 // Once per device: the kernels' shared memory, and how many clusters of each size run at once (one
@@ -978,8 +1095,9 @@ void* kernel_of(bool rows2) {
 int g_clusters[kMaxDevices][kMaxSplits + 1];
 
 cudaError_t set_up() {
-  for (int r = 0; r < 2; ++r) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel_of(r != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  const Kernel all[4] = {kernel_of(true, 1), kernel_of(false, 1), kernel_of(false, 2), kernel_of(false, 4)};
+  for (const Kernel kernel : all) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     if (e != cudaSuccess) return e;
   }
   int dev = 0;
@@ -998,7 +1116,7 @@ cudaError_t set_up() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, kernel_of(false), &cfg);
+    e = cudaOccupancyMaxActiveClusters(&n, kernel_of(false, 1), &cfg);
     if (e != cudaSuccess) return e;
     g_clusters[dev][s] = n > 0 ? n : 1;
   }
@@ -1007,7 +1125,7 @@ cudaError_t set_up() {
 
 struct AttnPlan {
   bool rows2;
-  int tiles, groups, splits;
+  int parts, tiles, groups, splits;
 };
 
 // Blocks along the rows and along the keys: the cheapest choice by a cost in SM cycles, rounds of
@@ -1016,10 +1134,12 @@ struct AttnPlan {
 // keys).
 AttnPlan make_plan(const clv_shape& s, int max_ctx_len, const int* clusters) {
   const int G = s.n_q_heads / s.n_kv_heads;
+  const int rows = s.n_nodes * G;
+  const int parts = rows <= BM / 4 ? 4 : rows <= BM / 2 ? 2 : 1;
   const int tiles = (s.n_nodes + BM / G - 1) / (BM / G);   // row tiles of BM / G whole nodes
   const int pieces = (max_ctx_len + PG - 1) / PG + (s.n_nodes + PG - 1) / PG;
   const int64_t units = (int64_t)s.batch * s.n_kv_heads;
-  AttnPlan best = {false, tiles, tiles, 1};
+  AttnPlan best = {false, parts, tiles, tiles, 1};
   double best_cost = 1e300;
   for (int r = 0; r < 2; ++r) {
     if (r && tiles < 2) break;
@@ -1028,8 +1148,10 @@ AttnPlan make_plan(const clv_shape& s, int max_ctx_len, const int* clusters) {
       if (sp > 1 && pieces < 2 * sp) break;   // at least one key tile per block
       const double rounds = (double)((units * groups + clusters[sp] - 1) / clusters[sp]);
       const double key_tiles = (double)((pieces + sp - 1) / sp) * 0.5;
-      const double cost = rounds * (key_tiles * (r ? 3200.0 : 1650.0) + (sp == 1 ? 18000.0 : r ? 36000.0 : 22500.0));
-      if (cost < best_cost) { best_cost = cost; best = {r != 0, tiles, groups, sp}; }
+      const double tile = r ? 3200.0 : parts > 1 ? 1200.0 : 1650.0;
+      const double besides = sp == 1 ? 18000.0 : r ? 36000.0 : parts > 1 ? 19500.0 : 22500.0;
+      const double cost = rounds * (key_tiles * tile + besides);
+      if (cost < best_cost) { best_cost = cost; best = {r != 0, parts, tiles, groups, sp}; }
     }
   }
   return best;
@@ -1060,7 +1182,7 @@ cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const vo
   alignas(64) Maps tm;
   const uint64_t cache_rows = c.paged ? (uint64_t)c.n_pages * CLV_PAGE_SIZE : (uint64_t)s.batch * c.cap_tokens;
   const uint64_t tree_rows = (uint64_t)s.batch * s.n_nodes;
-  if (!make_map_nodes(&tm.q, q, s, (uint32_t)G, (uint32_t)(BM / G)) ||
+  if (!make_map_nodes(&tm.q, q, s, (uint32_t)G, (uint32_t)(BM / plan.parts / G)) ||
       !make_map_nodes(&tm.out, out, s, (uint32_t)G, (uint32_t)(BM / G)) ||
       !make_map(&tm.kc, c.k, cache_rows, s.n_kv_heads, PG) || !make_map(&tm.vc, c.v, cache_rows, s.n_kv_heads, PG) ||
       !make_map(&tm.kt, k_tree, tree_rows, s.n_kv_heads, PG) || !make_map(&tm.vt, v_tree, tree_rows, s.n_kv_heads, PG))
@@ -1089,7 +1211,7 @@ cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const vo
   p.wait_limit = wait_limit_cycles();
   p.tickets = tickets;
   p.blocks_per_seq = s.n_kv_heads * plan.groups * plan.splits;
-  p.tile_nodes = BM / G;
+  p.tile_nodes = BM / plan.parts / G;
   p.by_splits = Divisor::of((unsigned)plan.splits);
   p.by_groups = Divisor::of((unsigned)plan.groups);
   p.by_kv_heads = Divisor::of((unsigned)s.n_kv_heads);
@@ -1109,8 +1231,7 @@ cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const vo
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return plan.rows2 ? cudaLaunchKernelEx(&cfg, tree_attn_kernel<true>, tm, p)
-                    : cudaLaunchKernelEx(&cfg, tree_attn_kernel<false>, tm, p);
+  return cudaLaunchKernelEx(&cfg, kernel_of(plan.rows2, plan.parts), tm, p);
 }
 
 }  // namespace clv

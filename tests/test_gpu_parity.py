@@ -264,6 +264,24 @@ def test_attention_splits_and_row_tiles(clv, oracle, batch, hq, hkv, ctx, n_node
     check_attention(oracle, w, st)
 
 
+@pytest.mark.parametrize("hq,hkv,n_nodes,ctx", [
+    (4, 4, 32, (0, 70)),        # 32 rows, four threads per row; one or two tiles, some parts without a key
+    (16, 16, 33, (190, 2100)),  # 33 rows, two threads per row
+    (14, 2, 4, (100, 600)),     # 28 rows of a group of 7: rows of a copy that no node has
+    (14, 2, 9, (65, 1300)),     # 63 rows
+    (2, 2, 64, (4000, 9000)),   # 64 rows, the keys over all blocks of a cluster
+    (1, 1, 1, (1, 40)),         # one row
+])
+def test_attention_rows_shared_by_threads(clv, oracle, hq, hkv, n_nodes, ctx):
+    cfg = W.small_config(batch=3, n_q_heads=hq, n_kv_heads=hkv, ctx=ctx, n_nodes=n_nodes, vocab=64,
+                         paged=n_nodes == 33, seed=W.BASE_SEED + 700 + n_nodes)
+    w = W.generate(cfg)
+    st = make_step(w)
+    st.tree_attn()
+    torch.cuda.synchronize()
+    check_attention(oracle, w, st)
+
+
 @pytest.mark.parametrize("n_nodes", [16, 128])
 def test_attention_scores_that_outgrow_the_first_tile(clv, oracle, n_nodes):
     # Keys 128 times larger from position 300 on: scores rise by far more than 2^32 between the tiles,
