@@ -382,10 +382,16 @@ cudaError_t launch_accept_sample(const clv_shape& s, const void* logits, int64_t
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((int64_t)rows * a.pieces), 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = even_share_smem((int64_t)rows * a.pieces, 2048 / kThreads);
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, softmax_stats_kernel, a);
+  static OncePerDevice once;
+  cudaError_t e = run_once_per_device(once, [] {
+    return cudaFuncSetAttribute(softmax_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+  });
+  if (e != cudaSuccess) return e;
+  e = cudaLaunchKernelEx(&cfg, softmax_stats_kernel, a);
   if (e != cudaSuccess) return e;
   WalkParams w;
   w.logits = a.logits;
@@ -404,6 +410,7 @@ cudaError_t launch_accept_sample(const clv_shape& s, const void* logits, int64_t
   w.next_token = next_token;
   w.status = status;
   cfg.gridDim = dim3((unsigned)s.batch, 1, 1);
+  cfg.dynamicSmemBytes = 0;
   return cudaLaunchKernelEx(&cfg, sample_walk_kernel, w);
 }
 

@@ -749,6 +749,12 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   const int R = k.R, per = k.per, first = k.first, mine = k.mine;
   const uint32_t smem0 = k.smem0, sRing = k.sRing;
   auto bar = [&](int idx) { return k.bar(idx); };
+  // Calls this short lose a tenth of their time between two launches.  The next kernel may be set up on the
+  // SMs that this grid leaves idle or has left, and waits for this grid's results itself (32 layers of
+  // 1 x 60 nodes x 1500 keys: 503 -> 466 us).  The other variants do not: what follows a long call is a
+  // stream over the logits at full occupancy, whose blocks then pile up on the idle SMs (4 x 64 nodes x
+  // 4096 keys with 256 rows of logits: 44.7 -> 45.9 us).
+  if (kParts > 1) cudaTriggerProgrammaticLaunchCompletion();
   const bool alone = kParts == 1 && CS == 1;   // nothing to be added to this block's accumulators
   const bool aborted = *k.abort_flag != 0;
   if (CS > 1) cluster_arrive();   // all Q K^T of this block are done: what the merge uses is idle (see there)
