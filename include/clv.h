@@ -387,7 +387,8 @@ clv_status clv_kv_commit(const clv_shape* shape, const clv_kv_cache* cache,
  * One whole verify step from HOST buffers (Sec. 2.1: attention, greedy choice, walk, commit in
  * that order).  The per-step inputs are copied from (preferably pinned) host memory to the
  * caller's device staging buffer, the four calls above run, and the results are copied back; all
- * on the given stream, without a synchronisation (results are valid once the stream has drained).
+ * in the given stream's order, without a synchronisation (results are valid once the stream has
+ * drained).  The logits travel on a stream of the library's that this one forks and joins.
  * The KV cache and ctx_len stay on the device; ctx_len is advanced in place.
  */
 typedef struct {          /* host memory; every pointer is a HOST pointer */

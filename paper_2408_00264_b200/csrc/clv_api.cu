@@ -1,5 +1,6 @@
 // C ABI of libclv: argument checks and dispatch.  No device memory is allocated here, nothing
-// synchronises, every launch goes to the caller's stream.
+// synchronises, every launch goes to the caller's stream (the whole step from host buffers also copies on a
+// stream of the library's, between an event of the caller's stream and a wait of it).
 #include <math.h>
 #include <stdint.h>
 #include <stdlib.h>
@@ -457,19 +458,41 @@ clv_status clv_verify_step_host(const clv_shape* shape, const clv_kv_cache* cach
                             reinterpret_cast<int32_t*>(d + L.aidx), reinterpret_cast<int32_t*>(d + L.next),
                             ctx_len, dstat + B, dstat + 2 * B);
   if (st != CLV_OK) return st;
-  cudaError_t e;
-#define CLV_COPY(dst, src, n, kind) \
-  if ((e = cudaMemcpyAsync(dst, src, n, kind, s)) != cudaSuccess) return cuda_fail(e)
-  CLV_COPY(d + L.q, in->q, qb, cudaMemcpyHostToDevice);
-  CLV_COPY(d + L.k_tree, in->k_tree, tb, cudaMemcpyHostToDevice);
-  CLV_COPY(d + L.v_tree, in->v_tree, tb, cudaMemcpyHostToDevice);
-  CLV_COPY(d + L.parent, in->parent, B * N * 4, cudaMemcpyHostToDevice);
-  CLV_COPY(d + L.tokens, in->tokens, B * N * 4, cudaMemcpyHostToDevice);
-  CLV_COPY(d + L.logits, in->logits, B * N * (size_t)in->ld * 2, cudaMemcpyHostToDevice);
-  st = clv_tree_attn(shape, cache, d + L.q, d + L.k_tree, d + L.v_tree,
-                     reinterpret_cast<int32_t*>(d + L.parent), ctx_len, max_ctx_len, softmax_scale,
-                     d + L.out, nullptr, dstat, workspace, workspace_bytes, cuda_stream);
+  // The logits are most of what comes from the host, and only the greedy choice reads them: they (and the
+  // tokens) come on a second stream, behind what the caller's stream holds so far, while attention
+  // runs and its output goes back.
+  SideStream* const side = take_side_stream(s);
+  const cudaStream_t s2 = side ? side->stream : s;
+  cudaError_t e = cudaSuccess;
+  auto copy = [&](void* dst, const void* src, size_t n, cudaMemcpyKind kind, cudaStream_t on) {
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, n, kind, on);
+  };
+  if (side) {
+    e = cudaEventRecord(side->fork, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s2, side->fork, 0);
+  }
+  copy(d + L.q, in->q, qb, cudaMemcpyHostToDevice, s);
+  copy(d + L.k_tree, in->k_tree, tb, cudaMemcpyHostToDevice, s);
+  copy(d + L.v_tree, in->v_tree, tb, cudaMemcpyHostToDevice, s);
+  copy(d + L.parent, in->parent, B * N * 4, cudaMemcpyHostToDevice, s);
+  copy(d + L.tokens, in->tokens, B * N * 4, cudaMemcpyHostToDevice, s2);
+  copy(d + L.logits, in->logits, B * N * (size_t)in->ld * 2, cudaMemcpyHostToDevice, s2);
+  if (side) {   // joined whatever happened: the side stream's next user is not to find this call's copies ahead of an error
+    const cudaError_t je = cudaEventRecord(side->join, s2);
+    if (e == cudaSuccess) e = je;
+  }
+  st = e != cudaSuccess ? cuda_fail(e)
+       : clv_tree_attn(shape, cache, d + L.q, d + L.k_tree, d + L.v_tree,
+                       reinterpret_cast<int32_t*>(d + L.parent), ctx_len, max_ctx_len, softmax_scale,
+                       d + L.out, nullptr, dstat, workspace, workspace_bytes, cuda_stream);
+  if (st == CLV_OK) copy(out->out, d + L.out, qb, cudaMemcpyDeviceToHost, s);
+  if (side) {
+    const cudaError_t we = cudaStreamWaitEvent(s, side->join, 0);
+    if (e == cudaSuccess) e = we;
+    give_side_stream(side);
+  }
   if (st != CLV_OK) return st;
+  if (e != cudaSuccess) return cuda_fail(e);
   st = clv_accept_argmax(shape, d + L.logits, in->ld, reinterpret_cast<int32_t*>(d + L.ids),
                          workspace, workspace_bytes, cuda_stream);
   if (st != CLV_OK) return st;
@@ -479,14 +502,18 @@ clv_status clv_verify_step_host(const clv_shape* shape, const clv_kv_cache* cach
                               reinterpret_cast<int32_t*>(d + L.aidx), reinterpret_cast<int32_t*>(d + L.next),
                               ctx_len, dstat + B, dstat + 2 * B, cuda_stream);
   if (st != CLV_OK) return st;
-  CLV_COPY(out->out, d + L.out, qb, cudaMemcpyDeviceToHost);
-  CLV_COPY(out->argmax_ids, d + L.ids, B * N * 4, cudaMemcpyDeviceToHost);
-  CLV_COPY(out->accept_len, d + L.alen, B * 4, cudaMemcpyDeviceToHost);
-  CLV_COPY(out->accept_idx, d + L.aidx, B * (size_t)shape->path_cap * 4, cudaMemcpyDeviceToHost);
-  CLV_COPY(out->next_token, d + L.next, B * 4, cudaMemcpyDeviceToHost);
-  CLV_COPY(out->status, d + L.status, 3 * B * 4, cudaMemcpyDeviceToHost);
-#undef CLV_COPY
-  return CLV_OK;
+  const size_t at[kHostArrays] = {L.ids, L.alen, L.aidx, L.next, L.status};
+  const size_t words[kHostArrays] = {B * N, B, B * (size_t)shape->path_cap, B, 3 * B};
+  int32_t* const to[kHostArrays] = {out->argmax_ids, out->accept_len, out->accept_idx, out->next_token, out->status};
+  int32_t* mapped[kHostArrays];
+  if (host_arrays_on_device(to, words, mapped)) {
+    const int32_t* from[kHostArrays];
+    for (int k = 0; k < kHostArrays; ++k) from[k] = reinterpret_cast<const int32_t*>(d + at[k]);
+    e = launch_host_results(from, mapped, words, s);
+  } else {
+    for (int k = 0; k < kHostArrays; ++k) copy(to[k], d + at[k], words[k] * 4, cudaMemcpyDeviceToHost, s);
+  }
+  return e == cudaSuccess ? CLV_OK : cuda_fail(e);
 }
 
 const char* clv_status_string(clv_status s) {

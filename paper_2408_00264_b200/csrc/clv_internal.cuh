@@ -105,6 +105,17 @@ cudaError_t launch_token_tree(int batch, int n_cand, int max_len, int node_cap, 
                               const int32_t* cand, const int32_t* cand_len, int32_t* tokens, int32_t* parent,
                               int32_t* n_nodes, int32_t* node_of, int32_t* status, cudaStream_t stream);
 
+// ---- whole step from host buffers
+struct SideStream {
+  cudaStream_t stream;
+  cudaEvent_t fork, join;
+};
+SideStream* take_side_stream(cudaStream_t s);   // null: none to be had, or `s` is being captured
+void give_side_stream(SideStream* s);
+constexpr int kHostArrays = 5;
+bool host_arrays_on_device(int32_t* const* host, const size_t* n, int32_t** device);
+cudaError_t launch_host_results(const int32_t* const* from, int32_t* const* to, const size_t* n, cudaStream_t stream);
+
 int sm_count();   // of the current device
 
 // SM cycles a bounded on-chip wait may last before the block gives up (default: about a second;

@@ -1,0 +1,120 @@
+// What the whole step from host buffers needs besides the step's own kernels: a second stream for the
+// copies that attention does not wait for, and one launch that writes the small results to the host.
+// The step is bound by the link: 1 x 64 nodes, 32000 logits each, are 5.6 MB up (108 us at 52 GB/s) and
+// 0.5 MB down.  Both copies up at once fill the gaps between them, attention and the copy down hide behind
+// the logits: 202 -> 147 us.  (With the logits behind Q and the tree's rows instead of beside them: 156.)
+#include <mutex>
+
+#include "clv_internal.cuh"
+
+namespace clv {
+namespace {
+
+struct SideSlot {
+  SideStream side = {};
+  bool made = false, taken = false;
+};
+constexpr int kSideSlots = 8;   // calls that may be in this function at once; any further one does without
+std::mutex g_side_mu;
+SideSlot g_side[kMaxDevices][kSideSlots];
+
+// Not allowed to disturb a capture that another host thread has under way.
+cudaError_t make_side(SideStream* s) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming);
+  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) {
+    if (s->fork) (void)cudaEventDestroy(s->fork);
+    if (s->stream) (void)cudaStreamDestroy(s->stream);
+    *s = SideStream{};
+    (void)cudaGetLastError();
+  }
+  return e;
+}
+
+struct HostArrays {
+  const int32_t* from[kHostArrays];
+  int32_t* to[kHostArrays];
+  int n[kHostArrays];
+};
+
+__global__ void __launch_bounds__(256) host_results_kernel(HostArrays a) {
+  cudaGridDependencySynchronize();
+  const int t = blockIdx.x * 256 + threadIdx.x, stride = gridDim.x * 256;
+#pragma unroll
+  for (int k = 0; k < kHostArrays; ++k)
+    for (int i = t; i < a.n[k]; i += stride) a.to[k][i] = a.from[k][i];
+}
+
+}  // namespace
+
+// The slot is the caller's until it is given back, which is when the call has enqueued its work: the
+// next user's events then replace this one's, whose waits have taken note of them already.
+SideStream* take_side_stream(cudaStream_t s) {
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone) {
+    (void)cudaGetLastError();
+    return nullptr;   // a side stream would belong to the capture until that ends
+  }
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_side_mu);
+  for (SideSlot& slot : g_side[dev]) {
+    if (slot.taken) continue;
+    if (!slot.made && make_side(&slot.side) != cudaSuccess) return nullptr;
+    slot.made = slot.taken = true;
+    return &slot.side;
+  }
+  return nullptr;
+}
+
+void give_side_stream(SideStream* s) {
+  std::lock_guard<std::mutex> lock(g_side_mu);
+  reinterpret_cast<SideSlot*>(s)->taken = false;   // the stream is the slot's first member
+}
+
+// Device addresses of pinned host arrays; false if one of them (its first or last word) is not pinned.
+bool host_arrays_on_device(int32_t* const* host, const size_t* n, int32_t** device) {
+  for (int k = 0; k < kHostArrays; ++k) {
+    void* at[2];
+    for (int end = 0; end < 2; ++end) {
+      cudaPointerAttributes a;
+      int32_t* const p = host[k] + (end ? n[k] - 1 : 0);
+      if (cudaPointerGetAttributes(&a, p) != cudaSuccess || a.type != cudaMemoryTypeHost || !a.devicePointer) {
+        (void)cudaGetLastError();
+        return false;
+      }
+      at[end] = a.devicePointer;
+    }
+    device[k] = static_cast<int32_t*>(at[0]);
+    if (device[k] + (n[k] - 1) != at[1]) return false;
+  }
+  return true;
+}
+
+// One launch in place of a copy per array: each costs 2 to 3 us of the copy engine, for a few hundred bytes.
+cudaError_t launch_host_results(const int32_t* const* from, int32_t* const* to, const size_t* n, cudaStream_t stream) {
+  HostArrays a;
+  size_t most = 1;
+  for (int k = 0; k < kHostArrays; ++k) {
+    a.from[k] = from[k];
+    a.to[k] = to[k];
+    a.n[k] = (int)n[k];
+    if (n[k] > most) most = n[k];
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((most + 255) / 256 < 64 ? (most + 255) / 256 : 64), 1, 1);
+  cfg.blockDim = dim3(256, 1, 1);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, host_results_kernel, a);
+}
+
+}  // namespace clv

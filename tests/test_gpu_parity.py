@@ -3,6 +3,8 @@
 Integer outputs (argmax ids, accepted path, next token, status, context lengths) and the committed
 cache bytes must match exactly; the attention output must be within max-abs 2e-2 and max-rel 1e-2
 of the checker's float64 result."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -570,6 +572,70 @@ def test_verify_step_from_host_buffers(clv, oracle):
                                           w.ctx_len)
     assert np.array_equal(st.ctx_len.cpu().numpy(), new_len)
     assert np.array_equal(bits(st.k_cache), kc) and np.array_equal(bits(st.v_cache), vc)
+
+
+@pytest.mark.parametrize("mode", ["pageable", "captured", "threads"])
+def test_host_step_ways_to_copy(clv, oracle, mode):
+    # Pageable results (a copy per array), a capture (no second stream), more callers at once than there
+    # are second streams; each caller steps twice from the same buffers.
+    def caller(seed):
+        cfg = W.small_config(batch=2, n_q_heads=4, n_kv_heads=2, ctx=(20, 300), n_nodes=20, vocab=3000,
+                             p_accept=0.8, seed=W.BASE_SEED + seed)
+        w = W.generate(cfg)
+        st = make_step(w, logits=False)
+        place = (lambda t: t) if mode == "pageable" else (lambda t: t.pin_memory())
+        host = [place(torch.from_numpy(a.view(np.int16) if a.dtype == np.uint16 else a))
+                for a in (w.q, w.k_tree, w.v_tree, w.parent, w.tokens, w.logits)]
+        n = (2, 20)
+        res = [place(torch.full(shape, -7, dtype=dtype)) for shape, dtype in (
+            ((*n, 4, 128), torch.int16), (n, torch.int32), ((2,), torch.int32), ((2, w.path_cap), torch.int32),
+            ((2,), torch.int32), ((3, 2), torch.int32))]
+        hin = clv.ClvHostInputs(*[t.data_ptr() for t in host], w.logits.shape[-1])
+        hout = clv.ClvHostOutputs(*[t.data_ptr() for t in res])
+        staging = torch.empty(clv.clv_staging_bytes(st.shape, w.logits.shape[-1]), dtype=torch.uint8, device="cuda")
+        start = st.ctx_len.clone()
+
+        def step():
+            st.ctx_len.copy_(start)
+            clv.clv_verify_step_host(st.shape, st.cache, hin, hout, st.ctx_len, st.max_ctx_len, st.scale, staging,
+                                     st.workspace)
+
+        def check():
+            ids = oracle.argmax(w.logits, w.cfg.vocab)
+            path = oracle.accept_walk(w.parent, w.tokens, ids, w.path_cap)[:3]
+            out = oracle.tree_attn(w.q, w.k_cache, w.v_cache, w.k_tree, w.v_tree, w.parent, w.ctx_len, w.scale)[0]
+            assert_attn_close(res[0].numpy().view(np.uint16), out, mode)
+            for got, ref in zip(res[1:5], (ids, *path)):
+                assert np.array_equal(got.numpy().reshape(-1), np.asarray(ref).reshape(-1))
+            assert (res[5].numpy() == 0).all()
+        return step, check, (st, host, staging)   # the last: kept alive
+
+    callers = [caller(900 + i) for i in range(12 if mode == "threads" else 1)]
+    if mode == "captured":
+        side = torch.cuda.Stream()
+        with torch.cuda.stream(side):
+            callers[0][0]()
+            side.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=side):
+                callers[0][0]()
+        for _ in range(2):
+            g.replay()
+    else:
+        torch.cuda.synchronize()
+
+        def work(step):
+            with torch.cuda.stream(torch.cuda.Stream()):
+                step()
+                step()
+        threads = [threading.Thread(target=work, args=(c[0],)) for c in callers]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+    torch.cuda.synchronize()
+    for c in callers:
+        c[1]()
 
 
 def test_host_step_with_a_bad_argument_leaves_the_stream_empty(clv, oracle):
