@@ -41,8 +41,7 @@ __device__ __forceinline__ int walk_sequence(WalkSmem& sm, int b, int lane, int 
       int found = INT_MAX;
       for (int c = cur + 1 + lane; c < N; c += 32)
         if (sp[c] == cur && st[c] == want) { found = c; break; }
-#pragma unroll
-      for (int s = 16; s > 0; s >>= 1) found = min(found, __shfl_xor_sync(0xFFFFFFFFu, found, s));
+      found = __reduce_min_sync(0xFFFFFFFFu, found);
       if (found == INT_MAX) break;
       if (len == path_cap || len == CLV_MAX_NODES) { bad = true; break; }
       if (lane == 0) path[len] = found;
