@@ -141,7 +141,7 @@ def time_model_step(w, n_layers, dev):
 
 def time_draft_head(rows, hidden, n_heads, vocab, dev):
     """clv_draft_head_step (Attention Decoder, output projector, norm + LM head, top-8) on `rows`
-    rows with random weights: microseconds per step (8 launches, replayed from a CUDA graph) and the
+    rows with random weights: microseconds per step (7 launches, replayed from a CUDA graph) and the
     rate at which the step streams its weights (1.22 GB at hidden 4096 and vocabulary 128256: far
     larger than the L2, so every step reads them from HBM)."""
     import torch
@@ -178,7 +178,7 @@ def time_draft_head(rows, hidden, n_heads, vocab, dev):
     wbytes = (3 * hidden * hidden + 2 * hidden * hidden + vocab * hidden) * 2
     bw_peak, bw_kind = measured_peaks()
     return {"rows": rows, "hidden": hidden, "n_heads": n_heads, "vocab": vocab, "k_top": k, "us": us,
-            "launches": 8, "status": st.cpu().tolist(), "weight_bytes": wbytes, "gbs": wbytes / us / 1e3,
+            "launches": 7, "status": st.cpu().tolist(), "weight_bytes": wbytes, "gbs": wbytes / us / 1e3,
             "frac_of_hbm_peak": {"of_%s_%.0f_GBps" % (bw_kind, bw_peak): wbytes / us / 1e3 / bw_peak}}
 
 
