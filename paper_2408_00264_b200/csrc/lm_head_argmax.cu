@@ -56,6 +56,7 @@ struct Params {
   int out_vec;                // `out` and its strides allow 16-byte accesses
   int two_acc;                // M <= 128: the two accumulators alternate between tiles, so that the
                               //   epilogue of one tile runs under the MMAs of the next
+  int weights_first;          // `out` and two_acc: the weights are the MMA's 128-row operand (see below)
   uint32_t a_tile_bytes;      // bytes one load of the row operand brings (a box of 8..128 rows)
   unsigned long long* keys;   // [M], zero between calls
   unsigned* queue;            // [0] items handed out beyond each block's first, [1] blocks that have stopped drawing; zero between calls
@@ -231,6 +232,16 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
         const uint64_t wd = smem_desc(sW(s), 16, 1024);
         for (int mt = 0; mt < m_tiles; ++mt) {
           const uint64_t ad = smem_desc(sA(s, mt), 16, 1024);
+          if (p.weights_first) {
+            for (int v = 0; v < (p.bn > BM ? 2 : 1); ++v) {
+              const uint64_t vd = wd + (uint64_t)((uint32_t)(v * (p.bn - BM)) * (BK * 2) >> 4);
+#pragma unroll
+              for (int ks = 0; ks < BK / 16; ++ks)
+                umma_bf16_if(el, tmem + (uint32_t)(acc * BN + v * BM), vd + (uint64_t)((ks * 32) >> 4), ad + (uint64_t)((ks * 32) >> 4),
+                             p.idesc, (kc > 0 || ks > 0) ? 1u : 0u);
+            }
+            continue;
+          }
 #pragma unroll
           for (int ks = 0; ks < BK / 16; ++ks)
             umma_bf16_if(el, tmem + (uint32_t)((mt + acc) * BN), ad + (uint64_t)((ks * 32) >> 4), wd + (uint64_t)((ks * 32) >> 4),
@@ -261,7 +272,23 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
       const bool group_used = p.two_acc || (p.M - wi.mb * MB) > mt * BM;
       float best_v = -INFINITY;
       int best_i = INT_MAX;
-      if (group_used) {
+      if (p.weights_first) {   // a lane per vocabulary entry, a column per row
+        float* const out = (wi.prob == 0 ? p.outs[0] : wi.prob == 1 ? p.outs[1] : p.outs[2]) + wi.part * p.out_split_stride;
+        for (int v = 0; v < (p.bn > BM ? 2 : 1); ++v) {
+          const int entry = v * (p.bn - BM) + row_in_tile;
+          const bool mine = wi.col0 + entry < lim && (v == 0 || entry >= BM);   // the two spans of 128 entries may overlap
+#pragma unroll 1
+          for (int c = 0; c < p.M; c += 16) {
+            uint32_t x[16];
+            tmem_ld_x16(tmem + lane_addr + (uint32_t)(mt * BN + v * BM + c), x);
+            tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (mine && c + j < p.M) out[(int64_t)(c + j) * p.ld_out + wi.col0 + entry] = __uint_as_float(x[j]);
+          }
+          __syncwarp();
+        }
+      } else if (group_used) {
 #pragma unroll 1
         for (int c = 0; c < p.bn; c += 32) {
           uint32_t x[32];
@@ -427,7 +454,6 @@ cudaError_t launch_rows_times_weights(int n_prob, const Product* pr, int64_t ld_
   p.V = vocab;
   p.n_tiles = (vocab + cut.bn - 1) / cut.bn;
   p.bn = cut.bn;
-  p.idesc = make_idesc(BM, cut.bn, false);
   p.m_blocks = (rows + MB - 1) / MB;
   p.ids = ids;
   p.out = pr[0].out;
@@ -438,6 +464,13 @@ cudaError_t launch_rows_times_weights(int n_prob, const Product* pr, int64_t ld_
   p.out_split_stride = out_split_stride;
   p.out_vec = p.out != nullptr && vec;
   p.two_acc = rows <= BM;
+  // A few rows against many weights: with the rows as the 128-row operand every MMA multiplies 128 rows, most
+  // of them whatever lies behind the real ones, and a step of the draft head runs into the power cap
+  // (in a loop: 920 W, 1.43-1.6 GHz, 225-241 us by card).  With the weights there, an MMA has 16 columns for up
+  // to 16 rows, and the step keeps 1.97 GHz at 800 W: 220 us.
+  // (The fused argmax keeps a thread per row.)
+  p.weights_first = p.two_acc && p.out != nullptr;
+  p.idesc = p.weights_first ? make_idesc(BM, a_box > 16 ? a_box : 16, false) : make_idesc(BM, cut.bn, false);
   p.a_tile_bytes = (uint32_t)a_box * BK * 2;
   p.queue = ws_queue(tickets);
   p.counter = tickets;
