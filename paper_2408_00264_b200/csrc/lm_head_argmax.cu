@@ -400,12 +400,22 @@ namespace {
 // rows are read more often), and some more per tile; what counts is the number of rounds over the SMs
 // times that.  60 rows x vocabulary 32000 x 4096: 143 tiles of 224 keep 143 SMs busy where 125 tiles of
 // 256 left 23 idle, 51.2 -> 47.4 us.  Below 128 entries a stage of the ring would bring too little.
+// Every stage brings the rows again beside its weights: they count one and a half times, for the bandwidth
+// and for the ring that they take (44 rows x 62745 x 2624: three rounds of tiles of 144 took 78 us, two
+// of 256 take 64).
 struct Cut {
   int bn, splits;
 };
+// rows one load of the row operand brings: the power of two that covers them, 8..128
+int row_box(int rows) {
+  int box = BM;
+  while (box > 8 && box / 2 >= rows) box /= 2;
+  return box;
+}
 Cut plan(int rows, int in_dim, int out_dim, int n, bool may_split) {
   const int m_blocks = (rows + MB - 1) / MB, chunks = in_dim / BK;
   const bool stream = rows <= BM;
+  const int box = row_box(rows);
   Cut best = {BN, 1};
   double best_cost = 1e300;
   for (int sp = 1; sp <= (may_split ? 8 : 1); sp *= 2) {
@@ -413,7 +423,7 @@ Cut plan(int rows, int in_dim, int out_dim, int n, bool may_split) {
     for (int bn = BN; bn >= 128; bn -= 16) {
       const int64_t items = (int64_t)((out_dim + bn - 1) / bn) * m_blocks * n * sp;
       const double rounds = (double)((items + sm_count() - 1) / sm_count());
-      const double cost = rounds * ((double)(chunks / sp) * (stream ? bn * 5.6 : (bn + 16) * 4.3) + (stream ? 700.0 : 4000.0)) + 200.0 * sp;
+      const double cost = rounds * ((double)(chunks / sp) * (stream ? (bn + 1.5 * box) * 5.6 : (bn + 16) * 4.3) + (stream ? 700.0 : 4000.0)) + 200.0 * sp;
       if (cost < best_cost) { best_cost = cost; best = {bn, sp}; }
     }
   }
@@ -437,8 +447,7 @@ cudaError_t launch_rows_times_weights(int n_prob, const Product* pr, int64_t ld_
   if (e0 != cudaSuccess) return e0;
   if (n_prob < 1 || n_prob > kMaxProb) return cudaErrorInvalidValue;
   Maps tm;
-  int a_box = BM;   // rows one load of the row operand brings: the power of two that covers them, 8..128
-  while (a_box > 8 && a_box / 2 >= rows) a_box /= 2;
+  const int a_box = row_box(rows);
   Params p;
   bool vec = (ld_out % 4) == 0 && (out_split_stride % 4) == 0;
   for (int i = 0; i < kMaxProb; ++i) {
