@@ -35,7 +35,8 @@
 // Split-KV: the blocks that share row tiles form a thread-block cluster (1..8 along the key axis).
 // Each sends the accumulator rows that another one finalises as fp16 (half a row scaled by a power of
 // two of its own: 2^-11 relative, against the output's 2^-9) with their reference and sum, by bulk
-// copies from its shared memory to the other's, into tile memory that is idle by then.
+// copies from its shared memory to the other's, into tile memory that is idle by then.  What is
+// added up within a block (the slots; the parts of a row if the block is alone) stays fp32.
 // No partial result touches global memory.
 // Every wait is bounded: on expiry the block raises a flag, all roles leave their loops, in-flight
 // copies and MMAs are drained and CLV_ERR_TIMEOUT is reported for the sequence.
@@ -192,6 +193,11 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap* tm, uint32_t src
 }
 __device__ __forceinline__ void st_shared16(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
   asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+__device__ __forceinline__ float4 ld_shared16(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
 }
 __device__ __forceinline__ void st_shared8(uint32_t a, float x, float y) {
   asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(a), "f"(x), "f"(y) : "memory");
@@ -860,6 +866,12 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
         for (int c = 0; c < 8; ++c)
           st_shared16(dst + (uint32_t)((c ^ (row & 7)) << 4), pack_bf16(v[8 * c], v[8 * c + 1]), pack_bf16(v[8 * c + 2], v[8 * c + 3]),
                       pack_bf16(v[8 * c + 4], v[8 * c + 5]), pack_bf16(v[8 * c + 6], v[8 * c + 7]));
+      } else if (kParts > 1 && CS == 1) {   // no row leaves the block: the parts stay fp32, 512 bytes per row where a cluster would receive
+        const uint32_t dst = rx + (uint32_t)row * 512u;
+#pragma unroll
+        for (int c = 0; c < 16; ++c)   // 16-byte piece c of row r sits at c ^ (r & 31)
+          st_shared16(dst + (uint32_t)(((half * 16 + c) ^ (row & 31)) << 4), __float_as_uint(v[4 * c]), __float_as_uint(v[4 * c + 1]),
+                      __float_as_uint(v[4 * c + 2]), __float_as_uint(v[4 * c + 3]));
       } else {
         float top[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -1009,6 +1021,33 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
         add(acc, j0, i, c, [&](int j) { return w[j]; });
       }
       if (o >= 0) write_row(acc, o, c);
+    }
+  } else if (CS == 1) {   // this block's parts, fp32, eight columns of a row per item
+#pragma unroll 1
+    for (int it = tid; it < mine * 16; it += kThreads) {
+      const int i = it >> 4, c = it & 15, o = row_outs[i];
+      float M = -INFINITY;
+#pragma unroll
+      for (int j = 0; j < kParts; ++j) M = fmaxf(M, own_sums[j * kRows + i].x);
+      const float mu = M == -INFINITY ? 0.f : M;
+      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, total = 0.f;
+#pragma unroll
+      for (int j = 0; j < kParts; ++j) {
+        const float4 m = own_sums[j * kRows + i];
+        const float w = ex2(m.x - mu);   // ex2(-inf) = 0
+        const uint32_t r = (uint32_t)(j * kRows + i), at = rx + r * 512u;
+        const float4 lo = ld_shared16(at + (((uint32_t)(2 * c) ^ (r & 31u)) << 4));
+        const float4 hi = ld_shared16(at + (((uint32_t)(2 * c + 1) ^ (r & 31u)) << 4));
+        const float x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+        total = fmaf(m.y, w, total);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] = fmaf(x[e], w, acc[e]);
+      }
+      const float inv = total > 0.f ? 1.f / total : 0.f;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) acc[e] *= inv;
+      if (o >= 0) write_row(acc, o, c);
+      if (c == 0) write_lse(o, M, total);
     }
   } else {   // up to 32 rows of many sources: eight lanes share a row's sources for one half of its columns
 #pragma unroll 1

@@ -58,6 +58,14 @@ def check_attention(oracle, w, st, rows=None):
     return ref
 
 
+def check_attention_status(oracle, w, st):
+    """The checker's attention output in float64, after a look at the per-sequence status."""
+    ref, _, _, status = oracle.tree_attn(w.q, w.k_cache, w.v_cache, w.k_tree, w.v_tree, w.parent, w.ctx_len, w.scale,
+                                         block_table=w.block_table)
+    assert np.array_equal(st.status[0].cpu().numpy(), status)
+    return ref
+
+
 def check_accept_and_commit(oracle, w, st):
     ids = oracle.argmax(w.logits, w.cfg.vocab)
     assert np.array_equal(st.ids.cpu().numpy(), ids)
@@ -282,6 +290,34 @@ def test_attention_rows_shared_by_threads(clv, oracle, hq, hkv, n_nodes, ctx):
     st.tree_attn()
     torch.cuda.synchronize()
     check_attention(oracle, w, st)
+
+
+@pytest.mark.parametrize("n_nodes,hq,batch", [
+    (13, 8, 40),    # 13 rows, four threads per row
+    (33, 8, 40),    # 33 rows, two threads per row
+    (48, 16, 30),   # 96 rows, one thread per row
+])
+def test_attention_of_a_block_alone_rounds_once(clv, oracle, n_nodes, hq, batch):
+    # More units than the machine takes at a time, so no unit's keys are shared out over blocks and
+    # nothing but the output is rounded to 16 bits.  With equal scores and whole values every
+    # probability and sum is exact in fp32; the quotient is within a few 2^-24, so the output is the
+    # bf16 number nearest to the exact mean, except where that lies within 2^-20 of a midpoint.
+    cfg = W.small_config(batch=batch, n_q_heads=hq, n_kv_heads=8, ctx=(90, 300), n_nodes=n_nodes, vocab=64,
+                         seed=W.BASE_SEED + 811 + n_nodes)
+    w = W.generate(cfg)
+    rng = np.random.default_rng(811)
+    w.q[:] = 0
+    for name in ("v_cache", "v_tree"):
+        v = rng.integers(1, 256, size=getattr(w, name).shape).astype(np.float32)
+        setattr(w, name, W.f32_to_bf16_bits(v))
+    st = make_step(w)
+    st.tree_attn()
+    torch.cuda.synchronize()
+    ref = check_attention_status(oracle, w, st)
+    nearest = [W.f32_to_bf16_bits((ref * (1 + d)).astype(np.float32)) for d in (-2.0 ** -20, 2.0 ** -20)]
+    got, sure = bits(st.out), nearest[0] == nearest[1]
+    assert sure.mean() > 0.99
+    assert np.array_equal(got[sure], nearest[0][sure])
 
 
 @pytest.mark.parametrize("n_nodes", [16, 128])
