@@ -27,8 +27,9 @@
 // Softmax: a thread takes its row's 128 scores into registers and writes P (bf16) back over the score
 // columns.  The exponentials of the first 64 keys are computed with the row's reference as it stands,
 // beside the maximum of all 128; the reference is replaced (O rescaled, those exponentials redone) only
-// when a score exceeds it by 2^32: P is bf16 and the sums are fp32, so a probability above 1 costs
-// no precision, and after a row's first tile the replacement is a rare event.
+// when a score exceeds it by 2^8: P is bf16 and the sums are fp32, so a probability above 1 costs
+// no precision, only range (an accumulator holds |V| up to about 2^120), and after a row's first tile the
+// replacement is a rare event.
 // The tree columns are masked with ancestor bitsets derived from parent[]; masked scores are replaced
 // by -inf, not added to, so they contribute exactly zero.
 //
@@ -68,7 +69,7 @@ constexpr uint32_t kPiece = PG * 64 * 2;       // 8 KB: [64 keys][64 d] swizzled
 constexpr uint32_t kStage = BN * HD * 2;       // 32 KB: a K (or V) tile, [64-wide half of d][128 keys][64 d]
 constexpr uint32_t kHalf = kStage / 2;
 constexpr uint32_t kTmemCols = 512;
-constexpr float kRefSlack = 32.f;      // log2 units a score may exceed the row's reference by
+constexpr float kRefSlack = 8.f;      // log2 units a score may exceed the row's reference by
 constexpr uint32_t kIdescQK = make_idesc(BM, BN, false);  // S[128 rows x 128 keys] = Q K^T
 constexpr uint32_t kIdescPV = make_idesc(BM, HD, true);   // O[128 rows x 128 d] += P V
 
@@ -877,10 +878,10 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
 #pragma unroll
         for (int j = 0; j < 64; j += 2) top[(j >> 1) & 3] = max3(top[(j >> 1) & 3], fabsf(v[j]), fabsf(v[j + 1]));
         const float amax = fmaxf(max3(top[0], top[1], top[2]), top[3]);
-        // scale 2^lc with amax * 2^lc in [2^13, 2^14); lc is clamped so that the scale and its
-        // inverse are normal numbers (zeros stay zeros, inf or NaN stay what they are)
+        // scale 2^lc with amax * 2^lc in [2^13, 2^14), up to the largest fp32 number; lc is clamped so that
+        // the scale and its inverse are normal numbers (zeros stay zeros, inf or NaN stay what they are)
         const int biased = (int)((__float_as_uint(amax) >> 23) & 255u);
-        const int lc = max(-100, min(100, 140 - biased));
+        const int lc = max(-114, min(100, 140 - biased));
         const float up = __uint_as_float((uint32_t)(127 + lc) << 23);
         asm volatile("st.shared.f32 [%0], %1;" ::"r"(meta + (uint32_t)seq_row * 16u + 8u + (uint32_t)half * 4u),
                      "f"(__uint_as_float((uint32_t)(127 - lc) << 23)) : "memory");

@@ -10,7 +10,7 @@ import pytest
 import torch
 
 from paper_2408_00264_b200 import workloads as W
-from parity_util import assert_attn_close, attn_errors, log_parity
+from parity_util import ATTN_MAX_REL, assert_attn_close, attn_errors, log_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -333,6 +333,32 @@ def test_attention_scores_that_outgrow_the_first_tile(clv, oracle, n_nodes):
     st.tree_attn()
     torch.cuda.synchronize()
     check_attention(oracle, w, st)
+
+
+@pytest.mark.parametrize("batch,hq,hkv,n_nodes", [
+    (2, 8, 8, 16),    # one row tile of 16 rows, of 128 (two slots share it), two row tiles per block;
+    (2, 8, 2, 32),    #   keys over several blocks
+    (2, 8, 2, 64),
+    (40, 8, 4, 64),   # blocks alone
+    (40, 4, 4, 20),
+])
+def test_attention_large_values_beside_rising_scores(clv, oracle, batch, hq, hkv, n_nodes):
+    # Scores rise by up to about 2^40 behind the first tiles and the values reach 2^112: a probability of
+    # 2^8 against the row's reference leaves room for that in an fp32 accumulator, one of 2^16 does not.
+    cfg = W.small_config(batch=batch, n_q_heads=hq, n_kv_heads=hkv, ctx=(420, 900), n_nodes=n_nodes, vocab=64,
+                         seed=W.BASE_SEED + 613)
+    w = W.generate(cfg)
+    w.k_cache[:, 300:] = _scale_bf16_by_pow2(w.k_cache[:, 300:], 3)
+    for name in ("v_cache", "v_tree"):
+        setattr(w, name, _scale_bf16_by_pow2(getattr(w, name), 110))
+    st = make_step(w)
+    st.tree_attn()
+    torch.cuda.synchronize()
+    ref = check_attention_status(oracle, w, st)
+    got = bits(st.out)
+    assert np.isfinite(W.bf16_bits_to_f64(got)).all()
+    _, rel = attn_errors(got, ref)
+    assert rel <= ATTN_MAX_REL, rel
 
 
 @pytest.mark.parametrize("n_nodes", [24, 128])   # one row tile per block / two row tiles per block
