@@ -162,6 +162,18 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
       : "l"(reinterpret_cast<unsigned long long&>(a)), "l"(reinterpret_cast<unsigned long long&>(b)));
   return d;
 }
+// Natural log-sum-exp of a row from its reference (in base 2) and its sum, in effect rounded once: the
+// sum is taken apart into 2^e * f, so that the logarithm is below 1, and ref + e keeps its remainder
+// (Knuth's two-sum).  (Base 2 with a product at the end has two roundings of the size of this one.)
+__device__ __forceinline__ float log_sum_exp(float ref, float total) {
+  if (!(total > 0.f && total < INFINITY)) return total > 0.f ? ref + total : total == 0.f ? ref : total;   // no key: ref is -inf
+  constexpr float kLn2 = 0x1.62e43p-1f, kLn2Rest = -0x1.05c61p-29f;
+  const uint32_t u = __float_as_uint(total);
+  const float e = (float)((int)(u >> 23) - 127), f = __uint_as_float((u & 0x007FFFFFu) | 0x3F800000u);
+  const float x = __fadd_rn(ref, e), part = __fsub_rn(x, ref);
+  const float rest = __fadd_rn(__fsub_rn(ref, __fsub_rn(x, part)), __fsub_rn(e, part));
+  return fmaf(x, kLn2, fmaf(rest, kLn2, fmaf(x, kLn2Rest, logf(f))));
+}
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
@@ -833,7 +845,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
       const float inv = ml.y > 0.f ? 1.f / ml.y : 0.f;
       w0 *= inv;
       w1 *= inv;
-      if (p.lse != nullptr && k.row_valid && (kRows2 || slot == 0)) p.lse[row_in_out] = (ml.x + log2f(ml.y)) * 0.6931471805599453f;
+      if (p.lse != nullptr && k.row_valid && (kRows2 || slot == 0)) p.lse[row_in_out] = log_sum_exp(ml.x, ml.y);
     }
     // the last P V of the accumulators this thread reads
     const bool has0 = kRows2 ? k.my_tiles > 0 : T > 0, has1 = !kRows2 && T > 1;
@@ -956,7 +968,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   constexpr int kRows = Cfg<kRows2, kParts>::kRows;
   auto sums_of = [&](int j, int i) { return j < received ? rx_sums[j * per + i] : own_sums[(j - received) * kRows + i]; };
   auto write_lse = [&](int o, float M, float total) {
-    if (p.lse != nullptr && o >= 0) p.lse[o] = (M + log2f(total)) * 0.6931471805599453f;
+    if (p.lse != nullptr && o >= 0) p.lse[o] = log_sum_exp(M, total);
   };
   // 8 columns of row i (16-byte piece c): sources j0 .. j0 + 3 with weights w
   auto add = [&](float (&acc)[8], int j0, int i, int c, auto weight) {

@@ -361,6 +361,22 @@ def test_attention_large_values_beside_rising_scores(clv, oracle, batch, hq, hkv
     assert rel <= ATTN_MAX_REL, rel
 
 
+@pytest.mark.parametrize("batch,hq,hkv,n_nodes,ctx", [(8, 16, 16, 20, (205, 215)), (3, 32, 8, 100, (240, 430))])
+def test_attention_lse_is_rounded_once(clv, oracle, batch, hq, hkv, n_nodes, ctx):
+    # Relative root mean square error of the log-sum-exp.  One rounding to fp32 has at most 2^-24 / sqrt(3) =
+    # 3.4e-8 (results just above a power of two); the fp32 sum of some 220 exponentials of 2^-22
+    # each, with either sign, adds about 2e-8: together below 4.3e-8.  (Two roundings: 4.8e-8 to 5.4e-8.)
+    cfg = W.small_config(batch=batch, n_q_heads=hq, n_kv_heads=hkv, ctx=ctx, n_nodes=n_nodes, vocab=64,
+                         seed=W.BASE_SEED + 619)
+    w = W.generate(cfg)
+    st = make_step(w)
+    st.tree_attn()
+    torch.cuda.synchronize()
+    lse = oracle.tree_attn(w.q, w.k_cache, w.v_cache, w.k_tree, w.v_tree, w.parent, w.ctx_len, w.scale)[2]
+    err = st.lse.cpu().numpy().astype(np.float64) / lse - 1
+    assert np.sqrt((err ** 2).mean()) <= 4.3e-8
+
+
 @pytest.mark.parametrize("n_nodes", [24, 128])   # one row tile per block / two row tiles per block
 def test_attention_wait_that_runs_out_is_reported_and_leaves_the_library_usable(clv, oracle, n_nodes):
     # Every on-chip wait of the attention kernel is bounded.  With the bound cut to a few dozen SM
