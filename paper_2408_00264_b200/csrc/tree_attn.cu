@@ -671,7 +671,9 @@ __device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Pa
 }
 
 // ------------------------------------------------------------------------------------ kernel
-template <bool kRows2, int kParts>
+// kOneBlock: of the variants with several threads per row, the one for a block that is not part of a cluster
+// (the code of neither case lies in the other's way: 1 x 16 nodes x 512 keys took 0.13 us longer in one kernel).
+template <bool kRows2, int kParts, bool kOneBlock>
 __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Params p) {
   constexpr int NST = Cfg<kRows2, kParts>::NST;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -692,7 +694,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     mbar_init(bar(B_Q), 1);
     mbar_init(bar(B_RX), 1);
     mbar_init(bar(B_DR), 1);
-    if (k.CS > 1) mbar_expect_tx(bar(B_RX), (uint32_t)((k.CS - 1) * kParts * k.mine) * 272u);   // what the other ranks will send
+    if (kParts > 1 ? !kOneBlock : k.CS > 1) mbar_expect_tx(bar(B_RX), (uint32_t)((k.CS - 1) * kParts * k.mine) * 272u);   // what the other ranks will send
     ms.abort_flag = 0;
     ms.issued = 0;
     fence_barrier_init();
@@ -774,9 +776,10 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   // stream over the logits at full occupancy, whose blocks then pile up on the idle SMs (4 x 64 nodes x
   // 4096 keys with 256 rows of logits: 44.7 -> 45.9 us).
   if (kParts > 1) cudaTriggerProgrammaticLaunchCompletion();
-  const bool alone = kParts == 1 && CS == 1;   // nothing to be added to this block's accumulators
+  const bool clustered = kParts > 1 ? !kOneBlock : CS > 1;
+  const bool alone = kParts == 1 && !clustered;   // nothing to be added to this block's accumulators
   const bool aborted = *k.abort_flag != 0;
-  if (CS > 1) cluster_arrive();   // all Q K^T of this block are done: what the merge uses is idle (see there)
+  if (clustered) cluster_arrive();   // all Q K^T of this block are done: what the merge uses is idle (see there)
   if (aborted) {
     // copies that were issued land on their own, MMAs that were issued finish: wait for both
     if (warp == kProducer && lane == 0) {
@@ -879,7 +882,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
         for (int c = 0; c < 8; ++c)
           st_shared16(dst + (uint32_t)((c ^ (row & 7)) << 4), pack_bf16(v[8 * c], v[8 * c + 1]), pack_bf16(v[8 * c + 2], v[8 * c + 3]),
                       pack_bf16(v[8 * c + 4], v[8 * c + 5]), pack_bf16(v[8 * c + 6], v[8 * c + 7]));
-      } else if (kParts > 1 && CS == 1) {   // no row leaves the block: the parts stay fp32, 512 bytes per row where a cluster would receive
+      } else if (kOneBlock) {   // no row leaves the block: the parts stay fp32, 512 bytes per row where a cluster would receive
         const uint32_t dst = rx + (uint32_t)row * 512u;
 #pragma unroll
         for (int c = 0; c < 16; ++c)   // 16-byte piece c of row r sits at c ^ (r & 31)
@@ -937,7 +940,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     return;
   }
 
-  if (CS > 1) {
+  if (clustered) {
     cluster_wait();   // every rank's receiving stages are idle
     const int d = tid / kParts, part = tid % kParts;
     if (d < CS && d != split) {   // a peer's rows, then what goes with them
@@ -1035,7 +1038,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
       }
       if (o >= 0) write_row(acc, o, c);
     }
-  } else if (CS == 1) {   // this block's parts, fp32, eight columns of a row per item
+  } else if constexpr (kOneBlock) {   // this block's parts, fp32, eight columns of a row per item
 #pragma unroll 1
     for (int it = tid; it < mine * 16; it += kThreads) {
       const int i = it >> 4, c = it & 15, o = row_outs[i];
@@ -1101,7 +1104,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     }
   }
   __syncwarp();
-  if (CS > 1) cluster_wait();   // no block may leave while a copy still reads its shared memory
+  if (clustered) cluster_wait();   // no block may leave while a copy still reads its shared memory
   publish();
 }
 
@@ -1144,8 +1147,11 @@ bool make_map_halves(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t 
 }
 
 using Kernel = void (*)(Maps, Params);
-Kernel kernel_of(bool rows2, int parts) {
-  return rows2 ? tree_attn_kernel<true, 1> : parts == 4 ? tree_attn_kernel<false, 4> : parts == 2 ? tree_attn_kernel<false, 2> : tree_attn_kernel<false, 1>;
+Kernel kernel_of(bool rows2, int parts, int splits) {
+  if (rows2) return tree_attn_kernel<true, 1, false>;
+  if (parts == 1) return tree_attn_kernel<false, 1, false>;
+  if (splits == 1) return parts == 4 ? tree_attn_kernel<false, 4, true> : tree_attn_kernel<false, 2, true>;
+  return parts == 4 ? tree_attn_kernel<false, 4, false> : tree_attn_kernel<false, 2, false>;
 }
 
 // Once per device: the kernels' shared memory, and how many clusters of each size run at once (one
@@ -1153,7 +1159,8 @@ Kernel kernel_of(bool rows2, int parts) {
 int g_clusters[kMaxDevices][kMaxSplits + 1];
 
 cudaError_t set_up() {
-  const Kernel all[4] = {kernel_of(true, 1), kernel_of(false, 1), kernel_of(false, 2), kernel_of(false, 4)};
+  const Kernel all[] = {kernel_of(true, 1, 1), kernel_of(false, 1, 1), kernel_of(false, 2, 1),
+                        kernel_of(false, 4, 1), kernel_of(false, 2, 2), kernel_of(false, 4, 2)};
   for (const Kernel kernel : all) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     if (e != cudaSuccess) return e;
@@ -1174,7 +1181,7 @@ cudaError_t set_up() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, kernel_of(false, 1), &cfg);
+    e = cudaOccupancyMaxActiveClusters(&n, kernel_of(false, 1, 1), &cfg);
     if (e != cudaSuccess) return e;
     g_clusters[dev][s] = n > 0 ? n : 1;
   }
@@ -1289,7 +1296,7 @@ cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const vo
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kernel_of(plan.rows2, plan.parts), tm, p);
+  return cudaLaunchKernelEx(&cfg, kernel_of(plan.rows2, plan.parts, plan.splits), tm, p);
 }
 
 }  // namespace clv
