@@ -88,6 +88,18 @@ __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) {
   const long long t0 = clock64();
   while (!mbar_try(bar, parity) && clock64() - t0 < kWaitLimitCycles) {}
 }
+// The same for a wait that can also run out: false if the phase took longer than `limit` cycles, but not
+// back before it is complete (or the long bound has passed), because what it waits for writes to this block.
+__device__ __forceinline__ bool mbar_drain_within(uint32_t bar, uint32_t parity, long long limit) {
+  const bool may_suspend = limit >= kSuspendFreeLimit;
+  const long long t0 = clock64();
+  while (!(may_suspend ? mbar_try(bar, parity) : mbar_test(bar, parity)))
+    if (clock64() - t0 > limit) {
+      mbar_drain(bar, parity);
+      return false;
+    }
+  return true;
+}
 __device__ __forceinline__ void fence_barrier_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }

@@ -40,7 +40,8 @@
 // added up within a block (the slots; the parts of a row if the block is alone) stays fp32.
 // No partial result touches global memory.
 // Every wait is bounded: on expiry the block raises a flag, all roles leave their loops, in-flight
-// copies and MMAs are drained and CLV_ERR_TIMEOUT is reported for the sequence.
+// copies and MMAs are drained and CLV_ERR_TIMEOUT is reported for the sequence.  That includes the
+// waits of the merge (the last P V, the other ranks' rows): no rows are written behind one that ran out.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <math.h>
@@ -88,7 +89,8 @@ struct Misc {                           // behind the tiles in dynamic shared me
   float2 ml[2 * BM];                    // (reference, sum) of every row of both slots
   unsigned long long bar[NBAR];
   uint32_t tmem;
-  int abort_flag;
+  int abort_flag;                       // a wait of the roles ran out
+  int late_flag;                        // the wait for the last P V did
   int seq, len;                         // the block's sequence and its context length
   int issued;                           // loads issued (producer)
   signed char parent[CLV_MAX_NODES];    // as far as valid, -1 otherwise
@@ -124,7 +126,7 @@ struct Params {
   int splits;         // blocks along the key axis = cluster size
   float scale_log2;
   long long wait_limit;   // SM cycles a bounded wait may last
-  unsigned* tickets;      // per sequence: [2b] blocks that have finished, [2b+1] error bits; zero between calls
+  unsigned* tickets;      // per sequence: [2b] blocks behind their last wait, [2b+1] what went wrong; zero between calls
   int blocks_per_seq;
   int tile_nodes;         // whole nodes of a row tile
   Divisor by_splits, by_groups, by_kv_heads, by_group_heads;
@@ -696,6 +698,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     mbar_init(bar(B_DR), 1);
     if (kParts > 1 ? !kOneBlock : k.CS > 1) mbar_expect_tx(bar(B_RX), (uint32_t)((k.CS - 1) * kParts * k.mine) * 272u);   // what the other ranks will send
     ms.abort_flag = 0;
+    ms.late_flag = 0;
     ms.issued = 0;
     fence_barrier_init();
     fence_async_smem();
@@ -796,22 +799,23 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     }
     __syncthreads();
   }
-  // status[b] is written once, by whichever block of the sequence finishes last: every block adds
-  // its error bits (1 malformed input, 2 a wait ran out) to the sequence's word in the workspace
-  // and then takes a ticket; the holder of the last ticket turns the bits into the status code and
-  // leaves both words zero for the next call.  The ticket is taken here and looked at when the block
-  // leaves, so that its round trip is hidden behind the merge.
-  unsigned my_ticket = 0;
-  if (tid == 32 * kIssuer) {
-    if (aborted) atomicOr(p.tickets + 2 * b + 1, 2u);
-    if (aborted || (k.group == 0 && split == 0 && kvh == 0)) __threadfence();   // error bits before the ticket
-    my_ticket = atomicInc(p.tickets + 2 * b, (unsigned)p.blocks_per_seq - 1);  // wraps to 0
-  }
+  // status[b] is written once, by whichever block of the sequence finishes last.  The sequence's two words in
+  // the workspace count the blocks that are behind their last wait, and with them, in the upper word, what
+  // went wrong (1: malformed input; 2 for each block in which a wait ran out), so that the holder of the last
+  // ticket has it all from one round trip, behind the final rows; it leaves both words zero for the next
+  // call.
+  unsigned long long* const tally = reinterpret_cast<unsigned long long*>(p.tickets + 2 * b);
+  unsigned long long ticket = 0;
+  auto take_ticket = [&](bool failed) {
+    if (tid != 32 * kIssuer) return;
+    if (k.group == 0 && split == 0 && kvh == 0) __threadfence();   // what the softmax threads reported comes first
+    ticket = atomicAdd(tally, failed ? (2ull << 32) + 1ull : 1ull) + (failed ? 2ull << 32 : 0ull);
+  };
   auto publish = [&]() {
-    if (tid != 32 * kIssuer || my_ticket != (unsigned)p.blocks_per_seq - 1) return;
-    __threadfence();
-    const unsigned bits = atomicExch(p.tickets + 2 * b + 1, 0u);
-    p.status[b] = (bits & 1u) ? CLV_ERR_TREE : (bits & 2u) ? CLV_ERR_TIMEOUT : CLV_OK;
+    if (tid != 32 * kIssuer || (unsigned)ticket != (unsigned)p.blocks_per_seq - 1) return;
+    *tally = 0ull;
+    const unsigned wrong = (unsigned)(ticket >> 32);
+    p.status[b] = (wrong & 1u) ? CLV_ERR_TREE : wrong ? CLV_ERR_TIMEOUT : CLV_OK;
   };
 
   // ---- merge.  Idle once all Q K^T of a block are done, which is when it arrives at the cluster
@@ -853,8 +857,9 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     // the last P V of the accumulators this thread reads
     const bool has0 = kRows2 ? k.my_tiles > 0 : T > 0, has1 = !kRows2 && T > 1;
     if (!aborted) {
-      if (has0) mbar_drain(bar(B_LAST + (kRows2 ? slot : 0)), 0);
-      if (has1) mbar_drain(bar(B_LAST + 1), 0);
+      bool done = true;
+      if (has0) done = wait_warp(bar(B_LAST + (kRows2 ? slot : 0)), 0, &ms.late_flag, p.wait_limit);
+      if (has1 && done) wait_warp(bar(B_LAST + 1), 0, &ms.late_flag, p.wait_limit);
     }
     __syncwarp();
     tc_fence_after();
@@ -923,10 +928,19 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     tc_fence_before();
   }
   __syncthreads();
-  if (warp == kIssuer) { tc_fence_after(); tmem_dealloc(k.tmem, kTmemCols); }
+  bool failed = aborted || *reinterpret_cast<volatile int*>(&ms.late_flag) != 0;   // neither flag is written any more
+  if (warp == kIssuer) {
+    if (failed && !aborted) {   // the last P V is still under way
+      umma_commit_if(elect_one(), bar(B_DR));
+      mbar_drain(bar(B_DR), 0);
+    }
+    tc_fence_after();
+    tmem_dealloc(k.tmem, kTmemCols);
+  }
 
+  if (!clustered) take_ticket(failed);
   if (alone) {
-    if (tid == 0) {
+    if (tid == 0 && !failed) {
 #pragma unroll
       for (int m = 0; m < Cfg<kRows2, kParts>::kQ; ++m) {
         if (m >= users) break;
@@ -953,14 +967,17 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
         bulk_to_peer(cluster_map(rx_meta(base) + at * 16u, (uint32_t)d), meta + (uint32_t)row0 * 16u, (uint32_t)n * 16u, their_bar);
       }
     }
-    mbar_drain(bar(B_RX), 0);
+    const bool got = mbar_drain_within(bar(B_RX), 0, p.wait_limit);
     __syncwarp();
     cluster_arrive();   // what this block was sent has arrived: its peers may leave
+    failed |= __syncthreads_or(got ? 0 : 1) != 0;
+    take_ticket(failed);
   }
   // ---- final rows.  A source of a row is a part of a block's accumulators: first what was received, by
   //      rank, then this block's own, always in this order, so that the result does not depend on timing.
   //      What counts here is the length of one thread's chain: the sources are loaded four at a time
   //      ahead of their sums (one after the other they cost 90 cycles each).
+  const int rows = failed ? 0 : mine;
   constexpr int kSources = kMaxSplits * kParts;
   const int received = (CS - 1) * kParts, sources = CS * kParts;
   const uint8_t* rx_rows = smem + (rx - smem0);                     // of source 0; the next source's are per rows on
@@ -1000,7 +1017,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   };
   if constexpr (kParts == 1) {   // up to 128 rows of few sources: their weights first, a thread per row
     float* weights = reinterpret_cast<float*>(smem + (meta + 8192u - smem0));   // [row][half][source]
-    for (int i = tid; i < mine; i += kThreads) {
+    for (int i = tid; i < rows; i += kThreads) {
       float4 m[kSources];
       float M = -INFINITY;
 #pragma unroll
@@ -1026,7 +1043,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
       write_lse(row_outs[i], M, total);
     }
     __syncthreads();
-    for (int it = tid; it < mine * 16; it += kThreads) {
+    for (int it = tid; it < rows * 16; it += kThreads) {
       const int i = it >> 4, c = it & 15, o = row_outs[i];
       float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -1040,7 +1057,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     }
   } else if constexpr (kOneBlock) {   // this block's parts, fp32, eight columns of a row per item
 #pragma unroll 1
-    for (int it = tid; it < mine * 16; it += kThreads) {
+    for (int it = tid; it < rows * 16; it += kThreads) {
       const int i = it >> 4, c = it & 15, o = row_outs[i];
       float M = -INFINITY;
 #pragma unroll
@@ -1067,8 +1084,8 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     }
   } else {   // up to 32 rows of many sources: eight lanes share a row's sources for one half of its columns
 #pragma unroll 1
-    for (int i0 = 2 * warp; i0 < mine; i0 += 2 * (kThreads / 32)) {
-      const int i = min(i0 + (lane >> 4), mine - 1), c = lane & 15, o = row_outs[i];
+    for (int i0 = 2 * warp; i0 < rows; i0 += 2 * (kThreads / 32)) {
+      const int i = min(i0 + (lane >> 4), rows - 1), c = lane & 15, o = row_outs[i];
       float4 m[kParts];   // sources (lane & 7) + 8 e
       float M = -INFINITY;
 #pragma unroll
@@ -1097,7 +1114,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
         const float scale = (c < 8 ? m[j0 >> 3].z : m[j0 >> 3].w) * (m[j0 >> 3].x * inv);
         add(acc, j0, i, c, [&](int j) { return __shfl_sync(0xFFFFFFFFu, scale, (j0 + j) & 7, 8); });
       }
-      if (i0 + (lane >> 4) < mine) {
+      if (i0 + (lane >> 4) < rows) {
         if (o >= 0) write_row(acc, o, c);
         if (c == 0) write_lse(o, M, total);
       }

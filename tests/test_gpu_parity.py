@@ -401,6 +401,41 @@ def test_attention_wait_that_runs_out_is_reported_and_leaves_the_library_usable(
     check_attention(oracle, w, st)
 
 
+@pytest.mark.parametrize("batch,hq,hkv,n_nodes", [
+    (3, 8, 8, 16),    # clusters: four threads per row, two, one, two row tiles
+    (3, 4, 4, 60),
+    (3, 8, 2, 32),
+    (2, 16, 2, 128),
+    (40, 8, 4, 13),   # blocks alone
+    (40, 8, 2, 32),
+])
+def test_attention_waits_that_run_out_anywhere_are_reported(clv, oracle, batch, hq, hkv, n_nodes):
+    # Bounds from below the first wait to above the last one: whichever wait runs out (for a tile, for the last
+    # product, for another block's rows), a sequence whose status is CLV_OK has the right rows.
+    cfg = W.small_config(batch=batch, n_q_heads=hq, n_kv_heads=hkv, ctx=(300, 2300), n_nodes=n_nodes, vocab=64,
+                         seed=W.BASE_SEED + 405)
+    w = W.generate(cfg)
+    st = make_step(w)
+    ref = oracle.tree_attn(w.q, w.k_cache, w.v_cache, w.k_tree, w.v_tree, w.parent, w.ctx_len, w.scale)[0]
+    seen = set()
+    for limit in [32, 200, 400, 600, 800, 1000, 1300, 1600, 2000, 2500, 3000, 4000, 6000, 9000, 20000, 100000, 0]:
+        st.out.fill_(float("nan"))
+        st.status.fill_(-7)
+        try:
+            clv.clv_test_set_wait_limit(limit)
+            st.tree_attn()
+            torch.cuda.synchronize()
+        finally:
+            clv.clv_test_set_wait_limit(0)
+        status = st.status[0].cpu().numpy()
+        seen.add((limit, bool(status.any())))
+        assert set(status.tolist()) <= {clv.CLV_OK, clv.CLV_ERR_TIMEOUT}, limit
+        done = status == clv.CLV_OK
+        if done.any():
+            assert_attn_close(bits(st.out)[done], ref[done], limit)
+    assert (32, True) in seen and (0, False) in seen
+
+
 # ------------------------------------------------------------------ argmax
 @pytest.mark.parametrize("vocab,ld_pad", [(1, 0), (7, 0), (8, 8), (2047, 0), (2049, 16),
                                           (32000, 0), (50257, 8), (128256, 0)])
