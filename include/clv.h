@@ -23,7 +23,9 @@
  *     The two descriptor structs live in host memory and are read during the call only.
  *   - The caller owns every buffer, including the workspace.  The library allocates no device
  *     memory, never synchronises, and only enqueues work on the given stream (a cudaStream_t
- *     passed as void*; NULL = the legacy default stream).
+ *     passed as void*; NULL = the legacy default stream).  One call, clv_verify_step_host, also uses
+ *     streams of the library's own, up to eight per device, each with two events, made when first
+ *     needed and kept until the process ends; they never order two of the caller's streams.
  *   - Inputs are const.  Only the documented outputs are written; clv_kv_commit writes cache
  *     rows [ctx_len[b], ctx_len[b] + accept_len[b]) of each sequence and nothing else.
  *   - bf16 tensors are dense, innermost dimension contiguous, base 16-byte aligned.
@@ -388,7 +390,9 @@ clv_status clv_kv_commit(const clv_shape* shape, const clv_kv_cache* cache,
  * that order).  The per-step inputs are copied from (preferably pinned) host memory to the
  * caller's device staging buffer, the four calls above run, and the results are copied back; all
  * in the given stream's order, without a synchronisation (results are valid once the stream has
- * drained).  The logits travel on a stream of the library's that this one forks and joins.
+ * drained).  The logits travel on a stream of the library's that this one forks and joins; there is
+ * one for each caller's stream with such a step under way, up to eight per device (a further one, or a
+ * stream being captured, takes all its copies itself).
  * The KV cache and ctx_len stay on the device; ctx_len is advanced in place.
  */
 typedef struct {          /* host memory; every pointer is a HOST pointer */

@@ -13,19 +13,23 @@ namespace {
 struct SideSlot {
   SideStream side = {};
   bool made = false, taken = false;
+  unsigned long long user = 0;   // id of the caller's stream that it served last
 };
-constexpr int kSideSlots = 8;   // calls that may be in this function at once; any further one does without
+constexpr int kSideSlots = 8;   // per device: callers' streams with a step under way; any further one does without
 std::mutex g_side_mu;
 SideSlot g_side[kMaxDevices][kSideSlots];
 
-// Not allowed to disturb a capture that another host thread has under way.
-cudaError_t make_side(SideStream* s) {
+// What is done in here may not disturb a capture that a host thread has under way.
+struct RelaxedCapture {
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  RelaxedCapture() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+cudaError_t make_side(SideStream* s) {
   cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming);
-  (void)cudaThreadExchangeStreamCaptureMode(&mode);
   if (e != cudaSuccess) {
     if (s->fork) (void)cudaEventDestroy(s->fork);
     if (s->stream) (void)cudaStreamDestroy(s->stream);
@@ -52,23 +56,41 @@ __global__ void __launch_bounds__(256) host_results_kernel(HostArrays a) {
 }  // namespace
 
 // The slot is the caller's until it is given back, which is when the call has enqueued its work: the
-// next user's events then replace this one's, whose waits have taken note of them already.
+// next user's events then replace this one's, whose waits have taken note of them already.  What the
+// call has put on the slot's stream waits for the caller's stream, so the next user may be a call on the
+// same stream, or any once that work is done: two streams of a caller's are never ordered by a slot.
 SideStream* take_side_stream(cudaStream_t s) {
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone) {
-    (void)cudaGetLastError();
-    return nullptr;   // a side stream would belong to the capture until that ends
-  }
+  unsigned long long id = 0;   // never used again for another stream, as a handle may be
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-  std::lock_guard<std::mutex> lock(g_side_mu);
-  for (SideSlot& slot : g_side[dev]) {
-    if (slot.taken) continue;
-    if (!slot.made && make_side(&slot.side) != cudaSuccess) return nullptr;
-    slot.made = slot.taken = true;
-    return &slot.side;
+  if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone ||
+      cudaStreamGetId(s, &id) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return nullptr;   // a capture: a side stream would belong to it until it ends
   }
-  return nullptr;
+  if (dev < 0 || dev >= kMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_side_mu);
+  RelaxedCapture relaxed;
+  SideSlot* pick = nullptr;
+  for (SideSlot& slot : g_side[dev])
+    if (slot.made && !slot.taken && slot.user == id) pick = &slot;
+  for (int i = 0; i < kSideSlots && !pick; ++i) {
+    SideSlot& slot = g_side[dev][i];
+    if (slot.taken) continue;
+    if (!slot.made) {
+      if (make_side(&slot.side) != cudaSuccess) return nullptr;
+      slot.made = true;
+      pick = &slot;
+    } else if (cudaEventQuery(slot.side.join) == cudaSuccess) {
+      pick = &slot;
+    } else {
+      (void)cudaGetLastError();   // not done
+    }
+  }
+  if (!pick) return nullptr;
+  pick->taken = true;
+  pick->user = id;
+  return &pick->side;
 }
 
 void give_side_stream(SideStream* s) {

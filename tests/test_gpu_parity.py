@@ -687,68 +687,120 @@ def test_verify_step_from_host_buffers(clv, oracle):
     assert np.array_equal(bits(st.k_cache), kc) and np.array_equal(bits(st.v_cache), vc)
 
 
-@pytest.mark.parametrize("mode", ["pageable", "captured", "threads"])
-def test_host_step_ways_to_copy(clv, oracle, mode):
-    # Pageable results (a copy per array), a capture (no second stream), more callers at once than there
-    # are second streams; each caller steps twice from the same buffers.
-    def caller(seed):
+class HostCaller:
+    """A small step from host buffers with its expected results; `clear` marks every result."""
+
+    def __init__(self, clv, oracle, seed, pinned=True):
         cfg = W.small_config(batch=2, n_q_heads=4, n_kv_heads=2, ctx=(20, 300), n_nodes=20, vocab=3000,
                              p_accept=0.8, seed=W.BASE_SEED + seed)
         w = W.generate(cfg)
-        st = make_step(w, logits=False)
-        place = (lambda t: t) if mode == "pageable" else (lambda t: t.pin_memory())
-        host = [place(torch.from_numpy(a.view(np.int16) if a.dtype == np.uint16 else a))
-                for a in (w.q, w.k_tree, w.v_tree, w.parent, w.tokens, w.logits)]
+        self.clv, self.st = clv, make_step(w, logits=False)
+        place = (lambda t: t.pin_memory()) if pinned else (lambda t: t)
+        self.host = [place(torch.from_numpy(a.view(np.int16) if a.dtype == np.uint16 else a))
+                     for a in (w.q, w.k_tree, w.v_tree, w.parent, w.tokens, w.logits)]
         n = (2, 20)
-        res = [place(torch.full(shape, -7, dtype=dtype)) for shape, dtype in (
+        self.res = [place(torch.full(shape, -7, dtype=dtype)) for shape, dtype in (
             ((*n, 4, 128), torch.int16), (n, torch.int32), ((2,), torch.int32), ((2, w.path_cap), torch.int32),
             ((2,), torch.int32), ((3, 2), torch.int32))]
-        hin = clv.ClvHostInputs(*[t.data_ptr() for t in host], w.logits.shape[-1])
-        hout = clv.ClvHostOutputs(*[t.data_ptr() for t in res])
-        staging = torch.empty(clv.clv_staging_bytes(st.shape, w.logits.shape[-1]), dtype=torch.uint8, device="cuda")
-        start = st.ctx_len.clone()
+        self.hin = clv.ClvHostInputs(*[t.data_ptr() for t in self.host], w.logits.shape[-1])
+        self.hout = clv.ClvHostOutputs(*[t.data_ptr() for t in self.res])
+        self.staging = torch.empty(clv.clv_staging_bytes(self.st.shape, w.logits.shape[-1]), dtype=torch.uint8, device="cuda")
+        self.start = self.st.ctx_len.clone()
+        ids = oracle.argmax(w.logits, w.cfg.vocab)
+        self.expected = (ids, *oracle.accept_walk(w.parent, w.tokens, ids, w.path_cap)[:3])
+        self.out = oracle.tree_attn(w.q, w.k_cache, w.v_cache, w.k_tree, w.v_tree, w.parent, w.ctx_len, w.scale)[0]
 
-        def step():
-            st.ctx_len.copy_(start)
-            clv.clv_verify_step_host(st.shape, st.cache, hin, hout, st.ctx_len, st.max_ctx_len, st.scale, staging,
-                                     st.workspace)
+    def clear(self):
+        for t in self.res:
+            t.fill_(-7)
+        self.staging.fill_(0x55)
 
-        def check():
-            ids = oracle.argmax(w.logits, w.cfg.vocab)
-            path = oracle.accept_walk(w.parent, w.tokens, ids, w.path_cap)[:3]
-            out = oracle.tree_attn(w.q, w.k_cache, w.v_cache, w.k_tree, w.v_tree, w.parent, w.ctx_len, w.scale)[0]
-            assert_attn_close(res[0].numpy().view(np.uint16), out, mode)
-            for got, ref in zip(res[1:5], (ids, *path)):
-                assert np.array_equal(got.numpy().reshape(-1), np.asarray(ref).reshape(-1))
-            assert (res[5].numpy() == 0).all()
-        return step, check, (st, host, staging)   # the last: kept alive
+    def step(self):
+        st = self.st
+        st.ctx_len.copy_(self.start)
+        self.clv.clv_verify_step_host(st.shape, st.cache, self.hin, self.hout, st.ctx_len, st.max_ctx_len, st.scale,
+                                      self.staging, st.workspace)
 
-    callers = [caller(900 + i) for i in range(12 if mode == "threads" else 1)]
+    def check(self):
+        assert_attn_close(self.res[0].numpy().view(np.uint16), self.out)
+        for got, ref in zip(self.res[1:5], self.expected):
+            assert np.array_equal(got.numpy().reshape(-1), np.asarray(ref).reshape(-1))
+        assert (self.res[5].numpy() == 0).all()
+
+
+@pytest.mark.parametrize("mode", ["pageable", "captured", "threads"])
+def test_host_step_ways_to_copy(clv, oracle, mode):
+    # Pageable results (a copy per array), a capture (no second stream), a dozen threads that step at the same
+    # time; the results of every step are marked before it.
+    callers = [HostCaller(clv, oracle, 900 + i, pinned=mode != "pageable") for i in range(12 if mode == "threads" else 1)]
     if mode == "captured":
         side = torch.cuda.Stream()
         with torch.cuda.stream(side):
-            callers[0][0]()
+            callers[0].step()
             side.synchronize()
             g = torch.cuda.CUDAGraph()
             with torch.cuda.graph(g, stream=side):
-                callers[0][0]()
+                callers[0].step()
         for _ in range(2):
+            callers[0].clear()
             g.replay()
-    else:
-        torch.cuda.synchronize()
-
-        def work(step):
-            with torch.cuda.stream(torch.cuda.Stream()):
-                step()
-                step()
-        threads = [threading.Thread(target=work, args=(c[0],)) for c in callers]
-        for t in threads:
-            t.start()
-        for t in threads:
-            t.join()
+            torch.cuda.synchronize()
+            callers[0].check()
+        return
     torch.cuda.synchronize()
-    for c in callers:
-        c[1]()
+    gate, failures = threading.Barrier(len(callers)), []
+
+    def work(c):
+        try:
+            s = torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                for _ in range(12):
+                    c.clear()
+                    gate.wait(60)
+                    c.step()
+                    s.synchronize()
+                    c.check()
+        except BaseException as e:  # noqa: B036
+            failures.append(e)
+            gate.abort()
+    threads = [threading.Thread(target=work, args=(c,)) for c in callers]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failures, failures
+
+
+@pytest.mark.parametrize("held", [1, 11])   # 11: more than the library has second streams
+def test_host_steps_of_different_streams_do_not_wait_for_each_other(clv, oracle, held):
+    # Steps on streams that are busy with something else for a while, then one on a free stream: that one is
+    # done first.  Two steps per held stream: the second follows the first wherever its copies travel.
+    # The device has eight queues for all streams, and a stream that shares one with a held stream waits
+    # whatever the library does, so a few are tried (with 11 held ones only the results count).
+    callers = [HostCaller(clv, oracle, 930 + i) for i in range(held + 1)]
+    overtook = 0
+    for attempt in range(9 if held == 1 else 2):   # the first time everything is made and loaded
+        done = [torch.cuda.Event() for _ in callers]
+        free, *streams = [torch.cuda.Stream() for _ in callers]
+        for c in callers:
+            c.clear()
+        torch.cuda.synchronize()
+        for c, s, e in zip(callers[:held], streams, done):
+            with torch.cuda.stream(s):
+                torch.cuda._sleep(300_000_000)   # about 0.15 s
+                c.step()
+                c.step()
+                e.record()
+        with torch.cuda.stream(free):
+            callers[held].step()
+            done[held].record()
+        done[held].synchronize()
+        overtook += not any(e.query() for e in done[:held])
+        callers[held].check()
+        torch.cuda.synchronize()
+        for c in callers:
+            c.check()
+    assert overtook or held > 1
 
 
 def test_host_step_with_a_bad_argument_leaves_the_stream_empty(clv, oracle):
