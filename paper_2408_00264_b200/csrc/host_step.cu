@@ -3,6 +3,7 @@
 // The step is bound by the link: 1 x 64 nodes, 32000 logits each, are 5.6 MB up (108 us at 52 GB/s) and
 // 0.5 MB down.  Both copies up at once fill the gaps between them, attention and the copy down hide behind
 // the logits: 202 -> 147 us.  (With the logits behind Q and the tree's rows instead of beside them: 156.)
+#include <algorithm>
 #include <mutex>
 
 #include "clv_internal.cuh"
@@ -98,21 +99,25 @@ void give_side_stream(SideStream* s) {
   reinterpret_cast<SideSlot*>(s)->taken = false;   // the stream is the slot's first member
 }
 
-// Device addresses of pinned host arrays; false if one of them (its first or last word) is not pinned.
+// Device addresses of pinned host arrays; false if one of them is not the kernel's to write: not pinned from end
+// to end (asked page by page: what is pinned is whole pages), not aligned, or so long that a copy is
+// as good.
 bool host_arrays_on_device(int32_t* const* host, const size_t* n, int32_t** device) {
+  constexpr size_t kPage = 4096, kMostPages = 64;
   for (int k = 0; k < kHostArrays; ++k) {
-    void* at[2];
-    for (int end = 0; end < 2; ++end) {
+    const uintptr_t begin = reinterpret_cast<uintptr_t>(host[k]), end = begin + n[k] * sizeof(int32_t);
+    if (begin % sizeof(int32_t) != 0 || end - begin > kMostPages * kPage) return false;
+    const uintptr_t last = end - sizeof(int32_t);
+    for (uintptr_t at = begin; at < end; at = at == last ? end : std::min((at / kPage + 1) * kPage, last)) {
       cudaPointerAttributes a;
-      int32_t* const p = host[k] + (end ? n[k] - 1 : 0);
-      if (cudaPointerGetAttributes(&a, p) != cudaSuccess || a.type != cudaMemoryTypeHost || !a.devicePointer) {
+      if (cudaPointerGetAttributes(&a, reinterpret_cast<const void*>(at)) != cudaSuccess || a.type != cudaMemoryTypeHost ||
+          !a.devicePointer) {
         (void)cudaGetLastError();
         return false;
       }
-      at[end] = a.devicePointer;
+      if (at == begin) device[k] = static_cast<int32_t*>(a.devicePointer);
+      else if (reinterpret_cast<uintptr_t>(a.devicePointer) - reinterpret_cast<uintptr_t>(device[k]) != at - begin) return false;
     }
-    device[k] = static_cast<int32_t*>(at[0]);
-    if (device[k] + (n[k] - 1) != at[1]) return false;
   }
   return true;
 }

@@ -690,7 +690,7 @@ def test_verify_step_from_host_buffers(clv, oracle):
 class HostCaller:
     """A small step from host buffers with its expected results; `clear` marks every result."""
 
-    def __init__(self, clv, oracle, seed, pinned=True):
+    def __init__(self, clv, oracle, seed, pinned=True, shift=0):
         cfg = W.small_config(batch=2, n_q_heads=4, n_kv_heads=2, ctx=(20, 300), n_nodes=20, vocab=3000,
                              p_accept=0.8, seed=W.BASE_SEED + seed)
         w = W.generate(cfg)
@@ -699,11 +699,12 @@ class HostCaller:
         self.host = [place(torch.from_numpy(a.view(np.int16) if a.dtype == np.uint16 else a))
                      for a in (w.q, w.k_tree, w.v_tree, w.parent, w.tokens, w.logits)]
         n = (2, 20)
-        self.res = [place(torch.full(shape, -7, dtype=dtype)) for shape, dtype in (
-            ((*n, 4, 128), torch.int16), (n, torch.int32), ((2,), torch.int32), ((2, w.path_cap), torch.int32),
-            ((2,), torch.int32), ((3, 2), torch.int32))]
+        self.dst = [(place(torch.zeros(np.prod(shape) * dtype.itemsize + shift, dtype=torch.uint8)), shape, dtype)
+                    for shape, dtype in (((*n, 4, 128), torch.int16), (n, torch.int32), ((2,), torch.int32),
+                                         ((2, w.path_cap), torch.int32), ((2,), torch.int32), ((3, 2), torch.int32))]
+        self.shift = shift   # bytes from the buffers' starts to the results
         self.hin = clv.ClvHostInputs(*[t.data_ptr() for t in self.host], w.logits.shape[-1])
-        self.hout = clv.ClvHostOutputs(*[t.data_ptr() for t in self.res])
+        self.hout = clv.ClvHostOutputs(*[d.data_ptr() + shift for d, _, _ in self.dst])
         self.staging = torch.empty(clv.clv_staging_bytes(self.st.shape, w.logits.shape[-1]), dtype=torch.uint8, device="cuda")
         self.start = self.st.ctx_len.clone()
         ids = oracle.argmax(w.logits, w.cfg.vocab)
@@ -711,8 +712,8 @@ class HostCaller:
         self.out = oracle.tree_attn(w.q, w.k_cache, w.v_cache, w.k_tree, w.v_tree, w.parent, w.ctx_len, w.scale)[0]
 
     def clear(self):
-        for t in self.res:
-            t.fill_(-7)
+        for d, _, _ in self.dst:
+            d.fill_(0xF9)
         self.staging.fill_(0x55)
 
     def step(self):
@@ -722,17 +723,19 @@ class HostCaller:
                                       self.staging, st.workspace)
 
     def check(self):
-        assert_attn_close(self.res[0].numpy().view(np.uint16), self.out)
-        for got, ref in zip(self.res[1:5], self.expected):
-            assert np.array_equal(got.numpy().reshape(-1), np.asarray(ref).reshape(-1))
-        assert (self.res[5].numpy() == 0).all()
+        res = [d[self.shift:].clone().view(dtype).view(shape).numpy() for d, shape, dtype in self.dst]
+        assert_attn_close(res[0].view(np.uint16), self.out)
+        for got, ref in zip(res[1:5], self.expected):
+            assert np.array_equal(got.reshape(-1), np.asarray(ref).reshape(-1))
+        assert (res[5] == 0).all()
 
 
-@pytest.mark.parametrize("mode", ["pageable", "captured", "threads"])
+@pytest.mark.parametrize("mode", ["pageable", "unaligned", "captured", "threads"])
 def test_host_step_ways_to_copy(clv, oracle, mode):
-    # Pageable results (a copy per array), a capture (no second stream), a dozen threads that step at the same
-    # time; the results of every step are marked before it.
-    callers = [HostCaller(clv, oracle, 900 + i, pinned=mode != "pageable") for i in range(12 if mode == "threads" else 1)]
+    # Pageable results and pinned ones at odd multiples of two bytes (a copy per array), a capture (no second
+    # stream), a dozen threads that step at the same time; the results of every step are marked before it.
+    callers = [HostCaller(clv, oracle, 900 + i, pinned=mode != "pageable", shift=2 * (mode == "unaligned"))
+               for i in range(12 if mode == "threads" else 1)]
     if mode == "captured":
         side = torch.cuda.Stream()
         with torch.cuda.stream(side):
