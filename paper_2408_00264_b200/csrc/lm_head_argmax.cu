@@ -168,6 +168,7 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
       if (p.early_weights) {   // the weights of the first item's first stages; the rows follow below
         const Item wi = decode_item(p, item);
         early = min(p.stages, k_chunks);
+        s_item[0] = item;   // ahead of the arrivals by which its readers are ordered
         for (int i = 0; i < early; ++i) load_w(wi, i, i);
         cudaGridDependencySynchronize();
       }
