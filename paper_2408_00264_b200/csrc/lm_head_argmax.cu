@@ -375,15 +375,10 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
 }
 
 bool make_map_2d(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t k, int64_t ld, uint32_t box_rows) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)k, rows};
   const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
   const cuuint32_t box[2] = {(cuuint32_t)BK, box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return encode_tile_map(tm, base, 2, dims, strides, box);
 }
 
 }  // namespace

@@ -214,5 +214,25 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
+// A 128-byte-swizzled bf16 tile map.  The encoder wants a current context, which a host thread has from its
+// first runtime call that needs one: where this is that call, the current device's is made current.
+bool encode_tile_map(CUtensorMap* tm, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                     const cuuint32_t* box) {
+  const EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  const cuuint32_t step[5] = {1, 1, 1, 1, 1};
+  auto encode = [&] {
+    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, step,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = encode();
+  int dev = 0;
+  if ((r == CUDA_ERROR_INVALID_CONTEXT || r == CUDA_ERROR_NOT_INITIALIZED) && cudaGetDevice(&dev) == cudaSuccess &&
+      cudaSetDevice(dev) == cudaSuccess)
+    r = encode();
+  return r == CUDA_SUCCESS;
+}
+
 }  // namespace
 }  // namespace clv

@@ -1126,21 +1126,12 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
 }
 
 // ------------------------------------------------------------------------------------ host side
-bool encode(CUtensorMap* tm, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  const cuuint32_t estr[4] = {1, 1, 1, 1};
-  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // bf16 tensor [rows][heads][128]; box = 64 elements x 1 head x box_rows, 128-byte swizzle
 bool make_map(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t heads, uint32_t box_rows) {
   const cuuint64_t dims[3] = {(cuuint64_t)HD, heads, rows};
   const cuuint64_t strides[2] = {(cuuint64_t)HD * 2, (cuuint64_t)HD * 2 * heads};
   const cuuint32_t box[3] = {64, 1, box_rows};
-  return encode(tm, base, 3, dims, strides, box);
+  return encode_tile_map(tm, base, 3, dims, strides, box);
 }
 
 // Q and the output: [B][N][Hq][128], box = 64 elements x G heads x `nodes` nodes of one sequence, so
@@ -1150,7 +1141,7 @@ bool make_map_nodes(CUtensorMap* tm, const void* base, const clv_shape& s, uint3
   const cuuint64_t row = (cuuint64_t)HD * 2 * s.n_q_heads;
   const cuuint64_t strides[3] = {(cuuint64_t)HD * 2, row, row * s.n_nodes};
   const cuuint32_t box[4] = {64, G, nodes, 1};
-  return encode(tm, base, 4, dims, strides, box);
+  return encode_tile_map(tm, base, 4, dims, strides, box);
 }
 
 // The cache seen as [rows][heads][2 halves of d][64]: a box of 64 x box_rows x 2 x 1 in the order
@@ -1160,7 +1151,7 @@ bool make_map_halves(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t 
   const cuuint64_t dims[4] = {64, rows, 2, heads};
   const cuuint64_t strides[3] = {(cuuint64_t)HD * 2 * heads, 128, (cuuint64_t)HD * 2};
   const cuuint32_t box[4] = {64, box_rows, 2, 1};
-  return encode(tm, base, 4, dims, strides, box);
+  return encode_tile_map(tm, base, 4, dims, strides, box);
 }
 
 using Kernel = void (*)(Maps, Params);

@@ -3,6 +3,9 @@
 Integer outputs (argmax ids, accepted path, next token, status, context lengths) and the committed
 cache bytes must match exactly; the attention output must be within max-abs 2e-2 and max-rel 1e-2
 of the checker's float64 result."""
+import os
+import subprocess
+import sys
 import threading
 
 import numpy as np
@@ -685,6 +688,40 @@ def test_verify_step_from_host_buffers(clv, oracle):
                                           w.ctx_len)
     assert np.array_equal(st.ctx_len.cpu().numpy(), new_len)
     assert np.array_equal(bits(st.k_cache), kc) and np.array_equal(bits(st.v_cache), vc)
+
+
+_FIRST_CALLS = """
+import sys, threading
+import torch
+from paper_2408_00264_b200 import binding as clv, workloads as W
+from paper_2408_00264_b200.step import VerifyStep
+torch.cuda.init()
+steps = [VerifyStep(W.generate(W.small_config(seed=W.BASE_SEED + i))) for i in range(8)]
+clv._load_calls()
+torch.cuda.synchronize()
+gate, failures = threading.Barrier(len(steps)), []
+def first(st):
+    try:
+        gate.wait(60)
+        st.tree_attn(torch.cuda.current_stream())
+    except Exception as e:
+        failures.append(repr(e))
+threads = [threading.Thread(target=first, args=(st,)) for st in steps]
+[t.start() for t in threads]
+[t.join() for t in threads]
+torch.cuda.synchronize()
+assert not failures, failures
+assert all(int(st.status[0].abs().sum()) == 0 for st in steps)
+"""
+
+
+def test_first_calls_of_a_process_from_several_threads(clv):
+    # What a process sets up once (the driver's tensor-map encoder, the kernels' attributes) is set up by
+    # whichever thread comes first, and the others wait for it; and a thread that has made no call of the
+    # runtime before has no current context: none is refused.
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    for _ in range(3):
+        subprocess.run([sys.executable, "-c", _FIRST_CALLS], check=True, cwd=root, timeout=120)
 
 
 class HostCaller:
