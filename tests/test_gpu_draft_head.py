@@ -55,6 +55,9 @@ def run_gpu(clv, h, e, wts, k_top):
                                          (4, 64, 4, 9000, 32),      # the widest one-pass selection, two levels
                                          (2, 64, 2, 3000, 40),      # beyond it: one pass per proposal
                                          (70, 192, 48, 2049, 2),    # head size 4; one entry in the second slice
+                                         # weights first, with 32, 64 and 128 columns of rows
+                                         (17, 256, 8, 20001, 4), (33, 128, 4, 40003, 8), (65, 192, 4, 3000, 2),
+                                         (130, 128, 4, 70003, 4),   # rows first, several tiles per block
                                          (1, 64, 1, 100, 3), (256, 64, 2, 300, 3)])   # fewest and most rows
 def test_draft_head_step(clv, oracle, R, H, nh, V, k):
     h, e, wts = W.make_draft_head(R, H, nh, V, seed=R + H + V)

@@ -56,12 +56,40 @@ def check_rows(oracle, h_bits, w_bits, got, rows=None):
 
 
 @pytest.mark.parametrize("rows,K,V", [(1, 64, 10), (5, 128, 255), (128, 64, 256), (129, 192, 257),
-                                       (300, 256, 1000), (64, 4096, 1500), (700, 128, 5000)])
+                                       (300, 256, 1000), (64, 4096, 1500), (700, 128, 5000),
+                                       (60, 4096, 32000)])
 def test_planted_winners_exact(clv, oracle, rows, K, V):
     h, w, win = W.make_lm_head(rows, K, V, seed=100 + rows + V)
     got = run_gpu(clv, h, w, ld_pad=8 if rows % 2 else 0)
     assert np.array_equal(got, win)
     assert np.array_equal(oracle.lm_head_argmax(h, w), win)
+
+
+@pytest.mark.parametrize("rows,K,V", [
+    (1, 64, 75827), (8, 128, 85321), (60, 64, 99457),       # tiles of 176, 208 and 240 entries, two to three per block
+    (128, 128, 42971), (60, 128, 106633),                   # 160 and 256
+    (129, 64, 37987), (300, 64, 60001), (700, 64, 66331),   # more than one accumulator of rows: 144, 208 and 240
+])
+def test_winners_at_the_edges_of_tiles_and_of_the_vocabulary(clv, rows, K, V):
+    # Blocks draw several tiles from the queue; the winners lie at both ends of every width of tile (a multiple
+    # of 16) and at the end of the vocabulary.  They lead by far: a row's others have a deviation of
+    # sqrt(1 + 40^2 / K) against 40, so fp32 sums cannot change the choice (looked at below).
+    gen = torch.Generator(device="cuda").manual_seed(rows + K + V)
+    w = torch.randn(V, K, dtype=torch.float32, device="cuda", generator=gen).mul_(K ** -0.5).bfloat16()
+    rng = np.random.default_rng(V)
+    ws = clv.new_workspace(clv.make_shape(1, 1, 1, 1, vocab=8), None, 0)
+    for call in range(max(2, 16 // rows)):
+        at = 16 * rng.integers(1, V // 16, size=rows) - rng.integers(0, 2, size=rows)
+        at[rng.integers(0, rows)] = V - 1 - call % 5
+        win = torch.from_numpy(at).cuda()
+        h = (torch.randn(rows, K, device="cuda", generator=gen) + 40.0 * w[win].float()).bfloat16()
+        top = (h.float() @ w.float().T).topk(2, dim=1)
+        assert torch.equal(top.indices[:, 0], win) and float((top.values[:, 0] - top.values[:, 1]).min()) > 1.0
+        ids = torch.full((rows,), -7, dtype=torch.int32, device="cuda")
+        status = torch.full((1,), -7, dtype=torch.int32, device="cuda")
+        clv.clv_lm_head_argmax(h, w, ids, status, ws)
+        assert int(status.item()) == 0
+        assert torch.equal(ids.long(), win)
 
 
 def test_unplanted_rows_are_valid_choices(clv, oracle):
