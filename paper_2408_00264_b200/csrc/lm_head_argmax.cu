@@ -1,9 +1,9 @@
 // LM head fused with the per-node greedy choice (Sec. 3.1: final norm and LM head of the target;
 // Sec. 4.2: greedy decoding at T = 0): ids[r] = argmax_v round_bf16(<hidden[r, :], W[v, :]>), lowest
-// v on ties.  The logits are never written: each 256 x 256 tile of them lives in tensor memory
-// only, and its row maxima go to one 64-bit key per row with atomicMax.
+// v on ties.  The logits are never written: each tile of them (up to 256 rows x 256 entries) lives in
+// tensor memory only, and its row maxima go to one 64-bit key per row with atomicMax.
 //
-// A persistent block per SM takes (vocabulary tile, row block) pairs from a queue.  Warp 0 streams
+// A persistent block per SM takes (vocabulary tile, row block) pairs, with few rows from a queue.  Warp 0 streams
 // 64-wide K chunks of the weight tile ([up to 256 vocabulary rows][64]) and of the hidden rows ([1 or 2 x
 // 128][64]) through a TMA ring, warp 1 issues tcgen05.mma (M 128, N = the tile's width, K 16; two
 // accumulators of 256 columns fill the tensor memory), warps 2..9 are the epilogue: one thread per row
@@ -12,8 +12,8 @@
 // With a handful of rows the kernel is a stream over the weights, and what is in flight sets its rate:
 // the ring is as deep as shared memory allows and holds only the rows there are (4 rows x 128256 x 4096:
 // 172.9 -> 159.5 us, the measured copy rate).  The width of a tile is chosen so that the tiles divide
-// evenly over the SMs (plan()).  With many rows the tensor core bounds it, at the power cap
-// (1024 rows: 795 -> 780 us, of which the queue is the most).
+// evenly over the SMs (plan()).  With many rows the tensor core bounds it, at the power cap (1024 rows of
+// 128256 x 4096: 840 us).
 #include <cuda_bf16.h>
 #include <limits.h>
 #include <math.h>
@@ -54,6 +54,7 @@ struct Params {
   int k_splits;               // with `out`: the K axis is cut in this many parts, part s writes its partial
   int64_t out_split_stride;   //   products to out + s * out_split_stride (the reader adds the parts up)
   int out_vec;                // `out` and its strides allow 16-byte accesses
+  int use_queue;              // a block's items after its first come from a queue, else every gridDim.x-th is its own
   int two_acc;                // M <= 128: the two accumulators alternate between tiles, so that the
                               //   epilogue of one tile runs under the MMAs of the next
   int weights_first;          // `out` and two_acc: the weights are the MMA's 128-row operand (see below)
@@ -153,9 +154,11 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
 
   if (warp == 0) {
     // =========================== TMA producer ===============================================
-    // A block's first item is its number; the others come from a queue, because the SMs do not get
-    // equal shares of the memory's bandwidth (with equal numbers of tiles the fastest was done after
-    // 0.75 of the time of the slowest).
+    // A block's first item is its number.  With few rows the others come from a queue, because the SMs do
+    // not get equal shares of the memory's bandwidth (with equal numbers of tiles the fastest was done after
+    // 0.75 of the time of the slowest).  With more than 128 the tensor core sets the pace, the same on every
+    // SM, and the queue's end cost more than it brought: a block takes every gridDim.x-th item (551 rows x 18771 x
+    // 2176: 54.7 -> 53.6 us, 513 x 32000 x 4096: 154.9 -> 149.6, 768 x 16384 x 1024: 31.0 -> 30.3).
     if (lane == 0) {
       bool ok = true;
       int s = 0, n = 0, item = blockIdx.x;
@@ -174,8 +177,9 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
       }
       for (; ok; ++n) {
         const bool end = item >= n_items;
+        if (end && !p.use_queue) break;
         unsigned ticket = 0;
-        if (!end) ticket = atomicAdd(p.queue, 1u);   // the next item, looked at when this one has been asked for
+        if (!end && p.use_queue) ticket = atomicAdd(p.queue, 1u);   // the next item, looked at when this one has been asked for
         const Item wi = decode_item(p, item);
         if (end) s_item[(n + 1) % kItems] = -1;
         s_item[n % kItems] = end ? -1 : item;
@@ -193,11 +197,12 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
           if (++s == p.stages) { s = 0; ++round; }
         }
         if (end) break;
-        item = (int)(ticket + gridDim.x);
+        item = (p.use_queue ? (int)ticket : item) + (int)gridDim.x;
       }
-      // the last block to stop drawing leaves the queue empty for the next call
-      __threadfence();
-      if (atomicInc(p.queue + 1, gridDim.x - 1) == gridDim.x - 1) *p.queue = 0u;
+      if (p.use_queue) {   // the last block to stop drawing leaves the queue empty for the next call
+        __threadfence();
+        if (atomicInc(p.queue + 1, gridDim.x - 1) == gridDim.x - 1) *p.queue = 0u;
+      }
     }
   } else if (warp == 1) {
     // =========================== MMA issuer ===================================================
@@ -214,9 +219,11 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
       return true;
     };
     for (int tile = 0; ok; ++tile) {
+      int item = (int)(blockIdx.x + tile * gridDim.x);
+      if (!p.use_queue && item >= n_items) break;
       ok = wait_warp(bar_full(s), round & 1u, abort_flag, wlim);
       if (!ok) break;
-      const int item = __shfl_sync(0xFFFFFFFFu, (int)s_item[tile % kItems], 0);
+      if (p.use_queue) item = __shfl_sync(0xFFFFFFFFu, (int)s_item[tile % kItems], 0);
       ok = acc_free(tile);
       if (!ok) break;
       const int acc = p.two_acc ? (tile & 1) : 0;
@@ -261,8 +268,10 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     for (int tile = p.two_acc ? mt : 0;; tile += p.two_acc ? 2 : 1) {
       const int acc = p.two_acc ? mt : 0;
+      int item = (int)(blockIdx.x + tile * gridDim.x);
+      if (!p.use_queue && item >= n_items) break;
       if (!wait_warp(bar_acc_full(acc), (p.two_acc ? (tile >> 1) : tile) & 1, abort_flag, wlim)) break;
-      const int item = s_item[tile % kItems];
+      if (p.use_queue) item = s_item[tile % kItems];
       if (item < 0) break;
       tc_fence_after();
       const Item wi = decode_item(p, item);
@@ -469,6 +478,7 @@ cudaError_t launch_rows_times_weights(int n_prob, const Product* pr, int64_t ld_
   p.out_split_stride = out_split_stride;
   p.out_vec = p.out != nullptr && vec;
   p.two_acc = rows <= BM;
+  p.use_queue = p.two_acc;
   // A few rows against many weights: with the rows as the 128-row operand every MMA multiplies 128 rows, most
   // of them whatever lies behind the real ones, and a step of the draft head runs into the power cap
   // (in a loop: 920 W, 1.43-1.6 GHz, 225-241 us by card).  With the weights there, an MMA has 16 columns for up
