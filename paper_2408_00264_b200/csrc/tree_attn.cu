@@ -63,6 +63,7 @@ constexpr int kThreads = 384;          // warps 0-3 and 4-7: the slots' softmax;
 // thread, so the third warpgroup's go to the first two while the roles work (256 x 216 + 128 x 72 =
 // 384 x 168; 4 x 64 nodes x 4096 keys: 28.0 -> 26.5 us).
 constexpr int kSoftmaxRegs = 216, kOtherRegs = 72, kLaunchRegs = 168;
+static_assert(2 * kSoftmaxRegs + kOtherRegs <= 3 * kLaunchRegs, "a block shares out the registers that it was launched with");
 constexpr int kSoftmaxWarps = 8, kProducer = 8, kIssuer = 9;
 constexpr int kMaxSplits = 8;          // portable cluster size
 constexpr uint32_t kQTile = BM * HD * 2;      // 32 KB: two [128 rows][64 d] swizzled halves
@@ -1170,7 +1171,10 @@ cudaError_t set_up() {
   const Kernel all[] = {kernel_of(true, 1, 1), kernel_of(false, 1, 1), kernel_of(false, 2, 1),
                         kernel_of(false, 4, 1), kernel_of(false, 2, 2), kernel_of(false, 4, 2)};
   for (const Kernel kernel : all) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e == cudaSuccess && a.numRegs < kLaunchRegs) e = cudaErrorInvalidKernelImage;   // a block would wait for registers that it was not launched with
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
     if (e != cudaSuccess) return e;
   }
   int dev = 0;
