@@ -91,8 +91,9 @@ typedef struct {
 } clv_kv_cache;
 
 /*
- * Workspace.  clv_tree_attn and clv_accept_argmax split their work over more thread blocks than
- * there are independent outputs and combine the pieces through the workspace.
+ * Workspace.  The calls split their work over more thread blocks than there are independent outputs:
+ * arrival counters and the greedy choice's and the sampling's partial results lie in the workspace
+ * (attention merges on chip and needs the counters only).
  * clv_workspace_bytes: bytes needed for this shape with contexts up to max_ctx_len (host call).
  * clv_workspace_init : must be enqueued ONCE on a fresh workspace before its first use (it clears
  *                      the arrival counters; every call leaves them cleared again).  One workspace
@@ -108,7 +109,9 @@ clv_status clv_workspace_init(void* workspace, size_t workspace_bytes, void* cud
  *            ancestor of i (row i of the tree's topology matrix),
  *   out    = softmax(softmax_scale * q . k) . v   over those keys, fp32 accumulation, rounded to
  *            bf16 (nearest even);   lse = natural-log sum-exp of the scaled scores (optional).
- * q/k are taken as given (rotary positions L_b + depth(i) are the caller's business).
+ * q/k are taken as given (rotary positions L_b + depth(i) are the caller's business); softmax_scale > 0.
+ * An accumulator holds values up to about 2^120.  Keys that a row does not see count exactly 0, but 0
+ * times a V that is not finite is NaN: keep the tree's and the cache's V finite.
  * Several roots (extra -1 parents) are accepted here.  L_b = 0 is allowed.
  * status[b] = CLV_ERR_TREE if parent[b] is malformed, L_b < 0, L_b exceeds the cache capacity or
  * a needed block-table entry is outside [0, n_pages); CLV_ERR_TIMEOUT if a bounded on-chip wait of
@@ -172,8 +175,8 @@ clv_status clv_accept_argmax_noalloc(const clv_shape* shape,
 
 /*
  * clv_accept_walk followed by clv_kv_commit in one launch (Sec. 2.1: the verification keeps the
- * drafts the target agrees with, and the cache must afterwards equal plain decoding's): a thread
- * block per sequence walks the tree and then copies the accepted rows.  Arguments, results, error
+ * drafts the target agrees with, and the cache must afterwards equal plain decoding's): a cluster of up
+ * to eight thread blocks per sequence walks the tree and then copies the accepted rows.  Arguments, results, error
  * codes and per-sequence statuses are those of the two calls (walk_status as clv_accept_walk's
  * status, commit_status as clv_kv_commit's); the result is identical to calling them in turn.
  */

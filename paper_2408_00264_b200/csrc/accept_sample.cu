@@ -11,11 +11,11 @@
 //
 // Two launches.  (1) One pass over all logits (an HBM stream like the argmax): every warp
 // reduces a slice of 4096 consecutive logits of a row to (maximum, sum of exponentials relative
-// to it) with an online update, in base-2 units.  (2) One block per sequence walks the tree: per
-// level it combines the slices of the current row, fetches the logits of all children's tokens
-// at once (one round trip to memory), and one thread runs the accept chain; the final draw
-// locates the slice by a running sum over the slices' weights (the weights of struck tokens
-// taken out) and then scans that one slice with the whole block, 16 logits per thread.
+// to it) with an online update, in base-2 units.  (2) One block per sequence fetches what any level of
+// the walk may need at once (every row's slices, every node's logit in its parent's row) and one
+// thread runs the accept chain in shared memory; the final draw locates the slice by a running sum over
+// the slices' weights (the weights of struck tokens taken out) and then scans that one slice with
+// the whole block, 16 logits per thread.
 #include <limits.h>
 #include <math.h>
 

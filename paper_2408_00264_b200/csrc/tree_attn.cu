@@ -16,8 +16,8 @@
 // below the other, and a row's keys are shared out over its copies: the softmax thread of a copy takes 64
 // (32) of a tile's 128 scores, has zeros for the others, and ends up with a partial result of its own.
 // The MMAs take what they take for 128 rows anyway; the softmax, which is what a short call waits for, is
-// half (a quarter) as long and keeps all four of the SM's quadrants busy (1 x 16 nodes x 512 keys:
-// 9.5 -> 8.2 us; 32 layers of 1 x 60 nodes x 1500 keys: 458 -> 425 us).
+// half (a quarter) as long and keeps all four of the SM's quadrants busy (whole steps in a loop, 1 x 16 nodes x
+// 512 keys: 15.8 -> 14.8 us; 32 layers of 1 x 60 nodes x 1500 keys and LM head: 500 -> 470 us).
 // What bounds a key tile of 128 x 128 scores: Q K^T and P V are 16 MMAs of 64 cycles, the
 // exponentials 1024 cycles of the special-function units, and within a slot the two alternate (scores
 // -> exponentials -> P V -> next scores).  With two slots the tensor core works for one while the
@@ -61,7 +61,8 @@ constexpr int CH = 32;                 // keys whose scores one load brings
 constexpr int kThreads = 384;          // warps 0-3 and 4-7: the slots' softmax; 8: TMA producer; 9: MMA issuer; 10, 11 idle
 // Registers per thread: the launch's 168 cannot hold a row's 128 scores and the rest of a softmax
 // thread, so the third warpgroup's go to the first two while the roles work (256 x 216 + 128 x 72 =
-// 384 x 168; 4 x 64 nodes x 4096 keys: 28.0 -> 26.5 us).
+// 384 x 168; 4 x 64 nodes x 4096 keys, launch to launch: 28.0 -> 26.5 us).  (The variant with two threads per row
+// spills: -Xptxas -v reports 4 bytes stored and 20 loaded.)
 constexpr int kSoftmaxRegs = 216, kOtherRegs = 72, kLaunchRegs = 168;
 static_assert(2 * kSoftmaxRegs + kOtherRegs <= 3 * kLaunchRegs, "a block shares out the registers that it was launched with");
 constexpr int kSoftmaxWarps = 8, kProducer = 8, kIssuer = 9;
@@ -776,7 +777,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   auto bar = [&](int idx) { return k.bar(idx); };
   // Calls this short lose a tenth of their time between two launches.  The next kernel may be set up on the
   // SMs that this grid leaves idle or has left, and waits for this grid's results itself (32 layers of
-  // 1 x 60 nodes x 1500 keys: 503 -> 466 us).  The other variants do not: what follows a long call is a
+  // 1 x 60 nodes x 1500 keys and LM head, in a loop: 486 -> 470 us).  The other variants do not: what follows a long call is a
   // stream over the logits at full occupancy, whose blocks then pile up on the idle SMs (4 x 64 nodes x
   // 4096 keys with 256 rows of logits: 44.7 -> 45.9 us).
   if (kParts > 1) cudaTriggerProgrammaticLaunchCompletion();
