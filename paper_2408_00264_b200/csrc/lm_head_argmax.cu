@@ -73,8 +73,24 @@ __device__ __forceinline__ unsigned long long pack_key(float v, int i) {
   const uint32_t ord = (f & 0x80000000u) ? ~f : (f | 0x80000000u);
   return ((unsigned long long)ord << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)i);
 }
-__device__ __forceinline__ float round_bf16(float x) {
-  return __bfloat162float(__float2bfloat16_rn(x));
+// A row's best logit of a tile so far, after rounding to bf16, for each of eight column positions (two per
+// register): the value and the group of eight columns in which it came first, 0xFFFF: nothing above -inf yet.
+// Branch free, four instructions per pair of columns.  A search of every chunk of 32 columns for its rounded
+// maximum took a warp some 350 instructions per chunk, and with more than 128 rows the tensor core waits for
+// the epilogue.
+struct Best {
+  __nv_bfloat162 v[4];
+  uint32_t at[4];
+};
+// columns [8 * group, 8 * group + 32) of the tile
+__device__ __forceinline__ void take_columns(Best& b, const uint32_t (&x)[32], uint32_t group) {
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const __nv_bfloat162 r = __floats2bfloat162_rn(__uint_as_float(x[2 * j]), __uint_as_float(x[2 * j + 1]));
+    const uint32_t above = __hgt2_mask(r, b.v[j & 3]);   // strictly: the first of equals stays; false for NaN
+    b.v[j & 3] = __hmax2(b.v[j & 3], r);                 // NaN operands are dropped
+    b.at[j & 3] = (b.at[j & 3] & ~above) | ((group + (uint32_t)(j >> 2)) * 0x00010001u & above);
+  }
 }
 
 // What a work item is: a vocabulary tile, a row block, with `out` also a part of the K axis and a
@@ -298,46 +314,56 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
           }
           __syncwarp();
         }
+      } else if (group_used && p.out == nullptr) {   // a chunk of 32 columns is fetched while the one before it is taken
+        Best best;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { best.v[j] = __float2bfloat162_rn(-INFINITY); best.at[j] = 0xFFFFFFFFu; }
+        uint32_t x[2][32];
+        const uint32_t acc_addr = tmem + lane_addr + (uint32_t)(mt * BN);
+        tmem_ld_x32(acc_addr, x[0]);
+#pragma unroll 1
+        for (int c0 = 0; c0 < p.bn; c0 += 64) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int c = c0 + 32 * h;
+            if (c >= p.bn) continue;
+            tmem_wait_ld();
+            if (c + 32 < p.bn) tmem_ld_x32(acc_addr + (uint32_t)(c + 32), x[h ^ 1]);
+            if (wi.col0 + c + 32 > lim) {   // the last chunk of a tile or of the vocabulary
+#pragma unroll
+              for (int j = 0; j < 32; ++j)
+                if (wi.col0 + c + j >= lim) x[h][j] = 0xFF800000u;
+            }
+            take_columns(best, x[h], (uint32_t)c >> 3);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t group = (j & 1) ? best.at[j >> 1] >> 16 : best.at[j >> 1] & 0xFFFFu;
+          const float v = (j & 1) ? __high2float(best.v[j >> 1]) : __low2float(best.v[j >> 1]);
+          const int i = wi.col0 + 8 * (int)group + j;
+          if (group != 0xFFFFu && (v > best_v || (v == best_v && i < best_i))) { best_v = v; best_i = i; }
+        }
       } else if (group_used) {
 #pragma unroll 1
         for (int c = 0; c < p.bn; c += 32) {
           uint32_t x[32];
           tmem_ld_x32(tmem + lane_addr + (uint32_t)(mt * BN + c), x);
           tmem_wait_ld();
-          if (p.out != nullptr) {   // plain product: this row's 32 values go to memory
-            if (row_valid) {
-              float* dst = (wi.prob == 0 ? p.outs[0] : wi.prob == 1 ? p.outs[1] : p.outs[2]) +
-                           wi.part * p.out_split_stride + (int64_t)row * p.ld_out + wi.col0 + c;
+          if (row_valid) {   // plain product: this row's 32 values go to memory
+            float* dst = (wi.prob == 0 ? p.outs[0] : wi.prob == 1 ? p.outs[1] : p.outs[2]) +
+                         wi.part * p.out_split_stride + (int64_t)row * p.ld_out + wi.col0 + c;
 #pragma unroll
-              for (int j = 0; j < 8; ++j) {   // four values at a time; the last of a tile or row one by one
-                const int at = wi.col0 + c + 4 * j;
-                if (p.out_vec && at + 4 <= lim) {
-                  reinterpret_cast<uint4*>(dst)[j] = make_uint4(x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
-                } else {
+            for (int j = 0; j < 8; ++j) {   // four values at a time; the last of a tile or row one by one
+              const int at = wi.col0 + c + 4 * j;
+              if (p.out_vec && at + 4 <= lim) {
+                reinterpret_cast<uint4*>(dst)[j] = make_uint4(x[4 * j], x[4 * j + 1], x[4 * j + 2], x[4 * j + 3]);
+              } else {
 #pragma unroll
-                  for (int t = 0; t < 4; ++t)
-                    if (at + t < lim) dst[4 * j + t] = __uint_as_float(x[4 * j + t]);
-                }
+                for (int t = 0; t < 4; ++t)
+                  if (at + t < lim) dst[4 * j + t] = __uint_as_float(x[4 * j + t]);
               }
             }
-            continue;
-          }
-          // rounding to bf16 is monotonic: the chunk's maximum first, the position only if it wins
-          float m = -INFINITY;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float v = (wi.col0 + c + j < lim) ? __uint_as_float(x[j]) : -INFINITY;
-            x[j] = __float_as_uint(v);
-            m = fmaxf(m, v);   // NaN operands are dropped
-          }
-          const float mr = round_bf16(m);
-          if (mr > best_v) {
-            int first = 31;
-#pragma unroll
-            for (int j = 31; j >= 0; --j)
-              if (round_bf16(__uint_as_float(x[j])) == mr) first = j;
-            best_v = mr;
-            best_i = wi.col0 + c + first;
           }
         }
       }

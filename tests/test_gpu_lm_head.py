@@ -92,6 +92,19 @@ def test_winners_at_the_edges_of_tiles_and_of_the_vocabulary(clv, rows, K, V):
         assert torch.equal(ids.long(), win)
 
 
+@pytest.mark.parametrize("rows,V", [(3, 600), (128, 48), (200, 529), (300, 1000)])
+def test_first_of_equal_logits_wherever_they_lie_in_a_tile(clv, rows, V):
+    # Whole numbers, so every logit is exact: row r reads column r % 64 of the matrix, whose highest value
+    # stands at two places; the lower one is the answer, whichever of a thread's positions they fall on.
+    rng = np.random.default_rng(rows + V)
+    w = rng.integers(-2, 2, size=(V, 64)).astype(np.float32)
+    for c in range(64):
+        w[rng.choice(V, size=2, replace=False), c] = 2.0
+    h = np.eye(64, dtype=np.float32)[np.arange(rows) % 64]
+    got = run_gpu(clv, W.f32_to_bf16_bits(h), W.f32_to_bf16_bits(w))
+    assert np.array_equal(got, (h @ w.T).argmax(axis=1))
+
+
 def test_unplanted_rows_are_valid_choices(clv, oracle):
     h, w, _ = W.make_lm_head(200, 512, 4000, seed=77, planted=0.0)
     got = run_gpu(clv, h, w)
