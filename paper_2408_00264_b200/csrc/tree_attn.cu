@@ -21,13 +21,17 @@
 // What bounds a key tile of 128 x 128 scores: Q K^T and P V are 16 MMAs of 64 cycles, the
 // exponentials 1024 cycles of the special-function units, and within a slot the two alternate (scores
 // -> exponentials -> P V -> next scores).  With two slots the tensor core works for one while the
-// other is in its exponentials, and P is handed over in three parts (64, 32, 32 keys), so that only
-// the last quarter of P V is left when the exponentials are done.
+// other is in its exponentials, and P is handed over in two parts (96 and 32 keys), so that only the last
+// quarter of P V is left when the exponentials are done.  (Three parts of 64, 32 and 32, the second after the
+// last exponentials: half of it was left; 3 x 64 nodes x 16384 keys 64.8 -> 62.2 us, 8 x 128 x 32768 508 -> 500.)
+// Leaving the exponentials out altogether does not shorten a call: what a tile takes is the chain through
+// both units and the waits between them, so what counts is the length of a thread's instructions.
 //
 // Softmax: a thread takes its row's 128 scores into registers and writes P (bf16) back over the score
 // columns.  The exponentials of the first 64 keys are computed with the row's reference as it stands,
-// beside the maximum of all 128; the reference is replaced (O rescaled, those exponentials redone) only
-// when a score exceeds it by 2^8: P is bf16 and the sums are fp32, so a probability above 1 costs
+// beside the maximum of the others; their sum, which the row needs anyway, says whether one of them is above
+// 2^8 (their maximum besides: 3 x 64 x 16384 62.9 -> 60.7 us, 8 x 128 x 32768 500 -> 487).  The reference is replaced
+// (O rescaled, those exponentials redone) only when a score exceeds it by 2^8 or their sum does: P is bf16 and the sums are fp32, so a probability above 1 costs
 // no precision, only range (an accumulator holds |V| up to about 2^120), and after a row's first tile the
 // replacement is a rare event.
 // The tree columns are masked with ancestor bitsets derived from parent[]; masked scores are replaced
@@ -73,6 +77,7 @@ constexpr uint32_t kStage = BN * HD * 2;       // 32 KB: a K (or V) tile, [64-wi
 constexpr uint32_t kHalf = kStage / 2;
 constexpr uint32_t kTmemCols = 512;
 constexpr float kRefSlack = 8.f;      // log2 units a score may exceed the row's reference by
+constexpr float kTopP = 256.f;        // the same for its probability
 constexpr uint32_t kIdescQK = make_idesc(BM, BN, false);  // S[128 rows x 128 keys] = Q K^T
 constexpr uint32_t kIdescPV = make_idesc(BM, HD, true);   // O[128 rows x 128 d] += P V
 
@@ -340,12 +345,12 @@ struct Block {
 
 // ---- the roles' work on the block's share of the keys
 
-// A tile's P is handed over in parts: keys 0-63, 64-95, 96-127 if a thread has all keys of its row, else
+// A tile's P is handed over in parts: keys 0-95, 96-127 if a thread has all keys of its row, else
 // the first and the second 32 of every thread's, or all at once.
 template <int kParts>
-__host__ __device__ constexpr int hand_overs() { return kParts == 1 ? 3 : kParts == 2 ? 2 : 1; }
+__host__ __device__ constexpr int hand_overs() { return kParts <= 2 ? 2 : 1; }
 template <int kParts>
-__host__ __device__ constexpr int handed_over_in(int c) { return kParts == 1 ? (c < 2 ? 0 : c - 1) : kParts == 2 ? (c & 1) : 0; }   // 32 keys c
+__host__ __device__ constexpr int handed_over_in(int c) { return kParts == 1 ? (c < 3 ? 0 : 1) : kParts == 2 ? (c & 1) : 0; }   // 32 keys c
 
 // Q needs nothing that is read from memory, so it is asked for ahead of the context length.
 template <bool kRows2, int kParts>
@@ -471,7 +476,7 @@ __device__ __forceinline__ bool issue(const Block<kRows2, kParts>& k, const Para
       const int keys[2] = {k.piece_keys(g0), k.piece_keys(g0 + 1)};
 #pragma unroll
       for (int h = 0; h < hand_overs<kParts>(); ++h) {
-        if (!ok || (kParts == 1 && h > 0 && keys[1] <= (h - 1) * CH)) continue;
+        if (!ok || (kParts == 1 && h > 0 && keys[1] <= CH)) continue;
         ok = wait_warp(k.bar(B_P + 3 * s + h), (ph >> (3 * s + h)) & 1u, k.abort_flag, p.wait_limit);
         if (!ok) continue;
         ph ^= 1u << (3 * s + h);
@@ -532,7 +537,7 @@ __device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Pa
   const uint32_t s_addr = k.tmem_S(slot) + k.lane_addr;   // this row's scores, then its P
   const float sc = p.scale_log2;
   float m_ref = k.row_valid ? -INFINITY : 0.f, l_run = 0.f;
-  auto hand_over = [&](int h) {   // part h of P: keys 0-63, 64-95, 96-127 of the tile
+  auto hand_over = [&](int h) {   // part h of P
     tmem_wait_st();
     tc_fence_before();
     __syncwarp();
@@ -571,8 +576,7 @@ __device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Pa
     vpos.advance(Cfg<kRows2, kParts>::kStep);
     if (kParts == 1 && !warp_active) {   // no row of this warp exists: its lanes of P may hold anything
       hand_over(0);
-      if (keys1 > 0) hand_over(1);
-      if (keys1 > CH) hand_over(2);
+      if (keys1 > CH) hand_over(1);
       continue;
     }
     const bool masked = !plain;   // rows that do not exist compute what nobody reads
@@ -663,7 +667,6 @@ __device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Pa
     load(2, x2);
     load(3, x3);
     if (masked) mask(0, x0);
-    take_max(x0);
     exps(x0);
     tmem_wait_ld();
     if (masked) {
@@ -671,40 +674,42 @@ __device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Pa
       mask(2, x2);
       mask(3, x3);
     }
-    take_max(x1);
     take_max(x2);
     take_max(x3);
     exps(x1);
-    const float m_new = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]) * sc;   // scale > 0; no allowed key: -inf
-    const bool need = m_new > m_ref + kRefSlack;
+    float m_new = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]) * sc;   // scale > 0; no allowed key: -inf
+    const float s01 = (sum[0].x + sum[0].y) + (sum[1].x + sum[1].y);   // no less than the largest of its 64 terms
+    bool need = s01 > kTopP || m_new > m_ref + kRefSlack || m_ref == -INFINITY;
     if (__any_sync(0xFFFFFFFFu, need)) {
-      new_reference(m_new, need);   // the scores of the first 64 keys are still in place
-      sum[0] = sum[1] = make_float2(0.f, 0.f);
-      load(0, x0);
+      load(0, x0);   // the scores of the first 64 keys are still in place
       load(1, x1);
       tmem_wait_ld();
       if (masked) {
         mask(0, x0);
         mask(1, x1);
       }
+      take_max(x0);
+      take_max(x1);
+      m_new = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]) * sc;
+      need = need && m_new > m_ref;
+      new_reference(m_new, need);
+      sum[0] = sum[1] = make_float2(0.f, 0.f);
       exps(x0);
       exps(x1);
     }
     store_p(0, x0);
     store_p(1, x1);
-    if (keys1 > CH) {   // a part's stores have the time of the next exponentials before they are waited for
+    if (keys1 > CH) {
       exps(x2);
-      hand_over(0);
       store_p(2, x2);
+      hand_over(0);
       exps(x3);
-      hand_over(1);
       store_p(3, x3);
-      hand_over(2);
+      hand_over(1);
     } else if (keys1 > 0) {
       exps(x2);
-      hand_over(0);
       store_p(2, x2);
-      hand_over(1);
+      hand_over(0);
     } else {
       hand_over(0);
     }
