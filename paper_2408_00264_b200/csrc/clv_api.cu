@@ -74,7 +74,8 @@ extern "C" {
 size_t clv_workspace_bytes(const clv_shape* shape, const clv_kv_cache* cache, int32_t max_ctx_len) {
   (void)cache;
   if (check_shape(shape) != CLV_OK) return 0;
-  size_t scratch = tree_attn_scratch_bytes(*shape, max_ctx_len);
+  (void)max_ctx_len;
+  size_t scratch = 0;   // attention merges on chip
   if (shape->vocab > 0) {
     const ArgmaxPlan gp = argmax_plan(shape->batch * shape->n_nodes, shape->vocab);
     if (gp.scratch_bytes > scratch) scratch = gp.scratch_bytes;
@@ -121,8 +122,7 @@ clv_status clv_tree_attn(const clv_shape* shape, const clv_kv_cache* cache, cons
                                            out, status, workspace, workspace_bytes);
   if (st != CLV_OK) return st;
   cudaError_t e = launch_tree_attn(*shape, *cache, q, k_tree, v_tree, parent, ctx_len, max_ctx_len, softmax_scale,
-                                   out, lse, status, ws_tickets(workspace), ws_scratch(workspace),
-                                   workspace_bytes - kWsFixedBytes, static_cast<cudaStream_t>(cuda_stream));
+                                   out, lse, status, ws_tickets(workspace), static_cast<cudaStream_t>(cuda_stream));
   return e == cudaSuccess ? CLV_OK : cuda_fail(e);
 }
 

@@ -79,9 +79,8 @@ cudaError_t launch_tree_from_intervals(int batch, int n_nodes, const int32_t* ti
 bool tree_attn_supported(const clv_shape& s, const clv_kv_cache& c);
 cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const void* q, const void* k_tree,
                              const void* v_tree, const int32_t* parent, const int32_t* ctx_len, int max_ctx_len,
-                             float scale, void* out, float* lse, int32_t* status, unsigned* tickets, void* scratch,
-                             size_t scratch_bytes, cudaStream_t stream);   // less scratch than it could use: another route
-size_t tree_attn_scratch_bytes(const clv_shape& s, int max_ctx_len);
+                             float scale, void* out, float* lse, int32_t* status, unsigned* tickets,
+                             cudaStream_t stream);
 
 // ---- LM head fused with the argmax (tcgen05 GEMM whose logits stay in tensor memory) ---------------
 bool lm_head_supported(int rows, int hidden, int vocab);

@@ -89,19 +89,8 @@ struct Cfg {
   static constexpr int kStep = kRows2 ? 2 : 4;   // loads from one tile of a slot to its next
 };
 
-// barriers: stage full [6] | stage empty [6] | S full [2] | part of P [2][3] | last P V done [2] | Q | merge | drain | Q read
-constexpr int B_FULL = 0, B_EMPTY = 6, B_S = 12, B_P = 14, B_LAST = 20, B_Q = 22, B_RX = 23, B_DR = 24, B_QFREE = 25, NBAR = 26;
-
-// What a role knows about its way through the units of its block's range (even shares).
-struct Way {
-  int b, head, len;                // the unit that comes next, its sequence's length
-  int base, at, end;               // where it starts in the row of all units, what is taken next, the range's end
-  int seq, kv_head, seq_len;       // the unit that is being worked on
-  int first_tile, end_tile;        //   the block's share of its tiles,
-  int tiles, unit;                 //   how many there are, where it starts
-  int loads_before, tiles_before;  // of the block's other units: loads of the ring, tiles of the thread's slot
-  uint32_t last_phases;            // bit s: parity of the next use of the barrier behind slot s's last P V
-};
+// barriers: stage full [6] | stage empty [6] | S full [2] | part of P [2][3] | last P V done [2] | Q | merge | drain
+constexpr int B_FULL = 0, B_EMPTY = 6, B_S = 12, B_P = 14, B_LAST = 20, B_Q = 22, B_RX = 23, B_DR = 24, NBAR = 25;
 
 struct Misc {                           // behind the tiles in dynamic shared memory
   float2 ml[2 * BM];                    // (reference, sum) of every row of both slots
@@ -111,11 +100,6 @@ struct Misc {                           // behind the tiles in dynamic shared me
   int late_flag;                        // the wait for the last P V did
   int seq, len;                         // the block's sequence and its context length
   int issued;                           // loads issued (producer)
-  int q_loads;                          // blocks that work on several units: loads of Q,
-  int last;                             //   whether this block had the last of a unit's keys,
-  int start, start_seq;                 //   where the block's range starts: position of a sequence's first unit
-  int total;                            //   length of the row of all units
-  Way way[8];                           //   of the softmax warps: kept in registers it would push their scores out
   signed char parent[CLV_MAX_NODES];    // as far as valid, -1 otherwise
 };
 constexpr uint32_t kMiscAt = 7 * kStage;   // either way: Q tiles + ring = 224 KB
@@ -153,9 +137,6 @@ struct Params {
   int blocks_per_seq;
   int tile_nodes;         // whole nodes of a row tile
   Divisor by_splits, by_groups, by_kv_heads, by_group_heads;
-  int ranges;             // even shares: ranges of each group's row of units
-  float4* parts;          //   partial results, two per block: fp32 rows, 16 bytes of all rows side by side,
-  float2* part_sums;      //   and (reference, sum) of each row
 };
 
 struct Maps {
@@ -263,7 +244,6 @@ struct Block {
   uint32_t smem0, sRing, bar0, tmem;
   volatile int* abort_flag;
   int tid, warp, lane;
-  unsigned block;
   int CS, split, group, kvh, b;            // cluster size, rank in the cluster, rows' group, kv head, sequence
   int N, G, tile_nodes, RT, tile0, users;  // whole nodes of a row tile and the rows they take; first row tile; slots that read one K/V tile
   int R, per, first, mine;                 // rows in use, numbered through the row tiles; rank d finalises [d * per, (d + 1) * per)
@@ -284,8 +264,7 @@ struct Block {
   __device__ __forceinline__ int slot_tiles(int s) const { return kRows2 ? (s < users ? T : 0) : (T - s + 1) / 2; }
 
   // the place in the grid (blocks of a cluster are neighbours along x)
-  __device__ __forceinline__ void place(const Params& p, uint8_t* sm, unsigned blk, int thread) {
-    block = blk;
+  __device__ __forceinline__ void place(const Params& p, uint8_t* sm, unsigned block, int thread) {
     smem = sm;
     smem0 = smem_u32(sm);
     sRing = smem0 + Cfg<kRows2, kParts>::kQ * kQTile;
@@ -312,24 +291,14 @@ struct Block {
   // and walks it in tiles of two; the last tile of a range may hold one piece only.  A bad length
   // reads the tree's own rows only.  Tiles [0, t_plain) consist of two complete pieces of context.
   __device__ __forceinline__ void range(const Params& p, int len) {
-    length(p, len);
-    thread_place(p);
-    share((int)p.by_splits.divide((unsigned)split * (unsigned)p_total), (int)p.by_splits.divide((unsigned)(split + 1) * (unsigned)p_total));
-  }
-  __device__ __forceinline__ void length(const Params& p, int len) {
     L = len;
     len_bad = (L < 0) || (p.paged ? ((L + PG - 1) / PG > p.max_pages) : (L > p.cap_tokens));
     p_cache = (!len_bad && L > 0) ? (L + PG - 1) / PG : 0;
     p_total = p_cache + (N + PG - 1) / PG;
-  }
-  __device__ __forceinline__ void share(int begin, int end) {
-    pc_begin = begin;
-    pc_end = end;
+    pc_begin = (int)p.by_splits.divide((unsigned)split * (unsigned)p_total);
+    pc_end = (int)p.by_splits.divide((unsigned)(split + 1) * (unsigned)p_total);
     T = (pc_end - pc_begin + 1) / 2;
     t_plain = max(0, (min(pc_end, len_bad ? 0 : L / PG) - pc_begin) / 2);
-    my_tiles = slot_tiles(slot);
-  }
-  __device__ __forceinline__ void thread_place(const Params& p) {
     tmem = misc().tmem;
     slot = (warp >> 2) & 1;
     row = (warp & 3) * 32 + lane;   // a warp may touch the 32 tensor-memory lanes of its number modulo 4
@@ -340,6 +309,7 @@ struct Block {
     node_in_tile = (int)p.by_group_heads.divide((unsigned)tile_row);
     node = rtile * tile_nodes + node_in_tile;
     row_valid = warp < kSoftmaxWarps && tile_row < RT && rtile < p.tiles && node < N;
+    my_tiles = slot_tiles(slot);
   }
 };
 
@@ -367,10 +337,12 @@ __device__ __forceinline__ void load_q(const Block<kRows2, kParts>& k, const Map
 }
 
 template <bool kRows2, int kParts>
-__device__ __forceinline__ bool produce(const Block<kRows2, kParts>& k, const Maps& tm, const Params& p, int issued) {   // loads so far
+__device__ __forceinline__ void produce(const Block<kRows2, kParts>& k, const Maps& tm, const Params& p) {
   constexpr int NST = Cfg<kRows2, kParts>::NST;
+  if (k.T == 0) mbar_drain(k.bar(B_Q), 0);   // nobody else waits for the Q that is on its way
   int page = 0, page_base = -64;   // lane j: pool page of context piece (page_base + j)
-  RingPos<NST> pos(issued);
+  RingPos<NST> pos(0);
+  int issued = 0;
   bool ok = true;
   for (int t = 0; t < k.T && ok; ++t) {
     const int g0 = k.pc_begin + 2 * t;
@@ -420,7 +392,6 @@ __device__ __forceinline__ bool produce(const Block<kRows2, kParts>& k, const Ma
     }
   }
   if (k.lane == 0) k.misc().issued = issued;   // for the drain of an aborted block
-  return ok;
 }
 
 // The whole warp walks the schedule and one elected lane issues: inside a divergent branch every
@@ -429,22 +400,16 @@ __device__ __forceinline__ bool produce(const Block<kRows2, kParts>& k, const Ma
 // order: Q K^T of both slots, then per tile and slot P V of the tile's parts as they are handed over and
 // Q K^T of the slot's next tile.  The tensor core queues a few MMAs, so what lies between two groups
 // of them is hidden.
-// What a block did before (not zero where it works on several units): loads of the ring, units.
-struct Before {
-  int loads, units;
-  uint32_t ph;   // bit 3 s + h: parity of the next use of the barrier for part h of slot s's P
-};
-template <bool kRows2, int kParts, bool kMany>
-__device__ __forceinline__ bool issue(const Block<kRows2, kParts>& k, const Params& p, Before& before) {
+template <bool kRows2, int kParts>
+__device__ __forceinline__ void issue(const Block<kRows2, kParts>& k, const Params& p) {
   constexpr int NST = Cfg<kRows2, kParts>::NST;
   const uint32_t el = elect_one();
-  if (k.T == 0 || !wait_warp(k.bar(B_Q), (uint32_t)before.units & 1u, k.abort_flag, p.wait_limit)) return false;
+  if (k.T == 0 || !wait_warp(k.bar(B_Q), 0, k.abort_flag, p.wait_limit)) return;
   const uint64_t q_desc = smem_desc(k.smem0, 16, 1024);
   const uint64_t k_desc = smem_desc(k.sRing, 16, 1024);
   const uint64_t v_desc = smem_desc(k.sRing, kHalf, 1024);   // lbo: the other half of d
-  RingPos<NST> kpos[2] = {RingPos<NST>(before.loads), RingPos<NST>(before.loads + (kRows2 ? 0 : 2))};
-  uint32_t ph = before.ph;
-  const int last_slot = k.slot_tiles(1) == k.slot_tiles(0) ? 1 : 0;   // whose Q K^T is the block's last
+  RingPos<NST> kpos[2] = {RingPos<NST>(0), RingPos<NST>(kRows2 ? 0 : 2)};
+  uint32_t ph = 0u;   // bit 3 s + h: parity of the next use of the barrier for part h of slot s's P
   auto issue_qk = [&](int s) -> bool {
     if (!wait_warp(k.bar(B_FULL + kpos[s].idx), kpos[s].ph, k.abort_flag, p.wait_limit)) return false;
     tc_fence_after();
@@ -462,7 +427,6 @@ __device__ __forceinline__ bool issue(const Block<kRows2, kParts>& k, const Para
   };
   bool ok = issue_qk(0);
   if (ok && k.slot_tiles(1) > 0) ok = issue_qk(1);
-  if (kMany && ok && k.slot_tiles(0) == 1) umma_commit_if(el, k.bar(B_QFREE));
 #pragma unroll 1
   for (int r = 0; r < k.slot_tiles(0) && ok; ++r) {
 #pragma unroll
@@ -493,18 +457,14 @@ __device__ __forceinline__ bool issue(const Block<kRows2, kParts>& k, const Para
       if (!ok) continue;
       umma_commit_if(el, k.bar(B_EMPTY + vpos.idx));
       kpos[s].advance(Cfg<kRows2, kParts>::kStep);
-      if (r + 1 < k.slot_tiles(s)) {
-        ok = issue_qk(s);
-        if (kMany && ok && s == last_slot && r + 2 == k.slot_tiles(0)) umma_commit_if(el, k.bar(B_QFREE));
-      } else umma_commit_if(el, k.bar(B_LAST + s));
+      if (r + 1 < k.slot_tiles(s)) ok = issue_qk(s);
+      else umma_commit_if(el, k.bar(B_LAST + s));
     }
   }
-  before.ph = ph;
-  return ok;
 }
 
 template <bool kRows2, int kParts>
-__device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Params& p, int par, int loads_before, int tiles_before) {
+__device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Params& p, int par) {
   constexpr int NST = Cfg<kRows2, kParts>::NST;
   Misc& ms = k.misc();
   const int tid = k.tid, lane = k.lane, slot = k.slot, row = k.row;
@@ -543,11 +503,11 @@ __device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Pa
     __syncwarp();
     mbar_arrive_if(lane == 0 ? 1u : 0u, k.bar(B_P + 3 * slot + h));
   };
-  RingPos<NST> vpos(loads_before + (kRows2 || slot == 0 ? 1 : 3));   // V stage of the current tile
+  RingPos<NST> vpos(kRows2 || slot == 0 ? 1 : 3);   // V stage of the current tile
 #pragma unroll 1
   for (int r = 0; r < k.my_tiles; ++r) {
     const int t = kRows2 ? r : 2 * r + slot;
-    if (!wait_warp(k.bar(B_S + slot), (uint32_t)(tiles_before + r) & 1u, k.abort_flag, p.wait_limit)) break;
+    if (!wait_warp(k.bar(B_S + slot), (uint32_t)r & 1u, k.abort_flag, p.wait_limit)) break;
     tc_fence_after();
     int keys0 = PG, keys1 = PG;    // real keys of the tile's pieces
     const bool plain = t < k.t_plain;
@@ -788,19 +748,14 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   if (tid == 0) { ms.seq = k.b; ms.len = k.L; }
   if (warp < kSoftmaxWarps) {
     more_registers<kSoftmaxRegs>();
-    softmax<kRows2, kParts>(k, p, par, 0, 0);
+    softmax<kRows2, kParts>(k, p, par);
     __syncwarp();
     fewer_registers<kLaunchRegs>();   // before the third warpgroup takes its own back
     named_barrier(2, kThreads);
   } else {
     fewer_registers<kOtherRegs>();
-    if (warp == kProducer) {
-      if (k.T == 0) mbar_drain(k.bar(B_Q), 0);   // nobody else waits for the Q that is on its way
-      produce<kRows2, kParts>(k, tm, p, 0);
-    } else if (warp == kIssuer) {
-      Before none = {0, 0, 0u};
-      issue<kRows2, kParts, false>(k, p, none);
-    }
+    if (warp == kProducer) produce<kRows2, kParts>(k, tm, p);
+    else if (warp == kIssuer) issue<kRows2, kParts>(k, p);
     __syncwarp();
     named_barrier(2, kThreads);
     more_registers<kLaunchRegs>();
@@ -1177,356 +1132,6 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   publish();
 }
 
-// ------------------------------------------------------------------------------------ even shares
-// One block per SM, and the key tiles of all (sequence, kv head) units, laid end to end, are shared out evenly:
-// block j of a group of row tiles takes range j, which may end one unit, hold some whole ones and begin another.
-// A unit that lies in one range is finished by its block.  Of the others each block leaves a partial result
-// (fp32 rows, reference and sum) in the workspace, and the block whose tiles complete the unit adds them up in
-// the order of the keys, so the result does not depend on timing; nobody waits for another block.
-// What it is for: long calls whose units do not divide over the machine, and ragged batches.  Clusters leave the
-// SMs idle that they do not divide, and every block of a unit takes as long as the longest sequence's.
-// The roles run on from unit to unit (the next unit's first tiles are loaded and multiplied while the
-// softmax threads store the previous one's rows); a fourth role (warp 10) loads Q.
-constexpr int kQLoader = 10;
-constexpr int kUnitStart = 2;     // tiles' worth of time that a unit takes besides its tiles
-constexpr int kMaxEvenBatch = 256;
-
-// A block's way through its range.  Positions count kUnitStart + tiles for each unit.
-template <class B>
-__device__ __forceinline__ bool next_unit(Way& w, B& k, const Params& p) {
-  while (w.at < w.end) {
-    k.b = w.b;
-    k.kvh = w.head;
-    w.seq = w.b;
-    w.kv_head = w.head;
-    w.seq_len = w.len;
-    k.length(p, w.len);
-    w.unit = w.base;
-    w.tiles = (k.p_total + 1) / 2;
-    const int unit_end = w.base + kUnitStart + w.tiles, stop = min(unit_end, w.end);
-    w.first_tile = max(0, w.at - w.base - kUnitStart);
-    w.end_tile = max(0, stop - w.base - kUnitStart);
-    w.at = stop;
-    if (stop == unit_end) {
-      w.base = unit_end;
-      if (++w.head == p.Hkv) {
-        w.head = 0;
-        ++w.b;
-        if (w.at < w.end && w.b < p.B) w.len = p.ctx_len[w.b];
-      }
-    }
-    if (w.end_tile > w.first_tile) {
-      k.split = w.first_tile;   // 0: the unit's first
-      k.share(2 * w.first_tile, min(2 * w.end_tile, k.p_total));
-      return true;
-    }
-  }
-  return false;
-}
-
-// What the softmax threads do when a block's share of a unit is through: the rows, or a partial result of them.
-template <bool kRows2>
-__device__ __forceinline__ void finish_unit(const Block<kRows2, 1>& k, const Params& p, const Way& w, int total) {
-  constexpr int kRows = kRows2 ? 2 * BM : BM;
-  constexpr int kCols = HD / 4;      // 16-byte pieces of a row
-  Misc& ms = k.misc();
-  const int slot = k.slot, row = k.row, rr = (kRows2 ? slot * BM : 0) + row;
-  const bool whole = w.first_tile == 0 && k.T == w.tiles;
-  float2 ml = ms.ml[slot * BM + row];
-  float w0 = 1.f, w1 = 0.f;
-  if (!kRows2) {   // the slots' shares of the keys
-    named_barrier(1, 32 * kSoftmaxWarps);
-    const float2 a = ms.ml[row], c = ms.ml[BM + row];
-    ml.x = fmaxf(a.x, c.x);
-    const float mu = ml.x == -INFINITY ? 0.f : ml.x;
-    w0 = ex2(a.x - mu);   // ex2(-inf) = 0
-    w1 = ex2(c.x - mu);
-    ml.y = a.y * w0 + c.y * w1;
-  }
-  const int64_t out_row = (int64_t)(k.b * k.N + k.node) * p.Hq + k.kvh * k.G + (row - k.node_in_tile * k.G);
-  if (whole) {
-    const float inv = ml.y > 0.f ? 1.f / ml.y : 0.f;
-    w0 *= inv;
-    w1 *= inv;
-  }
-  const bool has0 = kRows2 ? k.my_tiles > 0 : true, has1 = !kRows2 && k.T > 1;
-  bool done = true;
-  if (has0) done = wait_warp(k.bar(B_LAST + (kRows2 ? slot : 0)), (w.last_phases >> (kRows2 ? slot : 0)) & 1u, k.abort_flag, p.wait_limit);
-  if (has1 && done) wait_warp(k.bar(B_LAST + 1), (w.last_phases >> 1) & 1u, k.abort_flag, p.wait_limit);
-  __syncwarp();
-  tc_fence_after();
-  const unsigned groups = (unsigned)p.groups, range = p.by_groups.divide(k.block);
-  auto range_start = [&](unsigned j) { return (int)((unsigned long long)(unsigned)total * j / (unsigned)p.ranges); };
-  auto part_of = [&](unsigned j) {   // partial result of the group's block j for this unit: a block starts inside the unit or before it
-    return (int64_t)(2u * (j * groups + (unsigned)k.group) + (range_start(j) >= w.unit ? 0u : 1u));
-  };
-  auto write_half = [&](int half, const float (&v)[64]) {
-    uint4* dst = reinterpret_cast<uint4*>(p.out + out_row * HD + half * 64);
-#pragma unroll
-    for (int c = 0; c < 8; ++c)
-      dst[c] = make_uint4(pack_bf16(v[8 * c], v[8 * c + 1]), pack_bf16(v[8 * c + 2], v[8 * c + 3]),
-                          pack_bf16(v[8 * c + 4], v[8 * c + 5]), pack_bf16(v[8 * c + 6], v[8 * c + 7]));
-  };
-  const int64_t my_part = whole ? 0 : part_of(range);
-#pragma unroll 1
-  for (int half = kRows2 ? 0 : slot; half < (kRows2 ? 2 : slot + 1); ++half) {
-    float v[64];
-    {
-      uint32_t u[64], u1[64];
-      const uint32_t acc0 = (kRows2 ? k.tmem_O(slot) : k.tmem_O(0)) + k.lane_addr, acc1 = k.tmem_O(1) + k.lane_addr;
-      if (has0) tmem_ld_x64(acc0 + (uint32_t)(half * 64), u);
-      if (!kRows2 && has1) tmem_ld_x64(acc1 + (uint32_t)(half * 64), u1);
-      tmem_wait_ld();
-#pragma unroll
-      for (int j = 0; j < 64; ++j) {
-        v[j] = has0 ? __uint_as_float(u[j]) * w0 : 0.f;
-        if (!kRows2 && has1) v[j] = fmaf(__uint_as_float(u1[j]), w1, v[j]);
-      }
-    }
-    if (k.row_valid && whole) {
-      write_half(half, v);
-    } else if (k.row_valid) {
-      float4* dst = p.parts + my_part * (kRows * kCols) + half * (kCols / 2) * kRows + rr;
-#pragma unroll
-      for (int c = 0; c < kCols / 2; ++c) __stcg(dst + c * kRows, make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]));
-    }
-    __syncwarp();   // the next half's load takes the whole warp
-  }
-  if (k.row_valid && (kRows2 || slot == 0)) {
-    if (!whole) __stcg(p.part_sums + my_part * kRows + rr, ml);
-    else if (p.lse != nullptr) p.lse[out_row] = log_sum_exp(ml.x, ml.y);
-  }
-  // the threads' accumulators are read (the next unit's first P V follows their next hand-over), their parts and
-  // what they reported come before the unit's ticket
-  tc_fence_before();
-  __threadfence();
-  named_barrier(1, 32 * kSoftmaxWarps);
-  if (k.tid == 0) {
-    // the unit's word: tiles that are through, above them (8 bits) blocks that gave up a wait
-    unsigned* const word = p.tickets + 2 * p.B + ((unsigned)(k.b * p.Hkv + k.kvh) * groups + (unsigned)k.group);
-    unsigned through = (unsigned)k.T + (*k.abort_flag ? 1u << 24 : 0u);
-    if (!whole) through += atomicAdd(word, through);
-    int state = 0;   // 1: this block has the unit's last tiles, 2: and a wait of a block ran out
-    if ((through & 0xFFFFFFu) == (unsigned)w.tiles) {
-      state = through >> 24 ? 2 : 1;
-      if (!whole) *word = 0u;
-      unsigned long long* const tally = reinterpret_cast<unsigned long long*>(p.tickets + 2 * k.b);
-      const unsigned long long seen = atomicAdd(tally, state == 2 ? (2ull << 32) + 1ull : 1ull) + (state == 2 ? 2ull << 32 : 0ull);
-      if ((unsigned)seen == (unsigned)p.blocks_per_seq - 1u) {   // the sequence's last unit
-        *tally = 0ull;
-        const unsigned wrong = (unsigned)(seen >> 32);
-        p.status[k.b] = (wrong & 1u) ? CLV_ERR_TREE : wrong ? CLV_ERR_TIMEOUT : CLV_OK;
-      }
-    }
-    ms.last = whole ? 0 : state;
-  }
-  named_barrier(1, 32 * kSoftmaxWarps);
-  if (ms.last != 1 || !k.row_valid) return;
-  __threadfence();
-  // the blocks that had tiles of this unit: position x belongs to range ((x + 1) * ranges - 1) / total
-  const unsigned long long first = (unsigned)(w.unit + kUnitStart), last = first + (unsigned)w.tiles - 1;
-  const unsigned j0 = (unsigned)(((first + 1) * (unsigned)p.ranges - 1) / (unsigned)total);
-  const unsigned j1 = (unsigned)(((last + 1) * (unsigned)p.ranges - 1) / (unsigned)total);
-  float M = -INFINITY, sum = 0.f;
-  for (unsigned j = j0; j <= j1; ++j) {
-    if (range_start(j) == range_start(j + 1)) continue;
-    M = fmaxf(M, __ldcg(p.part_sums + part_of(j) * kRows + rr).x);
-  }
-  const float mu = M == -INFINITY ? 0.f : M;
-  for (unsigned j = j0; j <= j1; ++j) {
-    if (range_start(j) == range_start(j + 1)) continue;
-    const float2 m = __ldcg(p.part_sums + part_of(j) * kRows + rr);
-    sum = fmaf(m.y, ex2(m.x - mu), sum);
-  }
-  const float inv = sum > 0.f ? 1.f / sum : 0.f;
-#pragma unroll 1
-  for (int half = kRows2 ? 0 : slot; half < (kRows2 ? 2 : slot + 1); ++half) {
-    float acc[64];
-#pragma unroll
-    for (int i = 0; i < 64; ++i) acc[i] = 0.f;
-#pragma unroll 1
-    for (unsigned j = j0; j <= j1; ++j) {
-      if (range_start(j) == range_start(j + 1)) continue;
-      const int64_t part = part_of(j);
-      const float weight = ex2(__ldcg(p.part_sums + part * kRows + rr).x - mu) * inv;
-      const float4* src = p.parts + part * (kRows * kCols) + half * (kCols / 2) * kRows + rr;
-#pragma unroll
-      for (int c = 0; c < kCols / 2; ++c) {
-        const float4 x = __ldcg(src + c * kRows);
-        acc[4 * c] = fmaf(x.x, weight, acc[4 * c]);
-        acc[4 * c + 1] = fmaf(x.y, weight, acc[4 * c + 1]);
-        acc[4 * c + 2] = fmaf(x.z, weight, acc[4 * c + 2]);
-        acc[4 * c + 3] = fmaf(x.w, weight, acc[4 * c + 3]);
-      }
-    }
-    write_half(half, acc);
-  }
-  if (p.lse != nullptr && (kRows2 || slot == 0)) p.lse[out_row] = log_sum_exp(M, sum);
-}
-
-template <bool kRows2>
-__global__ void __launch_bounds__(kThreads, 1) tree_attn_even_kernel(const __grid_constant__ Maps tm, const __grid_constant__ Params p) {
-  constexpr int NST = Cfg<kRows2, 1>::NST;
-  extern __shared__ __align__(1024) uint8_t smem[];
-  Misc& ms = *reinterpret_cast<Misc*>(smem + kMiscAt);
-  Block<kRows2, 1> k;
-  k.place(p, smem, blockIdx.x, threadIdx.x);
-  const int tid = k.tid, warp = k.warp, lane = k.lane;
-  if (tid == 0) {
-    for (int i = 0; i < NST; ++i) { mbar_init(k.bar(B_FULL + i), 1); mbar_init(k.bar(B_EMPTY + i), (uint32_t)k.users); }
-    for (int i = 0; i < 2; ++i) { mbar_init(k.bar(B_S + i), 1); mbar_init(k.bar(B_LAST + i), 1); }
-    for (int i = 0; i < 6; ++i) mbar_init(k.bar(B_P + i), 4);
-    mbar_init(k.bar(B_Q), 1);
-    mbar_init(k.bar(B_QFREE), 1);
-    mbar_init(k.bar(B_DR), 1);
-    ms.abort_flag = 0;
-    ms.issued = 0;
-    ms.q_loads = 0;
-    fence_barrier_init();
-    fence_async_smem();
-  }
-  if (warp == kIssuer) tmem_alloc(smem_u32(&ms.tmem), kTmemCols);
-  if (tid == 32 * kProducer) {
-    tma_prefetch_desc(&tm.q);
-    if (p.pair_boxes) { tma_prefetch_desc(&tm.kc2); tma_prefetch_desc(&tm.vc2); }
-    tma_prefetch_desc(&tm.kc); tma_prefetch_desc(&tm.vc);
-    tma_prefetch_desc(&tm.kt); tma_prefetch_desc(&tm.vt);
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  cudaGridDependencySynchronize();
-
-  // ---- the block's range: a sum over the sequences' units up to each (a thread per sequence)
-  int* const warp_sums = reinterpret_cast<int*>(smem);   // the tiles are not in use yet
-  const unsigned range = p.by_groups.divide(blockIdx.x);
-  int units = 0;       // length of the thread's sequence's units
-  if (tid < p.B) {
-    k.length(p, p.ctx_len[tid]);
-    units = p.Hkv * (kUnitStart + (k.p_total + 1) / 2);
-  }
-  int upto = units;
-#pragma unroll
-  for (int d = 1; d < 32; d *= 2) {
-    const int v = __shfl_up_sync(0xFFFFFFFFu, upto, d);
-    if (lane >= d) upto += v;
-  }
-  if (lane == 31) warp_sums[warp] = upto;
-  __syncthreads();
-  int total = 0;
-  for (int i = 0; i < kThreads / 32; ++i) {
-    if (i < warp) upto += warp_sums[i];
-    total += warp_sums[i];
-  }
-  const int from = (int)((unsigned long long)(unsigned)total * range / (unsigned)p.ranges);
-  if (tid < p.B && from < upto && from >= upto - units) {
-    ms.start_seq = tid;
-    ms.start = upto - units;
-  }
-  __syncthreads();
-  Way w = {};
-  {
-    w.b = ms.start_seq;
-    w.len = p.ctx_len[w.b];
-    k.length(p, w.len);
-    const int unit = kUnitStart + (k.p_total + 1) / 2;
-    w.head = (from - ms.start) / unit;
-    w.base = ms.start + w.head * unit;
-    w.at = from;
-    w.end = (int)((unsigned long long)(unsigned)total * (range + 1) / (unsigned)p.ranges);
-  }
-  k.thread_place(p);
-  if (tid == 0) ms.total = total;
-  if (lane == 0 && warp < kSoftmaxWarps) ms.way[warp] = w;
-  fence_async_smem();   // the tiles are written by TMA next
-  __syncthreads();
-
-  if (warp < kSoftmaxWarps) {
-    more_registers<kSoftmaxRegs>();
-    auto here = [&](Block<kRows2, 1>& x) {   // worked out anew for each use (see the merge above)
-      unsigned block;
-      int thread;
-      asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(block));
-      asm volatile("mov.u32 %0, %%tid.x;" : "=r"(thread));
-      x.place(p, smem, block, thread);
-      x.thread_place(p);
-    };
-    for (;;) {
-      {
-        Block<kRows2, 1> x;
-        here(x);
-        Way v = ms.way[x.warp];
-        const bool more = next_unit(v, x, p);
-        __syncwarp();
-        if (!more) break;
-        if (x.lane == 0) ms.way[x.warp] = v;
-        __syncwarp();
-        const int par = x.tid < x.N ? p.parent[(int64_t)x.b * x.N + x.tid] : -1;
-        softmax<kRows2, 1>(x, p, par, v.loads_before, v.tiles_before);
-        __syncwarp();
-      }
-      Block<kRows2, 1> x;
-      here(x);
-      Way v = ms.way[x.warp];
-      x.b = v.seq;
-      x.kvh = v.kv_head;
-      x.length(p, v.seq_len);
-      x.share(2 * v.first_tile, min(2 * v.end_tile, x.p_total));
-      finish_unit<kRows2>(x, p, v, ms.total);
-      __syncwarp();
-      v.loads_before += 2 * x.T;
-      v.tiles_before += x.my_tiles;
-      v.last_phases ^= (x.slot_tiles(0) > 0 ? 1u : 0u) | (x.slot_tiles(1) > 0 ? 2u : 0u);
-      if (x.lane == 0) ms.way[x.warp] = v;
-      __syncwarp();
-    }
-    fewer_registers<kLaunchRegs>();   // before the third warpgroup takes its own back
-    named_barrier(2, kThreads);
-  } else {
-    fewer_registers<kOtherRegs>();
-    if (warp == kProducer) {
-      int loads = 0;
-      while (next_unit(w, k, p) && produce<kRows2, 1>(k, tm, p, loads)) loads += 2 * k.T;
-    } else if (warp == kIssuer) {
-      Before before = {0, 0, 0u};
-      while (next_unit(w, k, p) && issue<kRows2, 1, true>(k, p, before)) {
-        before.loads += 2 * k.T;
-        ++before.units;
-      }
-    } else if (warp == kQLoader) {
-      int n = 0;
-      for (; next_unit(w, k, p); ++n) {
-        if (n > 0 && !wait_warp(k.bar(B_QFREE), (uint32_t)(n - 1) & 1u, k.abort_flag, p.wait_limit)) break;
-        if (lane == 0) load_q<kRows2, 1>(k, tm);
-        __syncwarp();
-      }
-      if (lane == 0) ms.q_loads = n;
-    }
-    __syncwarp();
-    named_barrier(2, kThreads);
-    more_registers<kLaunchRegs>();
-  }
-  if (*k.abort_flag != 0) {   // copies that were issued land on their own, MMAs that were issued finish: wait for both
-    if (warp == kProducer && lane == 0) {
-      const int issued = ms.issued;
-      for (int i = max(0, issued - NST); i < issued; ++i) {
-        const RingPos<NST> pos(i);
-        mbar_drain(k.bar(B_FULL + pos.idx), pos.ph);
-      }
-      if (ms.q_loads > 0) mbar_drain(k.bar(B_Q), (uint32_t)(ms.q_loads - 1) & 1u);
-    }
-    if (warp == kIssuer) {
-      umma_commit_if(elect_one(), k.bar(B_DR));
-      mbar_drain(k.bar(B_DR), 0);
-    }
-  }
-  __syncthreads();
-  if (warp == kIssuer) {
-    tc_fence_after();
-    tmem_dealloc(ms.tmem, kTmemCols);
-  }
-}
-
 // ------------------------------------------------------------------------------------ host side
 // bf16 tensor [rows][heads][128]; box = 64 elements x 1 head x box_rows, 128-byte swizzle
 bool make_map(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t heads, uint32_t box_rows) {
@@ -1557,7 +1162,6 @@ bool make_map_halves(CUtensorMap* tm, const void* base, uint64_t rows, uint64_t 
 }
 
 using Kernel = void (*)(Maps, Params);
-Kernel even_kernel_of(bool rows2) { return rows2 ? tree_attn_even_kernel<true> : tree_attn_even_kernel<false>; }
 Kernel kernel_of(bool rows2, int parts, int splits) {
   if (rows2) return tree_attn_kernel<true, 1, false>;
   if (parts == 1) return tree_attn_kernel<false, 1, false>;
@@ -1571,8 +1175,7 @@ int g_clusters[kMaxDevices][kMaxSplits + 1];
 
 cudaError_t set_up() {
   const Kernel all[] = {kernel_of(true, 1, 1), kernel_of(false, 1, 1), kernel_of(false, 2, 1),
-                        kernel_of(false, 4, 1), kernel_of(false, 2, 2), kernel_of(false, 4, 2),
-                        even_kernel_of(true), even_kernel_of(false)};
+                        kernel_of(false, 4, 1), kernel_of(false, 2, 2), kernel_of(false, 4, 2)};
   for (const Kernel kernel : all) {
     cudaFuncAttributes a;
     cudaError_t e = cudaFuncGetAttributes(&a, kernel);
@@ -1606,38 +1209,20 @@ cudaError_t set_up() {
 struct AttnPlan {
   bool rows2;
   int parts, tiles, groups, splits;
-  int ranges;   // not 0: even shares, blocks of each group
 };
-
-// Partial results of even shares: two per block.
-size_t even_scratch_bytes(const AttnPlan& plan) {
-  return (size_t)plan.ranges * plan.groups * 2 * (plan.rows2 ? 2 : 1) * BM * (HD * sizeof(float) + sizeof(float2));
-}
-
-// What the even shares' arithmetic and the workspace's words hold: a thread per sequence, a word per unit and
-// group behind the sequences' two, 24 bits for a unit's tiles; and calls that are long enough at all.
-bool even_shares_fit(const clv_shape& s, int max_ctx_len) {
-  const int64_t words = (int64_t)s.batch * (2 + (int64_t)s.n_kv_heads * s.n_nodes);   // groups <= n_nodes
-  return s.batch <= kMaxEvenBatch && words <= kTickets && max_ctx_len >= 256;
-}
-// the row of all units, whatever lengths the device finds (a length beyond the cache counts as none)
-bool even_shares_fit(const clv_shape& s, const clv_kv_cache& c) {
-  const int64_t most = c.paged ? (int64_t)c.max_pages_per_seq * PG : c.cap_tokens;
-  return (int64_t)s.batch * s.n_kv_heads * (most / BN + CLV_MAX_NODES / BN + 4 + kUnitStart) < (1ll << 30) && most < (1ll << 30);
-}
 
 // Blocks along the rows and along the keys: the cheapest choice by a cost in SM cycles, rounds of
 // clusters over the machine times (key tiles of a block x cycles per tile + what a block takes
 // besides).  The figures are fitted to measurements of 22 shapes (batch 1-32, 1-8 row tiles, 350-16424
 // keys).
-AttnPlan make_plan(const clv_shape& s, const clv_kv_cache& c, int max_ctx_len, const int* clusters, size_t scratch_bytes) {
+AttnPlan make_plan(const clv_shape& s, int max_ctx_len, const int* clusters) {
   const int G = s.n_q_heads / s.n_kv_heads;
   const int rows = s.n_nodes * G;
   const int parts = rows <= BM / 4 ? 4 : rows <= BM / 2 ? 2 : 1;
   const int tiles = (s.n_nodes + BM / G - 1) / (BM / G);   // row tiles of BM / G whole nodes
   const int pieces = (max_ctx_len + PG - 1) / PG + (s.n_nodes + PG - 1) / PG;
   const int64_t units = (int64_t)s.batch * s.n_kv_heads;
-  AttnPlan best = {false, parts, tiles, tiles, 1, 0};
+  AttnPlan best = {false, parts, tiles, tiles, 1};
   double best_cost = 1e300;
   for (int r = 0; r < 2; ++r) {
     if (r && tiles < 2) break;
@@ -1649,21 +1234,13 @@ AttnPlan make_plan(const clv_shape& s, const clv_kv_cache& c, int max_ctx_len, c
       const double tile = r ? 3200.0 : parts > 1 ? 1200.0 : 1650.0;
       const double besides = sp == 1 ? 18000.0 : r ? 36000.0 : parts > 1 ? 19500.0 : 22500.0;
       const double cost = rounds * (key_tiles * tile + besides);
-      if (cost < best_cost) { best_cost = cost; best = {r != 0, parts, tiles, groups, sp, 0}; }
+      if (cost < best_cost) { best_cost = cost; best = {r != 0, parts, tiles, groups, sp}; }
     }
   }
-  (void)c;
-  (void)scratch_bytes;
   return best;
 }
 
 }  // namespace
-
-size_t tree_attn_scratch_bytes(const clv_shape& s, int max_ctx_len) {
-  (void)s;
-  (void)max_ctx_len;
-  return 0;   // no plan takes even shares yet
-}
 
 bool tree_attn_supported(const clv_shape& s, const clv_kv_cache& c) {
   const int G = s.n_q_heads / s.n_kv_heads;
@@ -1675,15 +1252,15 @@ bool tree_attn_supported(const clv_shape& s, const clv_kv_cache& c) {
 
 cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const void* q, const void* k_tree,
                              const void* v_tree, const int32_t* parent, const int32_t* ctx_len, int max_ctx_len,
-                             float scale, void* out, float* lse, int32_t* status, unsigned* tickets, void* scratch,
-                             size_t scratch_bytes, cudaStream_t stream) {
+                             float scale, void* out, float* lse, int32_t* status, unsigned* tickets,
+                             cudaStream_t stream) {
   static OncePerDevice once;
   cudaError_t e = run_once_per_device(once, set_up);
   if (e != cudaSuccess) return e;
   int dev = 0;
   e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const AttnPlan plan = make_plan(s, c, max_ctx_len, g_clusters[dev], scratch_bytes);
+  const AttnPlan plan = make_plan(s, max_ctx_len, g_clusters[dev]);
   const int G = s.n_q_heads / s.n_kv_heads;
   alignas(64) Maps tm;
   const uint64_t cache_rows = c.paged ? (uint64_t)c.n_pages * CLV_PAGE_SIZE : (uint64_t)s.batch * c.cap_tokens;
@@ -1712,14 +1289,11 @@ cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const vo
   p.tiles = plan.tiles;
   p.groups = plan.groups;
   p.splits = plan.splits;
-  p.longest_first = (plan.ranges == 0 && clusters * plan.splits > sm_count() && s.batch > 1 && s.batch <= 256) ? 1 : 0;
+  p.longest_first = (clusters * plan.splits > sm_count() && s.batch > 1 && s.batch <= 256) ? 1 : 0;
   p.scale_log2 = scale * 1.4426950408889634f;
   p.wait_limit = wait_limit_cycles();
   p.tickets = tickets;
-  p.blocks_per_seq = s.n_kv_heads * plan.groups * plan.splits;   // (even shares: units)
-  p.ranges = plan.ranges;
-  p.parts = static_cast<float4*>(scratch);
-  p.part_sums = reinterpret_cast<float2*>(p.parts + (size_t)plan.ranges * plan.groups * 2 * (plan.rows2 ? 2 : 1) * BM * (HD / 4));
+  p.blocks_per_seq = s.n_kv_heads * plan.groups * plan.splits;
   p.tile_nodes = BM / plan.parts / G;
   p.by_splits = Divisor::of((unsigned)plan.splits);
   p.by_groups = Divisor::of((unsigned)plan.groups);
@@ -1727,7 +1301,7 @@ cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const vo
   p.by_group_heads = Divisor::of((unsigned)G);
 
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(plan.ranges ? plan.ranges * plan.groups : clusters * plan.splits), 1, 1);
+  cfg.gridDim = dim3((unsigned)(clusters * plan.splits), 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = kSmem;
   cfg.stream = stream;
@@ -1740,7 +1314,7 @@ cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const vo
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, plan.ranges ? even_kernel_of(plan.rows2) : kernel_of(plan.rows2, plan.parts, plan.splits), tm, p);
+  return cudaLaunchKernelEx(&cfg, kernel_of(plan.rows2, plan.parts, plan.splits), tm, p);
 }
 
 }  // namespace clv
