@@ -338,6 +338,38 @@ def test_attention_scores_that_outgrow_the_first_tile(clv, oracle, n_nodes):
     check_attention(oracle, w, st)
 
 
+@pytest.mark.parametrize("pow2", [1, 3, 7])
+@pytest.mark.parametrize("start", [256, 319, 330, 383])
+def test_attention_reference_replaced_in_every_part_of_a_tile(clv, oracle, start, pow2):
+    # A tile's first 64 keys are judged by their sum of exponentials, the others by their maximum: scores rise
+    # (many by a little, or a few beyond fp32's range) from one key of a tile on, in each of its four chunks
+    # and at their edges.  Scores reach about 60 * 2^pow2 / 16, so fp32 resolves them within the tolerance.
+    cfg = W.small_config(batch=2, n_q_heads=4, n_kv_heads=2, ctx=(390, 700), n_nodes=48, vocab=64,
+                         seed=W.BASE_SEED + 640 + start)
+    w = W.generate(cfg)
+    w.k_cache[:, start:] = _scale_bf16_by_pow2(w.k_cache[:, start:], pow2)
+    st = make_step(w)
+    st.tree_attn()
+    torch.cuda.synchronize()
+    check_attention(oracle, w, st)
+
+
+@pytest.mark.parametrize("batch,hq,hkv,ctx,n_nodes", [
+    (20, 16, 4, (40, 900), 33),    # one row tile per block where equal lengths would take two
+    (20, 8, 4, (40, 900), 100),
+    (44, 8, 2, (10, 700), 70),     # two where equal lengths would take one
+])
+def test_attention_ragged_batches_in_a_small_pool(clv, oracle, batch, hq, hkv, ctx, n_nodes):
+    # the pool's pages bound the mean length, so the plan is one for blocks of unequal length
+    cfg = W.small_config(batch=batch, n_q_heads=hq, n_kv_heads=hkv, ctx=ctx, n_nodes=n_nodes, vocab=64, paged=True,
+                         seed=W.BASE_SEED + 660 + batch)
+    w = W.generate(cfg)
+    st = make_step(w)
+    st.tree_attn()
+    torch.cuda.synchronize()
+    check_attention(oracle, w, st)
+
+
 @pytest.mark.parametrize("batch,hq,hkv,n_nodes", [
     (2, 8, 8, 16),    # one row tile of 16 rows, of 128 (two slots share it), two row tiles per block;
     (2, 8, 2, 32),    #   keys over several blocks
