@@ -1,7 +1,9 @@
 // Greedy acceptance walk (Sec. 2.1 verification phase) and KV commit (equivalence requirement of
 // Sec. 2.1).  Both are latency-bound: one warp per sequence for the walk; the row copies of a sequence
 // are spread over a thread-block cluster, so that a row of many heads is a few loads per thread (walk and
-// commit of one sequence, 32 heads, 64 nodes: 6.4 us by one block, 3.7 by eight).
+// commit of one sequence, 32 heads, 64 nodes: 6.4 us by one block, 3.7 by eight; then the nodes fetched at once,
+// every node's accepted child found ahead of the walk and the pages fetched meanwhile: verify steps of 1 x 64 nodes 23.4 ->
+// 22.6 us, of 4 x 64 with grouped heads 44.0 -> 43.0, of 1 x 16 14.7 -> 14.4).
 #include <limits.h>
 
 #include "clv_internal.cuh"
@@ -11,8 +13,9 @@ namespace {
 
 // ------------------------------------------------------------------------------------ walk
 struct WalkSmem {
-  int sp[CLV_MAX_NODES], st[CLV_MAX_NODES], si[CLV_MAX_NODES], path[CLV_MAX_NODES];
+  int ids[CLV_MAX_NODES], next[CLV_MAX_NODES], path[CLV_MAX_NODES];
 };
+constexpr int kPerLane = CLV_MAX_NODES / 32;   // nodes of a lane
 
 // The walk of sequence b by one warp; returns the accepted length (0 if the tree is malformed).
 // The path is left in sm.path[0 .. len) for the caller (visible after a __syncwarp / barrier).
@@ -20,43 +23,56 @@ __device__ __forceinline__ int walk_sequence(WalkSmem& sm, int b, int lane, int 
                                              const int32_t* parent, const int32_t* tokens,
                                              const int32_t* ids, int32_t* accept_len, int32_t* accept_idx,
                                              int32_t* next_token, int32_t* status, bool write) {
-  int* sp = sm.sp; int* st = sm.st; int* si = sm.si; int* path = sm.path;
   const int64_t o = (int64_t)b * N;
+  // Everything the walk needs is asked for at once: one load behind the other's store to shared memory cost a
+  // round trip for every 32 nodes.
+  int p[kPerLane], token[kPerLane], id[kPerLane];
+#pragma unroll
+  for (int k = 0; k < kPerLane; ++k) {
+    const int i = lane + 32 * k;
+    p[k] = i < N ? parent[o + i] : -1;
+    token[k] = i < N ? tokens[o + i] : 0;
+    id[k] = i < N ? ids[o + i] : 0;
+  }
   bool bad = false;
-  for (int i = lane; i < N; i += 32) {
-    const int p = parent[o + i];
-    sp[i] = p;
-    st[i] = tokens[o + i];
-    si[i] = ids[o + i];
-    bad |= (i == 0) ? (p != -1) : (p < 0 || p >= i);  // node 0 is the only root
+#pragma unroll
+  for (int k = 0; k < kPerLane; ++k) {
+    const int i = lane + 32 * k;
+    sm.ids[i] = id[k];
+    sm.next[i] = INT_MAX;
+    bad |= i < N && (i == 0 ? p[k] != -1 : p[k] < 0 || p[k] >= i);   // node 0 is the only root
   }
   bad = __any_sync(0xFFFFFFFFu, bad) || path_cap < 1;
   __syncwarp();
+  // Every node's accepted child, the lowest that carries the target's choice there; the walk then is a load
+  // per step (a search among the nodes at each step: five dependent instructions and a reduction).
+  if (!bad) {
+#pragma unroll
+    for (int k = 0; k < kPerLane; ++k) {
+      const int i = lane + 32 * k;
+      if (i > 0 && i < N && token[k] == sm.ids[p[k]]) atomicMin(&sm.next[p[k]], i);
+    }
+  }
+  __syncwarp();
   int len = 0, cur = 0;
   if (!bad) {
-    if (lane == 0) path[0] = 0;
+    if (lane == 0) sm.path[0] = 0;
     len = 1;
-    for (int step = 1; step < N; ++step) {  // a path has at most N nodes
-      const int want = si[cur];
-      int found = INT_MAX;
-      for (int c = cur + 1 + lane; c < N; c += 32)
-        if (sp[c] == cur && st[c] == want) { found = c; break; }
-      found = __reduce_min_sync(0xFFFFFFFFu, found);
-      if (found == INT_MAX) break;
+    for (int child = sm.next[0]; child != INT_MAX; child = sm.next[cur]) {   // a child's number is higher than its parent's
       if (len == path_cap || len == CLV_MAX_NODES) { bad = true; break; }
-      if (lane == 0) path[len] = found;
+      if (lane == 0) sm.path[len] = child;
       ++len;
-      cur = found;
+      cur = child;
     }
   }
   __syncwarp();
   if (bad) len = 0;
   if (!write) return len;
   for (int j = lane; j < path_cap; j += 32)
-    accept_idx[(int64_t)b * path_cap + j] = (j < len) ? path[j] : -1;
+    accept_idx[(int64_t)b * path_cap + j] = (j < len) ? sm.path[j] : -1;
   if (lane == 0) {
     accept_len[b] = len;
-    next_token[b] = bad ? -1 : si[cur];
+    next_token[b] = bad ? -1 : sm.ids[cur];
     status[b] = bad ? CLV_ERR_TREE : CLV_OK;
   }
   return len;
@@ -92,7 +108,9 @@ struct CommitParams {
   int row_vec;  // 16-byte vectors per token row: Hkv * 128 * 2 / 16
 };
 
+constexpr int kPages = (CLV_MAX_NODES + CLV_PAGE_SIZE - 1) / CLV_PAGE_SIZE + 1;   // that a path may touch
 struct CommitSmem {
+  int pages[kPages];    // the block table's entries from the one that holds position L on
   int src[CLV_MAX_NODES];
   long long dst[CLV_MAX_NODES];  // destination token row (global row index)
   int L, len, ok;
@@ -101,13 +119,22 @@ struct CommitSmem {
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
+// The pages that the rows behind position L go to, by a warp that has nothing else to do while the path is
+// walked (paged caches: a round trip less before the copies).
+__device__ __forceinline__ void fetch_pages(CommitSmem& sm, const CommitParams& p, int b, int lane) {
+  if (!p.paged || lane >= kPages) return;
+  const int L = p.ctx_len[b];
+  const long long lp = (long long)(L / CLV_PAGE_SIZE) + lane;
+  sm.pages[lane] = L >= 0 && lp < p.max_pages ? p.block_table[(int64_t)b * p.max_pages + lp] : -1;
+}
+
 // The commit of sequence b by `ranks` thread blocks, of which this is number `rank`.  path: the accepted
 // nodes, sm.len of them (sm.len and sm.L are set by thread 0 of the caller).  kCluster: the blocks are a
 // cluster; ctx_len_out may be ctx_len, so it is written when every block has read it.
-template <bool kCluster>
+template <bool kCluster, bool kPagesFetched>
 __device__ __forceinline__ void commit_sequence(CommitSmem& sm, const CommitParams& p, int b, int tid, const int32_t* path,
                                                 int rank, int ranks) {
-  __syncthreads();   // sm.L, sm.len (and the path, if this block walked it)
+  __syncthreads();   // sm.L, sm.len (and the path and sm.pages, if this block walked it)
   if (kCluster) cluster_arrive();
   const int L = sm.L, len = sm.len;
   if (tid == 0) sm.ok = (L >= 0 && len >= 0 && len <= p.path_cap && len <= CLV_MAX_NODES) ? 1 : 0;
@@ -119,10 +146,9 @@ __device__ __forceinline__ void commit_sequence(CommitSmem& sm, const CommitPara
       long long row = -1;
       if (p.paged) {
         const long long lp = t / CLV_PAGE_SIZE;
-        if (lp < p.max_pages) {
-          const int pg = p.block_table[(int64_t)b * p.max_pages + lp];
-          if (pg >= 0 && pg < p.n_pages) row = (long long)pg * CLV_PAGE_SIZE + t % CLV_PAGE_SIZE;
-        }
+        const int pg = kPagesFetched ? sm.pages[lp - L / CLV_PAGE_SIZE]
+                       : lp < p.max_pages ? p.block_table[(int64_t)b * p.max_pages + lp] : -1;
+        if (pg >= 0 && pg < p.n_pages) row = (long long)pg * CLV_PAGE_SIZE + t % CLV_PAGE_SIZE;
       } else if (t < p.cap_tokens) {
         row = (long long)b * p.cap_tokens + t;
       }
@@ -173,7 +199,7 @@ __global__ void __launch_bounds__(256) commit_kernel(CommitParams p, int ranks) 
   cudaGridDependencySynchronize();  // programmatic launch: the walk's outputs are complete after this
   cudaTriggerProgrammaticLaunchCompletion();  // a following kernel may set up; it waits for this grid itself
   if (threadIdx.x == 0) { sm.L = p.ctx_len[b]; sm.len = p.accept_len[b]; }
-  commit_sequence<true>(sm, p, b, threadIdx.x, p.accept_idx + (int64_t)b * p.path_cap, rank, ranks);
+  commit_sequence<true, false>(sm, p, b, threadIdx.x, p.accept_idx + (int64_t)b * p.path_cap, rank, ranks);
 }
 
 // Walk and commit of a sequence in one launch: warp 0 of every block walks (the first block's writes
@@ -200,8 +226,10 @@ __global__ void __launch_bounds__(256) walk_commit_kernel(WalkArgs w, CommitPara
                                   w.accept_idx, w.next_token, w.status, rank == 0);
     if (threadIdx.x == 0) { csm.L = L; csm.len = len; }
     __syncwarp();
+  } else if (threadIdx.x < 64) {
+    fetch_pages(csm, p, b, threadIdx.x - 32);
   }
-  commit_sequence<true>(csm, p, b, threadIdx.x, wsm.path, rank, ranks);
+  commit_sequence<true, true>(csm, p, b, threadIdx.x, wsm.path, rank, ranks);
 }
 
 // The commit of every layer of a model in one launch: blocks (b, layer, *) copy the accepted rows of
@@ -220,7 +248,7 @@ __global__ void __launch_bounds__(256) commit_layers_kernel(CommitParams p, long
   p.k_tree += layer * tree_stride_vec;
   p.v_tree += layer * tree_stride_vec;
   if (threadIdx.x == 0) { sm.L = p.ctx_len[b]; sm.len = p.accept_len[b]; }
-  commit_sequence<false>(sm, p, b, threadIdx.x, p.accept_idx + (int64_t)b * p.path_cap, blockIdx.z, gridDim.z);
+  commit_sequence<false, false>(sm, p, b, threadIdx.x, p.accept_idx + (int64_t)b * p.path_cap, blockIdx.z, gridDim.z);
 }
 
 }  // namespace

@@ -656,6 +656,38 @@ def test_walk_commit_in_one_launch_with_errors(clv, oracle, paged):
     assert s1.tolist()[1:4] == [7, 7, 7] and s2.tolist()[4] == 7 and s2.tolist()[0] == 0
 
 
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("n_nodes", [1, 31, 32, 33, 64, 65, 97, 128])
+def test_walk_commit_at_the_edges_of_a_lane_s_nodes(clv, oracle, n_nodes, paged):
+    # Sizes around the nodes that a lane holds.  Sequence 0: a chain of which every edge agrees (128 nodes from
+    # position 40 on lie in three pages); 1: three tokens only, so siblings carry equal ones and the lowest
+    # matching child is taken; 2: nothing agrees.
+    cfg = W.small_config(batch=3, n_q_heads=4, n_kv_heads=2, ctx=40, n_nodes=n_nodes, max_depth=max(1, n_nodes - 1),
+                         vocab=64, paged=paged, seed=W.BASE_SEED + 90 + n_nodes)
+    w = W.generate(cfg)
+    w.path_cap = n_nodes
+    rng = np.random.default_rng(n_nodes)
+    ids = rng.integers(0, 3, size=(3, n_nodes)).astype(np.int32)
+    w.parent[0] = np.arange(n_nodes) - 1
+    w.tokens[0] = np.arange(n_nodes)
+    ids[0, :-1] = w.tokens[0, 1:]
+    w.tokens[1] = rng.integers(0, 3, size=n_nodes)
+    ids[2] = 63
+    w.tokens[2] = np.minimum(w.tokens[2], 62)
+    st = make_step(w)
+    st.ids.copy_(torch.from_numpy(ids))
+    st.accept_walk_commit()
+    torch.cuda.synchronize()
+    alen, aidx, nxt, s1 = oracle.accept_walk(w.parent, w.tokens, ids, w.path_cap)
+    kc, vc, new_len, s2 = oracle.kv_commit(w.k_cache, w.v_cache, w.k_tree, w.v_tree, aidx, alen, w.ctx_len,
+                                           block_table=w.block_table)
+    assert np.array_equal(st.accept_len.cpu().numpy(), alen) and np.array_equal(st.accept_idx.cpu().numpy(), aidx)
+    assert np.array_equal(st.next_token.cpu().numpy(), nxt) and np.array_equal(st.ctx_len_out.cpu().numpy(), new_len)
+    assert np.array_equal(st.status[1].cpu().numpy(), s1) and np.array_equal(st.status[2].cpu().numpy(), s2)
+    assert np.array_equal(bits(st.k_cache), kc) and np.array_equal(bits(st.v_cache), vc)
+    assert alen[0] == n_nodes and s2.tolist() == [0, 0, 0]
+
+
 def test_guard_bands_untouched(clv, oracle):
     # outputs live inside larger sentinel-filled buffers; nothing outside them may change
     cfg = W.small_config(batch=2, n_q_heads=8, n_kv_heads=2, ctx=(10, 333), n_nodes=19, vocab=4099)
