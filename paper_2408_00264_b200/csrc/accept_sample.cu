@@ -145,13 +145,15 @@ struct WalkParams {
 // One block per sequence.  What bounds it is the number of dependent round trips to memory, so everything
 // that any level of the walk may need is fetched at once: every row's statistics, and every node's
 // logit in its parent's row.  The walk itself then runs in shared memory, along lists of siblings
-// (statistics and walk, 5 sequences of 27 nodes, 50257 logits: 16.8 -> 12.8 us; 6 of 109 nodes: 42 -> 20).
+// (statistics and walk, 5 sequences of 27 nodes, 50257 logits: 16.8 -> 12.8 us; 6 of 109 nodes: 42 -> 20), the
+// statistics ahead of the tree that the logits' addresses come from, and kept for the draw (the whole step 35.0 -> 34.7).
 __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
   __shared__ int sp[CLV_MAX_NODES], st[CLV_MAX_NODES], path[CLV_MAX_NODES];
   __shared__ int s_first[CLV_MAX_NODES], s_next[CLV_MAX_NODES];   // a node's first child, its next sibling (N: none)
   __shared__ bool s_repeat[CLV_MAX_NODES];                         // an earlier sibling carries the same token
   __shared__ float su[CLV_MAX_NODES + 1], se[CLV_MAX_NODES], s_m[CLV_MAX_NODES], s_S[CLV_MAX_NODES];
   __shared__ float s_slice[kThreads];
+  __shared__ float2 s_stats[32 * CLV_MAX_NODES];   // every row's slices, if a row has no more than a warp's lanes
   __shared__ float s_before, s_target;
   __shared__ int s_found, s_bad, s_pick, s_lastv, s_len, s_cur;
   static_assert(kThreads == 2 * CLV_MAX_NODES, "two threads per node");
@@ -160,6 +162,18 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
   const int64_t o = (int64_t)b * N;
   cudaGridDependencySynchronize();
   cudaTriggerProgrammaticLaunchCompletion();
+  const int lane = tid & 31, warp = tid >> 5;
+  constexpr int kWarps = kThreads / 32, kRows = 4;   // a warp per row, four rows under way
+  const bool keep = n_sl <= 32;
+  auto fetch = [&](int r0, float2 (&v)[kRows]) {
+#pragma unroll
+    for (int u = 0; u < kRows; ++u) {
+      const int r = r0 + u * kWarps;
+      v[u] = (r < N && lane < n_sl) ? p.partial[(o + r) * n_sl + lane] : make_float2(-INFINITY, 0.f);
+    }
+  };
+  float2 v[kRows];
+  fetch(warp, v);   // under way before the tree, whose tokens the logits below wait for
   if (tid == 0) s_bad = (p.path_cap < 1) ? 1 : 0;
   if (tid < CLV_MAX_NODES) s_first[tid] = N;
   __syncthreads();
@@ -179,21 +193,15 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
   const bool in_vocab = child && tok >= 0 && tok < p.vocab;
   uint32_t logit = 0x7FC00000u;   // NaN: no mass
   if (tid < N && in_vocab) logit = (uint32_t)p.logits[(o + par) * p.ld + tok] << 16;
-  // ---- every row's maximum and sum from its slices, a warp per row, four rows under way
+  // ---- every row's maximum and sum from its slices
   {
-    const int lane = tid & 31, warp = tid >> 5;
-    constexpr int kWarps = kThreads / 32, kRows = 4;
     for (int r0 = warp; r0 < N; r0 += kWarps * kRows) {
-      float2 v[kRows];
-#pragma unroll
-      for (int u = 0; u < kRows; ++u) {
-        const int r = r0 + u * kWarps;
-        v[u] = (r < N && lane < n_sl) ? p.partial[(o + r) * n_sl + lane] : make_float2(-INFINITY, 0.f);
-      }
+      if (r0 != warp) fetch(r0, v);
       Stat a[kRows];
 #pragma unroll
       for (int u = 0; u < kRows; ++u) {
         const int r = min(r0 + u * kWarps, N - 1);
+        if (keep && r0 + u * kWarps < N && lane < n_sl) s_stats[(r0 + u * kWarps) * n_sl + lane] = v[u];
         a[u] = Stat{-INFINITY, 0.f};
         stat_merge(a[u], Stat{v[u].x, v[u].y});
         for (int i = lane + 32; i < n_sl; i += 32) {
@@ -266,7 +274,7 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
     // what is left, slice by slice (the first pass's sums minus the struck weights differ from a
     // fresh sum by rounding only); thread 0 walks the slices in vocabulary order
     for (int j = tid; j < n_sl; j += kThreads) {
-      const float2 sl = p.partial[(o + cur) * n_sl + j];
+      const float2 sl = keep ? s_stats[cur * n_sl + j] : p.partial[(o + cur) * n_sl + j];
       float sum = (sl.x > -INFINITY && m > -INFINITY) ? sl.y * ex2(sl.x - m) : 0.f;
       const int v0 = j * kSlice, v1 = min(p.vocab, v0 + kSlice);
       for (int c = s_first[cur]; c < N; c = s_next[c])
@@ -305,7 +313,6 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
       //      its start, and the first element whose running sum exceeds the target wins
       const float target = s_target;
       const int q0 = pick * kSlice, q1 = min(p.vocab, q0 + kSlice);
-      const int lane = tid & 31, warp = tid >> 5;
       const int v_base = q0 + tid * kPerThread;
       float e[kPerThread];
       {

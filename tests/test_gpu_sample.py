@@ -91,6 +91,23 @@ def compare(oracle, got, lg, vocab, parent, tokens, u, temperature, path_cap, mi
     return alen
 
 
+@pytest.mark.parametrize("vocab,n_nodes", [(131072, 33), (131080, 33), (4096, 128)])
+def test_sample_slices_of_a_row_kept_or_fetched_again(clv, oracle, vocab, n_nodes):
+    # a row of up to 32 slices stays in shared memory between its statistics and the draw; more nodes than
+    # the first fetch of all warps takes
+    B = 4
+    cfg = W.small_config(batch=B, n_nodes=n_nodes, vocab=vocab, seed=W.BASE_SEED + vocab + n_nodes)
+    w = W.generate(cfg)
+    lift = W.f32_to_bf16_bits(np.float32([np.log(vocab) + 1.0]))[0]
+    ids = oracle.argmax(w.logits, vocab)
+    for b in range(B):
+        for i in range(n_nodes):
+            w.logits[b, i, ids[b, i]] = lift
+    u = W.make_uniforms(B, n_nodes, seed=vocab)
+    got = run_gpu(clv, w.logits, vocab, w.parent, w.tokens, u, 1.0, w.path_cap)
+    compare(oracle, got, w.logits, vocab, w.parent, w.tokens, u, 1.0, w.path_cap, min_robust=0.0)
+
+
 @pytest.mark.parametrize("temperature", [1.0, 0.6, 1.7])
 @pytest.mark.parametrize("vocab,n_nodes", [(64, 9), (1000, 20), (4099, 33), (8192, 10), (32000, 64), (32771, 12),
                                            (128256, 64)])   # around the edges of the 4096-logit slices and 32768-logit pieces
