@@ -91,10 +91,10 @@ def compare(oracle, got, lg, vocab, parent, tokens, u, temperature, path_cap, mi
     return alen
 
 
-@pytest.mark.parametrize("vocab,n_nodes", [(131072, 33), (131080, 33), (4096, 128)])
+@pytest.mark.parametrize("vocab,n_nodes", [(131072, 16), (131080, 12), (4096, 64), (4096, 65)])
 def test_sample_slices_of_a_row_kept_or_fetched_again(clv, oracle, vocab, n_nodes):
-    # a row of up to 32 slices stays in shared memory between its statistics and the draw; more nodes than
-    # the first fetch of all warps takes
+    # up to 512 slices of rows of up to 32 stay in shared memory between the statistics and the draw; more nodes
+    # than the first fetch of all warps takes
     B = 4
     cfg = W.small_config(batch=B, n_nodes=n_nodes, vocab=vocab, seed=W.BASE_SEED + vocab + n_nodes)
     w = W.generate(cfg)
