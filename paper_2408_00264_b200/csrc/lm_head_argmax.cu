@@ -83,10 +83,10 @@ struct Best {
   __nv_bfloat162 v[4];
   uint32_t at[4];
 };
-// columns [8 * group, 8 * group + 32) of the tile
-__device__ __forceinline__ void take_columns(Best& b, const uint32_t (&x)[32], uint32_t group) {
+// columns [8 * group, 8 * group + 16) of the tile
+__device__ __forceinline__ void take_columns(Best& b, const uint32_t (&x)[16], uint32_t group) {
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
+  for (int j = 0; j < 8; ++j) {
     const __nv_bfloat162 r = __floats2bfloat162_rn(__uint_as_float(x[2 * j]), __uint_as_float(x[2 * j + 1]));
     const uint32_t above = __hgt2_mask(r, b.v[j & 3]);   // strictly: the first of equals stays; false for NaN
     b.v[j & 3] = __hmax2(b.v[j & 3], r);                 // NaN operands are dropped
@@ -315,24 +315,26 @@ lm_head_argmax_kernel(const __grid_constant__ Maps tm, const Params p) {
           }
           __syncwarp();
         }
-      } else if (group_used && p.out == nullptr) {   // a chunk of 32 columns is fetched while the one before it is taken
+      } else if (group_used && p.out == nullptr) {   // a chunk of 16 columns is fetched while the one before it is taken
+        // (chunks of 32 took 153 registers: the small kernels between the draft head's products found no room
+        // beside this one, 1 x 119116 x 2048: 109.4 -> 113.1 us)
         Best best;
 #pragma unroll
         for (int j = 0; j < 4; ++j) { best.v[j] = __float2bfloat162_rn(-INFINITY); best.at[j] = 0xFFFFFFFFu; }
-        uint32_t x[2][32];
+        uint32_t x[2][16];
         const uint32_t acc_addr = tmem + lane_addr + (uint32_t)(mt * BN);
-        tmem_ld_x32(acc_addr, x[0]);
+        tmem_ld_x16(acc_addr, x[0]);
 #pragma unroll 1
-        for (int c0 = 0; c0 < p.bn; c0 += 64) {
+        for (int c0 = 0; c0 < p.bn; c0 += 32) {
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            const int c = c0 + 32 * h;
+            const int c = c0 + 16 * h;   // a tile's width is a multiple of 16
             if (c >= p.bn) continue;
             tmem_wait_ld();
-            if (c + 32 < p.bn) tmem_ld_x32(acc_addr + (uint32_t)(c + 32), x[h ^ 1]);
-            if (wi.col0 + c + 32 > lim) {   // the last chunk of a tile or of the vocabulary
+            if (c + 16 < p.bn) tmem_ld_x16(acc_addr + (uint32_t)(c + 16), x[h ^ 1]);
+            if (wi.col0 + c + 16 > lim) {   // the last of the vocabulary
 #pragma unroll
-              for (int j = 0; j < 32; ++j)
+              for (int j = 0; j < 16; ++j)
                 if (wi.col0 + c + j >= lim) x[h][j] = 0xFF800000u;
             }
             take_columns(best, x[h], (uint32_t)c >> 3);
