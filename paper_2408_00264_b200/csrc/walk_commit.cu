@@ -131,9 +131,12 @@ __device__ __forceinline__ void fetch_pages(CommitSmem& sm, const CommitParams& 
 // The commit of sequence b by `ranks` thread blocks, of which this is number `rank`.  path: the accepted
 // nodes, sm.len of them (sm.len and sm.L are set by thread 0 of the caller).  kCluster: the blocks are a
 // cluster; ctx_len_out may be ctx_len, so it is written when every block has read it.
-template <bool kCluster, bool kPagesFetched>
+template <bool kCluster, bool kWalked>
 __device__ __forceinline__ void commit_sequence(CommitSmem& sm, const CommitParams& p, int b, int tid, const int32_t* path,
                                                 int rank, int ranks) {
+  // a path in memory is asked for beside its length and the context's, an entry per thread (the commit of 5 sequences
+  // alone: 2.35 -> 2.15 us)
+  const int entry = !kWalked && tid < min(p.path_cap, CLV_MAX_NODES) ? path[tid] : 0;
   __syncthreads();   // sm.L, sm.len (and the path and sm.pages, if this block walked it)
   if (kCluster) cluster_arrive();
   const int L = sm.L, len = sm.len;
@@ -141,12 +144,12 @@ __device__ __forceinline__ void commit_sequence(CommitSmem& sm, const CommitPara
   __syncthreads();
   if (sm.ok) {
     for (int j = tid; j < len; j += blockDim.x) {
-      const int a = path[j];
+      const int a = kWalked ? path[j] : entry;   // (len <= 128 < the block's threads: j is tid)
       const long long t = (long long)L + j;
       long long row = -1;
       if (p.paged) {
         const long long lp = t / CLV_PAGE_SIZE;
-        const int pg = kPagesFetched ? sm.pages[lp - L / CLV_PAGE_SIZE]
+        const int pg = kWalked ? sm.pages[lp - L / CLV_PAGE_SIZE]
                        : lp < p.max_pages ? p.block_table[(int64_t)b * p.max_pages + lp] : -1;
         if (pg >= 0 && pg < p.n_pages) row = (long long)pg * CLV_PAGE_SIZE + t % CLV_PAGE_SIZE;
       } else if (t < p.cap_tokens) {
