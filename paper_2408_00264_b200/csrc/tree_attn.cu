@@ -1214,24 +1214,18 @@ struct AttnPlan {
 // Blocks along the rows and along the keys: the cheapest choice by a cost in SM cycles, rounds of
 // clusters over the machine times (key tiles of a block x cycles per tile + what a block takes
 // besides).  The figures are fitted to measurements of 22 shapes (batch 1-32, 1-8 row tiles, 350-16424
-// keys).
-// Lengths are data of the device.  But the pages of a pool bound their mean (unless sequences share pages,
-// which costs speed only): if it is below 0.8 of the longest, the blocks of several rounds are not equally long, and
-// handed out longest first they fill the machine to within a fraction of the mean one.  All plans of 251
-// ragged paged shapes (batch 2-48, 200-32768 keys), measured: the plan taken was on average 3.9 % off the best
-// with the cost of equal lengths, and is 1.6 % off with this one (10 x 42 nodes, 28/4 heads, 3019-13316 keys: 113.6 -> 74.7
-// us; 3 of the shapes are slower by more than 3 %).  Equal lengths: 1.4 % off, and other figures gained less than 1 %.
-constexpr double kRagged = 0.8;
-
-AttnPlan make_plan(const clv_shape& s, const clv_kv_cache& c, int max_ctx_len, const int* clusters) {
+// keys).  Lengths are data of the device, so every sequence counts as long as the bound.  A pool's pages are no
+// measure of their mean: with n_pages / batch taken for it, ragged batches gained where the pool just held them (10 x 42 nodes,
+// 28/4 heads, 3019-13316 keys: 115.2 -> 74.1 us; not in a pool of three times the pages), but equally long ones lost with shared pages
+// (32 x 32, 8192 keys, 750 pages: 133.6 -> 147.1) or a loose bound (16 x 64, 4000 keys, bound 16384: 70.2 -> 98.5), and calls
+// of blocks alone, whose partial sums stay fp32, went to clusters, which exchange theirs as fp16.
+AttnPlan make_plan(const clv_shape& s, int max_ctx_len, const int* clusters) {
   const int G = s.n_q_heads / s.n_kv_heads;
   const int rows = s.n_nodes * G;
   const int parts = rows <= BM / 4 ? 4 : rows <= BM / 2 ? 2 : 1;
   const int tiles = (s.n_nodes + BM / G - 1) / (BM / G);   // row tiles of BM / G whole nodes
   const int pieces = (max_ctx_len + PG - 1) / PG + (s.n_nodes + PG - 1) / PG;
   const int64_t units = (int64_t)s.batch * s.n_kv_heads;
-  const double mean_pieces = c.paged && (double)c.n_pages / s.batch < pieces ? (double)c.n_pages / s.batch : (double)pieces;
-  const bool ragged = mean_pieces < kRagged * pieces;
   AttnPlan best = {false, parts, tiles, tiles, 1};
   double best_cost = 1e300;
   for (int r = 0; r < 2; ++r) {
@@ -1239,15 +1233,11 @@ AttnPlan make_plan(const clv_shape& s, const clv_kv_cache& c, int max_ctx_len, c
     const int groups = r ? (tiles + 1) / 2 : tiles;
     for (int sp = 1; sp <= kMaxSplits; ++sp) {
       if (sp > 1 && pieces < 2 * sp) break;   // at least one key tile per block
-      const double fill = (double)(units * groups) / clusters[sp], rounds = ceil(fill);
+      const double rounds = (double)((units * groups + clusters[sp] - 1) / clusters[sp]);
       const double key_tiles = (double)((pieces + sp - 1) / sp) * 0.5;
       const double tile = r ? 3200.0 : parts > 1 ? 1200.0 : 1650.0;
       const double besides = sp == 1 ? 18000.0 : r ? 36000.0 : parts > 1 ? 19500.0 : 22500.0;
-      double cost = rounds * (key_tiles * tile + besides);
-      if (ragged && rounds > 1.0) {
-        const double mean = mean_pieces / sp * 0.5 * tile + besides;
-        cost = fmax(key_tiles * tile + besides, mean * (fill + 0.3 + 0.2 * (rounds - fill)));
-      }
+      const double cost = rounds * (key_tiles * tile + besides);
       if (cost < best_cost) { best_cost = cost; best = {r != 0, parts, tiles, groups, sp}; }
     }
   }
@@ -1274,7 +1264,7 @@ cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const vo
   int dev = 0;
   e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const AttnPlan plan = make_plan(s, c, max_ctx_len, g_clusters[dev]);
+  const AttnPlan plan = make_plan(s, max_ctx_len, g_clusters[dev]);
   const int G = s.n_q_heads / s.n_kv_heads;
   alignas(64) Maps tm;
   const uint64_t cache_rows = c.paged ? (uint64_t)c.n_pages * CLV_PAGE_SIZE : (uint64_t)s.batch * c.cap_tokens;

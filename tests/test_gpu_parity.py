@@ -355,12 +355,12 @@ def test_attention_reference_replaced_in_every_part_of_a_tile(clv, oracle, start
 
 
 @pytest.mark.parametrize("batch,hq,hkv,ctx,n_nodes", [
-    (20, 16, 4, (40, 900), 33),    # one row tile per block where equal lengths would take two
+    (20, 16, 4, (40, 900), 33),    # two row tiles per block
     (20, 8, 4, (40, 900), 100),
-    (44, 8, 2, (10, 700), 70),     # two where equal lengths would take one
+    (44, 8, 2, (10, 700), 70),     # one
 ])
 def test_attention_ragged_batches_in_a_small_pool(clv, oracle, batch, hq, hkv, ctx, n_nodes):
-    # the pool's pages bound the mean length, so the plan is one for blocks of unequal length
+    # blocks of very unequal lengths, several to an SM
     cfg = W.small_config(batch=batch, n_q_heads=hq, n_kv_heads=hkv, ctx=ctx, n_nodes=n_nodes, vocab=64, paged=True,
                          seed=W.BASE_SEED + 660 + batch)
     w = W.generate(cfg)
@@ -368,6 +368,48 @@ def test_attention_ragged_batches_in_a_small_pool(clv, oracle, batch, hq, hkv, c
     st.tree_attn()
     torch.cuda.synchronize()
     check_attention(oracle, w, st)
+
+
+@pytest.mark.parametrize("batch,hq,hkv,ctx,n_nodes", [
+    (20, 8, 4, (60, 2500), 64),    # 80 units on 148 SMs: blocks are alone, partial sums stay fp32
+    (20, 8, 4, (60, 2500), 100),
+    (10, 16, 4, (60, 2500), 42),
+    (20, 16, 4, (40, 900), 33),
+    (44, 8, 2, (10, 700), 70),
+])
+def test_attention_of_a_paged_batch_whatever_the_pool(clv, oracle, batch, hq, hkv, ctx, n_nodes):
+    # The size of a pool says nothing about a batch's lengths: it may hold other batches' pages, and sequences may
+    # share theirs.  So the same bits come from a pool that just holds the batch and from one of three times the pages.
+    cfg = W.small_config(batch=batch, n_q_heads=hq, n_kv_heads=hkv, ctx=ctx, n_nodes=n_nodes, vocab=64, paged=True,
+                         seed=W.BASE_SEED + 680 + batch)
+    w = W.generate(cfg)
+    st = make_step(w)
+    st.tree_attn()
+    w.k_cache, w.v_cache = (np.concatenate([c, c[::-1], c]) for c in (w.k_cache, w.v_cache))
+    st2 = make_step(w)
+    st2.tree_attn()
+    torch.cuda.synchronize()
+    check_attention(oracle, w, st2)
+    assert torch.equal(st.out, st2.out) and torch.equal(st.lse, st2.lse) and torch.equal(st.status[0], st2.status[0])
+
+
+@pytest.mark.parametrize("batch,hq,hkv,n_nodes", [(20, 8, 4, 64), (16, 32, 8, 64), (12, 4, 4, 20), (3, 8, 2, 128)])
+def test_attention_with_shared_pages_and_a_loose_bound(clv, oracle, batch, hq, hkv, n_nodes):
+    # Every sequence begins with the same seven pages, and the bound is eight times the longest context, in a
+    # pool of a few pages per sequence.
+    cfg = W.small_config(batch=batch, n_q_heads=hq, n_kv_heads=hkv, ctx=(448, 700), n_nodes=n_nodes, vocab=64, paged=True,
+                         seed=W.BASE_SEED + 690 + batch)
+    w = W.generate(cfg)
+    w.block_table[:, :7] = w.block_table[0, :7]
+    used, w.block_table = np.unique(w.block_table, return_inverse=True)   # the pages that are left, numbered anew
+    w.block_table = w.block_table.reshape(batch, -1).astype(np.int32) - (1 if used[0] < 0 else 0)
+    w.k_cache, w.v_cache = (np.ascontiguousarray(c[used[used >= 0]]) for c in (w.k_cache, w.v_cache))
+    for bound in (1, 8):
+        st = make_step(w)
+        st.max_ctx_len *= bound
+        st.tree_attn()
+        torch.cuda.synchronize()
+        check_attention(oracle, w, st)
 
 
 @pytest.mark.parametrize("batch,hq,hkv,n_nodes", [
