@@ -89,8 +89,8 @@ struct Cfg {
   static constexpr int kStep = kRows2 ? 2 : 4;   // loads from one tile of a slot to its next
 };
 
-// barriers: stage full [6] | stage empty [6] | S full [2] | part of P [2][3] | last P V done [2] | Q | merge | drain
-constexpr int B_FULL = 0, B_EMPTY = 6, B_S = 12, B_P = 14, B_LAST = 20, B_Q = 22, B_RX = 23, B_DR = 24, NBAR = 25;
+// barriers: stage full [6] | stage empty [6] | S full [2] | part of P [2][2] | last P V done [2] | Q | merge | drain
+constexpr int B_FULL = 0, B_EMPTY = 6, B_S = 12, B_P = 14, B_LAST = 18, B_Q = 20, B_RX = 21, B_DR = 22, NBAR = 23;
 
 struct Misc {                           // behind the tiles in dynamic shared memory
   float2 ml[2 * BM];                    // (reference, sum) of every row of both slots
@@ -409,7 +409,7 @@ __device__ __forceinline__ void issue(const Block<kRows2, kParts>& k, const Para
   const uint64_t k_desc = smem_desc(k.sRing, 16, 1024);
   const uint64_t v_desc = smem_desc(k.sRing, kHalf, 1024);   // lbo: the other half of d
   RingPos<NST> kpos[2] = {RingPos<NST>(0), RingPos<NST>(kRows2 ? 0 : 2)};
-  uint32_t ph = 0u;   // bit 3 s + h: parity of the next use of the barrier for part h of slot s's P
+  uint32_t ph = 0u;   // bit 2 s + h: parity of the next use of the barrier for part h of slot s's P
   auto issue_qk = [&](int s) -> bool {
     if (!wait_warp(k.bar(B_FULL + kpos[s].idx), kpos[s].ph, k.abort_flag, p.wait_limit)) return false;
     tc_fence_after();
@@ -441,9 +441,9 @@ __device__ __forceinline__ void issue(const Block<kRows2, kParts>& k, const Para
 #pragma unroll
       for (int h = 0; h < hand_overs<kParts>(); ++h) {
         if (!ok || (kParts == 1 && h > 0 && keys[1] <= CH)) continue;
-        ok = wait_warp(k.bar(B_P + 3 * s + h), (ph >> (3 * s + h)) & 1u, k.abort_flag, p.wait_limit);
+        ok = wait_warp(k.bar(B_P + 2 * s + h), (ph >> (2 * s + h)) & 1u, k.abort_flag, p.wait_limit);
         if (!ok) continue;
-        ph ^= 1u << (3 * s + h);
+        ph ^= 1u << (2 * s + h);
         tc_fence_after();
 #pragma unroll
         for (int c = 0; c < BN / CH; ++c) {
@@ -501,7 +501,7 @@ __device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Pa
     tmem_wait_st();
     tc_fence_before();
     __syncwarp();
-    mbar_arrive_if(lane == 0 ? 1u : 0u, k.bar(B_P + 3 * slot + h));
+    mbar_arrive_if(lane == 0 ? 1u : 0u, k.bar(B_P + 2 * slot + h));
   };
   RingPos<NST> vpos(kRows2 || slot == 0 ? 1 : 3);   // V stage of the current tile
 #pragma unroll 1
@@ -699,7 +699,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   if (tid == 0) {
     for (int i = 0; i < NST; ++i) { mbar_init(bar(B_FULL + i), 1); mbar_init(bar(B_EMPTY + i), (uint32_t)k.users); }
     for (int i = 0; i < 2; ++i) { mbar_init(bar(B_S + i), 1); mbar_init(bar(B_LAST + i), 1); }
-    for (int i = 0; i < 6; ++i) mbar_init(bar(B_P + i), 4);
+    for (int i = 0; i < 4; ++i) mbar_init(bar(B_P + i), 4);
     mbar_init(bar(B_Q), 1);
     mbar_init(bar(B_RX), 1);
     mbar_init(bar(B_DR), 1);
