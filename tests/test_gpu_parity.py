@@ -338,20 +338,75 @@ def test_attention_scores_that_outgrow_the_first_tile(clv, oracle, n_nodes):
     check_attention(oracle, w, st)
 
 
-@pytest.mark.parametrize("pow2", [1, 3, 7])
-@pytest.mark.parametrize("start", [256, 319, 330, 383])
-def test_attention_reference_replaced_in_every_part_of_a_tile(clv, oracle, start, pow2):
-    # A tile's first 64 keys are judged by their sum of exponentials, the others by their maximum: scores rise
-    # (many by a little, or a few beyond fp32's range) from one key of a tile on, in each of its four chunks
-    # and at their edges.  Scores reach about 60 * 2^pow2 / 16, so fp32 resolves them within the tolerance.
-    cfg = W.small_config(batch=2, n_q_heads=4, n_kv_heads=2, ctx=(390, 700), n_nodes=48, vocab=64,
-                         seed=W.BASE_SEED + 640 + start)
+def judges_of_a_tile(w, tile, slots_share_keys):
+    """What the kernel's softmax judges a row's reference by at one key tile of the context, in float64: the sum of the
+    first 64 keys' probabilities, and the largest of the other 64 in log2 units above the reference.  A block that is
+    alone walks all tiles of its unit (with two row tiles per block), or every second one (one row tile, two slots)."""
+    B, N, Hq, D = w.q.shape
+    G = Hq // w.cfg.n_kv_heads
+    q, k = W.bf16_bits_to_f64(w.q), W.bf16_bits_to_f64(w.k_cache[:, :(tile + 1) * 128])
+    s = np.einsum("bnhd,bkhd->bnhk", q, np.repeat(k, G, axis=2), optimize=True) * (w.scale * np.log2(np.e))
+    ref = None
+    for t in range(tile % 2 if slots_share_keys else 0, tile + 1, 2 if slots_share_keys else 1):
+        x = s[..., t * 128:(t + 1) * 128]
+        if ref is None:
+            ref = x.max(-1)
+            continue
+        with np.errstate(over="ignore"):
+            total = np.exp2(x[..., :64] - ref[..., None]).sum(-1)
+        above = x[..., 64:].max(-1) - ref
+        if t < tile:   # nothing happens before the tile in question
+            assert total.max() < 256 and above.max() < 8
+    return s[..., tile * 128:], ref, total, above
+
+
+@pytest.mark.parametrize("n_nodes,tile,key", [
+    (64, 2, 0), (64, 2, 32), (64, 2, 63), (64, 2, 96),       # one row tile: the first slot,
+    (64, 3, 31), (64, 3, 64), (64, 3, 127),                  #   the second
+    (128, 3, 0), (128, 3, 63), (128, 3, 64), (128, 3, 95),   # two row tiles per block
+])
+def test_attention_reference_replaced_in_every_part_of_a_tile(clv, oracle, n_nodes, tile, key):
+    # Blocks are alone and take two to five tiles per slot.  In one tile behind a slot's first, one key is 128 times as
+    # large, so that about half of the rows' scores outgrow their reference by up to 2^700, and one judge only sees it: the
+    # sum for a tile's first 64 keys, the maximum for the others.  fp32 resolves such scores within the tolerance.
+    cfg = W.small_config(batch=40, n_q_heads=8, n_kv_heads=4, ctx=(520, 640), n_nodes=n_nodes, vocab=64,
+                         seed=W.BASE_SEED + 640 + key)
     w = W.generate(cfg)
-    w.k_cache[:, start:] = _scale_bf16_by_pow2(w.k_cache[:, start:], pow2)
+    at = tile * 128 + key
+    w.k_cache[:, at] = _scale_bf16_by_pow2(w.k_cache[:, at], 7)
+    _, _, total, above = judges_of_a_tile(w, tile, slots_share_keys=n_nodes == 64)
+    by_sum, by_max = total > 256, above > 8
+    assert (by_sum if key < 64 else by_max).mean() > 0.4 and not (by_max if key < 64 else by_sum).any()
     st = make_step(w)
     st.tree_attn()
     torch.cuda.synchronize()
     check_attention(oracle, w, st)
+
+
+@pytest.mark.parametrize("n_nodes,tile", [(64, 2), (64, 3), (128, 3)])
+def test_attention_reference_replaced_for_the_sum_alone(clv, oracle, n_nodes, tile):
+    # The first 64 keys of a tile are all about 2^6.5 above the rows' references: none reaches 2^8, their sum is
+    # about 2^12.  Values are positive and reach 2^118, so an accumulator against the old references would overflow.
+    cfg = W.small_config(batch=40, n_q_heads=8, n_kv_heads=4, ctx=(520, 640), n_nodes=n_nodes, vocab=64, seed=W.BASE_SEED + 648)
+    w = W.generate(cfg)
+    w.q[:] = _scale_bf16_by_pow2(w.q, -3)
+    w.q[..., 0] = W.f32_to_bf16_bits(np.float32([8.0]))[0]
+    w.k_cache[..., 0] = w.k_tree[..., 0] = 0
+    w.k_cache[:, tile * 128:tile * 128 + 64, :, 0] = W.f32_to_bf16_bits(np.float32([7 / (8 * w.scale * np.log2(np.e))]))[0]
+    rng = np.random.default_rng(648)
+    for name in ("v_cache", "v_tree"):
+        v = rng.uniform(1.0, 2.0, size=getattr(w, name).shape).astype(np.float32) * np.float32(2.0 ** 117)
+        setattr(w, name, W.f32_to_bf16_bits(v))
+    scores, ref, total, above = judges_of_a_tile(w, tile, slots_share_keys=n_nodes == 64)
+    assert (scores[..., :64].max(-1) - ref).max() < 8 and above.max() < 8 and total.min() > 2.0 ** 11.9
+    st = make_step(w)
+    st.tree_attn()
+    torch.cuda.synchronize()
+    want = check_attention_status(oracle, w, st)
+    got = bits(st.out)
+    assert np.isfinite(W.bf16_bits_to_f64(got)).all()
+    _, rel = attn_errors(got, want)
+    assert rel <= ATTN_MAX_REL, rel
 
 
 @pytest.mark.parametrize("batch,hq,hkv,ctx,n_nodes", [
