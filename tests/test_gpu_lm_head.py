@@ -105,6 +105,45 @@ def test_first_of_equal_logits_wherever_they_lie_in_a_tile(clv, rows, V):
     assert np.array_equal(got, (h @ w.T).argmax(axis=1))
 
 
+def special_logits(rows, V):
+    """Hidden rows and a vocabulary whose logits are exact in fp32, and the greedy choices: the lowest index of the
+    largest logit after rounding to bf16, NaN ignored, 0 if nothing but -inf and NaN is left.  Row r sees columns c and
+    c + 32 with c = r % 32, and c % 4 says what is special about its logits: 0: all overflow to -inf; 1: one is
+    finite in fp32 and infinite in bf16, behind the largest bf16 number and before one that overflows; 2: the
+    largest are zeros, one of them a negative number that rounds to -0; 3: two equal ones.  Two entries are NaN for
+    every row, and the last row is NaN throughout."""
+    rng = np.random.default_rng(1000 * rows + V)
+    h, w = np.zeros((rows, 64), dtype=np.float32), np.zeros((V, 64), dtype=np.float32)
+    best = np.zeros(32, dtype=np.int32)
+    for c in range(32):
+        at = np.sort(rng.choice(np.arange(1, V - 1), size=3, replace=False))
+        w[:, c] = rng.uniform(-2.0, -1.0, size=V)
+        if c % 4 == 0:
+            w[:, c] = -2.0 ** 100
+        elif c % 4 == 1:
+            w[at[:2], c], w[at[1], c + 32], w[at[2], c] = (2 - 2.0 ** -7) * 2.0 ** 63, 2.0 ** 55, 2.0 ** 100
+            best[c] = at[1]
+        elif c % 4 == 2:
+            w[at, c] = 0.0
+            w[at[c // 4 % 3], c] = -2.0 ** -70
+            best[c] = at[0]
+        else:
+            w[at[:2], c] = 1.0
+            best[c] = at[0]
+        h[c::32, c] = h[c::32, c + 32] = 2.0 ** (-70 if c % 4 == 2 else 64)
+    ids = best[np.arange(rows) % 32]
+    w[[0, V - 1]] = np.nan
+    h[-1], ids[-1] = np.nan, 0
+    return h, w, ids
+
+
+@pytest.mark.parametrize("rows,V", [(40, 48), (128, 600), (300, 1000)])
+def test_logits_that_are_nan_infinite_or_zero(clv, rows, V):
+    h, w, ids = special_logits(rows, V)
+    bf16 = lambda a: torch.from_numpy(a).bfloat16().view(torch.int16).numpy().view(np.uint16)  # noqa: E731
+    assert np.array_equal(run_gpu(clv, bf16(h), bf16(w)), ids)
+
+
 def test_unplanted_rows_are_valid_choices(clv, oracle):
     h, w, _ = W.make_lm_head(200, 512, 4000, seed=77, planted=0.0)
     got = run_gpu(clv, h, w)
