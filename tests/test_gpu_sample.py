@@ -105,7 +105,7 @@ def test_sample_slices_of_a_row_kept_or_fetched_again(clv, oracle, vocab, n_node
             w.logits[b, i, ids[b, i]] = lift
     u = W.make_uniforms(B, n_nodes, seed=vocab)
     got = run_gpu(clv, w.logits, vocab, w.parent, w.tokens, u, 1.0, w.path_cap)
-    compare(oracle, got, w.logits, vocab, w.parent, w.tokens, u, 1.0, w.path_cap, min_robust=0.0)
+    compare(oracle, got, w.logits, vocab, w.parent, w.tokens, u, 1.0, w.path_cap, min_robust=1.0)
 
 
 @pytest.mark.parametrize("temperature", [1.0, 0.6, 1.7])
