@@ -1,9 +1,10 @@
 // Per-node greedy choice: argmax over the vocabulary of each logits row (Sec. 4.2, T = 0).
 //
-// Pure HBM stream: every logit is read once with 16-byte loads that bypass L1.  A row is cut into
-// `chunks` pieces so that the grid covers the machine even for few rows; each block reduces its
-// piece to one (value, lowest index) pair, and the last block to arrive for a row takes the best of
-// its pieces.  The result is independent of the chunking and of block scheduling.
+// Pure HBM stream: every logit is read once with 16-byte loads that bypass L1.  With enough rows to cover the
+// machine a block takes a whole row; with fewer a row is cut into `chunks` pieces, one per block of a cluster,
+// whose (value, lowest index) pairs meet in the shared memory of the cluster's first block.  Very long rows in small
+// numbers are cut further, and the last block to arrive for a row takes the best of its pieces from global memory.
+// The result is independent of the cut and of block scheduling.
 #include <limits.h>
 
 #include "clv_internal.cuh"
@@ -11,9 +12,12 @@
 namespace clv {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kUnroll = 8;  // 16-byte loads in flight per thread (32 KB per block)
-constexpr int kMaxChunk = 2 * kUnroll * kThreads * 8;   // logits of a block
+constexpr int kUnroll = 8;  // 16-byte loads in flight per thread
+constexpr int kMaxCluster = 8;
+constexpr int kPieceThreads = 256;                           // of blocks that meet through global memory
+constexpr int kMaxPiece = 2 * kUnroll * kPieceThreads * 8;   // logits of such a block
+constexpr int kMaxWholeRow = 1 << 26;                        // visits of a thread are numbered in 16 bits
+enum Join { kWholeRow, kByCluster, kByTickets };
 
 __device__ __forceinline__ uint4 ld_stream16(const void* p) {
   uint4 r;
@@ -78,7 +82,22 @@ struct Params {
   uint2* partial;   // (value in unsigned order, index) per piece of a row
 };
 
-__global__ void __launch_bounds__(kThreads) argmax_kernel(Params p) {
+__device__ __forceinline__ void cluster_started() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// a pair to the shared memory of the cluster's first block
+__device__ __forceinline__ void st_first_block(const uint2* local, uint32_t x, uint32_t y) {
+  uint32_t at;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(local)));
+  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(at), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void take_better(uint32_t& value, uint32_t& index, uint2 k) {
+  if (k.x > value || (k.x == value && k.y < index)) { value = k.x; index = k.y; }
+}
+
+// 32 registers, so that as many blocks fit on an SM as its threads allow (with 34, 1024 rows of 128256: 39.0 -> 46.7 us)
+template <int kThreads, Join kJoin>
+__global__ void __launch_bounds__(kThreads, 2048 / kThreads) argmax_kernel(Params p) {
   const int row = blockIdx.x / p.chunks;
   const int chunk = blockIdx.x - row * p.chunks;
   const int begin = chunk * p.chunk_elems;
@@ -89,6 +108,7 @@ __global__ void __launch_bounds__(kThreads) argmax_kernel(Params p) {
   const int tid = threadIdx.x;
   // programmatic launch: the grid may be set up while the previous kernel of the stream drains;
   // nothing is read or written before that kernel's results are complete
+  if (kJoin == kByCluster) cluster_started();
   cudaGridDependencySynchronize();
 
   Track trk;
@@ -102,7 +122,19 @@ __global__ void __launch_bounds__(kThreads) argmax_kernel(Params p) {
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) { take_vec(trk, w[u], visit2); visit2 += 0x00010001u; }
   }
-  for (; i < nvec; i += kThreads) { take_vec(trk, ld_stream16(vp + i), visit2); visit2 += 0x00010001u; }
+  // what is left, in one or two batches of four (vector by vector each of them cost a round trip: 64 rows of 32000 in
+  // clusters of 4 3.14 -> 3.04 us, of 64000 5.8 -> 4.2)
+  auto four = [&](bool guarded) {
+    uint4 w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      w[u] = !guarded || i + u * kThreads < nvec ? ld_stream16(vp + i + u * kThreads) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { take_vec(trk, w[u], visit2); visit2 += 0x00010001u; }
+    i += 4 * kThreads;
+  };
+  if (i + 3 * kThreads < nvec) four(false);
+  if (i < nvec) four(true);
   // the thread's best of its 8 positions: visit k of this thread is vector tid + k * kThreads
   Best best = {-INFINITY, INT_MAX};
 #pragma unroll
@@ -125,20 +157,38 @@ __global__ void __launch_bounds__(kThreads) argmax_kernel(Params p) {
     }
   }
 
-  // Reduction in the order (value descending, index ascending): of a warp, of the block's warps, and by the
-  // last block to arrive of the row's pieces.  All by whole warps; what a small call takes is this chain
-  // (verify steps of 1 x 16 nodes 14.7 -> 14.2 us, of 1 x 64 22.9 -> 22.0, with the walk's minimum by one instruction).
-  __shared__ uint32_t s_value[kThreads / 32], s_index[kThreads / 32];
+  // Reduction in the order (value descending, index ascending), by whole warps: of a warp, of the row's or the
+  // block's warps, of the row's pieces.  What a small call takes is this chain: through global memory (result, fence,
+  // ticket, fence, results) it took 1.7 us of the 5 of 64 rows of 32000, which take 2.7 now.
   const int lane = tid & 31;
+  constexpr int kWarps = kThreads / 32;
   uint32_t value = ordered(best.v), index = (uint32_t)best.i;
   first_of_highest(value, index);
-  if (lane == 0) { s_value[tid >> 5] = value; s_index[tid >> 5] = index; }
-  __syncthreads();
-  if (tid >= 32) return;
-  value = lane < kThreads / 32 ? s_value[lane] : 0u;
-  index = lane < kThreads / 32 ? s_index[lane] : 0xFFFFFFFFu;
-  first_of_highest(value, index);
-  if (p.chunks > 1) {
+  if constexpr (kJoin == kByCluster) {
+    __shared__ uint2 s_pair[kMaxCluster * kWarps];
+    cluster_wait();   // every block of the row runs
+    if (lane == 0) st_first_block(&s_pair[chunk * kWarps + (tid >> 5)], value, index);
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    if (chunk != 0 || tid >= 32) return;
+    value = 0u;
+    index = 0xFFFFFFFFu;
+#pragma unroll
+    for (int c = 0; c < kMaxCluster * kWarps; c += 32)
+      if (c + lane < p.chunks * kWarps) take_better(value, index, s_pair[c + lane]);
+    first_of_highest(value, index);
+  } else {
+    __shared__ uint2 s_pair[kWarps];
+    if (lane == 0) s_pair[tid >> 5] = make_uint2(value, index);
+    __syncthreads();
+    if (tid >= 32) return;
+    const uint2 k = lane < kWarps ? s_pair[lane] : make_uint2(0u, 0xFFFFFFFFu);
+    value = k.x;
+    index = k.y;
+    first_of_highest(value, index);
+  }
+  if constexpr (kJoin == kByTickets) {
     uint2* mine = p.partial + (size_t)row * p.chunks;
     unsigned arrived = 0;
     if (lane == 0) {
@@ -148,10 +198,7 @@ __global__ void __launch_bounds__(kThreads) argmax_kernel(Params p) {
     }
     if (__shfl_sync(0xFFFFFFFFu, arrived, 0) != (unsigned)p.chunks - 1) return;
     __threadfence();
-    for (int c = lane; c < p.chunks; c += 32) {
-      const uint2 k = __ldcg(mine + c);
-      if (k.x > value || (k.x == value && k.y < index)) { value = k.x; index = k.y; }
-    }
+    for (int c = lane; c < p.chunks; c += 32) take_better(value, index, __ldcg(mine + c));
     first_of_highest(value, index);
   }
   if (lane == 0) p.ids[row] = (index == (uint32_t)INT_MAX) ? 0 : (int)index;  // a row of only -inf / NaN: first index
@@ -159,14 +206,13 @@ __global__ void __launch_bounds__(kThreads) argmax_kernel(Params p) {
 
 }  // namespace
 
+// How a call through tickets would cut its rows, which is also what a caller's workspace is sized for (whichever way
+// the call takes): 32768 logits (64 KB) per block, less where there are too few rows to cover the machine.
 ArgmaxPlan argmax_plan(int rows, int vocab) {
   ArgmaxPlan pl;
   pl.rows = rows;
-  // 32768 logits (64 KB) per block = two batches of kUnroll loads per thread (measured best on
-  // 128256-wide rows: 1024 blocks = one wave of 7 blocks per SM); fewer, smaller pieces only when
-  // there are too few rows to cover the machine.
-  const int unit = kThreads * 8;  // elements one pass of the block covers
-  int chunk_elems = kMaxChunk;
+  const int unit = kPieceThreads * 8;  // elements one pass of the block covers
+  int chunk_elems = kMaxPiece;
   const int want_blocks = 4 * sm_count();
   while (chunk_elems > unit && (int64_t)rows * ((vocab + chunk_elems - 1) / chunk_elems) < want_blocks)
     chunk_elems >>= 1;
@@ -176,35 +222,75 @@ ArgmaxPlan argmax_plan(int rows, int vocab) {
   return pl;
 }
 
+namespace {
+template <int kThreads, Join kJoin>
+cudaError_t launch(const Params& p, int rows, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((int64_t)rows * p.chunks), 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  // Small blocks that are launched early would pile up on the SMs that attention leaves idle (step of 1 x 64 nodes x 2048
+  // keys and 32000 logits: 21.6 -> 21.0 us).  Larger ones need the L1 that this would take for their loads in flight.
+  if (kJoin == kByCluster) {
+    cfg.dynamicSmemBytes = even_share_smem((int64_t)rows * p.chunks, 2048 / kThreads);
+    static OncePerDevice once;
+    const cudaError_t e = run_once_per_device(once, [] {
+      return cudaFuncSetAttribute(argmax_kernel<kThreads, kJoin>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    });
+    if (e != cudaSuccess) return e;
+  }
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)p.chunks;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = kJoin == kByCluster ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, argmax_kernel<kThreads, kJoin>, p);
+}
+}  // namespace
+
+// Rows that cover the SMs at least half are not cut, and their blocks are as large as lets one wave take them all;
+// fewer rows are shared by clusters of six blocks (of a row's best cut into 1, 2, 3, 4, 6, 8, six lost least), up to
+// rows for which eight blocks would be too few.  Back to back from a graph, cold, in us (before: all through tickets):
+//   rows x vocabulary     before   1024 threads    512    256   cluster of 6   taken
+//    16 x 32000              3.6            2.6    2.4    2.8            2.3   cluster
+//    64 x 32000              5.5            2.7    3.1    4.2            2.7   cluster
+//    64 x 128256             6.7            6.3    9.2   15.4            5.5   cluster
+//   100 x 128256             8.7            7.0    9.7   15.6            6.8   1024
+//   128 x 16000              5.7            3.2    3.3    4.9            4.0   1024
+//   192 x 32000              5.9            5.0    4.6    5.8            5.4   512
+//   256 x 128256            13.3           11.9   12.7   17.4           14.6   1024
+//   512 x 64000             14.1           13.5   12.1   13.5           15.5   512
+//   768 x 32000             10.1           11.7   11.0   10.1           14.9   256
+//  1024 x 128256            41.4           42.2   39.8   39.0           44.8   256
 cudaError_t launch_argmax(const ArgmaxPlan& plan, const void* logits, int64_t ld, int vocab,
                           int32_t* ids, unsigned* tickets, void* scratch, cudaStream_t stream) {
   Params p;
   p.logits = static_cast<const uint16_t*>(logits);
   p.ld = ld;
   p.vocab = vocab;
-  p.chunks = plan.chunks;
-  p.chunk_elems = plan.chunk_elems;
+  p.chunks = 1;
+  p.chunk_elems = vocab;
   p.ids = ids;
   p.tickets = tickets;
   p.partial = static_cast<uint2*>(scratch);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((int64_t)plan.rows * plan.chunks), 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  // Not for blocks of full size: their loads in flight need the L1 that this would take (4 x 64 rows of
-  // 128256: 44.7 -> 46.9 us for the step).
-  if (plan.chunk_elems < kMaxChunk) cfg.dynamicSmemBytes = even_share_smem((int64_t)plan.rows * plan.chunks, 2048 / kThreads);
-  static OncePerDevice once;
-  const cudaError_t e = run_once_per_device(once, [] {
-    return cudaFuncSetAttribute(argmax_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-  });
-  if (e != cudaSuccess) return e;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, argmax_kernel, p);
+  const int sms = sm_count();
+  if (2 * plan.rows > sms && vocab <= kMaxWholeRow) {
+    if (plan.rows <= sms || (plan.rows <= 2 * sms && vocab > kMaxPiece)) return launch<1024, kWholeRow>(p, plan.rows, stream);
+    if (plan.rows <= 4 * sms) return launch<512, kWholeRow>(p, plan.rows, stream);
+    return launch<256, kWholeRow>(p, plan.rows, stream);
+  }
+  if (2 * plan.rows > sms || vocab > kMaxCluster * kMaxPiece) {
+    p.chunks = plan.chunks;
+    p.chunk_elems = plan.chunk_elems;
+    return launch<kPieceThreads, kByTickets>(p, plan.rows, stream);
+  }
+  constexpr int kPieces = 6;
+  p.chunk_elems = ((vocab + kPieces - 1) / kPieces + 7) & ~7;
+  p.chunks = (vocab + p.chunk_elems - 1) / p.chunk_elems;
+  return launch<256, kByCluster>(p, plan.rows, stream);
 }
 
 // ---- variant whose scratch lives in the library image ------------------------------------------

@@ -652,6 +652,29 @@ def test_argmax_cuts_ties_and_ragged_rows(clv, oracle, rows_b, rows_n, vocab):
         ids.fill_(-5)
 
 
+@pytest.mark.parametrize("rows,vocab", [(1, 262144), (1, 262153), (3, 100003), (74, 2051), (75, 2051), (148, 4100), (149, 32768), (149, 32776),
+                                        (296, 32769), (297, 8195), (592, 6147), (593, 6147), (600, 8193)])
+def test_argmax_at_the_edges_of_its_blocks(clv, oracle, rows, vocab):
+    # How a row is shared depends on rows and vocabulary (148 SMs): both sides of every line, with remainders of the
+    # batches of loads.  Ties: a maximum in the last element and one anywhere before it.
+    ld = (vocab + 7) // 8 * 8 + 8
+    rng = np.random.default_rng(vocab + rows)
+    lg = np.empty((rows, ld), np.uint16)
+    lg[:, :vocab] = W.f32_to_bf16_bits(rng.standard_normal(vocab + 131).astype(np.float32))[np.arange(vocab) + np.arange(rows)[:, None] % 131]
+    lg[:, vocab:] = 0x7F00                        # huge values in the padding must be ignored
+    big = int(W.f32_to_bf16_bits(np.array([9.0], np.float32))[0])
+    lg[:, vocab - 1] = big
+    at = rng.integers(0, vocab, size=rows)
+    lg[np.arange(rows)[::2], at[::2]] = big
+    shape = clv.make_shape(rows, 1, 1, 1, vocab, 1)
+    ids = torch.full((rows, 1), -5, dtype=torch.int32, device="cuda")
+    clv.clv_accept_argmax(shape, torch.from_numpy(lg.view(np.int16)).cuda(), ld, ids, clv.new_workspace(shape, None, 0))
+    torch.cuda.synchronize()
+    ref = oracle.argmax(lg, vocab)
+    assert np.array_equal(ref[::2], at[::2]) and (ref[1::2] == vocab - 1).all()
+    assert np.array_equal(ids.cpu().numpy().reshape(-1), ref)
+
+
 # ------------------------------------------------------------------ walk and commit
 def test_walk_random_trees_and_errors(clv, oracle):
     rng = np.random.default_rng(5)
