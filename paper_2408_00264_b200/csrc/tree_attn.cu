@@ -62,14 +62,14 @@ constexpr int HD = CLV_HEAD_DIM;       // 128
 constexpr int BM = 128;                // rows per slot
 constexpr int BN = 128;                // keys per tile
 constexpr int CH = 32;                 // keys whose scores one load brings
-constexpr int kThreads = 384;          // warps 0-3 and 4-7: the slots' softmax; 8: TMA producer; 9: MMA issuer; 10, 11 idle
+constexpr int kThreads = 384;          // warps 0-3 and 4-7: the slots' softmax; 8: TMA producer; 9: MMA issuer; 10 reports; 11 idle
 // Registers per thread: the launch's 168 cannot hold a row's 128 scores and the rest of a softmax
 // thread, so the third warpgroup's go to the first two while the roles work (256 x 216 + 128 x 72 =
 // 384 x 168; 4 x 64 nodes x 4096 keys, launch to launch: 28.0 -> 26.5 us).  (The variant with two threads per row
 // spills: -Xptxas -v reports 4 bytes stored and 20 loaded.)
 constexpr int kSoftmaxRegs = 216, kOtherRegs = 72, kLaunchRegs = 168;
 static_assert(2 * kSoftmaxRegs + kOtherRegs <= 3 * kLaunchRegs, "a block shares out the registers that it was launched with");
-constexpr int kSoftmaxWarps = 8, kProducer = 8, kIssuer = 9;
+constexpr int kSoftmaxWarps = 8, kProducer = 8, kIssuer = 9, kWriter = 10;
 constexpr int kMaxSplits = 8;          // portable cluster size
 constexpr uint32_t kQTile = BM * HD * 2;      // 32 KB: two [128 rows][64 d] swizzled halves
 constexpr uint32_t kPiece = PG * 64 * 2;       // 8 KB: [64 keys][64 d] swizzled, one TMA box
@@ -89,16 +89,34 @@ struct Cfg {
   static constexpr int kStep = kRows2 ? 2 : 4;   // loads from one tile of a slot to its next
 };
 
+// What the merge sends of a row: its columns as fp16, and 16 bytes of reference, sum and scales (of either half of
+// the columns, where different warps send them).
+template <bool kRows2>
+constexpr uint32_t kRowBytes = HD * 2 + (kRows2 ? 16 : 32);
+
 // barriers: stage full [6] | stage empty [6] | S full [2] | part of P [2][2] | last P V done [2] | Q | merge | drain
 constexpr int B_FULL = 0, B_EMPTY = 6, B_S = 12, B_P = 14, B_LAST = 18, B_Q = 20, B_RX = 21, B_DR = 22, NBAR = 23;
 
+// What the merge needs to know about its block, the launch's constants among it (in shared memory meanwhile: see there).
+struct __align__(16) Place {
+  int b, split, kvh, users;
+  int T, R, per, first;
+  int mine, tile0, CS, N;
+  int G, Hq, tile_nodes, tiles;
+  int group_d;
+  unsigned group_m, meta;              // by_group_heads; where a third idle stage starts in the ring
+  uint16_t* out;
+  float* lse;
+  uint32_t rx[kMaxSplits];             // where each rank receives, in its ring
+};
 struct Misc {                           // behind the tiles in dynamic shared memory
   float2 ml[2 * BM];                    // (reference, sum) of every row of both slots
   unsigned long long bar[NBAR];
   uint32_t tmem;
   int abort_flag;                       // a wait of the roles ran out
   int late_flag;                        // the wait for the last P V did
-  int seq, len;                         // the block's sequence and its context length
+  int seq;                              // the block's sequence, if they are handed out by length
+  Place place;
   int issued;                           // loads issued (producer)
   signed char parent[CLV_MAX_NODES];    // as far as valid, -1 otherwise
 };
@@ -164,6 +182,13 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
         "l"(reinterpret_cast<unsigned long long&>(c)));
   return d;
 }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  float2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;"
+      : "=l"(reinterpret_cast<unsigned long long&>(d))
+      : "l"(reinterpret_cast<unsigned long long&>(a)), "l"(reinterpret_cast<unsigned long long&>(b)));
+  return d;
+}
 __device__ __forceinline__ float2 add2(float2 a, float2 b) {
   float2 d;
   asm("add.rn.f32x2 %0, %1, %2;"
@@ -221,8 +246,19 @@ __device__ __forceinline__ float4 ld_shared16(uint32_t a) {
   asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
   return v;
 }
+__device__ __forceinline__ void st_shared4(uint32_t a, uint32_t x) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(x) : "memory"); }
 __device__ __forceinline__ void st_shared8(uint32_t a, float x, float y) {
   asm volatile("st.shared.v2.f32 [%0], {%1,%2};" ::"r"(a), "f"(x), "f"(y) : "memory");
+}
+__device__ __forceinline__ uint32_t ld_shared4(uint32_t a) {
+  uint32_t x;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x) : "r"(a) : "memory");
+  return x;
+}
+__device__ __forceinline__ uint2 ld_shared8(uint32_t a) {
+  uint2 v;
+  asm volatile("ld.shared.v2.b32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory");
+  return v;
 }
 
 // a position in the ring of stages and the parity of its current round
@@ -463,6 +499,29 @@ __device__ __forceinline__ void issue(const Block<kRows2, kParts>& k, const Para
   }
 }
 
+// By an idle warp, meanwhile: what the merge needs to know, so that nothing but shared memory is read ahead of its copies.
+// Two neighbouring stages of the ring receive and a third holds this block's own sums: any but those of the last V tiles.
+template <bool kRows2, int kParts>
+__device__ __forceinline__ void note_place(const Block<kRows2, kParts>& k, const Params& p) {
+  constexpr int NST = Cfg<kRows2, kParts>::NST;
+  Place& at = k.misc().place;
+  if (k.lane < kMaxSplits) {   // other ranks write there, so the place is a function of the receiver's number of tiles
+    const unsigned d = min((unsigned)k.lane, (unsigned)k.CS - 1u);
+    const int tiles_of_rank = ((int)(p.by_splits.divide((d + 1u) * (unsigned)k.p_total) - p.by_splits.divide(d * (unsigned)k.p_total)) + 1) / 2;
+    const int i = (2 * tiles_of_rank) % NST, idx = i == NST - 1 ? 0 : i;
+    at.rx[k.lane] = (uint32_t)idx * kStage;
+    if ((int)d == k.split) at.meta = (uint32_t)((idx + 2) % NST) * kStage;
+  }
+  if (k.lane == 0) {
+    at.b = k.b; at.split = k.split; at.kvh = k.kvh;
+    at.users = k.users; at.T = k.T; at.R = k.R; at.per = k.per;
+    at.first = k.first; at.mine = k.mine; at.tile0 = k.tile0; at.CS = k.CS;
+    at.N = k.N; at.G = k.G; at.Hq = p.Hq; at.tile_nodes = k.tile_nodes;
+    at.tiles = p.tiles; at.group_d = (int)p.by_group_heads.d; at.group_m = p.by_group_heads.m;
+    at.out = p.out; at.lse = p.lse;
+  }
+}
+
 template <bool kRows2, int kParts>
 __device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Params& p, int par) {
   constexpr int NST = Cfg<kRows2, kParts>::NST;
@@ -480,7 +539,10 @@ __device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Pa
           const int e = p.block_table[(int64_t)k.b * p.max_pages + pg];
           bad |= (e < 0 || e >= p.n_pages);
         }
-      if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(p.tickets + 2 * k.b + 1, 1u);  // before this block's ticket
+      if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) {
+        atomicOr(p.tickets + 2 * k.b + 1, 1u);
+        __threadfence();   // before this block's ticket
+      }
     }
   }
   __syncwarp();
@@ -703,7 +765,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     mbar_init(bar(B_Q), 1);
     mbar_init(bar(B_RX), 1);
     mbar_init(bar(B_DR), 1);
-    if (kParts > 1 ? !kOneBlock : k.CS > 1) mbar_expect_tx(bar(B_RX), (uint32_t)((k.CS - 1) * kParts * k.mine) * 272u);   // what the other ranks will send
+    if (kParts > 1 ? !kOneBlock : k.CS > 1) mbar_expect_tx(bar(B_RX), (uint32_t)((k.CS - 1) * kParts * k.mine) * kRowBytes<kRows2>);   // what the other ranks will send
     ms.abort_flag = 0;
     ms.late_flag = 0;
     ms.issued = 0;
@@ -745,7 +807,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   __syncwarp();
   const int par = tid < k.N ? p.parent[(int64_t)k.b * k.N + tid] : -1;   // of node tid
   k.range(p, p.ctx_len[k.b]);
-  if (tid == 0) { ms.seq = k.b; ms.len = k.L; }
+  if (warp == kWriter) note_place(k, p);
   if (warp < kSoftmaxWarps) {
     more_registers<kSoftmaxRegs>();
     softmax<kRows2, kParts>(k, p, par);
@@ -763,23 +825,17 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   }
 
   // ---- every role has met here ------------------------------------------------------------------
-  // What is known about the block is worked out once more: kept in registers it would push the softmax
-  // threads' scores out of theirs (4 x 64 nodes x 4096 keys: 29.8 -> 27.7 us).
-  Block<kRows2, kParts> k;
-  {
-    unsigned block;
-    int thread;
-    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(block));
-    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(thread));
-    k.place(p, smem, block, thread);
-    k.b = ms.seq;
-    k.range(p, ms.len);
-  }
-  const int tid = k.tid, warp = k.warp, lane = k.lane, CS = k.CS, split = k.split, kvh = k.kvh, N = k.N, G = k.G;
-  const int tile_nodes = k.tile_nodes, tile0 = k.tile0, users = k.users, b = k.b, T = k.T;
-  const int R = k.R, per = k.per, first = k.first, mine = k.mine;
-  const uint32_t smem0 = k.smem0, sRing = k.sRing;
-  auto bar = [&](int idx) { return k.bar(idx); };
+  // What follows runs once per block, from a cold instruction cache, and that is what it takes its time by: compact
+  // loops, few instructions ahead of the copies.  What is known about the block comes from shared memory: kept in
+  // registers it would push the softmax threads' scores out of theirs (4 x 64 nodes x 4096 keys: 29.8 -> 27.7 us), and
+  // worked out once more it took 570 cycles instead of 90.
+  const Place& at = ms.place;
+  int tid;
+  asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+  const int warp = tid >> 5, lane = tid & 31, CS = at.CS, split = at.split, users = at.users, b = at.b, T = at.T;
+  const int R = at.R, per = at.per, first = at.first, mine = at.mine;
+  const uint32_t smem0 = smem_u32(smem), sRing = smem0 + Cfg<kRows2, kParts>::kQ * kQTile, tmem = ms.tmem;
+  auto bar = [&](int idx) { return smem_u32(&ms.bar[0]) + 8u * (uint32_t)idx; };
   // Calls this short lose a tenth of their time between two launches.  The next kernel may be set up on the
   // SMs that this grid leaves idle or has left, and waits for this grid's results itself (32 layers of
   // 1 x 60 nodes x 1500 keys and LM head, in a loop: 486 -> 470 us).  The other variants do not: what follows a long call is a
@@ -788,7 +844,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   if (kParts > 1) cudaTriggerProgrammaticLaunchCompletion();
   const bool clustered = kParts > 1 ? !kOneBlock : CS > 1;
   const bool alone = kParts == 1 && !clustered;   // nothing to be added to this block's accumulators
-  const bool aborted = *k.abort_flag != 0;
+  const bool aborted = *const_cast<volatile int*>(&ms.abort_flag) != 0;
   if (clustered) cluster_arrive();   // all Q K^T of this block are done: what the merge uses is idle (see there)
   if (aborted) {
     // copies that were issued land on their own, MMAs that were issued finish: wait for both
@@ -806,45 +862,57 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     }
     __syncthreads();
   }
-  // status[b] is written once, by whichever block of the sequence finishes last.  The sequence's two words in
-  // the workspace count the blocks that are behind their last wait, and with them, in the upper word, what
-  // went wrong (1: malformed input; 2 for each block in which a wait ran out), so that the holder of the last
-  // ticket has it all from one round trip, behind the final rows; it leaves both words zero for the next
-  // call.
+  // status[b] is written by whichever block of the sequence leaves its roles last.  The sequence's two words in the
+  // workspace count the blocks that have, and with them, in the upper word, what went wrong until then (1: malformed
+  // input; 2 for each block in which a wait ran out); the holder of the last ticket has it all from one round trip, which
+  // ends while the rows are staged, and leaves both words zero for the next call.  A wait of the merge that runs out comes
+  // after the block's ticket: such a block waits for the words to be zero and corrects the status behind the holder's.
   unsigned long long* const tally = reinterpret_cast<unsigned long long*>(p.tickets + 2 * b);
+  const bool clerk = tid == 32 * kWriter;
   unsigned long long ticket = 0;
-  auto take_ticket = [&](bool failed) {
-    if (tid != 32 * kIssuer) return;
-    if (k.group == 0 && split == 0 && kvh == 0) __threadfence();   // what the softmax threads reported comes first
-    ticket = atomicAdd(tally, failed ? (2ull << 32) + 1ull : 1ull) + (failed ? 2ull << 32 : 0ull);
-  };
+  if (clerk) ticket = atomicAdd(tally, aborted ? (2ull << 32) + 1ull : 1ull) + (aborted ? 2ull << 32 : 0ull);
   auto publish = [&]() {
-    if (tid != 32 * kIssuer || (unsigned)ticket != (unsigned)p.blocks_per_seq - 1) return;
-    *tally = 0ull;
+    if (!clerk || (unsigned)ticket != (unsigned)p.blocks_per_seq - 1) return;
     const unsigned wrong = (unsigned)(ticket >> 32);
-    p.status[b] = (wrong & 1u) ? CLV_ERR_TREE : wrong ? CLV_ERR_TIMEOUT : CLV_OK;
+    *const_cast<volatile int32_t*>(p.status + b) = (wrong & 1u) ? CLV_ERR_TREE : wrong ? CLV_ERR_TIMEOUT : CLV_OK;
+    __threadfence();
+    *const_cast<volatile unsigned long long*>(tally) = 0ull;
+  };
+  auto correct = [&](bool failed_late) {
+    if (!clerk || !failed_late) return;
+    const long long t0 = clock64();
+    while (*const_cast<volatile unsigned long long*>(tally) != 0ull && clock64() - t0 < kWaitLimitCycles) {}
+    __threadfence();
+    atomicCAS(p.status + b, CLV_OK, CLV_ERR_TIMEOUT);
   };
 
   // ---- merge.  Idle once all Q K^T of a block are done, which is when it arrives at the cluster
   //      barrier: the Q tiles (staging of the rows to be sent), and all ring stages but those of the
-  //      last V tiles.  Two neighbouring stages receive; since other ranks write there, the place is a
-  //      function of the receiver's number of tiles.  A third one holds what goes with this block's
-  //      own rows: 16 bytes per row (reference, sum, scales of its halves) | where each row's output
-  //      starts.
-  auto rx_index = [&](int tiles_of_rank) {
-    const int i = (2 * tiles_of_rank) % NST;
-    return i == NST - 1 ? 0 : i;
-  };
-  auto rank_tiles = [&](int d) {
-    return ((int)(p.by_splits.divide((unsigned)(d + 1) * (unsigned)k.p_total) - p.by_splits.divide((unsigned)d * (unsigned)k.p_total)) + 1) / 2;
-  };
-  auto rx_meta = [&](uint32_t rx_base) { return rx_base + (uint32_t)((CS - 1) * kParts * per) * 256u; };   // behind the rows
-  const uint32_t rx = sRing + (uint32_t)rx_index(T) * kStage;
-  const uint32_t meta = sRing + (uint32_t)((rx_index(T) + 2) % NST) * kStage;
-  const uint32_t row_at = meta + 4096u;
+  //      last V tiles.  Two neighbouring stages receive; a third one holds what goes with this block's
+  //      own rows (reference, sum, scales) | where each row's output starts | the sources' weights.
+  //      Rows are 128 bytes per half of their columns, 16-byte piece c of row r at c ^ (r & 7).
+  //      What counts is the number of instructions of one thread's chain, at about four cycles each: the same code, run
+  //      again with warm caches, takes as long.  Packed arithmetic, each warp's rows sent as they are staged, a lane per
+  //      source for the weights, addresses by increments: from where the roles meet to the end 6500 -> 5900 cycles for
+  //      1 x 16 nodes x 512 keys (MHA), 5600 -> 5400 for 4 x 64 x 4096 (8 KV heads); the step of 32 layers of 1 x 60 x 1500
+  //      and LM head 464 -> 451 us, of 4 x 64 x 4096 1010 -> 998.  (Stores from registers into the peers instead of staged
+  //      copies: 130 cycles each, 478 us; sums sent ahead and weights worked out by the other warps while rows are
+  //      staged, one copy per peer: 447 and 1010.)
+  constexpr int kRows = Cfg<kRows2, kParts>::kRows, kSlotRows = kRows2 ? 2 * BM : BM;   // rows of a part; of a staged half
+  constexpr uint32_t kHalfRows = (uint32_t)kSlotRows * 128u;
+  const int received = (CS - 1) * kParts, sources = CS * kParts;
+  auto rx_meta = [&](uint32_t rx_base) { return rx_base + (uint32_t)(received * per) * 256u; };   // behind the rows
+  const uint32_t rx = sRing + at.rx[split], meta = sRing + at.meta;
+  const uint32_t row_at = meta + 4096u, weights = meta + 8192u, lse_at = meta + 16384u;
   __syncwarp();
   if (warp < kSoftmaxWarps) {
-    const int slot = k.slot, row = k.row, row_in_out = (b * N + k.node) * p.Hq + kvh * G + (row % Cfg<kRows2, kParts>::kRows - k.node_in_tile * G);
+    const int slot = (warp >> 2) & 1, row = (warp & 3) * 32 + lane, part = row / kRows, tile_row = row % kRows;
+    const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
+    const int rtile = kRows2 ? at.tile0 + slot : at.tile0;
+    const int node_in_tile = (int)Divisor{(unsigned)at.group_d, at.group_m}.divide((unsigned)tile_row), node = rtile * at.tile_nodes + node_in_tile;
+    const bool row_valid = tile_row < at.tile_nodes * at.G && rtile < at.tiles && node < at.N;
+    const int row_in_out = (b * at.N + node) * at.Hq + at.kvh * at.G + (tile_row - node_in_tile * at.G);
+    const int seq_row = (kRows2 ? slot * BM : 0) + row;   // number of this row within the block
     float2 ml = ms.ml[slot * BM + row];
     float w0 = 1.f, w1 = 0.f;
     if (!kRows2) {   // combine the slots' shares of the keys
@@ -859,80 +927,121 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
       const float inv = ml.y > 0.f ? 1.f / ml.y : 0.f;
       w0 *= inv;
       w1 *= inv;
-      if (p.lse != nullptr && k.row_valid && (kRows2 || slot == 0)) p.lse[row_in_out] = log_sum_exp(ml.x, ml.y);
+      if (at.lse != nullptr && row_valid && (kRows2 || slot == 0)) at.lse[row_in_out] = log_sum_exp(ml.x, ml.y);
     }
+    // what the warp's lane d will send to rank d
+    int to_send = 0, send_from = 0;
+    uint32_t their_rows = 0u, their_sums = 0u, their_bar = 0u;
+    if (clustered && lane < CS && lane != split) {
+      const int d = lane, row0 = row - lane - part * kRows + (kRows2 ? slot * BM : 0);   // the warp's first row, as the ranks share them out
+      const int f = max(row0, d * per);
+      to_send = min(min(R, d * per + per), row0 + 32) - f;
+      send_from = f + part * kRows;
+      const int src = (split < d ? split : split - 1) * kParts + part, to = f - d * per;
+      const uint32_t base = cluster_map(sRing + at.rx[d], (uint32_t)d);
+      their_bar = cluster_map(bar(B_RX), (uint32_t)d);
+      their_rows = base + (uint32_t)(src * 2 * per + to) * 128u;
+      their_sums = rx_meta(base) + (uint32_t)((kRows2 ? src : src * 2 + slot) * per + to) * 16u;
+    }
+    __syncwarp();
     // the last P V of the accumulators this thread reads
-    const bool has0 = kRows2 ? k.my_tiles > 0 : T > 0, has1 = !kRows2 && T > 1;
+    const bool has0 = kRows2 ? slot < users && T > 0 : T > 0, has1 = !kRows2 && T > 1;
     if (!aborted) {
-      bool done = true;
-      if (has0) done = wait_warp(bar(B_LAST + (kRows2 ? slot : 0)), 0, &ms.late_flag, p.wait_limit);
-      if (has1 && done) wait_warp(bar(B_LAST + 1), 0, &ms.late_flag, p.wait_limit);
+      const uint32_t bar0 = bar(B_LAST + (kRows2 ? slot : 0));
+      bool done = (!has0 || mbar_test(bar0, 0)) & (!has1 || mbar_test(bar(B_LAST + 1), 0));   // both under way at once
+      if (!__all_sync(0xFFFFFFFFu, done)) {
+        done = !has0 || wait_warp(bar0, 0, &ms.late_flag, p.wait_limit);
+        if (has1 && done) wait_warp(bar(B_LAST + 1), 0, &ms.late_flag, p.wait_limit);
+      }
     }
     __syncwarp();
     tc_fence_after();
-    // half a row (64 columns) at a time: bf16 output if the block is alone, else fp16 for the rank
-    // that finalises the row
-    const int seq_row = (kRows2 ? slot * BM : 0) + row;   // number of this row within the block
-    const uint32_t acc0 = (kRows2 ? k.tmem_O(slot) : k.tmem_O(0)) + k.lane_addr, acc1 = k.tmem_O(1) + k.lane_addr;
+    // Half a row (64 columns) at a time: bf16 output if the block is alone (into the Q tile's place and layout; TMA
+    // stores it), fp32 if its parts are all there is to add up (512 bytes per row where a cluster would receive), else
+    // fp16 for the rank that finalises the row.
+    const uint32_t acc0 = tmem + (uint32_t)(2 * BN + (kRows2 ? slot * HD : 0)) + lane_addr, acc1 = tmem + (uint32_t)(2 * BN + HD) + lane_addr;
+    float downs[2] = {0.f, 0.f};   // what undoes the scales of the halves
 #pragma unroll 1
     for (int half = kRows2 ? 0 : slot; half < (kRows2 ? 2 : slot + 1); ++half) {
-      float v[64];
+      float2 v[32];
       {
-        uint32_t u[64], u1[64];
-        if (has0) tmem_ld_x64(acc0 + (uint32_t)(half * 64), u);
-        if (!kRows2 && has1) tmem_ld_x64(acc1 + (uint32_t)(half * 64), u1);
-        tmem_wait_ld();
+        const float2 ww0 = make_float2(w0, w0), ww1 = make_float2(w1, w1);
+        if (has1) {
+          uint32_t u[64], u1[64];
+          tmem_ld_x64(acc0 + (uint32_t)(half * 64), u);
+          tmem_ld_x64(acc1 + (uint32_t)(half * 64), u1);
+          tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < 64; ++j) {
-          v[j] = has0 ? __uint_as_float(u[j]) * w0 : 0.f;
-          if (!kRows2 && has1) v[j] = fmaf(__uint_as_float(u1[j]), w1, v[j]);
+          for (int j = 0; j < 32; ++j)
+            v[j] = fma2(make_float2(__uint_as_float(u1[2 * j]), __uint_as_float(u1[2 * j + 1])), ww1,
+                        mul2(make_float2(__uint_as_float(u[2 * j]), __uint_as_float(u[2 * j + 1])), ww0));
+        } else if (has0) {
+          uint32_t u[64];
+          tmem_ld_x64(acc0 + (uint32_t)(half * 64), u);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = mul2(make_float2(__uint_as_float(u[2 * j]), __uint_as_float(u[2 * j + 1])), ww0);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = make_float2(0.f, 0.f);
         }
       }
-      if (alone) {   // into the Q tile's place and layout; TMA stores it
-        const uint32_t dst = smem0 + (kRows2 ? slot * kQTile : 0u) + (uint32_t)half * (kQTile / 2) + (uint32_t)row * 128u;
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-          st_shared16(dst + (uint32_t)((c ^ (row & 7)) << 4), pack_bf16(v[8 * c], v[8 * c + 1]), pack_bf16(v[8 * c + 2], v[8 * c + 3]),
-                      pack_bf16(v[8 * c + 4], v[8 * c + 5]), pack_bf16(v[8 * c + 6], v[8 * c + 7]));
-      } else if (kOneBlock) {   // no row leaves the block: the parts stay fp32, 512 bytes per row where a cluster would receive
-        const uint32_t dst = rx + (uint32_t)row * 512u;
+      if (kOneBlock) {
+        const uint32_t to = rx + (uint32_t)row * 512u;
 #pragma unroll
         for (int c = 0; c < 16; ++c)   // 16-byte piece c of row r sits at c ^ (r & 31)
-          st_shared16(dst + (uint32_t)(((half * 16 + c) ^ (row & 31)) << 4), __float_as_uint(v[4 * c]), __float_as_uint(v[4 * c + 1]),
-                      __float_as_uint(v[4 * c + 2]), __float_as_uint(v[4 * c + 3]));
+          st_shared16(to + (uint32_t)(((half * 16 + c) ^ (row & 31)) << 4), __float_as_uint(v[2 * c].x), __float_as_uint(v[2 * c].y),
+                      __float_as_uint(v[2 * c + 1].x), __float_as_uint(v[2 * c + 1].y));
+        continue;
+      }
+      uint32_t h[32], to;
+      if (alone) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) h[j] = pack_bf16(v[j].x, v[j].y);
+        to = smem0 + (kRows2 ? slot * kQTile : 0u) + (uint32_t)half * (kQTile / 2) + (uint32_t)row * 128u;
       } else {
         float top[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int j = 0; j < 64; j += 2) top[(j >> 1) & 3] = max3(top[(j >> 1) & 3], fabsf(v[j]), fabsf(v[j + 1]));
+        for (int j = 0; j < 32; ++j) top[j & 3] = max3(top[j & 3], fabsf(v[j].x), fabsf(v[j].y));
         const float amax = fmaxf(max3(top[0], top[1], top[2]), top[3]);
         // scale 2^lc with amax * 2^lc in [2^13, 2^14), up to the largest fp32 number; lc is clamped so that
         // the scale and its inverse are normal numbers (zeros stay zeros, inf or NaN stay what they are)
-        const int biased = (int)((__float_as_uint(amax) >> 23) & 255u);
-        const int lc = max(-114, min(100, 140 - biased));
-        const float up = __uint_as_float((uint32_t)(127 + lc) << 23);
-        asm volatile("st.shared.f32 [%0], %1;" ::"r"(meta + (uint32_t)seq_row * 16u + 8u + (uint32_t)half * 4u),
-                     "f"(__uint_as_float((uint32_t)(127 - lc) << 23)) : "memory");
-        // 256 bytes per row; 16-byte piece c of row r sits at c ^ (r & 15)
-        const uint32_t dst = smem0 + (uint32_t)seq_row * 256u;
+        const int lc = max(-114, min(100, 140 - (int)((__float_as_uint(amax) >> 23) & 255u)));
+        const float up = __uint_as_float((uint32_t)(127 + lc) << 23), down = __uint_as_float((uint32_t)(127 - lc) << 23);
+        if (half) downs[1] = down; else downs[0] = down;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          uint32_t h[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const __half2 hv = __floats2half2_rn(v[8 * c + 2 * e] * up, v[8 * c + 2 * e + 1] * up);
-            h[e] = *reinterpret_cast<const uint32_t*>(&hv);
-          }
-          st_shared16(dst + (uint32_t)(((half * 8 + c) ^ (row & 15)) << 4), h[0], h[1], h[2], h[3]);
+        for (int j = 0; j < 32; ++j) {
+          const float2 x = mul2(v[j], make_float2(up, up));
+          const __half2 hv = __floats2half2_rn(x.x, x.y);
+          h[j] = *reinterpret_cast<const uint32_t*>(&hv);
         }
+        to = smem0 + (uint32_t)half * kHalfRows + (uint32_t)seq_row * 128u;
       }
+#pragma unroll
+      for (int c = 0; c < 8; ++c) st_shared16(to + (uint32_t)((c ^ (row & 7)) << 4), h[4 * c], h[4 * c + 1], h[4 * c + 2], h[4 * c + 3]);
     }
-    if (!alone && (kRows2 || slot == 0)) {
-      st_shared8(meta + (uint32_t)seq_row * 16u, ml.x, ml.y);
-      // where the row's output starts (in rows of 128), -1: the row does not exist
-      asm volatile("st.shared.b32 [%0], %1;" ::"r"(row_at + (uint32_t)seq_row * 4u), "r"(k.row_valid ? row_in_out : -1) : "memory");
+    if (!alone) {   // (of the scales, a reader takes the one of the half that it reads)
+      const float d0 = downs[0], d1 = downs[1];
+      st_shared16(meta + (uint32_t)((kRows2 ? 0 : slot * BM) + seq_row) * 16u, __float_as_uint(ml.x), __float_as_uint(ml.y), __float_as_uint(d0), __float_as_uint(d1));
     }
-    fence_async_smem();
+    if (alone || clustered) fence_async_smem();
     tc_fence_before();
+    __syncwarp();
+    if (clustered) {   // each warp sends its rows, a lane per peer
+      cluster_wait();   // every rank's receiving stages are idle
+      if (to_send > 0) {
+#pragma unroll
+        for (int half = 0; half < 2; ++half)
+          if (kRows2 || half == slot)
+            bulk_to_peer(their_rows + (uint32_t)(half * per) * 128u, smem0 + (uint32_t)half * kHalfRows + (uint32_t)send_from * 128u, (uint32_t)to_send * 128u, their_bar);
+        bulk_to_peer(their_sums, meta + (uint32_t)((kRows2 ? 0 : slot * BM) + send_from) * 16u, (uint32_t)to_send * 16u, their_bar);
+      }
+      __syncwarp();
+    }
+    if (!alone && (kRows2 || slot == 0))   // where the row's output starts (in rows of 128), -1: the row does not exist
+      st_shared4(row_at + (uint32_t)seq_row * 4u, (uint32_t)(row_valid ? row_in_out : -1));
+  } else if (clustered) {
+    cluster_wait();
   }
   __syncthreads();
   bool failed = aborted || *reinterpret_cast<volatile int*>(&ms.late_flag) != 0;   // neither flag is written any more
@@ -942,194 +1051,151 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
       mbar_drain(bar(B_DR), 0);
     }
     tc_fence_after();
-    tmem_dealloc(k.tmem, kTmemCols);
+    tmem_dealloc(tmem, kTmemCols);
   }
 
-  if (!clustered) take_ticket(failed);
+  publish();
+  __syncwarp();
   if (alone) {
     if (tid == 0 && !failed) {
 #pragma unroll
       for (int m = 0; m < Cfg<kRows2, kParts>::kQ; ++m) {
         if (m >= users) break;
-        tma_store_4d(&tm.out, smem0 + m * kQTile, 0, kvh * G, (tile0 + m) * tile_nodes, b);
-        tma_store_4d(&tm.out, smem0 + m * kQTile + kQTile / 2, 64, kvh * G, (tile0 + m) * tile_nodes, b);
+        tma_store_4d(&tm.out, smem0 + m * kQTile, 0, at.kvh * at.G, (at.tile0 + m) * at.tile_nodes, b);
+        tma_store_4d(&tm.out, smem0 + m * kQTile + kQTile / 2, 64, at.kvh * at.G, (at.tile0 + m) * at.tile_nodes, b);
       }
       asm volatile("cp.async.bulk.commit_group;" ::: "memory");
       asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
     }
-    publish();
+    correct(failed && !aborted);
     return;
   }
 
   if (clustered) {
-    cluster_wait();   // every rank's receiving stages are idle
-    const int d = tid / kParts, part = tid % kParts;
-    if (d < CS && d != split) {   // a peer's rows, then what goes with them
-      const int f = min(R, d * per), n = min(R, f + per) - f, row0 = part * Cfg<kRows2, kParts>::kRows + f;
-      if (n > 0) {
-        const uint32_t base = sRing + (uint32_t)rx_index(rank_tiles(d)) * kStage;
-        const uint32_t at = (uint32_t)(((split < d ? split : split - 1) * kParts + part) * per);
-        const uint32_t their_bar = cluster_map(bar(B_RX), (uint32_t)d);
-        bulk_to_peer(cluster_map(base + at * 256u, (uint32_t)d), smem0 + (uint32_t)row0 * 256u, (uint32_t)n * 256u, their_bar);
-        bulk_to_peer(cluster_map(rx_meta(base) + at * 16u, (uint32_t)d), meta + (uint32_t)row0 * 16u, (uint32_t)n * 16u, their_bar);
-      }
-    }
-    const bool got = mbar_drain_within(bar(B_RX), 0, p.wait_limit);
+    if (!mbar_drain_within(bar(B_RX), 0, p.wait_limit)) ms.late_flag = 1;   // looked at again behind the next barrier
     __syncwarp();
     cluster_arrive();   // what this block was sent has arrived: its peers may leave
-    failed |= __syncthreads_or(got ? 0 : 1) != 0;
-    take_ticket(failed);
   }
   // ---- final rows.  A source of a row is a part of a block's accumulators: first what was received, by
   //      rank, then this block's own, always in this order, so that the result does not depend on timing.
-  //      What counts here is the length of one thread's chain: the sources are loaded four at a time
-  //      ahead of their sums (one after the other they cost 90 cycles each).
-  const int rows = failed ? 0 : mine;
-  constexpr int kSources = kMaxSplits * kParts;
-  const int received = (CS - 1) * kParts, sources = CS * kParts;
-  const uint8_t* rx_rows = smem + (rx - smem0);                     // of source 0; the next source's are per rows on
-  const uint8_t* own_rows = smem + first * 256;                     // of part 0; the next part's are kRows rows on
-  const float4* rx_sums = reinterpret_cast<const float4*>(smem + (rx_meta(rx) - smem0));
-  const float4* own_sums = reinterpret_cast<const float4*>(smem + (meta - smem0)) + first;
-  const int* row_outs = reinterpret_cast<const int*>(smem + (row_at - smem0)) + first;
-  constexpr int kRows = Cfg<kRows2, kParts>::kRows;
-  auto sums_of = [&](int j, int i) { return j < received ? rx_sums[j * per + i] : own_sums[(j - received) * kRows + i]; };
-  auto write_lse = [&](int o, float M, float total) {
-    if (p.lse != nullptr && o >= 0) p.lse[o] = log_sum_exp(M, total);
-  };
-  // 8 columns of row i (16-byte piece c): sources j0 .. j0 + 3 with weights w
-  auto add = [&](float (&acc)[8], int j0, int i, int c, auto weight) {
-    const uint32_t at = (uint32_t)i * 256u + (uint32_t)((c ^ ((first + i) & 15)) << 4);
-    uint4 u[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (j0 + j < sources)
-        u[j] = *reinterpret_cast<const uint4*>((j0 + j < received ? rx_rows + (j0 + j) * per * 256 : own_rows + (j0 + j - received) * (kRows * 256)) + at);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const float w = weight(j);
-      if (j0 + j >= sources) continue;
-      const uint32_t h[4] = {u[j].x, u[j].y, u[j].z, u[j].w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 f = half2_bits_to_float2(h[e]);
-        acc[2 * e] = fmaf(f.x, w, acc[2 * e]);
-        acc[2 * e + 1] = fmaf(f.y, w, acc[2 * e + 1]);
-      }
-    }
-  };
-  auto write_row = [&](const float (&acc)[8], int o, int c) {
-    *reinterpret_cast<uint4*>(p.out + (int64_t)o * HD + c * 8) =
-        make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
-  };
-  if constexpr (kParts == 1) {   // up to 128 rows of few sources: their weights first, a thread per row
-    float* weights = reinterpret_cast<float*>(smem + (meta + 8192u - smem0));   // [row][half][source]
-    for (int i = tid; i < rows; i += kThreads) {
-      float4 m[kSources];
-      float M = -INFINITY;
-#pragma unroll
-      for (int j = 0; j < kSources; ++j) {
-        m[j] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
-        if (j < sources) m[j] = sums_of(j, i);
-        M = fmaxf(M, m[j].x);
-      }
-      const float mu = M == -INFINITY ? 0.f : M;
-      float total = 0.f;
-#pragma unroll
-      for (int j = 0; j < kSources; ++j) {
-        m[j].x = ex2(m[j].x - mu);   // ex2(-inf) = 0
-        total = fmaf(m[j].y, m[j].x, total);
-      }
-      const float inv = total > 0.f ? 1.f / total : 0.f;
-#pragma unroll
-      for (int j = 0; j < kSources; ++j) {
-        if (j >= sources) continue;
-        weights[i * 2 * kSources + j] = m[j].x * m[j].z * inv;
-        weights[i * 2 * kSources + kSources + j] = m[j].x * m[j].w * inv;
-      }
-      write_lse(row_outs[i], M, total);
-    }
-    __syncthreads();
-    for (int it = tid; it < rows * 16; it += kThreads) {
-      const int i = it >> 4, c = it & 15, o = row_outs[i];
-      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int j0 = 0; j0 < kSources; j0 += 4) {
-        if (j0 >= sources) break;
-        const float4 w4 = *reinterpret_cast<const float4*>(weights + i * 2 * kSources + (c >> 3) * kSources + j0);
-        const float w[4] = {w4.x, w4.y, w4.z, w4.w};
-        add(acc, j0, i, c, [&](int j) { return w[j]; });
-      }
-      if (o >= 0) write_row(acc, o, c);
-    }
-  } else if constexpr (kOneBlock) {   // this block's parts, fp32, eight columns of a row per item
+  int rows = failed ? 0 : mine;
+  if constexpr (kOneBlock) {   // this block's parts, fp32, eight columns of a row per item
+    const uint32_t own_sums = meta + (uint32_t)first * 16u;
 #pragma unroll 1
     for (int it = tid; it < rows * 16; it += kThreads) {
-      const int i = it >> 4, c = it & 15, o = row_outs[i];
+      const int i = it >> 4, c = it & 15, o = (int)ld_shared4(row_at + (uint32_t)(first + i) * 4u);
       float M = -INFINITY;
 #pragma unroll
-      for (int j = 0; j < kParts; ++j) M = fmaxf(M, own_sums[j * kRows + i].x);
+      for (int j = 0; j < kParts; ++j) M = fmaxf(M, ld_shared16(own_sums + (uint32_t)(j * kRows + i) * 16u).x);
       const float mu = M == -INFINITY ? 0.f : M;
       float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, total = 0.f;
 #pragma unroll
       for (int j = 0; j < kParts; ++j) {
-        const float4 m = own_sums[j * kRows + i];
+        const uint32_t r = (uint32_t)(j * kRows + i), from = rx + r * 512u;
+        const float4 m = ld_shared16(own_sums + r * 16u);
         const float w = ex2(m.x - mu);   // ex2(-inf) = 0
-        const uint32_t r = (uint32_t)(j * kRows + i), at = rx + r * 512u;
-        const float4 lo = ld_shared16(at + (((uint32_t)(2 * c) ^ (r & 31u)) << 4));
-        const float4 hi = ld_shared16(at + (((uint32_t)(2 * c + 1) ^ (r & 31u)) << 4));
+        const float4 lo = ld_shared16(from + (((uint32_t)(2 * c) ^ (r & 31u)) << 4));
+        const float4 hi = ld_shared16(from + (((uint32_t)(2 * c + 1) ^ (r & 31u)) << 4));
         const float x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
         total = fmaf(m.y, w, total);
 #pragma unroll
         for (int e = 0; e < 8; ++e) acc[e] = fmaf(x[e], w, acc[e]);
       }
       const float inv = total > 0.f ? 1.f / total : 0.f;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[e] *= inv;
-      if (o >= 0) write_row(acc, o, c);
-      if (c == 0) write_lse(o, M, total);
+      if (o < 0) continue;
+      *reinterpret_cast<uint4*>(at.out + (int64_t)o * HD + c * 8) = make_uint4(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv),
+                                                                           pack_bf16(acc[4] * inv, acc[5] * inv), pack_bf16(acc[6] * inv, acc[7] * inv));
+      if (c == 0 && at.lse != nullptr) at.lse[o] = log_sum_exp(M, total);
     }
-  } else {   // up to 32 rows of many sources: eight lanes share a row's sources for one half of its columns
+  } else {
+    // The sources' weights, a lane per source (2^n lanes per row, so that a row is a chain of two short reductions),
+    // for either half of the columns.
+    constexpr int kMetaStep = kRows2 ? 16 : 32;   // times per: from a source's to the next's
+    const int lanes_log = sources <= 2 ? 1 : sources <= 4 ? 2 : sources <= 8 ? 3 : sources <= 16 ? 4 : 5;
 #pragma unroll 1
-    for (int i0 = 2 * warp; i0 < rows; i0 += 2 * (kThreads / 32)) {
-      const int i = min(i0 + (lane >> 4), rows - 1), c = lane & 15, o = row_outs[i];
-      float4 m[kParts];   // sources (lane & 7) + 8 e
-      float M = -INFINITY;
-#pragma unroll
-      for (int e = 0; e < kParts; ++e) {
-        const int j = (lane & 7) + 8 * e;
-        m[e] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
-        if (j < sources) m[e] = sums_of(j, i);
-        M = fmaxf(M, m[e].x);
+    for (int it0 = warp * 32; it0 < rows << lanes_log; it0 += kThreads) {
+      const int i = (it0 + lane) >> lanes_log, j = (it0 + lane) & ((1 << lanes_log) - 1);
+      const bool here = i < rows && j < sources;
+      float4 m0 = make_float4(-INFINITY, 0.f, 0.f, 0.f), m1 = m0;
+      if (here) {
+        const uint32_t at0 = j < received ? rx_meta(rx) + (uint32_t)(j * per * kMetaStep + i * 16) : meta + (uint32_t)((j - received) * kRows + first + i) * 16u;
+        m0 = ld_shared16(at0);
+        m1 = kRows2 ? m0 : ld_shared16(at0 + (j < received ? (uint32_t)per * 16u : (uint32_t)BM * 16u));
       }
+      float M = m0.x;
 #pragma unroll
-      for (int d = 1; d < 8; d *= 2) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, d));
-      const float mu = M == -INFINITY ? 0.f : M;
-      float total = 0.f;
+      for (int d = 1; d < 32; d *= 2)
+        if (d < 1 << lanes_log) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, d));
+      const float w = ex2(m0.x - (M == -INFINITY ? 0.f : M));   // ex2(-inf) = 0
+      float total = m0.y * w;
 #pragma unroll
-      for (int e = 0; e < kParts; ++e) {
-        m[e].x = ex2(m[e].x - mu);   // ex2(-inf) = 0
-        total = fmaf(m[e].y, m[e].x, total);
-      }
-#pragma unroll
-      for (int d = 1; d < 8; d *= 2) total += __shfl_xor_sync(0xFFFFFFFFu, total, d);
+      for (int d = 1; d < 32; d *= 2)
+        if (d < 1 << lanes_log) total += __shfl_xor_sync(0xFFFFFFFFu, total, d);
       const float inv = total > 0.f ? 1.f / total : 0.f;
-      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      if (here) {
+        const uint32_t to = weights + (uint32_t)(i * 2 * sources + j) * 4u;
+        st_shared4(to, __float_as_uint(w * m0.z * inv));
+        st_shared4(to + (uint32_t)sources * 4u, __float_as_uint(w * m1.w * inv));
+        if (j == 0) st_shared8(lse_at + (uint32_t)i * 8u, M, total);
+      }
+    }
+    __syncthreads();
+    if (clustered && *reinterpret_cast<volatile int*>(&ms.late_flag) != 0) {
+      failed = true;
+      rows = 0;
+    }
+    if (at.lse != nullptr)   // by the last warps, which have fewer items below
+      for (int i = kThreads - 1 - tid; i < rows; i += kThreads) {
+        const int o = (int)ld_shared4(row_at + (uint32_t)(first + i) * 4u);
+        const uint2 m = ld_shared8(lse_at + (uint32_t)i * 8u);
+        if (o >= 0) at.lse[o] = log_sum_exp(__uint_as_float(m.x), __uint_as_float(m.y));
+      }
+    // kCols columns of a row per item, so that there are items for all threads; a source is a load, its weight another
+    constexpr int kCols = kParts > 2 ? 4 : 8, kItems = HD / kCols;
+#pragma unroll 1
+    for (int it = tid; it < rows * kItems; it += kThreads) {
+      const int i = it / kItems, c = it % kItems, half = c / (kItems / 2);
+      const uint32_t piece = (uint32_t)(((c * kCols / 8) & 7) ^ (i & 7)) * 16u + (kCols == 4 ? (uint32_t)(c & 1) * 8u : 0u);   // first and per are multiples of 8
+      float acc[kCols];
 #pragma unroll
-      for (int j0 = 0; j0 < kSources; j0 += 4) {
-        if (j0 >= sources) break;
-        const float scale = (c < 8 ? m[j0 >> 3].z : m[j0 >> 3].w) * (m[j0 >> 3].x * inv);
-        add(acc, j0, i, c, [&](int j) { return __shfl_sync(0xFFFFFFFFu, scale, (j0 + j) & 7, 8); });
-      }
-      if (i0 + (lane >> 4) < rows) {
-        if (o >= 0) write_row(acc, o, c);
-        if (c == 0) write_lse(o, M, total);
-      }
+      for (int e = 0; e < kCols; ++e) acc[e] = 0.f;
+      auto take = [&](uint32_t from, uint32_t w_at) {
+        uint32_t h[kCols / 2];
+        if constexpr (kCols == 8) {
+          const float4 u = ld_shared16(from);
+          h[0] = __float_as_uint(u.x); h[1] = __float_as_uint(u.y); h[2] = __float_as_uint(u.z); h[3] = __float_as_uint(u.w);
+        } else {
+          const uint2 u = ld_shared8(from);
+          h[0] = u.x; h[1] = u.y;
+        }
+        const float w = __uint_as_float(ld_shared4(w_at));
+#pragma unroll
+        for (int x = 0; x < kCols / 2; ++x) {
+          const float2 f = half2_bits_to_float2(h[x]);
+          acc[2 * x] = fmaf(f.x, w, acc[2 * x]);
+          acc[2 * x + 1] = fmaf(f.y, w, acc[2 * x + 1]);
+        }
+      };
+      uint32_t w_at = weights + (uint32_t)((i * 2 + half) * sources) * 4u;
+      uint32_t from = rx + (uint32_t)(half * per + i) * 128u + piece;
+      const uint32_t step = (uint32_t)per * 256u;
+#pragma unroll 4
+      for (int j = 0; j < received; ++j, from += step, w_at += 4u) take(from, w_at);
+      from = smem0 + (uint32_t)half * kHalfRows + (uint32_t)(first + i) * 128u + piece;
+#pragma unroll
+      for (int j = 0; j < kParts; ++j) take(from + (uint32_t)(j * kRows) * 128u, w_at + 4u * (uint32_t)j);
+      const int o = (int)ld_shared4(row_at + (uint32_t)(first + i) * 4u);
+      if (o < 0) continue;
+      uint16_t* out = at.out + (int64_t)o * HD + c * kCols;
+      if constexpr (kCols == 8)
+        *reinterpret_cast<uint4*>(out) = make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
+      else
+        *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]));
     }
   }
   __syncwarp();
   if (clustered) cluster_wait();   // no block may leave while a copy still reads its shared memory
-  publish();
+  correct(failed && !aborted);
 }
 
 // ------------------------------------------------------------------------------------ host side
