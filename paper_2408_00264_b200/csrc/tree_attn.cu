@@ -62,14 +62,14 @@ constexpr int HD = CLV_HEAD_DIM;       // 128
 constexpr int BM = 128;                // rows per slot
 constexpr int BN = 128;                // keys per tile
 constexpr int CH = 32;                 // keys whose scores one load brings
-constexpr int kThreads = 384;          // warps 0-3 and 4-7: the slots' softmax; 8: TMA producer; 9: MMA issuer; 10 reports; 11 idle
+constexpr int kThreads = 384;          // warps 0-3 and 4-7: the slots' softmax; 8: TMA producer; 9: MMA issuer; 10 reports; 11 asks ahead
 // Registers per thread: the launch's 168 cannot hold a row's 128 scores and the rest of a softmax
 // thread, so the third warpgroup's go to the first two while the roles work (256 x 216 + 128 x 72 =
 // 384 x 168; 4 x 64 nodes x 4096 keys, launch to launch: 28.0 -> 26.5 us).  (The variant with two threads per row
 // spills: -Xptxas -v reports 4 bytes stored and 20 loaded.)
 constexpr int kSoftmaxRegs = 216, kOtherRegs = 72, kLaunchRegs = 168;
 static_assert(2 * kSoftmaxRegs + kOtherRegs <= 3 * kLaunchRegs, "a block shares out the registers that it was launched with");
-constexpr int kSoftmaxWarps = 8, kProducer = 8, kIssuer = 9, kWriter = 10;
+constexpr int kSoftmaxWarps = 8, kProducer = 8, kIssuer = 9, kWriter = 10, kScout = 11;
 constexpr int kMaxSplits = 8;          // portable cluster size
 constexpr uint32_t kQTile = BM * HD * 2;      // 32 KB: two [128 rows][64 d] swizzled halves
 constexpr uint32_t kPiece = PG * 64 * 2;       // 8 KB: [64 keys][64 d] swizzled, one TMA box
@@ -145,6 +145,7 @@ struct Params {
   int B, N, Hq, Hkv, G;
   int paged, cap_tokens, n_pages, max_pages;
   int longest_first;  // hand out sequences in order of decreasing context length
+  int ask_ahead;      // the first key tiles into L2 ahead of the previous kernel's end
   int pair_boxes;     // the 4-D tensor maps exist: a whole 128-key tile of a contiguous cache is one copy
   int tiles;          // row tiles per (sequence, kv head)
   int groups;         // blocks along the rows: tiles, or pairs of tiles (kRows2)
@@ -370,6 +371,38 @@ __device__ __forceinline__ void load_q(const Block<kRows2, kParts>& k, const Map
     tma_load_4d(dst, &tm.q, 0, k.kvh * k.G, node0, k.b, k.bar(B_Q));
     tma_load_4d(dst + kQTile / 2, &tm.q, 64, k.kvh * k.G, node0, k.b, k.bar(B_Q));
   }
+}
+
+// Ahead of the previous kernel's end, by an idle warp: the block's first key tiles of context are asked for into L2, a lane
+// per piece.  Length and block table are read as hints (an earlier kernel may still be writing them): whatever they say,
+// the addresses are in range, and what is loaded in the end goes by what they say then.  For the short variants, whose
+// loads would otherwise start from nothing when the previous grid is gone (1 x 64 nodes x 2048 keys, whole step: 20.5 -> 18.9
+// us; 32 layers of 1 x 60 x 1500 and LM head: 450 -> 432; with three tiles 1 % less, with four or eight 2; attention behind a
+// kernel that is not launched ahead of its end: 15.2 -> 14.9).  The other variants lost: where their loop is bound by the
+// tensor core, or the memory is busy anyway, it is traffic in the way (one tile, 32 layers of 4 x 64 x 4096: 985 -> 995;
+// 32 x 32 paged: 137.4 -> 138.4).
+constexpr int kAhead = 2;
+constexpr int kAheadFrom = 3;   // key tiles of a block, by the bound of the lengths: with fewer there is nothing to gain
+template <bool kRows2, int kParts>
+__device__ __forceinline__ void scout(const Block<kRows2, kParts>& k, const Maps& tm, const Params& p) {
+  const int most = p.paged ? p.max_pages * PG : p.cap_tokens;
+  const int len = max(0, min(ld_hint(p.ctx_len + k.b), most));
+  const int p_cache = (len + PG - 1) / PG, p_total = p_cache + (k.N + PG - 1) / PG;
+  const int begin = (int)p.by_splits.divide((unsigned)k.split * (unsigned)p_total);
+  const int end = min(min(p_cache, begin + 2 * kAhead), (int)p.by_splits.divide((unsigned)(k.split + 1) * (unsigned)p_total));
+  for (int g = begin + k.lane; g < end; g += 32) {
+    int row = k.b * p.cap_tokens + g * PG;
+    if (p.paged) {
+      const int pg = ld_hint(p.block_table + (int64_t)k.b * p.max_pages + g);
+      if (pg < 0 || pg >= p.n_pages) continue;
+      row = pg * PG;
+    }
+    tma_prefetch_3d(&tm.kc, 0, k.kvh, row);
+    tma_prefetch_3d(&tm.kc, 64, k.kvh, row);
+    tma_prefetch_3d(&tm.vc, 0, k.kvh, row);
+    tma_prefetch_3d(&tm.vc, 64, k.kvh, row);
+  }
+  __syncwarp();
 }
 
 template <bool kRows2, int kParts>
@@ -780,6 +813,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     tma_prefetch_desc(&tm.kt); tma_prefetch_desc(&tm.vt);
   }
   tc_fence_before();
+  if (kParts > 1 && p.ask_ahead && warp == kScout) scout(k, tm, p);
   __syncthreads();
   tc_fence_after();
   cudaGridDependencySynchronize();
@@ -1360,6 +1394,8 @@ cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const vo
   p.groups = plan.groups;
   p.splits = plan.splits;
   p.longest_first = (clusters * plan.splits > sm_count() && s.batch > 1 && s.batch <= 256) ? 1 : 0;
+  const int pieces = (max_ctx_len + PG - 1) / PG + (s.n_nodes + PG - 1) / PG;
+  p.ask_ahead = plan.parts > 1 && !p.longest_first && pieces >= 2 * kAheadFrom * plan.splits ? 1 : 0;
   p.scale_log2 = scale * 1.4426950408889634f;
   p.wait_limit = wait_limit_cycles();
   p.tickets = tickets;

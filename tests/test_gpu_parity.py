@@ -248,6 +248,43 @@ def test_attention_flags_bad_sequences(clv, oracle):
 
 
 @pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("n_nodes", [16, 50])
+def test_attention_asks_ahead_by_hints_that_are_wrong(clv, oracle, n_nodes, paged):
+    # Key tiles are asked for into L2 by the lengths and pages as they stand ahead of the previous kernel's end (row tiles of up to
+    # 64 rows, three key tiles per block and more): lengths and pages out of range, and lengths that the commit in front changes.
+    w = W.generate(W.small_config(batch=4, n_q_heads=4, n_kv_heads=4, ctx=4000, n_nodes=n_nodes, paged=paged))
+    st = make_step(w)
+    st.tree_attn()
+    torch.cuda.synchronize()
+    check_attention(oracle, w, st)
+    good = w.ctx_len.copy()
+    alen, aidx = torch.tensor([3, 0, 2, 1], dtype=torch.int32, device="cuda"), torch.zeros(4, w.path_cap, dtype=torch.int32, device="cuda")
+    aidx[:, :3] = torch.arange(3, device="cuda", dtype=torch.int32)
+    before = torch.from_numpy(good - np.array([3, 0, 2, 1], np.int32)).cuda()
+    moved = st.k_cache.clone(), st.v_cache.clone()
+    for _ in range(3):      # the commit advances the lengths to `good` and overwrites rows that attention reads right behind it
+        st.k_cache.copy_(moved[0]); st.v_cache.copy_(moved[1]); st.ctx_len.copy_(before)
+        clv.clv_kv_commit(st.shape, st.cache, st.k_tree, st.v_tree, aidx, alen, st.ctx_len, st.ctx_len, st.status[2])
+        st.tree_attn()
+    torch.cuda.synchronize()
+    assert np.array_equal(st.ctx_len.cpu().numpy(), good)
+    w.k_cache[:], w.v_cache[:] = bits(st.k_cache), bits(st.v_cache)
+    check_attention(oracle, w, st)
+    bad = good.copy()
+    bad[1], bad[2] = -5, 1 << 30
+    st.ctx_len.copy_(torch.from_numpy(bad))
+    flagged = [0, clv.CLV_ERR_TREE, clv.CLV_ERR_TREE, 0]
+    if paged:
+        table = w.block_table.copy()
+        table[3, :5] = [-7, w.n_pages, 1 << 30, -1, w.n_pages + 5]
+        st.block_table.copy_(torch.from_numpy(table))
+        flagged[3] = clv.CLV_ERR_TREE
+    st.tree_attn()
+    torch.cuda.synchronize()
+    assert st.status[0].cpu().tolist() == flagged
+
+
+@pytest.mark.parametrize("paged", [False, True])
 def test_attention_units_of_many_row_tiles(clv, oracle, paged):
     # four row tiles per (sequence, kv head) (GQA 4 x 128 nodes = 512 rows): such units are worked
     # by blocks of two row tiles; ragged contexts, one of them shorter than a key tile, key splits
