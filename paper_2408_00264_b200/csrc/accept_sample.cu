@@ -26,7 +26,9 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kPiece = 32768;   // logits per block of the statistics pass (64 KB)
-constexpr int kUnroll = 8;
+// Vectors of a batch of the statistics pass, whose registers let six blocks of it share an SM (eight vectors: three blocks,
+// 16 x 64 rows of 128256 59 us instead of 54, or five with a few registers spilled, 55.5; 5 x 27 of 50257 the same).
+constexpr int kUnroll = 4;
 constexpr int kSlice = kPiece / (kThreads / 32);   // 4096 logits per warp: the unit of the running sums
 constexpr int kPerThread = kSlice / kThreads;       // 16: what a thread scans of the chosen slice
 static_assert(kSlice == 4096 && kPerThread == 16, "a slice is scanned in one round of the block");
@@ -55,29 +57,58 @@ __device__ __forceinline__ void stat_merge(Stat& a, const Stat& b) {
   a.s = a.s * ex2(a.m - ref) + b.s * ex2(b.m - ref);   // 2^(-inf) = 0 for an empty side
   a.m = m;
 }
-// A batch of kUnroll vectors at once: one maximum and at most one rescale for the 64 values, then
-// their exponentials into four running sums (no long chain of dependent additions).
-__device__ __forceinline__ void stat_take_batch(Stat& st, const uint4 (&w)[kUnroll], float k) {
-  float mx = -INFINITY;
+__device__ __forceinline__ __nv_bfloat162 as_bf162(uint32_t u) { return *reinterpret_cast<__nv_bfloat162*>(&u); }
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+  return (unsigned long long)__float_as_uint(y) << 32 | __float_as_uint(x);
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ float low(unsigned long long v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float high(unsigned long long v) { return __uint_as_float((uint32_t)(v >> 32)); }
+
+// A batch of kUnroll vectors at once: one maximum and at most one rescale for the 32 values, then
+// their exponentials into four running sums (no long chain of dependent additions).  Beside the stream this is bound by
+// its instructions, so the maximum is taken of packed bf16 (a positive factor does not change which it is, and the
+// maximum with -inf drops a NaN, which carries no mass), and products, differences and sums are packed fp32 (statistics and walk of
+// 16 x 64 rows of 128256 64.3 -> 59.2 us, of 5 x 27 of 50257 11.8 -> 10.7 with the walk's changes).
+__device__ __forceinline__ void stat_take_batch(Stat& st, uint4 (&w)[kUnroll], float k) {
+  const __nv_bfloat162 none = as_bf162(0xFF80FF80u);
+  __nv_bfloat162 top[2] = {none, none};
 #pragma unroll
   for (int u = 0; u < kUnroll; ++u) {
-    const uint32_t r[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+    uint32_t* r = reinterpret_cast<uint32_t*>(&w[u]);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) mx = fmaxf(mx, fmaxf(bf16_lo(r[j]) * k, bf16_hi(r[j]) * k));   // NaN operands are dropped
+    for (int j = 0; j < 4; ++j) {
+      const __nv_bfloat162 x = __hmax2(as_bf162(r[j]), none);
+      r[j] = *reinterpret_cast<const uint32_t*>(&x);
+      top[j & 1] = __hmax2(top[j & 1], x);
+    }
   }
+  const __nv_bfloat162 t = __hmax2(top[0], top[1]);
+  const float mx = fmaxf(__low2float(t), __high2float(t)) * k;
   if (!(mx > -INFINITY)) return;   // nothing but -inf (or NaN): no mass
   if (mx > st.m) { st.s *= ex2(st.m - mx); st.m = mx; }
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+  const unsigned long long kk = pack2(k, k), mm = pack2(-st.m, -st.m);
+  unsigned long long acc[2] = {0ull, 0ull};
 #pragma unroll
   for (int u = 0; u < kUnroll; ++u) {
     const uint32_t r[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const float a = bf16_lo(r[j]) * k, b = bf16_hi(r[j]) * k;
-      acc[j] += ((a == a) ? ex2(a - st.m) : 0.f) + ((b == b) ? ex2(b - st.m) : 0.f);   // a NaN logit carries no mass
+      const unsigned long long x = fma2(pack2(bf16_lo(r[j]), bf16_hi(r[j])), kk, mm);
+      acc[j & 1] = add2(acc[j & 1], pack2(ex2(low(x)), ex2(high(x))));
     }
   }
-  st.s += (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  const unsigned long long sum = add2(acc[0], acc[1]);
+  st.s += low(sum) + high(sum);
 }
 
 struct StatParams {
@@ -88,7 +119,7 @@ struct StatParams {
   float2* partial;   // [rows][pieces * 8]: one (maximum, sum) per slice
 };
 
-__global__ void __launch_bounds__(kThreads) softmax_stats_kernel(StatParams p) {
+__global__ void __launch_bounds__(kThreads, 6) softmax_stats_kernel(StatParams p) {
   const int row = blockIdx.x / p.pieces;
   const int piece = blockIdx.x - row * p.pieces;
   const int begin = piece * kPiece;
@@ -146,21 +177,35 @@ struct WalkParams {
 // what runs before and behind it: 4 x 109 nodes, 56488 logits, the whole step: 35 -> 43 us.
 constexpr int kKept = 512;
 
+constexpr int kMaskWords = CLV_MAX_NODES / 32;
+// f(node) for every node of a mask below `end`, in increasing order
+template <class F>
+__device__ __forceinline__ void for_each_below(const uint32_t (&mask)[kMaskWords], int end, F f) {
+#pragma unroll 1
+  for (int w = 0; 32 * w < end; ++w) {
+    uint32_t bits = mask[w];
+    if (end - 32 * w < 32) bits &= (1u << (end - 32 * w)) - 1u;
+    for (; bits; bits &= bits - 1u) f(32 * w + __ffs(bits) - 1);
+  }
+}
+
 // One block per sequence.  What bounds it is the number of dependent round trips to memory, so everything
 // that any level of the walk may need is fetched at once: every row's statistics, and every node's
-// logit in its parent's row.  The walk itself then runs in shared memory, along lists of siblings
+// logit in its parent's row.  Siblings are bits of their parent's mask; every node's test is made by a thread of its own
+// ahead of the walk, which is then one load per level (one thread that tested and walked took 1.2 us for 27 nodes, 1.8 for
+// 109; now 0.3 and 0.4).
 // (statistics and walk, 5 sequences of 27 nodes, 50257 logits: 16.8 -> 12.8 us; 6 of 109 nodes: 42 -> 20), the
 // statistics ahead of the tree that the logits' addresses come from, and kept for the draw (the whole step 35.0 -> 34.7).
 __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
-  __shared__ int sp[CLV_MAX_NODES], st[CLV_MAX_NODES], path[CLV_MAX_NODES];
-  __shared__ int s_first[CLV_MAX_NODES], s_next[CLV_MAX_NODES];   // a node's first child, its next sibling (N: none)
-  __shared__ bool s_repeat[CLV_MAX_NODES];                         // an earlier sibling carries the same token
+  __shared__ int st[CLV_MAX_NODES], path[CLV_MAX_NODES];
+  __shared__ uint32_t s_kids[CLV_MAX_NODES][kMaskWords];           // a node's children
+  __shared__ int s_accepted[CLV_MAX_NODES];                        // the first of them that its test accepts (INT_MAX: none)
   __shared__ float su[CLV_MAX_NODES + 1], se[CLV_MAX_NODES], s_m[CLV_MAX_NODES], s_S[CLV_MAX_NODES];
-  __shared__ float s_slice[kThreads];
+  __shared__ float s_slice[kThreads], s_before_slice[kThreads];
   __shared__ float2 s_stats[kKept];   // every row's slices, if they are few
   __shared__ float s_before, s_target;
   __shared__ int s_found, s_bad, s_pick, s_lastv, s_len, s_cur;
-  static_assert(kThreads == 2 * CLV_MAX_NODES, "two threads per node");
+  static_assert(kThreads >= CLV_MAX_NODES, "a thread per node");
   const int b = blockIdx.x, tid = threadIdx.x, N = p.N;
   const int n_sl = p.pieces * (kPiece / kSlice);   // slices of a row
   const int64_t o = (int64_t)b * N;
@@ -179,24 +224,26 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
   float2 v[kRows];
   fetch(warp, v);   // under way before the tree, whose tokens the logits below wait for
   if (tid == 0) s_bad = (p.path_cap < 1) ? 1 : 0;
-  if (tid < CLV_MAX_NODES) s_first[tid] = N;
+  if (tid < CLV_MAX_NODES) {
+    s_accepted[tid] = INT_MAX;
+#pragma unroll
+    for (int w = 0; w < kMaskWords; ++w) s_kids[tid][w] = 0u;
+  }
   __syncthreads();
-  const int node = tid & (CLV_MAX_NODES - 1);
+  const int node = tid;
   int par = -1, tok = -1;
   if (node < N) {
     par = p.parent[o + node];
     tok = p.tokens[o + node];
-    if (tid < N) {
-      sp[node] = par;
-      st[node] = tok;
-      if ((node == 0) ? (par != -1) : (par < 0 || par >= node)) s_bad = 1;   // node 0 is the only root
-    }
+    st[node] = tok;
+    if ((node == 0) ? (par != -1) : (par < 0 || par >= node)) s_bad = 1;   // node 0 is the only root
   }
   for (int i = tid; i <= N; i += kThreads) su[i] = p.uniforms[(int64_t)b * (N + 1) + i];
   const bool child = node > 0 && node < N && par >= 0 && par < node;
+  if (child) atomicOr(&s_kids[par][node >> 5], 1u << (node & 31));
   const bool in_vocab = child && tok >= 0 && tok < p.vocab;
   uint32_t logit = 0x7FC00000u;   // NaN: no mass
-  if (tid < N && in_vocab) logit = (uint32_t)p.logits[(o + par) * p.ld + tok] << 16;
+  if (in_vocab) logit = (uint32_t)p.logits[(o + par) * p.ld + tok] << 16;
   // ---- every row's maximum and sum from its slices
   {
     for (int r0 = warp; r0 < N; r0 += kWarps * kRows) {
@@ -226,38 +273,31 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
   }
   __syncthreads();
   bool bad = s_bad != 0;
-  // ---- siblings: one thread of a node looks at those before it, the other at those behind; and the
-  //      weights 2^(x - m) of all nodes in their parents' rows
+  // ---- the weight 2^(x - m) of every node in its parent's row; a token that an earlier sibling carries was struck with
+  //      that sibling and carries nothing
   if (!bad && child) {
-    if (tid < N) {
-      bool repeat = false;
-      for (int d = 1; d < node; ++d) repeat |= (sp[d] == par && st[d] == tok);
-      s_repeat[node] = repeat;
-      atomicMin(&s_first[par], node);
-      const float l = __uint_as_float(logit) * p.k, m = s_m[par];
-      se[node] = (in_vocab && m > -INFINITY && l == l) ? ex2(l - m) : 0.f;
-    } else {
-      int next = N;
-      for (int d = N - 1; d > node; --d) next = sp[d] == par ? d : next;
-      s_next[node] = next;
-    }
+    bool repeat = false;
+    for_each_below(s_kids[par], node, [&](int d) { repeat |= st[d] == tok; });
+    const float l = __uint_as_float(logit) * p.k, m = s_m[par];
+    se[node] = (!repeat && in_vocab && m > -INFINITY && l == l) ? ex2(l - m) : 0.f;
   }
   __syncthreads();
-  if (tid == 0) {   // the accept chain: at every level the children in node order
+  // ---- every node's test, should the walk come to its parent: what is left of that row when its earlier siblings were
+  //      rejected, in node order
+  if (!bad && child) {
+    float rej = 0.f;
+    for_each_below(s_kids[par], node, [&](int d) { rej += se[d]; });
+    const float left = s_S[par] - rej;
+    const float a = (left > 0.f) ? se[node] / left : 0.f;
+    if (su[node] < a) atomicMin(&s_accepted[par], node);
+  }
+  __syncthreads();
+  if (tid == 0) {   // the accept chain
     int len = 1, cur = 0;
     path[0] = 0;
     while (!bad) {
-      const float S = s_S[cur];
-      float rej = 0.f;
-      int found = -1;
-      for (int c = s_first[cur]; c < N; c = s_next[c]) {
-        const float e = s_repeat[c] ? 0.f : se[c];   // a token that was struck already carries nothing
-        const float left = S - rej;
-        const float a = (left > 0.f) ? e / left : 0.f;
-        if (su[c] < a) { found = c; break; }
-        rej += e;
-      }
-      if (found < 0) break;
+      const int found = s_accepted[cur];
+      if (found == INT_MAX) break;
       if (len == p.path_cap || len == CLV_MAX_NODES) { bad = true; break; }
       path[len++] = found;
       cur = found;
@@ -281,32 +321,49 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
       const float2 sl = keep ? s_stats[cur * n_sl + j] : p.partial[(o + cur) * n_sl + j];
       float sum = (sl.x > -INFINITY && m > -INFINITY) ? sl.y * ex2(sl.x - m) : 0.f;
       const int v0 = j * kSlice, v1 = min(p.vocab, v0 + kSlice);
-      for (int c = s_first[cur]; c < N; c = s_next[c])
-        if (st[c] >= v0 && st[c] < v1 && !s_repeat[c]) sum -= se[c];   // a token carried by two siblings is struck once
+      for_each_below(s_kids[cur], N, [&](int c) {
+        if (st[c] >= v0 && st[c] < v1) sum -= se[c];   // (a token carried by two siblings is struck once)
+      });
       sum = fmaxf(sum, 0.f);
       if (j < kThreads) s_slice[j] = sum;
     }
     __syncthreads();
-    if (tid == 0) {
-      const int n_here = n_sl;   // at most one slice per thread: larger vocabularies are refused by the host
+    if (warp == 0) {
+      // the running sums in vocabulary order (one thread: the sums of all slices in this order are what is drawn from),
+      // then every lane looks at slices of its own for the one that the target falls into
       float total = 0.f;
-      for (int j = 0; j < n_here; ++j) total += s_slice[j];
+      if (lane == 0) {
+#pragma unroll 8
+        for (int j = 0; j < n_sl; ++j) {   // at most one slice per thread: larger vocabularies are refused by the host
+          s_before_slice[j] = total;
+          total += s_slice[j];
+        }
+      }
+      __syncwarp();
+      total = __shfl_sync(0xFFFFFFFFu, total, 0);
       const float target = su[N] * total;
-      float run = 0.f;
-      int pick = -1, last = -1;
-      for (int j = 0; j < n_here; ++j) {
-        if (s_slice[j] > 0.f) last = j;
-        if (pick < 0 && s_slice[j] > 0.f && run + s_slice[j] > target) { pick = j; s_before = run; }
-        if (pick < 0) run += s_slice[j];
+      int pick = INT_MAX, last = -1;
+      for (int j = lane; j < n_sl; j += 32) {
+        const float here = s_slice[j];
+        if (here > 0.f) {
+          last = j;
+          if (pick == INT_MAX && s_before_slice[j] + here > target) pick = j;
+        }
       }
-      if (pick < 0 && last >= 0) {   // rounding: the target lies at the very end
-        pick = last;
-        s_before = total - s_slice[last];
+      pick = __reduce_min_sync(0xFFFFFFFFu, pick);
+      last = __reduce_max_sync(0xFFFFFFFFu, last);
+      if (lane == 0) {
+        if (pick != INT_MAX) {
+          s_before = s_before_slice[pick];
+        } else {
+          pick = last;   // rounding: the target lies at the very end (-1: a row without any mass)
+          if (last >= 0) s_before = total - s_slice[last];
+        }
+        s_pick = pick;
+        s_target = target;
+        s_found = INT_MAX;   // first element of the slice whose running sum exceeds the target
+        s_lastv = -1;        // last element of the slice that carries any weight
       }
-      s_pick = pick;
-      s_target = target;
-      s_found = INT_MAX;   // first element of the slice whose running sum exceeds the target
-      s_lastv = -1;        // last element of the slice that carries any weight
     }
     __syncthreads();
     const int pick = s_pick;
@@ -325,8 +382,9 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
         for (int h = 0; h < 2; ++h)   // past the row's end: the last vector again (cut by index below)
           w[h] = ld_stream16(row + min(v_base + 8 * h, (q1 - 1) & ~7));
         uint32_t struck = 0;
-        for (int c = s_first[cur]; c < N; c = s_next[c])
+        for_each_below(s_kids[cur], N, [&](int c) {
           if (st[c] >= v_base && st[c] < v_base + kPerThread) struck |= 1u << (st[c] - v_base);
+        });
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const float x[8] = {bf16_lo(w[h].x), bf16_hi(w[h].x), bf16_lo(w[h].y), bf16_hi(w[h].y),

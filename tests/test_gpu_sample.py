@@ -108,6 +108,21 @@ def test_sample_slices_of_a_row_kept_or_fetched_again(clv, oracle, vocab, n_node
     compare(oracle, got, w.logits, vocab, w.parent, w.tokens, u, 1.0, w.path_cap, min_robust=1.0)
 
 
+@pytest.mark.parametrize("n_nodes", [31, 32, 33, 64, 65, 97, 128])
+def test_sample_siblings_at_the_edges_of_their_masks(clv, oracle, n_nodes):
+    # A node's children are bits of four words: stars and trees of few levels, whose siblings lie in all of them, with tokens that
+    # siblings share (struck once) and tokens outside the vocabulary.
+    B, vocab, ld = 24, 300, 304
+    rng = np.random.default_rng(n_nodes)
+    lg = W.f32_to_bf16_bits(rng.normal(0, 2, size=(B, n_nodes, ld)).astype(np.float32))
+    lg[:, :, vocab:] = 0x7F00
+    parent = np.array([[-1] + [0 if b % 3 == 0 else int(rng.integers(0, min(i, 1 + b % 5))) for i in range(1, n_nodes)] for b in range(B)], np.int32)
+    tokens = rng.integers(0, vocab + 20, size=(B, n_nodes)).astype(np.int32)
+    u = W.make_uniforms(B, n_nodes, seed=n_nodes)
+    got = run_gpu(clv, lg, vocab, parent, tokens, u, 1.0, 9)
+    compare(oracle, got, lg, vocab, parent, tokens, u, 1.0, 9)
+
+
 @pytest.mark.parametrize("temperature", [1.0, 0.6, 1.7])
 @pytest.mark.parametrize("vocab,n_nodes", [(64, 9), (1000, 20), (4099, 33), (8192, 10), (32000, 64), (32771, 12),
                                            (128256, 64)])   # around the edges of the 4096-logit slices and 32768-logit pieces
