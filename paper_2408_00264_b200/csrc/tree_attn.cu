@@ -152,7 +152,7 @@ struct Params {
   int splits;         // blocks along the key axis = cluster size
   float scale_log2;
   long long wait_limit;   // SM cycles a bounded wait may last
-  unsigned* tickets;      // per sequence: [2b] blocks behind their last wait, [2b+1] what went wrong; zero between calls
+  unsigned* tickets;      // per sequence: [2b] blocks whose roles have met, [2b+1] what went wrong; zero between calls
   int blocks_per_seq;
   int tile_nodes;         // whole nodes of a row tile
   Divisor by_splits, by_groups, by_kv_heads, by_group_heads;
