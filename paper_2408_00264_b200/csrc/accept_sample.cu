@@ -48,7 +48,13 @@ __device__ __forceinline__ float ex2(float x) {
 __device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
 
-// (m, s): s = sum of 2^(x - m) over the values seen so far, m their maximum (s = 0 while m = -inf)
+// A token's weight beside a maximum m: 2^(x k - m) in one rounding, as the statistics' packed form has it.  Wherever the same
+// logit is weighed the number is the same, whatever the compiler makes of a product and a difference: m is rounded to 2^-24
+// of itself, so a row's sum by one form and a weight by the other differ by that much of |x k| (T = 0.01 and a logit of 30:
+// 1.7e-4 of a token that is certain).
+__device__ __forceinline__ float weight(float x, float k, float m) { return ex2(fmaf(x, k, -m)); }
+
+// (m, s): s = sum of the weights beside m of the values seen so far, m their maximum (s = 0 while m = -inf)
 struct Stat {
   float m, s;
 };
@@ -146,8 +152,8 @@ __global__ void __launch_bounds__(kThreads, 6) softmax_stats_kernel(StatParams p
   {  // ragged end of the row: at most 7 scalars, taken by the warp whose slice holds them
     const int t0 = begin + 8 * nvec + lane;
     if (t0 < end && (t0 - begin) / kSlice == warp) {
-      const float x = __uint_as_float((uint32_t)base[t0] << 16) * p.k;
-      if (x > -INFINITY) { Stat one = {x, 1.f}; stat_merge(st, one); }
+      const float x = __uint_as_float((uint32_t)base[t0] << 16), m = x * p.k;
+      if (m > -INFINITY) { Stat one = {m, m < INFINITY ? weight(x, p.k, m) : 1.f}; stat_merge(st, one); }
     }
   }
 #pragma unroll
@@ -273,13 +279,13 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
   }
   __syncthreads();
   bool bad = s_bad != 0;
-  // ---- the weight 2^(x - m) of every node in its parent's row; a token that an earlier sibling carries was struck with
+  // ---- the weight of every node in its parent's row; a token that an earlier sibling carries was struck with
   //      that sibling and carries nothing
   if (!bad && child) {
     bool repeat = false;
     for_each_below(s_kids[par], node, [&](int d) { repeat |= st[d] == tok; });
-    const float l = __uint_as_float(logit) * p.k, m = s_m[par];
-    se[node] = (!repeat && in_vocab && m > -INFINITY && l == l) ? ex2(l - m) : 0.f;
+    const float x = __uint_as_float(logit), m = s_m[par];
+    se[node] = (!repeat && in_vocab && m > -INFINITY && x == x) ? weight(x, p.k, m) : 0.f;
   }
   __syncthreads();
   // ---- every node's test, should the walk come to its parent: what is left of that row when its earlier siblings were
@@ -391,9 +397,8 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
                               bf16_lo(w[h].z), bf16_hi(w[h].z), bf16_lo(w[h].w), bf16_hi(w[h].w)};
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const float l = x[j] * p.k;
-            const bool in = (v_base + 8 * h + j < q1) && !((struck >> (8 * h + j)) & 1u) && l == l && m > -INFINITY;
-            e[8 * h + j] = in ? ex2(l - m) : 0.f;
+            const bool in = (v_base + 8 * h + j < q1) && !((struck >> (8 * h + j)) & 1u) && x[j] == x[j] && m > -INFINITY;
+            e[8 * h + j] = in ? weight(x[j], p.k, m) : 0.f;
           }
         }
       }

@@ -154,6 +154,21 @@ def test_sample_low_temperature_is_the_greedy_walk(clv, oracle):
     assert np.array_equal(got[3], st)
 
 
+@pytest.mark.parametrize("temperature", [1.7, 1.0, 0.1, 1e-2, 1e-3, 1e-4])
+@pytest.mark.parametrize("vocab,at", [(4096, 0), (4096, 4095), (4099, 2500), (4099, 4098), (13, 3), (13, 12)])   # 4098 and 12: behind the last whole vector
+def test_sample_a_certain_token_is_certain(clv, vocab, at, temperature):
+    # All of a row's mass is one token's: its probability is 1 and above every uniform, whatever the rounding of logit / T.
+    # The row's sum and the token's weight come from different kernels and have to be the same number.
+    B, N = 256, 3
+    ld = (vocab + 7) // 8 * 8
+    lg = W.f32_to_bf16_bits(np.full((B, N, ld), -300, np.float32))
+    lg[:, :, at] = W.f32_to_bf16_bits(np.random.default_rng(vocab + at).uniform(15, 40, size=(B, N)).astype(np.float32))
+    parent, tokens = np.tile(np.array([-1, 0, 1], np.int32), (B, 1)), np.full((B, N), at, np.int32)
+    u = np.full((B, N + 1), 1 - 2.0 ** -24, np.float32)
+    alen, aidx, nxt, st = run_gpu(clv, lg, vocab, parent, tokens, u, temperature, N)
+    assert (st == 0).all() and (alen == 3).all() and (aidx == [0, 1, 2]).all() and (nxt == at).all()
+
+
 def test_sample_special_values_and_bad_trees(clv, oracle):
     vocab, N, ld = 50, 4, 56
     lg = np.zeros((4, N, ld), np.uint16)
