@@ -116,8 +116,8 @@ clv_status clv_workspace_init(void* workspace, size_t workspace_bytes, void* cud
  * status[b] = CLV_ERR_TREE if parent[b] is malformed, L_b < 0, L_b exceeds the cache capacity or
  * a needed block-table entry is outside [0, n_pages); CLV_ERR_TIMEOUT if a bounded on-chip wait of
  * one of the sequence's thread blocks ran out (about a second; never seen on a healthy device);
- * CLV_OK otherwise.  With a non-zero status that sequence's outputs are unspecified; the word is
- * written once per call, by the last thread block of the sequence to finish.
+ * CLV_OK otherwise.  With a non-zero status that sequence's outputs are unspecified.  The word
+ * is final when the call's work on the stream is (a failure late in the call corrects it).
  * max_ctx_len (host): an upper bound of ctx_len[], used only to choose the split count; the
  * result does not depend on it.
  * workspace: required (CLV_ERR_WORKSPACE), at least clv_workspace_bytes(); batch <= 32768.

@@ -51,6 +51,7 @@
 #include <math.h>
 
 #include "clv_internal.cuh"
+#include "seq_status.cuh"
 #include "tc_ptx.cuh"
 #include "tmem_access.cuh"
 
@@ -152,7 +153,7 @@ struct Params {
   int splits;         // blocks along the key axis = cluster size
   float scale_log2;
   long long wait_limit;   // SM cycles a bounded wait may last
-  unsigned* tickets;      // per sequence: [2b] blocks whose roles have met, [2b+1] what went wrong; zero between calls
+  unsigned* tickets;      // per sequence: the word of seq_status.cuh; zero between calls
   int blocks_per_seq;
   int tile_nodes;         // whole nodes of a row tile
   Divisor by_splits, by_groups, by_kv_heads, by_group_heads;
@@ -774,6 +775,23 @@ __device__ __forceinline__ void softmax(const Block<kRows2, kParts>& k, const Pa
   ms.ml[slot * BM + row] = make_float2(m_ref, l_run);
 }
 
+// The words of a sequence for seq_status.cuh.  The wait for its publisher outlasts the publisher's own.
+struct TallyWords {
+  unsigned long long* tally;
+  int32_t* status;
+  long long wait_limit, since = 0;
+  __device__ __forceinline__ unsigned long long add(unsigned long long v) { return atomicAdd(tally, v); }
+  __device__ __forceinline__ unsigned count() { return *reinterpret_cast<volatile unsigned*>(tally); }
+  __device__ __forceinline__ void put(int s) { *const_cast<volatile int32_t*>(status) = s; }
+  __device__ __forceinline__ void fence() { __threadfence(); }
+  __device__ __forceinline__ void correct() { atomicCAS(status, CLV_OK, CLV_ERR_TIMEOUT); }
+  __device__ __forceinline__ bool expired() {
+    const long long now = clock64();
+    if (since == 0) since = now;
+    return now - since > wait_limit + kWaitLimitCycles;
+  }
+};
+
 // ------------------------------------------------------------------------------------ kernel
 // kOneBlock: of the variants with several threads per row, the one for a block that is not part of a cluster
 // (the code of neither case lies in the other's way: 1 x 16 nodes x 512 keys took 0.13 us longer in one kernel).
@@ -896,29 +914,12 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     }
     __syncthreads();
   }
-  // status[b] is written by whichever block of the sequence leaves its roles last.  The sequence's two words in the
-  // workspace count the blocks that have, and with them, in the upper word, what went wrong until then (1: malformed
-  // input; 2 for each block in which a wait ran out); the holder of the last ticket has it all from one round trip, which
-  // ends while the rows are staged, and leaves both words zero for the next call.  A wait of the merge that runs out comes
-  // after the block's ticket: such a block waits for the words to be zero and corrects the status behind the holder's.
-  unsigned long long* const tally = reinterpret_cast<unsigned long long*>(p.tickets + 2 * b);
+  // The status is settled by one thread (see seq_status.cuh).  The block is counted here, so that the addition's round trip
+  // ends while the rows are staged; the waits of the merge come after it.
+  TallyWords words = {reinterpret_cast<unsigned long long*>(p.tickets + 2 * b), p.status + b, p.wait_limit};
   const bool clerk = tid == 32 * kWriter;
-  unsigned long long ticket = 0;
-  if (clerk) ticket = atomicAdd(tally, aborted ? (2ull << 32) + 1ull : 1ull) + (aborted ? 2ull << 32 : 0ull);
-  auto publish = [&]() {
-    if (!clerk || (unsigned)ticket != (unsigned)p.blocks_per_seq - 1) return;
-    const unsigned wrong = (unsigned)(ticket >> 32);
-    *const_cast<volatile int32_t*>(p.status + b) = (wrong & 1u) ? CLV_ERR_TREE : wrong ? CLV_ERR_TIMEOUT : CLV_OK;
-    __threadfence();
-    *const_cast<volatile unsigned long long*>(tally) = 0ull;
-  };
-  auto correct = [&](bool failed_late) {
-    if (!clerk || !failed_late) return;
-    const long long t0 = clock64();
-    while (*const_cast<volatile unsigned long long*>(tally) != 0ull && clock64() - t0 < kWaitLimitCycles) {}
-    __threadfence();
-    atomicCAS(p.status + b, CLV_OK, CLV_ERR_TIMEOUT);
-  };
+  unsigned long long found = 0;
+  if (clerk) found = add_block(words, aborted);
 
   // ---- merge.  Idle once all Q K^T of a block are done, which is when it arrives at the cluster
   //      barrier: the Q tiles (staging of the rows to be sent), and all ring stages but those of the
@@ -1088,7 +1089,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
     tmem_dealloc(tmem, kTmemCols);
   }
 
-  publish();
+  if (clerk) publish_if_last(words, found, (unsigned)p.blocks_per_seq);
   __syncwarp();
   if (alone) {
     if (tid == 0 && !failed) {
@@ -1101,7 +1102,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
       asm volatile("cp.async.bulk.commit_group;" ::: "memory");
       asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
     }
-    correct(failed && !aborted);
+    if (clerk && failed && !aborted) report_late(words, (unsigned)p.blocks_per_seq);
     return;
   }
 
@@ -1229,7 +1230,7 @@ __global__ void __launch_bounds__(kThreads, 1) tree_attn_kernel(const __grid_con
   }
   __syncwarp();
   if (clustered) cluster_wait();   // no block may leave while a copy still reads its shared memory
-  correct(failed && !aborted);
+  if (clerk && failed && !aborted) report_late(words, (unsigned)p.blocks_per_seq);
 }
 
 // ------------------------------------------------------------------------------------ host side

@@ -605,6 +605,30 @@ def test_attention_waits_that_run_out_anywhere_are_reported(clv, oracle, batch, 
     assert (32, True) in seen and (0, False) in seen
 
 
+def test_attention_waits_that_run_out_in_a_sequence_of_more_blocks_than_run_at_once(clv, oracle):
+    # 149 heads in clusters of two: 298 blocks of one sequence, 148 of them at a time, so that blocks whose waits run out
+    # late are gone before the last are counted.  Their failures must reach the status all the same, and promptly.
+    w = W.generate(W.small_config(batch=1, n_q_heads=149, n_kv_heads=149, ctx=6000, n_nodes=16, vocab=64, seed=W.BASE_SEED + 406))
+    st = make_step(w)
+    rows = np.array([[0, i, h] for h in range(149) for i in (0, 15)], np.int64)
+    ref = oracle.tree_attn(w.q, w.k_cache, w.v_cache, w.k_tree, w.v_tree, w.parent, w.ctx_len, w.scale, rows=rows)[0]
+    for limit in [32, 400, 800, 1300, 2000, 3000, 4000, 5000, 6000, 9000, 20000, 100000, 0]:
+        for _ in range(3):
+            st.out.fill_(float("nan"))
+            st.status.fill_(-7)
+            try:
+                clv.clv_test_set_wait_limit(limit)
+                st.tree_attn()
+                torch.cuda.synchronize()
+            finally:
+                clv.clv_test_set_wait_limit(0)
+            status = int(st.status[0, 0])
+            assert status in (clv.CLV_OK, clv.CLV_ERR_TIMEOUT) and (limit or status == clv.CLV_OK)
+            if status == clv.CLV_OK:
+                assert not torch.isnan(st.out).any()
+                assert_attn_close(bits(st.out)[rows[:, 0], rows[:, 1], rows[:, 2]], ref, limit)
+
+
 # ------------------------------------------------------------------ argmax
 @pytest.mark.parametrize("vocab,ld_pad", [(1, 0), (7, 0), (8, 8), (2047, 0), (2049, 16),
                                           (32000, 0), (50257, 8), (128256, 0)])
