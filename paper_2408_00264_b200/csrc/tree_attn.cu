@@ -125,6 +125,9 @@ constexpr uint32_t kMiscAt = 7 * kStage;   // either way: Q tiles + ring = 224 K
 constexpr uint32_t kSmem = kMiscAt + (uint32_t)sizeof(Misc);
 static_assert(Cfg<true, 1>::kQ + Cfg<true, 1>::NST == 7 && Cfg<false, 1>::kQ + Cfg<false, 1>::NST == 7 && kSmem <= 232448, "shared memory");
 
+// pieces of n >= 0 keys, up to the largest length there is (n + PG - 1 does not fit in an int for the last 63 of them)
+__host__ __device__ __forceinline__ int pieces_of(int n) { return (int)(((unsigned)n + (unsigned)(PG - 1)) / PG); }
+
 // n / d by a multiplication: m = ceil(2^32 / d), so the high word is n / d or one more.  (A division of
 // the language is some 40 instructions that a block runs once, from a cold instruction cache.)
 struct Divisor {
@@ -330,9 +333,9 @@ struct Block {
   // reads the tree's own rows only.  Tiles [0, t_plain) consist of two complete pieces of context.
   __device__ __forceinline__ void range(const Params& p, int len) {
     L = len;
-    len_bad = (L < 0) || (p.paged ? ((L + PG - 1) / PG > p.max_pages) : (L > p.cap_tokens));
-    p_cache = (!len_bad && L > 0) ? (L + PG - 1) / PG : 0;
-    p_total = p_cache + (N + PG - 1) / PG;
+    len_bad = (L < 0) || (p.paged ? (pieces_of(L) > p.max_pages) : (L > p.cap_tokens));
+    p_cache = len_bad ? 0 : pieces_of(L);
+    p_total = p_cache + pieces_of(N);
     pc_begin = (int)p.by_splits.divide((unsigned)split * (unsigned)p_total);
     pc_end = (int)p.by_splits.divide((unsigned)(split + 1) * (unsigned)p_total);
     T = (pc_end - pc_begin + 1) / 2;
@@ -386,9 +389,8 @@ constexpr int kAhead = 2;
 constexpr int kAheadFrom = 3;   // key tiles of a block, by the bound of the lengths: with fewer there is nothing to gain
 template <bool kRows2, int kParts>
 __device__ __forceinline__ void scout(const Block<kRows2, kParts>& k, const Maps& tm, const Params& p) {
-  const int most = p.paged ? p.max_pages * PG : p.cap_tokens;
-  const int len = max(0, min(ld_hint(p.ctx_len + k.b), most));
-  const int p_cache = (len + PG - 1) / PG, p_total = p_cache + (k.N + PG - 1) / PG;
+  const int len = max(0, ld_hint(p.ctx_len + k.b));
+  const int p_cache = p.paged ? min(pieces_of(len), p.max_pages) : pieces_of(min(len, p.cap_tokens)), p_total = p_cache + pieces_of(k.N);
   const int begin = (int)p.by_splits.divide((unsigned)k.split * (unsigned)p_total);
   const int end = min(min(p_cache, begin + 2 * kAhead), (int)p.by_splits.divide((unsigned)(k.split + 1) * (unsigned)p_total));
   for (int g = begin + k.lane; g < end; g += 32) {
@@ -1325,7 +1327,7 @@ AttnPlan make_plan(const clv_shape& s, int max_ctx_len, const int* clusters) {
   const int rows = s.n_nodes * G;
   const int parts = rows <= BM / 4 ? 4 : rows <= BM / 2 ? 2 : 1;
   const int tiles = (s.n_nodes + BM / G - 1) / (BM / G);   // row tiles of BM / G whole nodes
-  const int pieces = (max_ctx_len + PG - 1) / PG + (s.n_nodes + PG - 1) / PG;
+  const int pieces = pieces_of(max_ctx_len) + pieces_of(s.n_nodes);
   const int64_t units = (int64_t)s.batch * s.n_kv_heads;
   AttnPlan best = {false, parts, tiles, tiles, 1};
   double best_cost = 1e300;
@@ -1395,7 +1397,7 @@ cudaError_t launch_tree_attn(const clv_shape& s, const clv_kv_cache& c, const vo
   p.groups = plan.groups;
   p.splits = plan.splits;
   p.longest_first = (clusters * plan.splits > sm_count() && s.batch > 1 && s.batch <= 256) ? 1 : 0;
-  const int pieces = (max_ctx_len + PG - 1) / PG + (s.n_nodes + PG - 1) / PG;
+  const int pieces = pieces_of(max_ctx_len) + pieces_of(s.n_nodes);
   p.ask_ahead = plan.parts > 1 && !p.longest_first && pieces >= 2 * kAheadFrom * plan.splits ? 1 : 0;
   p.scale_log2 = scale * 1.4426950408889634f;
   p.wait_limit = wait_limit_cycles();

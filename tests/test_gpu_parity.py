@@ -248,6 +248,29 @@ def test_attention_flags_bad_sequences(clv, oracle):
 
 
 @pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("hq,hkv,n_nodes", [(4, 4, 16), (4, 4, 50), (8, 2, 32), (8, 2, 128)])
+def test_attention_flags_the_largest_lengths_there_are(clv, oracle, hq, hkv, n_nodes, paged):
+    # The number of a length's pages is worked out without adding to the length: the last 63 integers are refused like any
+    # other length beyond the table, by every variant, and as the bound of the lengths the largest integer is as good as any.
+    w = W.generate(W.small_config(batch=4, n_q_heads=hq, n_kv_heads=hkv, ctx=1200, n_nodes=n_nodes, paged=paged))
+    ref = oracle.tree_attn(w.q, w.k_cache, w.v_cache, w.k_tree, w.v_tree, w.parent, w.ctx_len, w.scale, block_table=w.block_table)[0]
+    most = 2 ** 31 - 1
+    st = make_step(w)
+    for bad in ([most, most - 62], [most - 63, most - 31], [-most - 1, most - 1]):
+        lens = w.ctx_len.copy()
+        lens[1], lens[2] = bad
+        st.ctx_len.copy_(torch.from_numpy(lens))
+        for bound in (1200, most):
+            st.out.fill_(float("nan"))
+            clv.clv_tree_attn(st.shape, st.cache, st.q, st.k_tree, st.v_tree, st.parent, st.ctx_len, bound, w.scale, st.out, st.lse,
+                              st.status[0], st.workspace)
+            torch.cuda.synchronize()
+            assert st.status[0].cpu().tolist() == [0, clv.CLV_ERR_TREE, clv.CLV_ERR_TREE, 0]
+            for b in (0, 3):
+                assert_attn_close(bits(st.out)[b], ref[b], "beside lengths of %s" % bad)
+
+
+@pytest.mark.parametrize("paged", [False, True])
 @pytest.mark.parametrize("n_nodes", [16, 50])
 def test_attention_asks_ahead_by_hints_that_are_wrong(clv, oracle, n_nodes, paged):
     # Key tiles are asked for into L2 by the lengths and pages as they stand ahead of the previous kernel's end (row tiles of up to
