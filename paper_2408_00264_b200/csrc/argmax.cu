@@ -13,7 +13,8 @@ namespace clv {
 namespace {
 
 constexpr int kUnroll = 8;  // 16-byte loads in flight per thread
-constexpr int kMaxCluster = 8;
+constexpr int kPieces = 6;                                   // of a row that a cluster shares
+constexpr int kOnePerSm = 226 * 1024;                        // shared memory that only one block of an SM can have
 constexpr int kPieceThreads = 256;                           // of blocks that meet through global memory
 constexpr int kMaxPiece = 2 * kUnroll * kPieceThreads * 8;   // logits of such a block
 constexpr int kMaxWholeRow = 1 << 26;                        // visits of a thread are numbered in 16 bits
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(kThreads, 2048 / kThreads) argmax_kernel(Param
   uint32_t value = ordered(best.v), index = (uint32_t)best.i;
   first_of_highest(value, index);
   if constexpr (kJoin == kByCluster) {
-    __shared__ uint2 s_pair[kMaxCluster * kWarps];
+    __shared__ uint2 s_pair[kPieces * kWarps];
     cluster_wait();   // every block of the row runs
     if (lane == 0) st_first_block(&s_pair[chunk * kWarps + (tid >> 5)], value, index);
     __syncwarp();
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(kThreads, 2048 / kThreads) argmax_kernel(Param
     value = 0u;
     index = 0xFFFFFFFFu;
 #pragma unroll
-    for (int c = 0; c < kMaxCluster * kWarps; c += 32)
+    for (int c = 0; c < kPieces * kWarps; c += 32)
       if (c + lane < p.chunks * kWarps) take_better(value, index, s_pair[c + lane]);
     first_of_highest(value, index);
   } else {
@@ -223,6 +224,24 @@ ArgmaxPlan argmax_plan(int rows, int vocab) {
 }
 
 namespace {
+// SMs that run a block each, of as much shared memory as there is, when all blocks are of clusters of kPieces
+cudaError_t sms_of_clusters(void (*kernel)(Params), int threads, int* sms) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kPieces;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(kPieces * sm_count()), 1, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = kOnePerSm;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+  *sms = n > 0 ? n * kPieces : kPieces;
+  return e;
+}
+
 template <int kThreads, Join kJoin>
 cudaError_t launch(const Params& p, int rows, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
@@ -230,13 +249,21 @@ cudaError_t launch(const Params& p, int rows, cudaStream_t stream) {
   cfg.blockDim = dim3(kThreads, 1, 1);
   // Small blocks that are launched early would pile up on the SMs that attention leaves idle (step of 1 x 64 nodes x 2048
   // keys and 32000 logits: 21.6 -> 21.0 us).  Larger ones need the L1 that this would take for their loads in flight.
+  // A cluster's SMs are of one GPC, so the share is one of the SMs that clusters can have (of all of them, 23-24, 47-49 and
+  // 72-74 rows had their last clusters wait for a wave: 24 x 128256 8.2 us, where 25 rows took 4.7).
   if (kJoin == kByCluster) {
-    cfg.dynamicSmemBytes = even_share_smem((int64_t)rows * p.chunks, 2048 / kThreads);
     static OncePerDevice once;
-    const cudaError_t e = run_once_per_device(once, [] {
-      return cudaFuncSetAttribute(argmax_kernel<kThreads, kJoin>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-    });
+    static int cluster_sms[kMaxDevices];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+      e = run_once_per_device(once, [&] {
+        cudaError_t set = cudaFuncSetAttribute(argmax_kernel<kThreads, kJoin>, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePerSm);
+        if (set == cudaSuccess && dev < kMaxDevices) set = sms_of_clusters(argmax_kernel<kThreads, kJoin>, kThreads, &cluster_sms[dev]);
+        return set;
+      });
     if (e != cudaSuccess) return e;
+    cfg.dynamicSmemBytes = even_share_smem((int64_t)rows * p.chunks, 2048 / kThreads, dev < kMaxDevices ? cluster_sms[dev] : sm_count());
   }
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -282,12 +309,11 @@ cudaError_t launch_argmax(const ArgmaxPlan& plan, const void* logits, int64_t ld
     if (plan.rows <= 4 * sms) return launch<512, kWholeRow>(p, plan.rows, stream);
     return launch<256, kWholeRow>(p, plan.rows, stream);
   }
-  if (2 * plan.rows > sms || vocab > kMaxCluster * kMaxPiece) {
+  if (2 * plan.rows > sms || vocab > 8 * kMaxPiece) {
     p.chunks = plan.chunks;
     p.chunk_elems = plan.chunk_elems;
     return launch<kPieceThreads, kByTickets>(p, plan.rows, stream);
   }
-  constexpr int kPieces = 6;
   p.chunk_elems = ((vocab + kPieces - 1) / kPieces + 7) & ~7;
   p.chunks = (vocab + p.chunk_elems - 1) / p.chunk_elems;
   return launch<256, kByCluster>(p, plan.rows, stream);

@@ -147,8 +147,9 @@ inline cudaError_t run_once_per_device(OncePerDevice& st, Fn fn) {
 // Dynamic shared memory with which no more blocks of a one-wave grid of small blocks fit on an SM than its
 // even share.  A grid that is launched while the previous kernel of the stream still runs would
 // otherwise pile up, as deep as its blocks go, on the few SMs that are free.  0: no limit needed.
-inline size_t even_share_smem(int64_t blocks, int natural_limit) {
-  const int64_t per_sm = (blocks + sm_count() - 1) / sm_count();
+// sms: those that the grid's blocks can have.
+inline size_t even_share_smem(int64_t blocks, int natural_limit, int sms = sm_count()) {
+  const int64_t per_sm = (blocks + sms - 1) / sms;
   if (per_sm >= natural_limit) return 0;
   constexpr int64_t kPerSm = 228 * 1024, kReserved = 1024, kStatic = 1024;   // the kernels' own is below kStatic
   return (size_t)(kPerSm / per_sm - kReserved - kStatic);

@@ -759,6 +759,37 @@ def test_argmax_at_the_edges_of_its_blocks(clv, oracle, rows, vocab):
     assert np.array_equal(ids.cpu().numpy().reshape(-1), ref)
 
 
+def argmax_time(clv, rows, vocab):
+    """Shortest time of a call among others, in ms, over logits that change from call to call."""
+    ld, calls = (vocab + 7) // 8 * 8, 24
+    sets = max(2, min(calls, (1 << 28) // (2 * rows * ld)))
+    lg = torch.randn(sets, rows, ld, dtype=torch.bfloat16, device="cuda")
+    shape = clv.make_shape(rows, 1, 1, 1, vocab, 1)
+    ids, ws = torch.zeros(rows, 1, dtype=torch.int32, device="cuda"), clv.new_workspace(shape, None, 0)
+    clv.clv_accept_argmax(shape, lg[0], ld, ids, ws)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for k in range(calls):
+            clv.clv_accept_argmax(shape, lg[k % sets], ld, ids, ws)
+    best = 1e9
+    for _ in range(9):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        g.replay()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) / calls)
+    return best
+
+
+@pytest.mark.parametrize("rows,others", [(22, 25), (23, 25), (24, 25), (47, 50), (48, 50), (49, 50), (72, 66), (74, 66)])
+def test_argmax_has_no_last_cluster_that_waits_for_a_wave(clv, rows, others):
+    # Clusters of six fill a GPU's parts only so far: a grid whose blocks were shared out evenly over all SMs took up to 1.7 times
+    # what a few rows more or less took.  The bound is what the rows' number explains and a quarter.
+    assert argmax_time(clv, rows, 128256) <= 1.25 * max(1.0, rows / others) * argmax_time(clv, others, 128256)
+
+
 # ------------------------------------------------------------------ walk and commit
 def test_walk_random_trees_and_errors(clv, oracle):
     rng = np.random.default_rng(5)
