@@ -2,7 +2,7 @@
 //
 // Pure HBM stream: every logit is read once with 16-byte loads that bypass L1.  With enough rows to cover the
 // machine a block takes a whole row; with fewer a row is cut into `chunks` pieces, one per block of a cluster,
-// whose (value, lowest index) pairs meet in the shared memory of the cluster's first block.  Very long rows in small
+// whose (value, lowest index) pairs meet in the shared memory of the cluster's first block.  Long rows in small
 // numbers are cut further, and the last block to arrive for a row takes the best of its pieces from global memory.
 // The result is independent of the cut and of block scheduling.
 #include <limits.h>
@@ -135,7 +135,13 @@ __global__ void __launch_bounds__(kThreads, 2048 / kThreads) argmax_kernel(Param
     i += 4 * kThreads;
   };
   if (i + 3 * kThreads < nvec) four(false);
-  if (i < nvec) four(true);
+  // (blocks through tickets take the same number of visits by all threads but in a row's last one: a single visit left
+  // is not worth the three it would be filled up to, 8 x 262144 5.7 -> 5.1)
+  if (kJoin == kByTickets && i + kThreads >= nvec) {
+    if (i < nvec) take_vec(trk, ld_stream16(vp + i), visit2);
+  } else if (i < nvec) {
+    four(true);
+  }
   // the thread's best of its 8 positions: visit k of this thread is vector tid + k * kThreads
   Best best = {-INFINITY, INT_MAX};
 #pragma unroll
@@ -248,22 +254,23 @@ cudaError_t launch(const Params& p, int rows, cudaStream_t stream) {
   cfg.gridDim = dim3((unsigned)((int64_t)rows * p.chunks), 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
   // Small blocks that are launched early would pile up on the SMs that attention leaves idle (step of 1 x 64 nodes x 2048
-  // keys and 32000 logits: 21.6 -> 21.0 us).  Larger ones need the L1 that this would take for their loads in flight.
-  // A cluster's SMs are of one GPC, so the share is one of the SMs that clusters can have (of all of them, 23-24, 47-49 and
-  // 72-74 rows had their last clusters wait for a wave: 24 x 128256 8.2 us, where 25 rows took 4.7).
-  if (kJoin == kByCluster) {
+  // keys: with 32000 logits, clusters, 21.6 -> 21.0 us; with 200000, tickets, 25.2 -> 24.2).  Larger ones need the L1 that this
+  // would take for their loads in flight.  A cluster's SMs are of one GPC, so its share is one of the SMs that clusters can
+  // have (of all of them, 23-24, 47-49 and 72-74 rows had their last clusters wait for a wave: 24 x 128256 8.2 us, where 25
+  // rows took 4.7).
+  if (kJoin == kByCluster || (kJoin == kByTickets && p.chunk_elems < kMaxPiece)) {
     static OncePerDevice once;
     static int cluster_sms[kMaxDevices];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
+    const bool by_cluster = kJoin == kByCluster && dev < kMaxDevices;
     if (e == cudaSuccess)
       e = run_once_per_device(once, [&] {
-        cudaError_t set = cudaFuncSetAttribute(argmax_kernel<kThreads, kJoin>, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePerSm);
-        if (set == cudaSuccess && dev < kMaxDevices) set = sms_of_clusters(argmax_kernel<kThreads, kJoin>, kThreads, &cluster_sms[dev]);
-        return set;
+        const cudaError_t set = cudaFuncSetAttribute(argmax_kernel<kThreads, kJoin>, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePerSm);
+        return set == cudaSuccess && by_cluster ? sms_of_clusters(argmax_kernel<kThreads, kJoin>, kThreads, &cluster_sms[dev]) : set;
       });
     if (e != cudaSuccess) return e;
-    cfg.dynamicSmemBytes = even_share_smem((int64_t)rows * p.chunks, 2048 / kThreads, dev < kMaxDevices ? cluster_sms[dev] : sm_count());
+    cfg.dynamicSmemBytes = even_share_smem((int64_t)rows * p.chunks, 2048 / kThreads, by_cluster ? cluster_sms[dev] : sm_count());
   }
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -278,9 +285,35 @@ cudaError_t launch(const Params& p, int rows, cudaStream_t stream) {
 }
 }  // namespace
 
+namespace {
+// Logits up to which six blocks are enough for one of a few rows, and up to which rows that leave up to half of the SMs idle
+// are not cut.  Back to back from a graph, cold, in us:
+//    rows x vocabulary   cluster of 6   1024 threads   tickets
+//       4 x 128256                4.4                      4.0   (a step of 1 x 4 nodes x 2048 keys: 17.7, 18.8)
+//      50 x 152064                6.1                      6.5
+//      74 x 153600                7.3                      7.5
+//      74 x 163840                8.7                      7.5
+//      32 x 200000                6.7                      6.1
+//       4 x 262144                6.8                      4.3
+//      75 x 180000                               8.1       9.7
+//     100 x 196608                               9.3      10.0
+//      80 x 200000                               9.3       8.7
+//      75 x 400000                              15.4      12.5
+//     111 x 400000                              17.4      18.9
+constexpr int kLongForClusters = 153600, kLongForHalfAWave = 196608;
+constexpr int kLongForTwo = 32768;   // logits from which an SM's two rows are taken by 1024 threads each, rather than 512
+
+// Which way a call takes.
+Join argmax_join(int rows, int vocab) {
+  const int sms = sm_count();
+  if (2 * rows <= sms) return vocab <= kLongForClusters ? kByCluster : kByTickets;
+  return vocab <= (4 * rows < 3 * sms ? kLongForHalfAWave : kMaxWholeRow) ? kWholeRow : kByTickets;
+}
+}  // namespace
+
 // Rows that cover the SMs at least half are not cut, and their blocks are as large as lets one wave take them all;
-// fewer rows are shared by clusters of six blocks (of a row's best cut into 1, 2, 3, 4, 6, 8, six lost least), up to
-// rows for which eight blocks would be too few.  Back to back from a graph, cold, in us (before: all through tickets):
+// fewer rows are shared by clusters of six blocks (of a row's best cut into 1, 2, 3, 4, 6, 8, six lost least); long rows that
+// would leave much of the GPU idle are cut finely and go through tickets.  Back to back from a graph, cold, in us (before: all through tickets):
 //   rows x vocabulary     before   1024 threads    512    256   cluster of 6   taken
 //    16 x 32000              3.6            2.6    2.4    2.8            2.3   cluster
 //    64 x 32000              5.5            2.7    3.1    4.2            2.7   cluster
@@ -303,16 +336,18 @@ cudaError_t launch_argmax(const ArgmaxPlan& plan, const void* logits, int64_t ld
   p.ids = ids;
   p.tickets = tickets;
   p.partial = static_cast<uint2*>(scratch);
-  const int sms = sm_count();
-  if (2 * plan.rows > sms && vocab <= kMaxWholeRow) {
-    if (plan.rows <= sms || (plan.rows <= 2 * sms && vocab > kMaxPiece)) return launch<1024, kWholeRow>(p, plan.rows, stream);
-    if (plan.rows <= 4 * sms) return launch<512, kWholeRow>(p, plan.rows, stream);
-    return launch<256, kWholeRow>(p, plan.rows, stream);
-  }
-  if (2 * plan.rows > sms || vocab > 8 * kMaxPiece) {
-    p.chunks = plan.chunks;
-    p.chunk_elems = plan.chunk_elems;
-    return launch<kPieceThreads, kByTickets>(p, plan.rows, stream);
+  switch (argmax_join(plan.rows, vocab)) {
+    case kWholeRow: {
+      const int sms = sm_count();
+      if (plan.rows <= sms || (plan.rows <= 2 * sms && vocab > kLongForTwo)) return launch<1024, kWholeRow>(p, plan.rows, stream);
+      if (plan.rows <= 4 * sms) return launch<512, kWholeRow>(p, plan.rows, stream);
+      return launch<256, kWholeRow>(p, plan.rows, stream);
+    }
+    case kByTickets:
+      p.chunks = plan.chunks;
+      p.chunk_elems = plan.chunk_elems;
+      return launch<kPieceThreads, kByTickets>(p, plan.rows, stream);
+    case kByCluster: break;
   }
   p.chunk_elems = ((vocab + kPieces - 1) / kPieces + 7) & ~7;
   p.chunks = (vocab + p.chunk_elems - 1) / p.chunk_elems;

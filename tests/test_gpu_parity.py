@@ -736,7 +736,7 @@ def test_argmax_cuts_ties_and_ragged_rows(clv, oracle, rows_b, rows_n, vocab):
         ids.fill_(-5)
 
 
-@pytest.mark.parametrize("rows,vocab", [(1, 262144), (1, 262153), (3, 100003), (74, 2051), (75, 2051), (148, 4100), (149, 32768), (149, 32776),
+@pytest.mark.parametrize("rows,vocab", [(1, 262144), (1, 262153), (74, 153600), (74, 153601), (75, 196608), (110, 196615), (111, 196609), (3, 100003), (74, 2051), (75, 2051), (148, 4100), (149, 32768), (149, 32776),
                                         (296, 32769), (297, 8195), (592, 6147), (593, 6147), (600, 8193)])
 def test_argmax_at_the_edges_of_its_blocks(clv, oracle, rows, vocab):
     # How a row is shared depends on rows and vocabulary (148 SMs): both sides of every line, with remainders of the
@@ -788,6 +788,12 @@ def test_argmax_has_no_last_cluster_that_waits_for_a_wave(clv, rows, others):
     # Clusters of six fill a GPU's parts only so far: a grid whose blocks were shared out evenly over all SMs took up to 1.7 times
     # what a few rows more or less took.  The bound is what the rows' number explains and a quarter.
     assert argmax_time(clv, rows, 128256) <= 1.25 * max(1.0, rows / others) * argmax_time(clv, others, 128256)
+
+
+@pytest.mark.parametrize("rows,vocab,other_rows,other_vocab", [(4, 200000, 4, 262152), (25, 262144, 25, 262152), (75, 1 << 20, 74, 1 << 20)])
+def test_argmax_takes_no_longer_for_fewer_logits(clv, rows, vocab, other_rows, other_vocab):
+    # a few long rows are cut finely enough to fill the GPU: whole rows and clusters of six left half of it idle (1.2 to 1.4 times)
+    assert argmax_time(clv, rows, vocab) <= 1.1 * argmax_time(clv, other_rows, other_vocab)
 
 
 # ------------------------------------------------------------------ walk and commit
