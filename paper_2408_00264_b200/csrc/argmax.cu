@@ -390,8 +390,9 @@ cudaError_t launch_argmax_static(const void* logits, int64_t ld, int rows, int v
   }
   unsigned char* base = g_static_ptr[dev];
   const ArgmaxPlan plan = argmax_plan(rows, vocab);
-  if (plan.chunks > 1) {
-    // the counters must start at zero whatever an earlier (possibly aborted) call left behind
+  if (argmax_join(rows, vocab) == kByTickets) {
+    // the counters must start at zero whatever an earlier (possibly aborted) call left behind (without the fill
+    // 64 rows of 128256 that stay in L2 take 3.5 us instead of 7.4)
     e = cudaMemsetAsync(base, 0, sizeof(unsigned) * (size_t)rows, stream);
     if (e != cudaSuccess) return e;
   }

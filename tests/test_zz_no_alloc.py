@@ -91,9 +91,25 @@ def test_noalloc_allocates_nothing(clv):
     assert free1 == free0
 
 
+@pytest.mark.parametrize("rows,vocab,nodes", [(1, 2048, 1), (16, 32000, 1), (74, 128256, 1), (200, 50257, 1), (4, 262144, 2), (75, 400000, 2)])
+def test_noalloc_clears_its_counters_only_where_they_are_used(clv, rows, vocab, nodes):
+    # the nodes of a recorded call: a launch, and a fill ahead of it if a row's pieces meet through the counters
+    from cuda.bindings import runtime
+    shape, ids = clv.make_shape(rows, 1, 1, 1, vocab, 1), torch.zeros(rows, 1, dtype=torch.int32, device="cuda")
+    ld = (vocab + 7) // 8 * 8
+    d = torch.zeros(rows, ld, dtype=torch.bfloat16, device="cuda")
+    clv.clv_accept_argmax_noalloc(shape, d, ld, ids)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        clv.clv_accept_argmax_noalloc(shape, d, ld, ids)
+    err, _, n = runtime.cudaGraphGetNodes(runtime.cudaGraph_t(init_value=g.raw_cuda_graph()))
+    assert int(err) == 0 and n == nodes
+
+
 def test_noalloc_call_can_be_captured_in_a_graph(clv, oracle):
-    # after the first call on the device (which looks up the array's address) a call is a clearing
-    # of the counters and a launch on the caller's stream: both can be recorded and replayed
+    # after the first call on the device (which looks up the array's address) a call is a launch on the caller's stream, with
+    # a clearing of the counters ahead of it where they are used: both can be recorded and replayed
     vocab, rows = 5000, 24
     lg, ld = _logits(rows, vocab, seed=9)
     d = torch.from_numpy(lg.view(np.int16)).cuda()
