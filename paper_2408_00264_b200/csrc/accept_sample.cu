@@ -472,6 +472,8 @@ cudaError_t launch_accept_sample(const clv_shape& s, const void* logits, int64_t
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((int64_t)rows * a.pieces), 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
+  // (up to eight blocks per SM, of which registers let six run: the others do better behind an even share all the same, 7 x 128
+  // rows of 32000 24.1 us instead of 27.9, 4 x 64 of 128256 22.8 instead of 23.6)
   cfg.dynamicSmemBytes = even_share_smem((int64_t)rows * a.pieces, 2048 / kThreads);
   cfg.stream = stream;
   cfg.attrs = attr;

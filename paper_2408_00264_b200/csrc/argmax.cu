@@ -301,7 +301,9 @@ namespace {
 //      75 x 400000                              15.4      12.5
 //     111 x 400000                              17.4      18.9
 constexpr int kLongForClusters = 153600, kLongForHalfAWave = 196608;
-constexpr int kLongForTwo = 32768;   // logits from which an SM's two rows are taken by 1024 threads each, rather than 512
+// Logits from which an SM's two rows are taken by 1024 threads each, rather than 512: 180 rows of 24000 4.4 us (512: 4.0), of
+// 40000 6.0 (5.1), of 50257 6.2 (5.9), of 64000 6.2 (6.6), of 128256 9.4 (10.8); 149 and 296 rows likewise.
+constexpr int kLongForTwo = 57344;
 
 // Which way a call takes.
 Join argmax_join(int rows, int vocab) {

@@ -736,7 +736,7 @@ def test_argmax_cuts_ties_and_ragged_rows(clv, oracle, rows_b, rows_n, vocab):
         ids.fill_(-5)
 
 
-@pytest.mark.parametrize("rows,vocab", [(1, 262144), (1, 262153), (74, 153600), (74, 153601), (75, 196608), (110, 196615), (111, 196609), (3, 100003), (74, 2051), (75, 2051), (148, 4100), (149, 32768), (149, 32776),
+@pytest.mark.parametrize("rows,vocab", [(1, 262144), (1, 262153), (74, 153600), (74, 153601), (75, 196608), (110, 196615), (111, 196609), (3, 100003), (74, 2051), (75, 2051), (148, 4100), (149, 32768), (149, 32776), (149, 57344), (296, 57345),
                                         (296, 32769), (297, 8195), (592, 6147), (593, 6147), (600, 8193)])
 def test_argmax_at_the_edges_of_its_blocks(clv, oracle, rows, vocab):
     # How a row is shared depends on rows and vocabulary (148 SMs): both sides of every line, with remainders of the
