@@ -120,14 +120,15 @@ __device__ __forceinline__ void stat_take_batch(Stat& st, uint4 (&w)[kUnroll], f
 struct StatParams {
   const uint16_t* logits;
   int64_t ld;
-  int vocab, pieces;
+  int vocab, pieces, rows;
+  int rows_first;    // all rows' first pieces, then all second ones
   float k;           // log2(e) / T
   float2* partial;   // [rows][pieces * 8]: one (maximum, sum) per slice
 };
 
 __global__ void __launch_bounds__(kThreads, 6) softmax_stats_kernel(StatParams p) {
-  const int row = blockIdx.x / p.pieces;
-  const int piece = blockIdx.x - row * p.pieces;
+  const int row = p.rows_first ? blockIdx.x % p.rows : blockIdx.x / p.pieces;
+  const int piece = p.rows_first ? blockIdx.x / p.rows : blockIdx.x - row * p.pieces;
   const int begin = piece * kPiece;
   const int end = min(p.vocab, begin + kPiece);
   const uint16_t* base = p.logits + (int64_t)row * p.ld;
@@ -464,6 +465,13 @@ cudaError_t launch_accept_sample(const clv_shape& s, const void* logits, int64_t
   a.ld = ld;
   a.vocab = s.vocab;
   a.pieces = sample_pieces(s.vocab);
+  a.rows = rows;
+  // A row's last piece may be short.  If the pieces' number is even, as the SMs' is, blocks in the rows' order give the short
+  // ones to the same SMs time and again (7 x 120 rows of 33000 27.8 us, by pieces 23.4; 4 x 110 of 33000 22.9, 20.1, of 50257
+  // 25.1, 23.7; 1 x 128 of 100000 18.7, 17.8).  Otherwise rows stay together (16 x 64 of 128256 53.2, by pieces 53.6; 10 x 90 of
+  // 70000 36.8, 37.5), and so they do where an SM has up to three blocks (5 x 36 of 50257 14.1, 14.6).
+  const int last_piece = s.vocab - (a.pieces - 1) * kPiece;
+  a.rows_first = a.pieces % 2 == 0 && 4 * last_piece < 3 * kPiece && (int64_t)rows * a.pieces > 3 * sm_count();
   a.k = k;
   a.partial = static_cast<float2*>(scratch);
   cudaLaunchAttribute attr[1];

@@ -108,6 +108,19 @@ def test_sample_slices_of_a_row_kept_or_fetched_again(clv, oracle, vocab, n_node
     compare(oracle, got, w.logits, vocab, w.parent, w.tokens, u, 1.0, w.path_cap, min_robust=1.0)
 
 
+@pytest.mark.parametrize("batch,n_nodes,vocab", [(2, 111, 40000), (3, 74, 40000), (2, 112, 40000), (3, 75, 40005), (2, 128, 100003), (2, 128, 57344)])
+def test_sample_blocks_by_rows_and_by_pieces(clv, oracle, batch, n_nodes, vocab):
+    # the statistics' blocks in the rows' order or the pieces': on both sides of 444 blocks (148 SMs), short and long last pieces
+    w = W.generate(W.small_config(batch=batch, n_nodes=n_nodes, vocab=vocab, seed=W.BASE_SEED + vocab + n_nodes))
+    lift = W.f32_to_bf16_bits(np.float32([np.log(vocab) + 1.0]))[0]
+    ids = oracle.argmax(w.logits, vocab)
+    bi, ni = np.meshgrid(np.arange(batch), np.arange(n_nodes), indexing="ij")
+    w.logits[bi, ni, ids] = lift
+    u = W.make_uniforms(batch, n_nodes, seed=vocab)
+    compare(oracle, run_gpu(clv, w.logits, vocab, w.parent, w.tokens, u, 1.0, w.path_cap), w.logits, vocab, w.parent, w.tokens, u, 1.0,
+            w.path_cap, min_robust=1.0)
+
+
 @pytest.mark.parametrize("n_nodes", [31, 32, 33, 64, 65, 97, 128])
 def test_sample_siblings_at_the_edges_of_their_masks(clv, oracle, n_nodes):
     # A node's children are bits of four words: stars and trees of few levels, whose siblings lie in all of them, with tokens that
