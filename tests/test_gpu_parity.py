@@ -308,6 +308,45 @@ def test_attention_asks_ahead_by_hints_that_are_wrong(clv, oracle, n_nodes, page
 
 
 @pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("n_nodes", [16, 50])
+def test_attention_asks_ahead_by_hints_of_other_tiles(clv, oracle, n_nodes, paged):
+    # The kernel in front of attention writes the lengths, or the block table: what stands there until then is a length pages and
+    # splits away (or none), pages of other sequences or none.  A commit of empty paths writes its input's lengths to another
+    # array and lets the next kernel be set up meanwhile, so attention's hints are the old words.
+    w = W.generate(W.small_config(batch=4, n_q_heads=4, n_kv_heads=4, ctx=4000, n_nodes=n_nodes, paged=paged))
+    st = make_step(w)
+    w.ctx_len[:] = [191, 1281, 4000, 2048]
+    ref = oracle.tree_attn(w.q, w.k_cache, w.v_cache, w.k_tree, w.v_tree, w.parent, w.ctx_len, w.scale, block_table=w.block_table)[0]
+
+    def writer(words, out):   # a commit that leaves `words` in `out`
+        n = words.size
+        src, zero = torch.from_numpy(np.ascontiguousarray(words.reshape(-1))).cuda(), torch.zeros(n, 1, dtype=torch.int32, device="cuda")
+        tree, k, v = (torch.zeros(n, 1, 1, 128, dtype=torch.bfloat16, device="cuda") for _ in range(3))
+        shape, status = clv.make_shape(n, 1, 1, 1, 1, 1), torch.zeros(n, dtype=torch.int32, device="cuda")
+        return lambda: clv.clv_kv_commit(shape, clv.make_cache(k, v), tree, tree, zero, zero, src, out, status)
+
+    real = {"lengths": (w.ctx_len, st.ctx_len)}
+    stale = {"lengths": [[4000, 1, 0, 3841], [0, 4000, 63, 4000], [-1, 2 ** 31 - 1, 1 << 30, 65]]}
+    if paged:
+        real["pages"] = (w.block_table, st.block_table)
+        stale["pages"] = [np.roll(w.block_table, 1, axis=0), np.full_like(w.block_table, -1), np.full_like(w.block_table, w.n_pages),
+                          w.block_table[:, ::-1]]
+    put = {name: writer(words.astype(np.int32), out) for name, (words, out) in real.items()}
+    for last in real:
+        for old in stale[last]:
+            for name, (words, out) in real.items():
+                out.copy_(torch.from_numpy(np.ascontiguousarray(words)))
+            real[last][1].copy_(torch.from_numpy(np.ascontiguousarray(np.int32(old))))
+            st.out.fill_(float("nan"))
+            put[last]()
+            st.tree_attn()
+            torch.cuda.synchronize()
+            assert st.status[0].cpu().tolist() == [0, 0, 0, 0]
+            assert np.array_equal(st.ctx_len.cpu().numpy(), w.ctx_len)
+            assert_attn_close(bits(st.out), ref, "%s of %s" % (last, old))
+
+
+@pytest.mark.parametrize("paged", [False, True])
 def test_attention_units_of_many_row_tiles(clv, oracle, paged):
     # four row tiles per (sequence, kv head) (GQA 4 x 128 nodes = 512 rows): such units are worked
     # by blocks of two row tiles; ragged contexts, one of them shorter than a key tile, key splits
