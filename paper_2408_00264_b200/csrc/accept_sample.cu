@@ -52,7 +52,21 @@ __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u 
 // logit is weighed the number is the same, whatever the compiler makes of a product and a difference: m is rounded to 2^-24
 // of itself, so a row's sum by one form and a weight by the other differ by that much of |x k| (T = 0.01 and a logit of 30:
 // 1.7e-4 of a token that is certain).
-__device__ __forceinline__ float weight(float x, float k, float m) { return ex2(fmaf(x, k, -m)); }
+//
+// The rounding of m alone is up to 2^-24 |m|, which must not become a weight of its own: a slice of masked logits (-1e30) had
+// weights of 2^(+-1e23), and infinity beside a rescale by 0 made the whole row's sum NaN.  From 2^20 on k and m are scaled by the
+// power of two that brings m to [2^20, 2^21): an equal logit's weight stays within 2^(+-1/16), and any other bf16 logit, at
+// least 2^-8 |m| below, has none either way.
+struct Exponent {
+  float k, m;
+  __device__ __forceinline__ float weight(float x) const { return ex2(fmaf(x, k, -m)); }
+};
+__device__ __forceinline__ Exponent exponent_of(float k, float m) {
+  const uint32_t e = (__float_as_uint(m) >> 23) & 255u;
+  if (e < 127u + 20u || e == 255u) return {k, m};   // 255: infinite
+  const float scale = __uint_as_float((2u * 127u + 20u - e) << 23);
+  return {k * scale, m * scale};
+}
 
 // (m, s): s = sum of the weights beside m of the values seen so far, m their maximum (s = 0 while m = -inf)
 struct Stat {
@@ -102,7 +116,8 @@ __device__ __forceinline__ void stat_take_batch(Stat& st, uint4 (&w)[kUnroll], f
   const float mx = fmaxf(__low2float(t), __high2float(t)) * k;
   if (!(mx > -INFINITY)) return;   // nothing but -inf (or NaN): no mass
   if (mx > st.m) { st.s *= ex2(st.m - mx); st.m = mx; }
-  const unsigned long long kk = pack2(k, k), mm = pack2(-st.m, -st.m);
+  const Exponent e = exponent_of(k, st.m);
+  const unsigned long long kk = pack2(e.k, e.k), mm = pack2(-e.m, -e.m);
   unsigned long long acc[2] = {0ull, 0ull};
 #pragma unroll
   for (int u = 0; u < kUnroll; ++u) {
@@ -154,7 +169,7 @@ __global__ void __launch_bounds__(kThreads, 6) softmax_stats_kernel(StatParams p
     const int t0 = begin + 8 * nvec + lane;
     if (t0 < end && (t0 - begin) / kSlice == warp) {
       const float x = __uint_as_float((uint32_t)base[t0] << 16), m = x * p.k;
-      if (m > -INFINITY) { Stat one = {m, m < INFINITY ? weight(x, p.k, m) : 1.f}; stat_merge(st, one); }
+      if (m > -INFINITY) { Stat one = {m, m < INFINITY ? exponent_of(p.k, m).weight(x) : 1.f}; stat_merge(st, one); }
     }
   }
 #pragma unroll
@@ -286,7 +301,7 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
     bool repeat = false;
     for_each_below(s_kids[par], node, [&](int d) { repeat |= st[d] == tok; });
     const float x = __uint_as_float(logit), m = s_m[par];
-    se[node] = (!repeat && in_vocab && m > -INFINITY && x == x) ? weight(x, p.k, m) : 0.f;
+    se[node] = (!repeat && in_vocab && m > -INFINITY && x == x) ? exponent_of(p.k, m).weight(x) : 0.f;
   }
   __syncthreads();
   // ---- every node's test, should the walk come to its parent: what is left of that row when its earlier siblings were
@@ -388,6 +403,7 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
 #pragma unroll
         for (int h = 0; h < 2; ++h)   // past the row's end: the last vector again (cut by index below)
           w[h] = ld_stream16(row + min(v_base + 8 * h, (q1 - 1) & ~7));
+        const Exponent ex = exponent_of(p.k, m);   // (once: 16 times it took 0.4 us)
         uint32_t struck = 0;
         for_each_below(s_kids[cur], N, [&](int c) {
           if (st[c] >= v_base && st[c] < v_base + kPerThread) struck |= 1u << (st[c] - v_base);
@@ -399,7 +415,7 @@ __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const bool in = (v_base + 8 * h + j < q1) && !((struck >> (8 * h + j)) & 1u) && x[j] == x[j] && m > -INFINITY;
-            e[8 * h + j] = in ? weight(x[j], p.k, m) : 0.f;
+            e[8 * h + j] = in ? ex.weight(x[j]) : 0.f;
           }
         }
       }

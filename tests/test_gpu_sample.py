@@ -182,6 +182,42 @@ def test_sample_a_certain_token_is_certain(clv, vocab, at, temperature):
     assert (st == 0).all() and (alen == 3).all() and (aidx == [0, 1, 2]).all() and (nxt == at).all()
 
 
+@pytest.mark.parametrize("mask,temperature", [(-1e4, 1.0), (-1e9, 0.8), (-1e10, 0.8), (-3e10, 1.0), (-1e20, 1.0), (-1e20, 1.7), (-1e30, 1.0), (-1e30, 1.7),
+                                              (-3.3895e38, 1.0), (-3.3895e38, 1.7), (-3.3895e38, 2.0), (-3.3895e38, 100.0), (-np.inf, 0.8)])
+def test_sample_masked_logits(clv, oracle, mask, temperature):
+    # All logits but a few are a mask's value, among them whole slices of 4096 and the scalars behind the last whole vector: they
+    # carry no mass beside the others, and where a row holds nothing else, they share it evenly.
+    B, N, vocab = 64, 6, 3 * 4096 + 5
+    rng = np.random.default_rng(17)
+    lg = W.f32_to_bf16_bits(np.full((B, N, vocab + 3), mask, np.float32))
+    kept = np.sort(4096 + rng.permutation(4096)[:5])
+    lg[:, :, kept] = W.f32_to_bf16_bits(rng.normal(0, 1.3, size=(B, N, 5)).astype(np.float32))
+    parent = np.tile(np.array([-1, 0, 0, 1, 1, 2], np.int32), (B, 1))
+    tokens = np.tile(kept[[0, 1, 3, 0, 4, 2]].astype(np.int32), (B, 1))
+    if 1.4427 * abs(mask) / temperature < 3.4e38:
+        lg[:8, 1] = lg[0, 0, 0]
+    u = W.make_uniforms(B, N, seed=23)
+    alen = compare(oracle, run_gpu(clv, lg, vocab, parent, tokens, u, temperature, N), lg, vocab, parent, tokens, u, temperature, N)
+    assert alen.max() == 3
+
+
+@pytest.mark.parametrize("temperature", [1e-5, 1e-6, 1e-7, 1e-8, 1e-10, 1e-20, 1e-36])
+@pytest.mark.parametrize("top", [1, 2, 3])   # tokens that share the highest logit
+def test_sample_temperatures_near_zero(clv, oracle, temperature, top):
+    # Only the highest logit counts, wherever logit / T is finite: a token is certain, or has an even share beside its equals (in
+    # another slice, behind the last whole vector).
+    B, N, vocab = 256, 3, 4096 + 3
+    lg = W.f32_to_bf16_bits(np.random.default_rng(5).normal(0, 3, size=(B, N, vocab + 5)).astype(np.float32))
+    best = W.f32_to_bf16_bits(np.random.default_rng(6).uniform(15, 40, size=(B, N)).astype(np.float32))
+    for at in [7, 4098, 2000][:top]:
+        lg[:, :, at] = best
+    parent, tokens = np.tile(np.array([-1, 0, 1], np.int32), (B, 1)), np.full((B, N), 7, np.int32)
+    u = W.make_uniforms(B, N, seed=29)
+    got = run_gpu(clv, lg, vocab, parent, tokens, u, temperature, N)
+    compare(oracle, got, lg, vocab, parent, tokens, u, temperature, N)
+    assert (got[3] == 0).all() and np.isin(got[2], [7, 4098, 2000][:top]).all() and (top > 1 or (got[0] == 3).all())
+
+
 def test_sample_special_values_and_bad_trees(clv, oracle):
     vocab, N, ld = 50, 4, 56
     lg = np.zeros((4, N, ld), np.uint16)
