@@ -213,11 +213,11 @@ __device__ __forceinline__ void for_each_below(const uint32_t (&mask)[kMaskWords
 
 // One block per sequence.  What bounds it is the number of dependent round trips to memory, so everything
 // that any level of the walk may need is fetched at once: every row's statistics, and every node's
-// logit in its parent's row.  Siblings are bits of their parent's mask; every node's test is made by a thread of its own
-// ahead of the walk, which is then one load per level (one thread that tested and walked took 1.2 us for 27 nodes, 1.8 for
-// 109; now 0.3 and 0.4).
-// (statistics and walk, 5 sequences of 27 nodes, 50257 logits: 16.8 -> 12.8 us; 6 of 109 nodes: 42 -> 20), the
-// statistics ahead of the tree that the logits' addresses come from, and kept for the draw (the whole step 35.0 -> 34.7).
+// logit in its parent's row (statistics and walk, 5 sequences of 27 nodes, 50257 logits: 16.8 -> 12.8 us; 6 of 109 nodes:
+// 42 -> 20).  The statistics are asked for ahead of the tree, from which the logits' addresses come, and kept for the
+// draw (the whole step 35.0 -> 34.7).  Siblings are bits of their parent's mask; every node's test is made by a thread of its
+// own ahead of the walk, which is then one load per level (one thread that tested and walked took 1.2 us for 27 nodes, 1.8
+// for 109; now 0.3 and 0.4).
 __global__ void __launch_bounds__(kThreads) sample_walk_kernel(WalkParams p) {
   __shared__ int st[CLV_MAX_NODES], path[CLV_MAX_NODES];
   __shared__ uint32_t s_kids[CLV_MAX_NODES][kMaskWords];           // a node's children

@@ -12,7 +12,7 @@
 namespace clv {
 namespace {
 
-constexpr int kUnroll = 8;  // 16-byte loads in flight per thread
+constexpr int kUnroll = 8;  // 16-byte loads of a batch (the results of about four at a time fit beside the maxima in 32 registers)
 constexpr int kPieces = 6;                                   // of a row that a cluster shares
 constexpr int kOnePerSm = 226 * 1024;                        // shared memory that only one block of an SM can have
 constexpr int kPieceThreads = 256;                           // of blocks that meet through global memory

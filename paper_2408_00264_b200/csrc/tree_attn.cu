@@ -66,8 +66,7 @@ constexpr int CH = 32;                 // keys whose scores one load brings
 constexpr int kThreads = 384;          // warps 0-3 and 4-7: the slots' softmax; 8: TMA producer; 9: MMA issuer; 10 reports; 11 asks ahead
 // Registers per thread: the launch's 168 cannot hold a row's 128 scores and the rest of a softmax
 // thread, so the third warpgroup's go to the first two while the roles work (256 x 216 + 128 x 72 =
-// 384 x 168; 4 x 64 nodes x 4096 keys, launch to launch: 28.0 -> 26.5 us).  (The variant with two threads per row
-// spills: -Xptxas -v reports 4 bytes stored and 20 loaded.)
+// 384 x 168; 4 x 64 nodes x 4096 keys, launch to launch: 28.0 -> 26.5 us).  No variant spills (-Xptxas -v).
 constexpr int kSoftmaxRegs = 216, kOtherRegs = 72, kLaunchRegs = 168;
 static_assert(2 * kSoftmaxRegs + kOtherRegs <= 3 * kLaunchRegs, "a block shares out the registers that it was launched with");
 constexpr int kSoftmaxWarps = 8, kProducer = 8, kIssuer = 9, kWriter = 10, kScout = 11;
