@@ -783,6 +783,7 @@ struct TallyWords {
   long long wait_limit, since = 0;
   __device__ __forceinline__ unsigned long long add(unsigned long long v) { return atomicAdd(tally, v); }
   __device__ __forceinline__ unsigned count() { return *reinterpret_cast<volatile unsigned*>(tally); }
+  __device__ __forceinline__ void clear() { *const_cast<volatile unsigned long long*>(tally) = 0ull; }
   __device__ __forceinline__ void put(int s) { *const_cast<volatile int32_t*>(status) = s; }
   __device__ __forceinline__ void fence() { __threadfence(); }
   __device__ __forceinline__ void correct() { atomicCAS(status, CLV_OK, CLV_ERR_TIMEOUT); }

@@ -35,6 +35,7 @@ struct Words {
     g_tasks[g_now].polls = false;
     return (unsigned)g_word;
   }
+  void clear() { step(); g_word = 0; }
   void put(int s) { step(); g_status = s; }
   void fence() {}
   void correct() { step(); if (g_status == CLV_OK) g_status = CLV_ERR_TIMEOUT; }
