@@ -393,10 +393,10 @@ ATTN_BOUND = {"C1": "hbm", "C2": "hbm", "C3": "hbm", "C4": "hbm", "C5": "tensor"
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from ncu captures of the library whose
 # clv_version() is the first element; a different library version reports null instead
 NCU_TRAFFIC = {
-    (116, "C1", "tree_attn"): 8.86e6, (116, "C2", "tree_attn"): 35.2e6, (116, "C3", "tree_attn"): 72.4e6,
-    (116, "C4", "tree_attn"): 522.1e6, (116, "C5", "tree_attn"): 1090.2e6,
-    (116, "C1", "accept_argmax"): 1.04e6, (116, "C2", "accept_argmax"): 4.11e6, (116, "C3", "accept_argmax"): 65.7e6,
-    (116, "C4", "accept_argmax"): 262.8e6, (116, "C5", "accept_argmax"): 262.7e6,
+    (117, "C1", "tree_attn"): 8.86e6, (117, "C2", "tree_attn"): 35.2e6, (117, "C3", "tree_attn"): 72.5e6,
+    (117, "C4", "tree_attn"): 522.8e6, (117, "C5", "tree_attn"): 1090.2e6,
+    (117, "C1", "accept_argmax"): 1.04e6, (117, "C2", "accept_argmax"): 4.11e6, (117, "C3", "accept_argmax"): 65.7e6,
+    (117, "C4", "accept_argmax"): 262.8e6, (117, "C5", "accept_argmax"): 262.8e6,
 }
 MIN_TIMED_MS = 200.0   # the --steps loop is repeated until this much has been timed
 

@@ -95,8 +95,8 @@ __device__ __forceinline__ float low(unsigned long long v) { return __uint_as_fl
 __device__ __forceinline__ float high(unsigned long long v) { return __uint_as_float((uint32_t)(v >> 32)); }
 
 // A batch of kUnroll vectors at once: one maximum and at most one rescale for the 32 values, then
-// their exponentials into four running sums (no long chain of dependent additions).  Beside the stream this is bound by
-// its instructions, so the maximum is taken of packed bf16 (a positive factor does not change which it is, and the
+// their exponentials into four running sums (no long chain of dependent additions).  Beside the stream (DRAM 65 %) it is
+// the issue slots, 61 % of the active cycles, and the exponentials, two thirds of theirs, that set the pace, so the maximum is taken of packed bf16 (a positive factor does not change which it is, and the
 // maximum with -inf drops a NaN, which carries no mass), and products, differences and sums are packed fp32 (statistics and walk of
 // 16 x 64 rows of 128256 64.3 -> 59.2 us, of 5 x 27 of 50257 11.8 -> 10.7 with the walk's changes).
 __device__ __forceinline__ void stat_take_batch(Stat& st, uint4 (&w)[kUnroll], float k) {
